@@ -29,9 +29,10 @@ namespace gdn {
 //                                          a word that says for which shape the plan was built (plan_magic)
 //   unit_list uint32[..][4]                one record per group, the groups of a tree next to one another, the trees
 //                                          in the order in which their plan CTAs got there: (tree, first row of the
-//                                          tree, first position | own nodes << 16, n_prefix | node at the first
-//                                          position << 16).  A tree of at most 64 nodes is its own single group
-//                                          (., ., T << 16, 0xFFFF): identity numbering, tables in depth / anc8.  The
+//                                          tree, first position | own nodes << 16 | k << 24 of the tree's k-th group,
+//                                          n_prefix | groups of the tree << 8 | node at the first position << 16).  A
+//                                          tree of at most 64 nodes is its own single group (., ., T << 16,
+//                                          0xFF | 1 << 8): identity numbering, tables in depth / anc8.  The
 //                                          tensor-core verify kernel walks this list, so that its units are real
 //                                          groups only and spread evenly over the CTAs whatever the tree sizes.
 //   dfs_node  uint16[N]                    node id at position r

@@ -118,13 +118,13 @@ __device__ __forceinline__ void plan_tree(const PlanArgs &a, const int b)
     if (threadIdx.x == 0) tree_ok[b] = any_err ? 0 : 1;
     if (any_err || !grouped) {
         // a tree that fits one tile is its own single group with the identity numbering, marked by n_prefix =
-        // 0xFFFF (no group at all if the tree was rejected or is empty)
+        // 0xFF (no group at all if the tree was rejected or is empty)
         // (a call with a single tree keeps the count itself; otherwise the counter was zeroed in front of this grid)
         const bool one = !any_err && T > 0 && T <= GDN_GROUP_TILE;
         if (threadIdx.x == 0 && n_seq == 1) *unit_count = one ? 1 : 0;
         if (threadIdx.x == 0 && one)
             unit_list[n_seq == 1 ? 0 : atomicAdd(unit_count, 1)] =
-                make_uint4((uint32_t)b, (uint32_t)lo, (uint32_t)T << 16, 0xFFFFu);
+                make_uint4((uint32_t)b, (uint32_t)lo, (uint32_t)T << 16, 0xFFu | (1u << 8));
         return;
     }
 
@@ -171,7 +171,7 @@ __device__ __forceinline__ void plan_tree(const PlanArgs &a, const int b)
     for (int k = threadIdx.x; k <= GDN_MAX_GROUPS; k += PLAN_THREADS)
         group_start[(size_t)b * (GDN_MAX_GROUPS + 1) + k] = gstart_s[k];
     // one record per group in the unit list, the groups of this tree next to one another
-    __shared__ int list_base_s;
+    __shared__ int list_base_s, n_groups_s;
     if (threadIdx.x == 0) {
         int n_groups = 0;
         while (n_groups < GDN_MAX_GROUPS && gstart_s[n_groups] < T) ++n_groups;
@@ -181,13 +181,15 @@ __device__ __forceinline__ void plan_tree(const PlanArgs &a, const int b)
         } else {
             list_base_s = atomicAdd(unit_count, n_groups);
         }
+        n_groups_s = n_groups;
     }
     __syncthreads();
     for (int k = threadIdx.x; k < GDN_MAX_GROUPS; k += PLAN_THREADS) {
         const int g0 = gstart_s[k], own = gstart_s[k + 1] - g0;
-        if (own > 0)   // (first position, own nodes), (n_prefix, node at the first position)
-            unit_list[list_base_s + k] = make_uint4((uint32_t)b, (uint32_t)lo, (uint32_t)g0 | ((uint32_t)own << 16),
-                                                    (uint32_t)(depth_at_s[g0] - 1) | ((uint32_t)dfs_node[lo + g0] << 16));
+        if (own > 0)   // (first position, own nodes, k), (n_prefix, groups of the tree, node at the first position)
+            unit_list[list_base_s + k] =
+                make_uint4((uint32_t)b, (uint32_t)lo, (uint32_t)g0 | ((uint32_t)own << 16) | ((uint32_t)k << 24),
+                           (uint32_t)(depth_at_s[g0] - 1) | ((uint32_t)n_groups_s << 8) | ((uint32_t)dfs_node[lo + g0] << 16));
     }
     // Root path of every node in the virtual indices of its group: an ancestor before the group's first
     // position is an ancestor of the group's first node and gets index depth-1; one inside the group gets
