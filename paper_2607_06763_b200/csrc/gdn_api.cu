@@ -180,7 +180,10 @@ extern "C" int gdn_tree_verify(const gdn_shape_t *shape, const float *S0, const 
     const WorkspaceLayout lay = workspace_layout(s);
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const PlanPtrs plan = plan_ptrs(workspace, lay);
-    // trees of at most 64 nodes on the tensor-core path: that kernel builds the tree metadata itself
+    // trees of at most 64 nodes: the kernels build the tree metadata themselves
+    if (!verify_sm100_supported(s) && verify_generic_small_supported(s))
+        return launch_verify_generic_small(s, S0, q, k, v, g, beta, parent, node_offsets, o, status_dev, stream) == cudaSuccess
+                   ? GDN_OK : GDN_ERR_CUDA;
     if (!verify_sm100_single_group(s) &&
         launch_plan(s, parent, node_offsets, nullptr, plan, status_dev, stream) != cudaSuccess)
         return GDN_ERR_CUDA;

@@ -116,6 +116,12 @@ cudaError_t launch_verify_generic(const gdn_shape_t &s, const float *S0, const v
                                   const int32_t *node_offsets, void *o, const PlanPtrs &plan,
                                   cudaStream_t stream);
 
+// The same for trees of at most 64 nodes, which need no plan: the metadata is derived from parent[] on chip.
+bool verify_generic_small_supported(const gdn_shape_t &s);
+cudaError_t launch_verify_generic_small(const gdn_shape_t &s, const float *S0, const void *q, const void *k,
+                                        const void *v, const void *g, const void *beta, const int32_t *parent,
+                                        const int32_t *node_offsets, void *o, int32_t *status_dev, cudaStream_t stream);
+
 // Tensor-core fast path (d_k = d_v = 128, bf16 inputs, trees <= 64 nodes, root paths <= 16 nodes).
 bool verify_sm100_supported(const gdn_shape_t &s);
 bool verify_sm100_single_group(const gdn_shape_t &s);   // every tree fits one CTA (<= 64 nodes): fusable with commit

@@ -176,6 +176,302 @@ __global__ void __launch_bounds__(VG_THREADS, 1) verify_generic_kernel(const Ver
     }
 }
 
+// ---------------------------------------------------------------------------------------- trees of at most 64 nodes
+// The same triangular form with the solve moved to the query side, so that no node waits for another one.  With
+// X(l, t) = beta_l dec(l, t) (k_l.k_t) and y_it = dec(i, t) (q_i.k_t) along the root path of node i, row i of
+// Z = Y (I + X)^-1 is a back-substitution over that path alone, and
+//     o_i = S0^T q'_i + sum_t scale z_it beta_t v_t,      q'_i = scale (a_i q_i - sum_t z_it beta_t a_t k_t).
+// One CTA per (tree, value head, block of VS_NODES nodes); the tree metadata is derived from parent[] by every CTA (64
+// nodes: a walk of at most max_depth steps per thread), so no plan kernel runs in front.  Bound by FMA issue in the state
+// product (two rows of 32 key positions per thread against one read of q': 64 FMA per 8 shared-memory loads) and by
+// latency for small batches.  Against the kernel above, which visits the nodes of a tree one after the other: 8 trees of
+// 9..64 nodes, 32 heads of 128 components, fp32, verification and commit
+// 228 -> 79 us (the commit is 15 of them); one tree of 8 nodes, 4 heads of 32 components 26.6 -> 17.0 us.
+constexpr int VS_THREADS = 256;
+constexpr int VS_TREE = 64;      // largest tree
+constexpr int VS_NODES = 16;     // nodes per CTA
+constexpr int VS_SPLIT = 4;      // lanes sharing two value components
+
+struct VerifySmallParams {
+    int h_qk, h_v, d_k, d_v, max_depth, max_tree_nodes, total_nodes, n_seq, n_blocks;
+    float scale;
+    const float *S0;
+    const void *q, *k, *v, *g, *beta;
+    const int32_t *parent, *node_offsets;
+    void *o;
+    int32_t *status_dev;
+};
+
+template <typename T> __device__ __forceinline__ float4 load4_as_float(const T *p);
+template <> __device__ __forceinline__ float4 load4_as_float<float>(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
+template <> __device__ __forceinline__ float4 load4_as_float<__nv_bfloat16>(const __nv_bfloat16 *p)
+{
+    const uint2 w = __ldg(reinterpret_cast<const uint2 *>(p));
+    return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xFFFF0000u), __uint_as_float(w.y << 16),
+                       __uint_as_float(w.y & 0xFFFF0000u));
+}
+
+struct VerifySmallSmem {
+    float ks[VS_TREE][VG_DK];              // k rows of the nodes this block needs
+    float qp[VS_NODES][VG_DK];             // q'
+    float x[VS_TREE][VS_TREE];             // decays, then X(l, .): entry j belongs to the j-th node up the root path of l
+    float y[VS_NODES][VS_TREE];            // y, then the weights of the k rows; same order
+    float zv[VS_NODES][VS_TREE];           // weights of the v rows
+    float a[VS_TREE], beta[VS_TREE], g[VS_TREE];
+    unsigned long long mask[VS_TREE];      // nodes on the root path
+    int par[VS_TREE];
+    uint8_t up[VS_TREE][VS_TREE];          // j-th node up the root path (0 = the node itself)
+    uint8_t depth[VS_TREE];
+};
+
+template <typename TIn, typename TOut>
+__global__ void __launch_bounds__(VS_THREADS, 2) verify_generic_small_kernel(const VerifySmallParams p)
+{
+    extern __shared__ __align__(16) uint8_t vs_smem[];
+    VerifySmallSmem &sm = *reinterpret_cast<VerifySmallSmem *>(vs_smem);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int blk = blockIdx.x % p.n_blocks, bh = blockIdx.x / p.n_blocks, b = bh / p.h_v, h = bh % p.h_v;
+    const int hk = h / (p.h_v / p.h_qk), i0 = blk * VS_NODES;
+    const int d_k = p.d_k, d_v = p.d_v;
+    const TIn *q = static_cast<const TIn *>(p.q), *k = static_cast<const TIn *>(p.k);
+    const TIn *v = static_cast<const TIn *>(p.v), *g = static_cast<const TIn *>(p.g), *beta = static_cast<const TIn *>(p.beta);
+    TOut *o = static_cast<TOut *>(p.o);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+
+    const int base = p.node_offsets[b], end = p.node_offsets[b + 1], T = end - base;
+    bool offsets_ok = base >= 0 && T >= 0 && T <= p.max_tree_nodes && T <= VS_TREE && end <= p.total_nodes;
+    if (b == 0) offsets_ok = offsets_ok && base == 0;
+    if (b == p.n_seq - 1) offsets_ok = offsets_ok && end == p.total_nodes;
+    if (!offsets_ok) {
+        if (tid == 0) report_status(p.status_dev, GDN_ERR_TREE);
+        return;
+    }
+    if (i0 >= T) return;
+    if (tid < T) {
+        sm.par[tid] = p.parent[base + tid];
+        sm.g[tid] = load_as_float(g + (size_t)(base + tid) * p.h_v + h);
+        sm.beta[tid] = load_as_float(beta + (size_t)(base + tid) * p.h_v + h);
+    }
+    // State slice: rows c, c + 1; sreg[r][8 m + e] holds key position 16 j + 4 s + e, m = j / 2 (zero beyond d_k / d_v).
+    const int c = (tid / VS_SPLIT) * 2, s = tid % VS_SPLIT;
+    float2 sreg[2][VG_DK / VS_SPLIT / 2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const float *row = p.S0 + ((size_t)(b * p.h_v + h) * d_v + (c + r < d_v ? c + r : 0)) * d_k;
+#pragma unroll
+        for (int j = 0; j < VG_DK / 16; ++j) {
+            const int at = 16 * j + 4 * s;
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (c + r < d_v && at < d_k) x = __ldg(reinterpret_cast<const float4 *>(row + at));
+            sreg[r][2 * j] = make_float2(x.x, x.y);
+            sreg[r][2 * j + 1] = make_float2(x.z, x.w);
+        }
+    }
+    __syncthreads();
+
+    // Root paths, by one thread per node; decays as sums of g from the ancestor's child down to the node, so that no large
+    // exponents cancel.  A bad parent[] or a path of more than max_depth nodes rejects the tree.
+    int err = 0;
+    if (tid < T) {
+        int d = 0, cur = tid;
+        float sfx = 0.f;
+        unsigned long long m = 0;
+        while (cur >= 0) {
+            if (d == p.max_depth) { err = GDN_ERR_DEPTH; break; }
+            sm.up[tid][d] = (uint8_t)cur;
+            sm.x[tid][d] = expf(sfx);
+            m |= 1ull << cur;
+            sfx += sm.g[cur];
+            ++d;
+            const int up = sm.par[cur];
+            if (up < -1 || up >= cur) { err = GDN_ERR_TREE; break; }
+            cur = up;
+        }
+        sm.depth[tid] = (uint8_t)d;
+        sm.mask[tid] = m;
+        sm.a[tid] = expf(sfx);
+    }
+    if (err) report_status(p.status_dev, err);
+    if (__syncthreads_or(err != 0)) return;
+    const int nn = min(VS_NODES, T - i0);
+    unsigned long long need = 0;   // the block's nodes and their ancestors
+    for (int i = 0; i < nn; ++i) need |= sm.mask[i0 + i];
+    const int vecs = d_k / 4;
+    for (int idx = tid; idx < T * 32; idx += VS_THREADS) {
+        const int t = idx >> 5, r = idx & 31;
+        if (((need >> t) & 1) && r < vecs)
+            *reinterpret_cast<float4 *>(&sm.ks[t][4 * r]) = load4_as_float(k + ((size_t)(base + t) * p.h_qk + hk) * d_k + 4 * r);
+    }
+    __syncthreads();
+
+    // X and y: a warp per node, its lanes four key positions each
+    for (int l = warp; l < T; l += VS_THREADS / 32) {
+        if (!((need >> l) & 1)) continue;
+        const bool own = l >= i0 && l < i0 + nn;
+        float4 kl = make_float4(0.f, 0.f, 0.f, 0.f), ql = kl;
+        if (lane < vecs) {
+            kl = *reinterpret_cast<const float4 *>(&sm.ks[l][4 * lane]);
+            if (own) ql = load4_as_float(q + ((size_t)(base + l) * p.h_qk + hk) * d_k + 4 * lane);
+        }
+        const int d = sm.depth[l];
+        const float be = sm.beta[l];
+#pragma unroll 2
+        for (int j = own ? 0 : 1; j < d; ++j) {
+            float4 kt = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (lane < vecs) kt = *reinterpret_cast<const float4 *>(&sm.ks[sm.up[l][j]][4 * lane]);
+            float kk = fmaf(kl.x, kt.x, fmaf(kl.y, kt.y, fmaf(kl.z, kt.z, kl.w * kt.w)));
+            float qk = fmaf(ql.x, kt.x, fmaf(ql.y, kt.y, fmaf(ql.z, kt.z, ql.w * kt.w)));
+            // lanes 0..15 end up with kk, lanes 16..31 with qk
+            const float other = __shfl_xor_sync(0xffffffffu, lane & 16 ? kk : qk, 16);
+            float w = (lane & 16 ? qk : kk) + other;
+#pragma unroll
+            for (int m = 8; m > 0; m >>= 1) w += __shfl_xor_sync(0xffffffffu, w, m);
+            const float dec = sm.x[l][j];
+            __syncwarp();
+            if (lane == 0) sm.x[l][j] = be * dec * w;   // (entry 0, the node itself, is never read)
+            if (lane == 16 && own) sm.y[l - i0][j] = dec * w;
+        }
+    }
+    __syncthreads();
+
+    // z by back-substitution: 16 lanes per node, lane ln owning the entries ln, ln + 16, ... ; once z_j is final it is
+    // subtracted, times X(up_j, .), from the entries further up
+    {
+        const int i = tid >> 4, ln = tid & 15, n = i0 + i;
+        const int d = i < nn ? sm.depth[n] : 0;
+        const int d_warp = __reduce_max_sync(0xffffffffu, d);
+        float z[VS_TREE / 16];
+#pragma unroll
+        for (int e = 0; e < VS_TREE / 16; ++e) z[e] = ln + 16 * e < d ? sm.y[i][ln + 16 * e] : 0.f;
+#pragma unroll
+        for (int e = 0; e < VS_TREE / 16; ++e) {
+            if (16 * e >= d_warp - 1) break;
+#pragma unroll 1
+            for (int l = 0; l < 16; ++l) {
+                const int j = 16 * e + l;
+                if (j >= d_warp - 1) break;
+                const float zj = __shfl_sync(0xffffffffu, z[e], (lane & 16) | l);
+                if (j < d - 1) {
+                    const float *xr = sm.x[sm.up[n][j]];
+#pragma unroll
+                    for (int f = e; f < VS_TREE / 16; ++f) {
+                        const int t = ln + 16 * f;
+                        if (t > j && t < d) z[f] = fmaf(-zj, xr[t - j], z[f]);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < VS_TREE / 16; ++e) {
+            const int t = ln + 16 * e;
+            if (t < d) {
+                const int m = sm.up[n][t];
+                const float w = p.scale * z[e] * sm.beta[m];
+                sm.zv[i][t] = w;
+                sm.y[i][t] = w * sm.a[m];
+            }
+        }
+    }
+    __syncthreads();
+
+    // q': 16 lanes per node, eight key positions each
+    {
+        const int i = tid >> 4, ln = tid & 15, n = i0 + i;
+        if (i < nn) {
+            const int d = sm.depth[n];
+            const float sa = p.scale * sm.a[n];
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                const int r = half * 64 + ln * 4;
+                float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (r < d_k) {
+                    w = load4_as_float(q + ((size_t)(base + n) * p.h_qk + hk) * d_k + r);
+                    w = make_float4(sa * w.x, sa * w.y, sa * w.z, sa * w.w);
+                    for (int t = 0; t < d; ++t) {
+                        const float cf = -sm.y[i][t];
+                        const float4 kt = *reinterpret_cast<const float4 *>(&sm.ks[sm.up[n][t]][r]);
+                        w = make_float4(fmaf(cf, kt.x, w.x), fmaf(cf, kt.y, w.y), fmaf(cf, kt.z, w.z), fmaf(cf, kt.w, w.w));
+                    }
+                }
+                *reinterpret_cast<float4 *>(&sm.qp[i][r]) = w;
+            }
+        }
+    }
+    __syncthreads();
+
+    // outputs, four nodes at a time: the four lanes of a row pair share key positions and path entries; the eight sums
+    // (four nodes x two rows) are folded into one another so that lane s ends up with those of node s
+#pragma unroll 1
+    for (int ib = 0; ib < nn; ib += 4) {
+        float acc[4][2];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = ib + u;
+            float2 s0 = make_float2(0.f, 0.f), s1 = s0;
+            if (i < nn) {
+#pragma unroll
+                for (int j = 0; j < VG_DK / 16; ++j) {
+                    const float4 x = *reinterpret_cast<const float4 *>(&sm.qp[i][16 * j + 4 * s]);
+                    s0 = __ffma2_rn(sreg[0][2 * j], make_float2(x.x, x.y), s0);
+                    s1 = __ffma2_rn(sreg[1][2 * j], make_float2(x.x, x.y), s1);
+                    s0 = __ffma2_rn(sreg[0][2 * j + 1], make_float2(x.z, x.w), s0);
+                    s1 = __ffma2_rn(sreg[1][2 * j + 1], make_float2(x.z, x.w), s1);
+                }
+                const int d = sm.depth[i0 + i];
+                if (c < d_v) {
+                    const int c1 = c + 1 < d_v ? c + 1 : c;
+#pragma unroll 2
+                    for (int t = s; t < d; t += VS_SPLIT) {
+                        const TIn *vr = v + ((size_t)(base + sm.up[i0 + i][t]) * p.h_v + h) * d_v;
+                        const float w = sm.zv[i][t];
+                        s0.x = fmaf(w, load_as_float(vr + c), s0.x);
+                        s1.x = fmaf(w, load_as_float(vr + c1), s1.x);
+                    }
+                }
+            }
+            acc[u][0] = s0.x + s0.y;
+            acc[u][1] = s1.x + s1.y;
+        }
+        float half_sum[2][2], out[2];
+        const bool odd = (s & 1) != 0, high = (s & 2) != 0;
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int r = 0; r < 2; ++r)   // keep nodes u * 2 + (s & 1)
+                half_sum[u][r] = (odd ? acc[2 * u + 1][r] : acc[2 * u][r]) +
+                                 __shfl_xor_sync(0xffffffffu, odd ? acc[2 * u][r] : acc[2 * u + 1][r], 1);
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+            out[r] = (high ? half_sum[1][r] : half_sum[0][r]) + __shfl_xor_sync(0xffffffffu, high ? half_sum[0][r] : half_sum[1][r], 2);
+        if (ib + s < nn) {
+            TOut *dst = o + ((size_t)(base + i0 + ib + s) * p.h_v + h) * d_v + c;
+            if (c < d_v) store_from_float(dst, out[0]);
+            if (c + 1 < d_v) store_from_float(dst + 1, out[1]);
+        }
+    }
+}
+
+template <typename TIn, typename TOut>
+cudaError_t launch_small_typed(const VerifySmallParams &p, cudaStream_t stream)
+{
+    const int grid = p.n_seq * p.h_v * p.n_blocks;
+    cudaError_t e = cudaFuncSetAttribute(verify_generic_small_kernel<TIn, TOut>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(VerifySmallSmem));
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(VS_THREADS);
+    cfg.dynamicSmemBytes = sizeof(VerifySmallSmem);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, verify_generic_small_kernel<TIn, TOut>, p);
+}
+
 template <typename TIn, typename TOut>
 cudaError_t launch_typed(const gdn_shape_t &s, const VerifyGenericParams &p, cudaStream_t stream)
 {
@@ -190,6 +486,28 @@ cudaError_t launch_typed(const gdn_shape_t &s, const VerifyGenericParams &p, cud
 }
 
 }  // namespace
+
+// The grid has (tree, head, block) CTAs whatever the tree sizes: blocks beyond a tree return at once.
+bool verify_generic_small_supported(const gdn_shape_t &s)
+{
+    return s.max_tree_nodes <= VS_TREE &&
+           (long long)s.n_seq * s.h_v * ((s.max_tree_nodes + VS_NODES - 1) / VS_NODES) <= 0x7fffffffLL;
+}
+
+cudaError_t launch_verify_generic_small(const gdn_shape_t &s, const float *S0, const void *q, const void *k,
+                                        const void *v, const void *g, const void *beta, const int32_t *parent,
+                                        const int32_t *node_offsets, void *o, int32_t *status_dev, cudaStream_t stream)
+{
+    if (s.n_seq == 0 || s.total_nodes == 0) return cudaSuccess;
+    const VerifySmallParams p{s.h_qk, s.h_v, s.d_k, s.d_v, s.max_depth, s.max_tree_nodes, s.total_nodes, s.n_seq,
+                              (s.max_tree_nodes + VS_NODES - 1) / VS_NODES, s.scale, S0, q, k, v, g, beta, parent,
+                              node_offsets, o, status_dev};
+    const bool in_bf = s.in_dtype == GDN_BF16, out_bf = s.out_dtype == GDN_BF16;
+    if (in_bf && out_bf) return launch_small_typed<__nv_bfloat16, __nv_bfloat16>(p, stream);
+    if (in_bf) return launch_small_typed<__nv_bfloat16, float>(p, stream);
+    if (out_bf) return launch_small_typed<float, __nv_bfloat16>(p, stream);
+    return launch_small_typed<float, float>(p, stream);
+}
 
 cudaError_t launch_verify_generic(const gdn_shape_t &s, const float *S0, const void *q, const void *k,
                                   const void *v, const void *g, const void *beta,

@@ -110,6 +110,25 @@ def test_edge_shapes(tl, name, dims):
     _check_full(tl, w, f"{name} {dims}")
 
 
+@pytest.mark.parametrize("dims", [(2, 6, 128, 127, synth.F32, synth.F32), (1, 2, 4, 1, synth.F32, synth.F32),
+                                  (2, 2, 100, 65, synth.BF16, synth.BF16)])
+def test_general_path_node_blocks(tl, dims):
+    """General path on trees around its block of 16 nodes, with root paths of up to 64 nodes (tolerance: fp32 sums)."""
+    h_qk, h_v, d_k, d_v, idt, odt = dims
+    rng = np.random.default_rng(71)
+    trees = [synth.tree_geo(rng, T) for T in (1, 15, 16, 17, 33, 63)] + [synth.tree_chain(64)]
+    _check_full(tl, synth.random_case(72, trees, h_qk, h_v, d_k, d_v, idt, odt), f"blocks {dims}", max_depth=64)
+
+
+@pytest.mark.parametrize("out_dtype", [synth.BF16, synth.F32])
+@pytest.mark.parametrize("sizes", [(1, 15, 16, 17, 31, 32, 33, 48, 63, 64), (65, 113, 128, 200, 40)])
+def test_verify_shares_rows_and_state_between_units(tl, sizes, out_dtype):
+    """Tree sizes around the 16-node pieces and the 64-node unit, three value heads per key head."""
+    rng = np.random.default_rng(73)
+    w = synth.random_case(74, [synth.tree_geo(rng, T) for T in sizes], 3, 9, 128, 128, synth.BF16, out_dtype)
+    _check_full(tl, w, f"sizes {sizes}")
+
+
 def test_deep_chain_needs_larger_max_depth(tl):
     w = synth.random_case(5, [synth.tree_chain(40)], 1, 2, 64, 64, synth.F32, synth.F32,
                           paths=[np.arange(40, dtype=np.int32)])
