@@ -11,9 +11,11 @@
 // are fetched once into shared memory; the state is read once and written once.  The state loads
 // are issued before anything else so that the path checks and the k-row staging run under their
 // latency, and the kernel keeps to 64 registers so that two CTAs (32 warps) share an SM.
+#include <atomic>
+
+#include "gdn_fragments.cuh"
 #include "gdn_internal.cuh"
 #include "gdn_plan.cuh"
-#include "gdn_replay.cuh"
 
 namespace gdn {
 
@@ -174,10 +176,16 @@ __global__ void __launch_bounds__(CM_THREADS, 2) commit_generic_kernel(const Com
     }
 }
 
-// Fast form for d_k = d_v = 128, bf16 inputs, paths of at most 16 nodes: 256 threads hold the tile as the
-// tensor-core verify kernel does (eight lanes per row, 32-byte accesses) and replay the path in the scaled form
-// (gdn_replay.cuh).  One CTA per (tree, value head), two CTAs per SM; the state loads go first, the path is fetched
-// and checked by one warp with shuffles, its k/v rows arrive by cp.async.
+// Fast forms for d_k = d_v = 128, bf16 inputs, paths of at most 16 nodes: one CTA of 256 threads per (tree, value head);
+// the state loads go first, the path is fetched and checked by one warp with shuffles, its k/v rows arrive by cp.async.
+// Two forms of the arithmetic, chosen by how many CTAs the call has for how many SMs (commit_form):
+//   step by step (commit_replay_unit): 64 state registers per thread, two CTAs per SM; the shortest chain, the better one
+//     while all CTAs of the call are resident at once that way;
+//   as matrix products (commit_fragment_unit, gdn_fragments.cuh): 32 state registers, the tile read twice, the second time
+//     out of L2; three or four CTAs per SM, so that the loads of some run under the arithmetic of others.
+// Measured (us; 32 heads per slot, path of 7; two by two / three / four per SM): 4 slots 8.2 / 8.9 / 9.3, 8 slots 10.6 /
+// 13.3 / 12.7, 12 slots 16.6 / 13.4 / 16.0, 14 slots 18.4 / 18.4 / 16.6, 32 slots 36.2 / 33.9 / 31.1, 48 slots 49.5 /
+// 45.8 / 43.0 (path of 12: 56.8 / 50.7 / 49.1; HBM alone: 31).
 constexpr int CF_THREADS = 256;
 constexpr int CF_MD = 16;
 
@@ -185,8 +193,13 @@ __device__ __forceinline__ void cf_cp_async_16(uint32_t dst, const void *src)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
+__device__ __forceinline__ void cf_cp_async_4(uint32_t dst, const void *src, bool valid)   // zero-fills where not valid
+{
+    const int n = valid ? 4 : 0;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+}
 
-__device__ __forceinline__ void commit_tile128_unit(const CommitParams &p, const int unit)
+__device__ __forceinline__ void commit_replay_unit(const CommitParams &p, const int unit)
 {
     __shared__ __align__(16) uint16_t pk_s[CF_MD * GDN_TILE_D];
     __shared__ __align__(16) uint16_t pv_s[CF_MD * GDN_TILE_D];
@@ -292,22 +305,176 @@ __device__ __forceinline__ void commit_tile128_unit(const CommitParams &p, const
     }
 }
 
-__global__ void __launch_bounds__(CF_THREADS, 2) commit_tile128_kernel(const CommitParams p)
+__device__ __forceinline__ void commit_fragment_unit(const CommitParams &p, const int unit)
 {
-    commit_tile128_unit(p, (int)blockIdx.x);
+    __shared__ __align__(16) uint8_t pk_s[CF_MD * GDN_PK_STRIDE];
+    __shared__ __align__(16) uint16_t pv_s[CF_MD * GDN_TILE_D];
+    __shared__ __align__(16) float couple_s[CF_MD * 16];
+    __shared__ __align__(16) float4 scal_s[CF_MD];
+    __shared__ int len_s;
+    __shared__ float decay_s;
+
+    const int b = unit / p.h_v, h = unit % p.h_v;
+    const int hk = h / (p.h_v / p.h_qk);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid < 4)   // L2 may be asked for the tile meanwhile (a prefetch consumes nothing)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;"
+                     ::"l"(p.S + (size_t)unit * GDN_TILE_D * GDN_TILE_D + (size_t)tid * 4096), "r"(16384) : "memory");
+    wait_for_previous_kernel();
+    const int tree = p.t_pad ? b % p.n_trees : b;
+    const int pp0 = p.t_pad ? tree * p.path_stride : p.path_offsets[b];
+    int len = p.t_pad ? p.path_len[tree] : p.path_offsets[b + 1] - pp0;
+    if (len == 0) return;   // nothing accepted from this tree: state untouched
+
+    // the state first: its latency covers the path fetch below
+    const int row = warp * 16 + (lane >> 2);
+    float *S = p.S + (size_t)unit * GDN_TILE_D * GDN_TILE_D + (size_t)row * GDN_TILE_D + (lane & 3) * 8;
+    float x[2][4][4];
+    load_chunk(S, 0, x[0]);
+    load_chunk(S, 1, x[1]);
+
+    const int pb = p.t_pad ? b * p.t_pad : p.node_offsets[b];
+    const int pT = p.t_pad ? min(p.n_nodes[tree], p.t_pad) : p.node_offsets[b + 1] - pb;
+    const __nv_bfloat16 *k = static_cast<const __nv_bfloat16 *>(p.k), *v = static_cast<const __nv_bfloat16 *>(p.v);
+    const bool shape_ok = len > 0 && len <= CF_MD && len <= p.max_depth && pT > 0 && pp0 >= 0;
+    const uint32_t pk = (uint32_t)__cvta_generic_to_shared(pk_s);
+    // Every thread reads the path entry whose row piece it fetches (no hand-over through shared memory in front of the
+    // row fetch); an entry outside the tree is skipped here and reported by the check below.  k rows word by word into the
+    // fragment order, zero up to the next multiple of eight rows.
+    if (shape_ok) {
+#pragma unroll 2
+        for (int idx = tid; idx < ((len + 7) & ~7) * 64; idx += CF_THREADS) {
+            const int t = idx >> 6, w = idx & 63;
+            int nt = t < len ? p.path[pp0 + t] : 0;
+            const bool valid = t < len && nt >= 0 && nt < pT;
+            if (!valid) nt = 0;
+            cf_cp_async_4(pk + t * GDN_PK_STRIDE + path_row_word(w), k + ((size_t)(pb + nt) * p.h_qk + hk) * GDN_TILE_D + w * 2, valid);
+        }
+        if (tid < len * 16) {
+            const int t = tid >> 4, c16 = tid & 15, nt = p.path[pp0 + t];
+            if (nt >= 0 && nt < pT)
+                cf_cp_async_16((uint32_t)__cvta_generic_to_shared(pv_s + t * GDN_TILE_D + c16 * 8),
+                               v + ((size_t)(pb + nt) * p.h_v + h) * GDN_TILE_D + c16 * 8);
+        }
+    }
+    float G = 0.f, be = 0.f;   // of step `lane` (warp 0)
+    if (warp == 0) {
+        // lane t: entry t of the path and that node's parent; the path must be a chain from a root inside the tree
+        const int ppar = p.t_pad ? tree * p.t_pad : pb;   // first entry of the tree in parent[]
+        const bool mine = shape_ok && lane < len;
+        int n = -1, parent_n = -2;
+        if (mine) {
+            n = p.path[pp0 + lane];
+            if (n >= 0 && n < pT) {
+                if (p.parent) parent_n = p.parent[ppar + n];
+                const size_t i = (size_t)(pb + n) * p.h_v + h;
+                G = gate_log_decay(static_cast<const unsigned short *>(p.g)[i], p.raw_gates != 0);
+                be = gate_beta(static_cast<const unsigned short *>(p.beta)[i], p.raw_gates != 0);
+            }
+        }
+        const int n_up = __shfl_up_sync(0xffffffffu, n, 1);
+        bool bad = false;
+        if (mine) {
+            if (n < 0 || n >= pT) bad = true;
+            else if (p.parent) bad = parent_n != (lane ? n_up : -1);
+            else if (lane && n <= n_up) bad = true;   // without parent[] only the topological order can be checked
+        }
+        if (__any_sync(0xffffffffu, bad) || !shape_ok) {
+            if (lane == 0) report_status(p.status_dev, GDN_ERR_PATH);
+            len = 0;
+        }
+        // sums of g along the path over the lanes, and the per-step scalars
+#pragma unroll
+        for (int off = 1; off < CF_MD; off <<= 1) {
+            const float up = __shfl_up_sync(0xffffffffu, G, off);
+            if (lane >= off) G += up;
+        }
+        const float G_L = __shfl_sync(0xffffffffu, G, max(len - 1, 0));
+        if (lane < len) scal_s[lane] = make_float4(be, be * expf(G), expf(G_L - G), 0.f);
+        if (lane == 0) {
+            len_s = len;
+            decay_s = expf(G_L);
+        }
+    }
+    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    len = len_s;
+    if (len == 0) return;   // rejected path: this state stays as it was
+    const bool two = len > 8;
+    const uint32_t operand = path_operand(pk, lane);
+    if (warp == 0 && len > 1) path_coupling(pk, len, G, be, couple_s, lane);
+    PathUpdate up;
+    {
+        PathProducts a;
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) a.z[i][e] = a.rest[i][e] = 0.f;
+#pragma unroll 1
+        for (int j = 0; j < 4; j += 2)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                path_products_chunk(x[i], j + i, two, operand, a);
+                load_chunk(S, (j + i + 2) & 3, x[i]);   // (the first two again, for the update)
+            }
+        __syncthreads();   // the coupling table
+        path_solve(a, len, PathTile{pv_s, scal_s, couple_s}, row, lane, up);
+    }
+    const float A_L = decay_s;
+#pragma unroll 1
+    for (int j = 0; j < 4; j += 2)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            path_update_chunk(x[i], j + i, two, operand, A_L, up);
+            store_chunk(S, j + i, x[i]);
+            if (j == 0) load_chunk(S, i + 2, x[i]);
+        }
+}
+
+// CTAS: CTAs per SM (2: step by step, otherwise as matrix products)
+template <int CTAS> __device__ __forceinline__ void commit_unit(const CommitParams &p, const int unit)
+{
+    if constexpr (CTAS == 2) commit_replay_unit(p, unit);
+    else commit_fragment_unit(p, unit);
+}
+
+template <int CTAS> __global__ void __launch_bounds__(CF_THREADS, CTAS) commit_tile128_kernel(const CommitParams p)
+{
+    commit_unit<CTAS>(p, (int)blockIdx.x);
 }
 
 // The fused call on trees of more than 64 nodes: the plans of the NEW trees do not depend on the commit of the previous
 // step's paths, so they are built by the first n_seq CTAs of the same grid instead of by a launch of their own in
 // between (one launch and one dependency hop less in front of the verify kernel).
 static_assert(PLAN_THREADS == CF_THREADS, "the plan CTAs and the commit CTAs share a block size");
-__global__ void __launch_bounds__(CF_THREADS, 2) commit_plan_kernel(const CommitParams p, const PlanArgs a)
+template <int CTAS> __global__ void __launch_bounds__(CF_THREADS, CTAS) commit_plan_kernel(const CommitParams p, const PlanArgs a)
 {
     if ((int)blockIdx.x < a.n_seq) {
         wait_for_previous_kernel();
         plan_tree(a, (int)blockIdx.x);
     } else
-        commit_tile128_unit(p, (int)blockIdx.x - a.n_seq);
+        commit_unit<CTAS>(p, (int)blockIdx.x - a.n_seq);
+}
+
+// CTAs per SM for a call of `units` tiles: the fewest with which they are all resident at once.
+int commit_form(int units)
+{
+    static std::atomic<int> sm_count[64];
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 2;
+    if (dev < 64) sms = sm_count[dev].load(std::memory_order_relaxed);
+    if (sms == 0) {
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 2;
+        if (dev < 64) sm_count[dev].store(sms, std::memory_order_relaxed);
+    }
+    return units <= 2 * sms ? 2 : units <= 3 * sms ? 3 : 4;
+}
+
+cudaError_t launch_tile128(const CommitParams &p, int units, cudaStream_t stream)
+{
+    const int form = commit_form(units);
+    return launch_overlapped(form == 2 ? commit_tile128_kernel<2> : form == 3 ? commit_tile128_kernel<3> : commit_tile128_kernel<4>,
+                             units, CF_THREADS, 0, stream, p);
 }
 
 }  // namespace
@@ -322,7 +489,7 @@ cudaError_t launch_commit_generic(const gdn_shape_t &s, float *S, const void *k,
     CommitParams p{s.h_qk, s.h_v, s.d_k, s.d_v, s.max_depth, S, k, v, g, beta,
                    parent, node_offsets, path, path_offsets, status_dev, 0, 0, 0, 0, nullptr, nullptr};
     if (s.d_k == GDN_TILE_D && s.d_v == GDN_TILE_D && s.in_dtype == GDN_BF16 && s.max_depth <= CF_MD)
-        return launch_overlapped(commit_tile128_kernel, grid, CF_THREADS, 0, stream, p);
+        return launch_tile128(p, grid, stream);
     const size_t smem = sizeof(float) * ((size_t)s.max_depth * CM_DK + 4 * (size_t)s.max_depth);
     cudaError_t e;
     if (s.in_dtype == GDN_BF16) {
@@ -354,9 +521,9 @@ cudaError_t launch_commit_plan(const gdn_shape_t &s, float *S, const void *k, co
     }
     CommitParams p{s.h_qk, s.h_v, s.d_k, s.d_v, s.max_depth, S, k, v, g, beta, parent_prev, node_offsets_prev, path,
                    path_offsets, status_dev, 0, 0, 0, 0, nullptr, nullptr};
-    const int grid = s.n_seq + s.n_seq * s.h_v;
-    return launch_overlapped(commit_plan_kernel, grid, CF_THREADS, 0, stream, p,
-                             plan_args(s, parent, node_offsets, nullptr, plan, status_dev));
+    const int grid = s.n_seq + s.n_seq * s.h_v, form = commit_form(s.n_seq * s.h_v);
+    return launch_overlapped(form == 2 ? commit_plan_kernel<2> : form == 3 ? commit_plan_kernel<3> : commit_plan_kernel<4>, grid,
+                             CF_THREADS, 0, stream, p, plan_args(s, parent, node_offsets, nullptr, plan, status_dev));
 }
 
 bool commit_padded_supported(const gdn_shape_t &s)
@@ -373,7 +540,7 @@ cudaError_t launch_commit_padded(const gdn_shape_t &s, int n_trees, bool raw_gat
     if (grid == 0) return cudaSuccess;
     CommitParams p{s.h_qk, s.h_v, s.d_k, s.d_v, s.max_depth, S, k, v, g, beta, parent, nullptr, path, nullptr,
                    status_dev, s.max_tree_nodes, n_trees, s.max_depth, raw_gates ? 1 : 0, n_nodes, path_len};
-    return launch_overlapped(commit_tile128_kernel, grid, CF_THREADS, 0, stream, p);
+    return launch_tile128(p, grid, stream);
 }
 
 }  // namespace gdn

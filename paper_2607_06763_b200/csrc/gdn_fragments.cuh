@@ -1,0 +1,233 @@
+// The commit (Eq. 7 along an accepted path, the delayed commit of Section 3.4) on a 128 x 128 fp32 state tile taken
+// through registers as accumulator fragments of the warp-level tensor-core instruction m16n8k16, so that both halves of
+// the work -- the products k_t.s of every step with the old state, and the rank-L update -- are matrix products on the
+// registers as they are.  Against the step-by-step replay (gdn_replay.cuh) the work per tile hardly grows with the length
+// of the path: 0.45 K + 0.09 K per step instead of 0.68 K per step cycles with two tiles per SM (7 steps: 4.0 K against
+// 4.8 K, 16 steps: 6.0 K against 10.5 K), and a tile needs 32 registers per thread instead of 64.
+//
+// Thread layout: a warp owns 16 rows (rows = value components, contiguous in memory along the key dimension), taken in
+// four chunks of 32 key positions; lane = 4 g + l4 holds of rows g and g + 8 the key positions 32 jj + 8 l4 + e (e = 0..7)
+// of chunk jj: x[e >> 1][2 r + (e & 1)] for row g + 8 r, i.e. 32 contiguous bytes per lane and row.  As a fragment, x[n]
+// is the n-th 16 x 8 tile of the chunk in a permuted column order (column 2 l4 + (e & 1) of tile e >> 1); the other operand
+// of every product, the path's k rows in shared memory, is stored in that order (path_row_word).
+#pragma once
+
+#include <cuda_bf16.h>
+#include <stdint.h>
+
+#include "gdn_replay.cuh"
+
+namespace gdn {
+
+constexpr int GDN_PK_STRIDE = 272;   // bytes from one path row to the next: eight rows of a 16-byte column hit all banks once
+
+// Byte place of 4-byte word `w` (0..63) of a k row in the permuted order.
+__device__ __forceinline__ uint32_t path_row_word(int w) { return (uint32_t)((w & ~15) + (w & 3) * 4 + ((w >> 2) & 3)) * 4u; }
+
+__device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t (&r)[4])
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t (&r)[4])
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma_1688(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t b0)
+{
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(b0));
+}
+__device__ __forceinline__ uint32_t pack_bf16_pair(float2 x)
+{
+    __nv_bfloat162 t = __floats2bfloat162_rn(x.x, x.y);
+    return *reinterpret_cast<uint32_t *>(&t);
+}
+// x minus the bf16 pair h, two values at a time (exact)
+__device__ __forceinline__ float2 bf16_rest(float2 x, uint32_t h)
+{
+    return make_float2(x.x - __uint_as_float(h << 16), x.y - __uint_as_float(h & 0xFFFF0000u));
+}
+// x = hi + mid + lo in three bf16 terms (|x - hi - mid - lo| <= 2^-26 |x|: fp32 precision), two values at a time
+__device__ __forceinline__ void split3_bf16(float x0, float x1, uint32_t &hi, uint32_t &mid, uint32_t &lo)
+{
+    float2 x = make_float2(x0, x1);
+    hi = pack_bf16_pair(x);
+    x = bf16_rest(x, hi);
+    mid = pack_bf16_pair(x);
+    lo = pack_bf16_pair(bf16_rest(x, mid));
+}
+
+// One chunk of a warp's 16 rows: global memory <-> fragments.  src: this lane's first row at its first key position.
+__device__ __forceinline__ void load_chunk(const float *src, int jj, float (&x)[4][4])
+{
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        float4 a, b;
+        ldg_v8(src + r * 8 * GDN_TILE_D + jj * 32, a, b);
+        x[0][2 * r] = a.x; x[0][2 * r + 1] = a.y; x[1][2 * r] = a.z; x[1][2 * r + 1] = a.w;
+        x[2][2 * r] = b.x; x[2][2 * r + 1] = b.y; x[3][2 * r] = b.z; x[3][2 * r + 1] = b.w;
+    }
+}
+__device__ __forceinline__ void store_chunk(float *dst, int jj, const float (&x)[4][4])
+{
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+        stg_v8(dst + r * 8 * GDN_TILE_D + jj * 32, make_float4(x[0][2 * r], x[0][2 * r + 1], x[1][2 * r], x[1][2 * r + 1]),
+               make_float4(x[2][2 * r], x[2][2 * r + 1], x[3][2 * r], x[3][2 * r + 1]));
+}
+
+// An accepted path in shared memory: k rows in the permuted order (zero up to the next multiple of eight rows), v rows
+// bf16 [..][128], and per step t: scal (beta_t, beta_t A_t, E_t, .) with A_t = exp(G_t), E_t = exp(G_L - G_t), G = sum of g
+// along the path; coupling[u][t] = beta_t exp(G_t - G_u) k_t.k_u for t > u, 0 otherwise (row stride 16).
+struct PathTile {
+    const uint16_t *pv;
+    const float4 *scal;
+    const float *coupling;
+};
+
+// S <- S after L steps (1 <= L <= 16).  With u_t = beta_t (v_t - A_t k_t.S) - sum_{u < t} coupling_ut u_u (the triangular
+// form of Section 3.4.1 on the path alone), S_L = A_L S + sum_t E_t u_t k_t^T; every factor is at most 1, so nothing can
+// overflow whatever the decays.  The products run on bf16 operands that are exact (k) or three-term splits (S, E u), i.e.
+// at fp32 precision.  The tile passes through the registers twice: once for the products, once for the update.
+struct PathProducts {     // steps 2 l4, 2 l4 + 1 (+ 8 in the second entry) of rows g (entries 0, 1) and g + 8 (2, 3)
+    float z[2][4], rest[2][4];   // the mid and lo terms go to accumulators of their own (shorter chains)
+};
+__device__ __forceinline__ uint32_t path_operand(uint32_t pk, int lane)
+{
+    return pk + (uint32_t)(lane & 7) * GDN_PK_STRIDE + (uint32_t)(lane >> 3) * 16;
+}
+__device__ __forceinline__ void path_products_chunk(const float (&x)[4][4], int jj, bool two, uint32_t operand, PathProducts &a)
+{
+    uint32_t b0[4], b1[4];
+    ldmatrix_x4(operand + jj * 64, b0);
+    if (two) ldmatrix_x4(operand + 8 * GDN_PK_STRIDE + jj * 64, b1);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        uint32_t hi[4], mid[4], lo[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) split3_bf16(x[2 * h + (i >> 1)][2 * (i & 1)], x[2 * h + (i >> 1)][2 * (i & 1) + 1], hi[i], mid[i], lo[i]);
+        mma_16816(a.z[0], hi, b0[2 * h], b0[2 * h + 1]);
+        mma_16816(a.rest[0], mid, b0[2 * h], b0[2 * h + 1]);
+        mma_16816(a.rest[0], lo, b0[2 * h], b0[2 * h + 1]);
+        if (two) {
+            mma_16816(a.z[1], hi, b1[2 * h], b1[2 * h + 1]);
+            mma_16816(a.rest[1], mid, b1[2 * h], b1[2 * h + 1]);
+            mma_16816(a.rest[1], lo, b1[2 * h], b1[2 * h + 1]);
+        }
+    }
+}
+// products -> E_t u_t in three bf16 terms, the other operand of the update.  row: this lane's first row
+struct PathUpdate { uint32_t hi[4], mid[4], lo[4]; };
+__device__ __forceinline__ void path_solve(PathProducts &a, int L, const PathTile &p, int row, int lane, PathUpdate &u)
+{
+    const int l4 = lane & 3;
+    const bool two = L > 8;   // (warp-uniform)
+    float (&z)[2][4] = a.z;
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int t = 8 * i + 2 * l4 + e;
+            const bool on = t < L;
+            const float4 sc = on ? p.scal[t] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const float v = on ? __uint_as_float((uint32_t)p.pv[t * GDN_TILE_D + row + 8 * r] << 16) : 0.f;
+                z[i][2 * r + e] = on ? fmaf(-sc.y, z[i][2 * r + e] + a.rest[i][2 * r + e], sc.x * v) : 0.f;
+            }
+        }
+    // forward substitution: once u_t is final its four lanes subtract its share from the later steps (coupling is zero
+    // for the others)
+#pragma unroll 1
+    for (int t = 0; t < L - 1; ++t) {
+        const int src = (lane & ~3) | ((t & 7) >> 1);
+        const float2 c0 = *reinterpret_cast<const float2 *>(p.coupling + t * 16 + 2 * l4);
+        const float a0 = t & 8 ? z[1][0] : z[0][0], a1 = t & 8 ? z[1][1] : z[0][1];
+        const float a2 = t & 8 ? z[1][2] : z[0][2], a3 = t & 8 ? z[1][3] : z[0][3];
+        const float u0 = __shfl_sync(0xffffffffu, t & 1 ? a1 : a0, src), u1 = __shfl_sync(0xffffffffu, t & 1 ? a3 : a2, src);
+        z[0][0] = fmaf(-c0.x, u0, z[0][0]); z[0][1] = fmaf(-c0.y, u0, z[0][1]);
+        z[0][2] = fmaf(-c0.x, u1, z[0][2]); z[0][3] = fmaf(-c0.y, u1, z[0][3]);
+        if (two) {
+            const float2 c1 = *reinterpret_cast<const float2 *>(p.coupling + t * 16 + 8 + 2 * l4);
+            z[1][0] = fmaf(-c1.x, u0, z[1][0]); z[1][1] = fmaf(-c1.y, u0, z[1][1]);
+            z[1][2] = fmaf(-c1.x, u1, z[1][2]); z[1][3] = fmaf(-c1.y, u1, z[1][3]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int t = 8 * i + 2 * l4;
+        const float e0 = t < L ? p.scal[t].z : 0.f, e1 = t + 1 < L ? p.scal[t + 1].z : 0.f;
+        split3_bf16(t < L ? e0 * z[i][0] : 0.f, t + 1 < L ? e1 * z[i][1] : 0.f, u.hi[2 * i], u.mid[2 * i], u.lo[2 * i]);
+        split3_bf16(t < L ? e0 * z[i][2] : 0.f, t + 1 < L ? e1 * z[i][3] : 0.f, u.hi[2 * i + 1], u.mid[2 * i + 1], u.lo[2 * i + 1]);
+    }
+}
+__device__ __forceinline__ void path_update_chunk(float (&x)[4][4], int jj, bool two, uint32_t operand, float A_L, const PathUpdate &u)
+{
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[n][e] *= A_L;
+    uint32_t b0[4], b1[4];
+    ldmatrix_x4_trans(operand + jj * 64, b0);
+    if (two) {
+        ldmatrix_x4_trans(operand + 8 * GDN_PK_STRIDE + jj * 64, b1);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) mma_16816(x[q], u.lo, b0[q], b1[q]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) mma_16816(x[q], u.mid, b0[q], b1[q]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) mma_16816(x[q], u.hi, b0[q], b1[q]);
+    } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) mma_1688(x[q], u.lo[0], u.lo[1], b0[q]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) mma_1688(x[q], u.mid[0], u.mid[1], b0[q]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) mma_1688(x[q], u.hi[0], u.hi[1], b0[q]);
+    }
+}
+
+// The coupling table of a path whose k rows are in shared memory, by one warp (lane t: G_t, beta_t of step t; rows beyond
+// L up to the next multiple of eight are zero).
+__device__ __forceinline__ void path_coupling(uint32_t pk, int L, float G, float beta, float *coupling, int lane)
+{
+    const int g = lane >> 2, l4 = lane & 3;
+    const bool two = L > 8;
+    float k[2][2][4];   // [parity of the chunk][tile of u]: k_t.k_u, rows t = g (entries 0, 1) and g + 8 (2, 3)
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) k[0][i][e] = k[1][i][e] = 0.f;
+    const int half = (lane >> 3) & 1;   // ldmatrix: matrices (rows 0-7, chunk c), (rows 8-15, c), (rows 0-7, c + 1), (rows 8-15, c + 1)
+    const uint32_t addr = pk + (uint32_t)((lane & 7) + (two ? 8 * half : 0)) * GDN_PK_STRIDE + (uint32_t)(lane >> 4) * 16;
+#pragma unroll 2
+    for (int c = 0; c < 8; ++c) {
+        uint32_t a[4];
+        ldmatrix_x4(addr + c * 32, a);
+        mma_16816(k[c & 1][0], a, a[0], a[2]);
+        if (two) mma_16816(k[c & 1][1], a, a[1], a[3]);
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {   // t = g + 8 r
+        const int t = g + 8 * r;
+        const float Gt = __shfl_sync(0xffffffffu, G, t), bt = __shfl_sync(0xffffffffu, beta, t);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int u = 8 * i + 2 * l4 + e;
+                const float Gu = __shfl_sync(0xffffffffu, G, u);
+                if ((two || (r == 0 && i == 0)) && u < L)
+                    coupling[u * 16 + t] = t > u && t < L ? bt * expf(Gt - Gu) * (k[0][i][2 * r + e] + k[1][i][2 * r + e]) : 0.f;
+            }
+    }
+}
+
+}  // namespace gdn

@@ -714,6 +714,24 @@ def test_commit_tile_kernel_paths(tl):
     assert bool((d3.S0 == before3).all())
 
 
+@pytest.mark.parametrize("slots", [10, 17])
+def test_commit_tile_kernel_forms_of_large_calls(tl, slots):
+    """More tiles than are resident at two / at three per SM (32 heads per slot): path lengths 0..16, a path that decays
+    below what fp32 can invert, and a rejected path."""
+    paths = [np.arange((5 * i) % 17, dtype=np.int32) for i in range(slots)]
+    paths[3] = np.array([0, 2], np.int32)
+    trees = [synth.tree_chain(16)] * slots
+    make = lambda ps: synth.random_case(47, trees, 2, 32, 128, 128, synth.BF16, synth.BF16, paths=ps)
+    w, w_ref = make(paths), make([np.zeros(0, np.int32) if i == 3 else p for i, p in enumerate(paths)])
+    for x in (w, w_ref):
+        x.g[16:32] = synth.f32_to_bf16_bits(np.float32([-30.0]))[0]
+    dc = tl.DeviceCase(w)
+    before = dc.S0.clone()
+    assert dc.commit() == 0 and dc.device_status() == -9
+    tl.assert_state_close(dc.S0.cpu().numpy().astype(np.float64), tl.oracle_commit(w_ref), what="tile commit")
+    assert bool((dc.S0[3] == before[3]).all()) and bool((dc.S0[0] == before[0]).all())
+
+
 def test_fused_call_on_large_trees(tl):
     """Trees beyond one CTA tile: the fused entry point runs the commit tile kernel and the grouped verify kernel back
     to back; results as for the small-tree kernel."""
