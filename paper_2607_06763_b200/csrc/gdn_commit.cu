@@ -11,8 +11,6 @@
 // are fetched once into shared memory; the state is read once and written once.  The state loads
 // are issued before anything else so that the path checks and the k-row staging run under their
 // latency, and the kernel keeps to 64 registers so that two CTAs (32 warps) share an SM.
-#include <atomic>
-
 #include "gdn_fragments.cuh"
 #include "gdn_internal.cuh"
 #include "gdn_plan.cuh"
@@ -459,14 +457,9 @@ template <int CTAS> __global__ void __launch_bounds__(CF_THREADS, CTAS) commit_p
 // CTAs per SM for a call of `units` tiles: the fewest with which they are all resident at once.
 int commit_form(int units)
 {
-    static std::atomic<int> sm_count[64];
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 2;
-    if (dev < 64) sms = sm_count[dev].load(std::memory_order_relaxed);
-    if (sms == 0) {
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 2;
-        if (dev < 64) sm_count[dev].store(sms, std::memory_order_relaxed);
-    }
+    static PerDevice seen;
+    int sms = 0;
+    if (device_sms(seen, nullptr, 0, &sms) != cudaSuccess) return 2;
     return units <= 2 * sms ? 2 : units <= 3 * sms ? 3 : 4;
 }
 
@@ -490,19 +483,9 @@ cudaError_t launch_commit_generic(const gdn_shape_t &s, float *S, const void *k,
                    parent, node_offsets, path, path_offsets, status_dev, 0, 0, 0, 0, nullptr, nullptr};
     if (s.d_k == GDN_TILE_D && s.d_v == GDN_TILE_D && s.in_dtype == GDN_BF16 && s.max_depth <= CF_MD)
         return launch_tile128(p, grid, stream);
-    const size_t smem = sizeof(float) * ((size_t)s.max_depth * CM_DK + 4 * (size_t)s.max_depth);
-    cudaError_t e;
-    if (s.in_dtype == GDN_BF16) {
-        e = cudaFuncSetAttribute(commit_generic_kernel<__nv_bfloat16>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        return launch_overlapped(commit_generic_kernel<__nv_bfloat16>, grid, CM_THREADS, smem, stream, p);
-    } else {
-        e = cudaFuncSetAttribute(commit_generic_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem);
-        if (e != cudaSuccess) return e;
-        return launch_overlapped(commit_generic_kernel<float>, grid, CM_THREADS, smem, stream, p);
-    }
+    const size_t smem = sizeof(float) * ((size_t)s.max_depth * CM_DK + 4 * (size_t)s.max_depth);   // at most 33 KB
+    return launch_overlapped(s.in_dtype == GDN_BF16 ? commit_generic_kernel<__nv_bfloat16> : commit_generic_kernel<float>, grid,
+                             CM_THREADS, smem, stream, p);
 }
 
 bool commit_tile128_supported(const gdn_shape_t &s) { return commit_padded_supported(s); }

@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "gdn_tree.h"
 
 namespace gdn {
@@ -103,6 +105,24 @@ inline PlanPtrs plan_ptrs(void *workspace, const WorkspaceLayout &w)
             reinterpret_cast<uint8_t *>(b + w.dfs_anc8), reinterpret_cast<uint16_t *>(b + w.group_start),
             reinterpret_cast<int32_t *>(b + w.unit_count), reinterpret_cast<uint4 *>(b + w.unit_list),
             reinterpret_cast<float *>(b + w.utilde)};
+}
+
+// What a launcher needs of the current device, asked for once per device and kernel (the runtime calls cost about a
+// microsecond each): the number of SMs, and the kernel's dynamic shared memory limit raised to `smem` bytes.
+struct PerDevice {
+    std::atomic<int> sms[64];   // 0 = not asked yet
+};
+inline cudaError_t device_sms(PerDevice &seen, const void *kernel, size_t smem, int *sms)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    *sms = dev < 64 ? seen.sms[dev].load(std::memory_order_acquire) : 0;
+    if (*sms != 0) return cudaSuccess;
+    e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess && kernel) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess && dev < 64) seen.sms[dev].store(*sms, std::memory_order_release);
+    return e;
 }
 
 // Host launchers (each returns the cudaError_t of its launch).

@@ -455,9 +455,11 @@ __global__ void __launch_bounds__(VS_THREADS, 2) verify_generic_small_kernel(con
 template <typename TIn, typename TOut>
 cudaError_t launch_small_typed(const VerifySmallParams &p, cudaStream_t stream)
 {
+    static PerDevice seen;
     const int grid = p.n_seq * p.h_v * p.n_blocks;
-    cudaError_t e = cudaFuncSetAttribute(verify_generic_small_kernel<TIn, TOut>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(VerifySmallSmem));
+    int sms = 0;
+    const cudaError_t e = device_sms(seen, reinterpret_cast<const void *>(verify_generic_small_kernel<TIn, TOut>),
+                                     sizeof(VerifySmallSmem), &sms);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)grid);

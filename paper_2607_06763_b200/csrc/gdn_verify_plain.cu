@@ -25,8 +25,6 @@
 // What bounds it: the chain of a unit (Gram -> lists -> back-substitution -> C -> q' -> output product -> rows), not memory
 // and not the tensor pipe; so the unit has as few instructions and barriers as could be found, two CTAs share an SM and
 // fill each other's waits, and a CTA takes neighbouring units, which have much in common.
-#include <atomic>
-
 #include "gdn_internal.cuh"
 #include "gdn_replay.cuh"
 #include "gdn_tc.cuh"
@@ -799,21 +797,12 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
     if (warp == 0) tmem_dealloc(tmem, TM_COLS);
 }
 
-// SMs of the current device and the shared-memory limit of the kernel, looked up and raised once per kernel and device.
 template <typename TOut, bool PADDED, bool GROUPED> cudaError_t launch_kernel(const VerifyPlainParams &p, cudaStream_t stream)
 {
-    static std::atomic<int> sm_count[64];
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    static PerDevice seen;
+    int sms = 0;
+    const cudaError_t e = device_sms(seen, reinterpret_cast<const void *>(verify_plain_kernel<TOut, PADDED, GROUPED>), SP_ALLOC, &sms);
     if (e != cudaSuccess) return e;
-    if (dev < 64) sms = sm_count[dev].load(std::memory_order_acquire);
-    if (sms == 0) {
-        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(verify_plain_kernel<TOut, PADDED, GROUPED>, cudaFuncAttributeMaxDynamicSharedMemorySize, SP_ALLOC);
-        if (e != cudaSuccess) return e;
-        if (dev < 64) sm_count[dev].store(sms, std::memory_order_release);
-    }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(p.n_units < 2 * sms ? p.n_units : 2 * sms));   // persistent CTAs, two per SM
     cfg.blockDim = dim3(VP_THREADS);

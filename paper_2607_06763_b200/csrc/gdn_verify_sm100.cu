@@ -1241,9 +1241,13 @@ cudaError_t launch_fast_typed(const gdn_shape_t &s, const VerifyFastParams &p, c
             kernel = small ? verify_sm100_persistent_kernel<TOut, FUSED, true, true, false>
                            : verify_sm100_persistent_kernel<TOut, FUSED, false, true, false>;
     }
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_ALLOC);
+    static PerDevice seen[4];
+    int sms = 0;
+    const cudaError_t e = device_sms(seen[(padded ? 2 : 0) + (s.max_tree_nodes <= 32 ? 1 : 0)], reinterpret_cast<const void *>(kernel),
+                                     SM_ALLOC, &sms);
     if (e != cudaSuccess) return e;
-    const int grid = pt.n_units < p.prefetch_dist ? pt.n_units : p.prefetch_dist;
+    pt.prefetch_dist = 2 * sms;
+    const int grid = pt.n_units < pt.prefetch_dist ? pt.n_units : pt.prefetch_dist;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(FV_THREADS);
@@ -1261,10 +1265,8 @@ VerifyFastParams make_params(const gdn_shape_t &s, const float *S0, const void *
                              const void *g, const void *beta, const int32_t *node_offsets, void *o,
                              const PlanPtrs &plan, int32_t *status_dev)
 {
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     VerifyFastParams p{};
-    p.h_qk = s.h_qk; p.h_v = s.h_v; p.n_units = s.n_seq * s.h_v; p.prefetch_dist = 2 * sms; p.scale = s.scale;
+    p.h_qk = s.h_qk; p.h_v = s.h_v; p.n_units = s.n_seq * s.h_v; p.scale = s.scale;
     p.S0 = S0;
     p.q = static_cast<const __nv_bfloat16 *>(q); p.k = static_cast<const __nv_bfloat16 *>(k);
     p.v = static_cast<const __nv_bfloat16 *>(v); p.g = static_cast<const __nv_bfloat16 *>(g);
