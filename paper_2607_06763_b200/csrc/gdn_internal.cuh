@@ -150,7 +150,7 @@ bool verify_sm100_single_group(const gdn_shape_t &s);   // every tree fits one C
 cudaError_t launch_verify_sm100(const gdn_shape_t &s, const float *S0, const void *q, const void *k,
                                 const void *v, const void *g, const void *beta, const int32_t *parent,
                                 const int32_t *node_offsets, void *o, const PlanPtrs &plan,
-                                int32_t *status_dev, cudaStream_t stream);
+                                int32_t *status_dev, cudaStream_t stream, bool behind_commit = false);
 
 // Same kernel with the commit of the previous step's accepted paths fused in front of the verify:
 // the state tile is read once, advanced along the path (Eq. 7), written back, and the new tree is
@@ -170,7 +170,7 @@ cudaError_t launch_commit_verify_sm100(const gdn_shape_t &s, float *S, const voi
 cudaError_t launch_verify_sm100_padded(const gdn_shape_t &s, int n_trees, bool raw_gates, const float *S0,
                                        const void *q, const void *k, const void *v, const void *g, const void *beta,
                                        const int32_t *parent, const int32_t *n_nodes, void *o, int32_t *status_dev,
-                                       cudaStream_t stream);
+                                       cudaStream_t stream, bool behind_commit = false);
 cudaError_t launch_commit_verify_sm100_padded(const gdn_shape_t &s, int n_trees, bool raw_gates, float *S,
                                               int prev_t_pad, const void *k_prev, const void *v_prev,
                                               const void *g_prev, const void *beta_prev, const int32_t *parent_prev,

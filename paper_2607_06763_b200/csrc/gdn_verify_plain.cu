@@ -90,6 +90,7 @@ struct VerifyPlainParams {
     int t_pad, n_trees;
     const int32_t *n_nodes;
     int raw_gates;                                     // g / beta arrive as raw gate inputs ("scalars" stage on chip)
+    int state_late;                                    // the kernel in front writes the state alone (see the wait)
     // grouped verification of trees with more than 64 nodes (only read by the GROUPED instantiation)
     int groups_per_tree, anc_stride;                   // upper bound of the groups of a tree (sizes the grid); entries
                                                        // per row of anc16
@@ -168,10 +169,16 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
             }
         }
     }
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    // ... and whatever is launched behind this grid with the same attribute (the next call's kernel, which itself waits
-    // for this grid to complete before it reads or writes anything) may be made resident as CTAs leave.
-    asm volatile("griddepcontrol.launch_dependents;");
+    // state_late: the kernel in front is the commit of the same call, which itself has waited for everything before it and
+    // writes nothing but the state; only the first use of a state tile waits for it.
+    bool state_late = !GROUPED && p.state_late;
+    auto wait_for_previous_kernel = [&]() {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        // ... and whatever is launched behind this grid with the same attribute (the next call's kernel, which itself waits
+        // for this grid to complete before it reads or writes anything) may be made resident as CTAs leave.
+        asm volatile("griddepcontrol.launch_dependents;");
+    };
+    if (!state_late) wait_for_previous_kernel();
 
     // ------------------------------------------------------------------------------------ the units of this CTA
     // Unit = slot b * h_v + head h; GROUPED: E = records in the plan's list (the groups of a tree next to one another),
@@ -479,7 +486,9 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
     while (have) {
         // State tile, as 16 x 8 fragments in a permuted column order: lane = 4 g + l4 holds rows g and g + 8 of the warp's
         // sixteen, and of each the key positions 32 jj + 8 l4 + e (e = 0..7) as x[4 jj + (e >> 1)][2 r + (e & 1)], i.e. 32
-        // contiguous bytes per lane and load.  Asked for at the top, needed behind the coefficients.
+        // contiguous bytes per lane and load.  Asked for at the top, needed behind the coefficients; in two pieces, or, beside
+        // the row copies of the grouped mode, in four (256-node trees, fused call: 278.5 -> 275.5 us; plain trees are 2 % slower
+        // that way).
         float x[16][4];
         const size_t tile = (size_t)(un.b * p.h_v + un.h) * VP_D * VP_D + (size_t)(row0 + (lane >> 2)) * VP_D + (lane & 3) * 8;
         auto load_state = [&](int j0, int j1) {
@@ -495,7 +504,7 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
                     }
             }
         };
-        load_state(0, 2);
+        if (!state_late) load_state(0, GROUPED ? 1 : 2);
         if (new_rows) {
             if (!mbar_wait_bounded(mbar_kq, gram_parity)) *flag = 1;
             if (!mbar_wait_bounded(mbar_g, gram_parity)) *flag = 1;
@@ -503,7 +512,7 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
             gram_parity ^= 1;
         }
         __syncthreads();   // tables; the output stage has been read
-        load_state(2, 4);
+        if (!state_late) load_state(GROUPED ? 1 : 2, GROUPED ? 2 : 4);
         // a tree whose parent[] was rejected while its tables were built runs as a tree of no nodes
         const bool bad = *bad_s != 0;
         const int T = bad ? 0 : un.T;
@@ -533,6 +542,7 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
             tc_fence_before();
             __syncthreads();
         }
+        if constexpr (GROUPED) load_state(2, 3);
         // (2) w by back-substitution over the root path (column-oriented: once w_l is final, subtract w_l kappa(n_l, t) from
         // every entry t < l); four threads per node, thread sq of the quad owning path positions 4 sq .. 4 sq + 3
         const int zi = tid >> 2, sq = tid & 3;
@@ -597,6 +607,7 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
                 }
             }
         }
+        if constexpr (GROUPED) load_state(3, 4);
         if (!mbar_wait_bounded(mbar_v, par)) *flag = 1;
         // k and v rows between the tree and the next multiple of 16 belong to another tree (or are padding): they meet zero
         // weights in the products, which have to be zero whatever they hold
@@ -638,6 +649,11 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
             tables_load(nx, nr);
             if (tid < 4 && (!GROUPED || nx.fresh))   // ... and its state tile into L2
                 prefetch_l2_bulk(p.S0 + (size_t)(nx.b * p.h_v + nx.h) * VP_D * VP_D + (size_t)tid * 4096, 16384);
+        }
+        if (state_late) {
+            wait_for_previous_kernel();
+            state_late = false;
+            load_state(0, 4);
         }
         // (5) the state tile as bf16 hi + lo, the operand of the last product; a warp writes the lanes it can reach
         if (!GROUPED || un.fresh) {
@@ -790,6 +806,7 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
         have = have_n;
     }
 
+    if (state_late) wait_for_previous_kernel();   // (no unit had work: this grid must not end before the one in front)
     if (*flag != 0 && tid == 0) report_status(p.status_dev, GDN_ERR_TIMEOUT);
     cp_async_wait_all();
     tc_fence_before();
@@ -866,10 +883,11 @@ VerifyPlainParams make_params(const gdn_shape_t &s, const float *S0, const void 
 cudaError_t launch_verify_sm100_padded(const gdn_shape_t &s, int n_trees, bool raw_gates, const float *S0,
                                        const void *q, const void *k, const void *v, const void *g, const void *beta,
                                        const int32_t *parent, const int32_t *n_nodes, void *o, int32_t *status_dev,
-                                       cudaStream_t stream)
+                                       cudaStream_t stream, bool behind_commit)
 {
     if (s.n_seq == 0 || s.total_nodes == 0) return cudaSuccess;
     VerifyPlainParams p = make_params(s, S0, q, k, v, g, beta, nullptr, o, PlanPtrs{}, status_dev);
+    p.state_late = behind_commit ? 1 : 0;
     p.parent = parent;
     p.t_pad = s.max_tree_nodes; p.n_trees = n_trees; p.n_nodes = n_nodes; p.raw_gates = raw_gates ? 1 : 0;
     return launch_plain<false>(s, p, stream);
@@ -901,11 +919,12 @@ bool verify_sm100_single_group(const gdn_shape_t &s) { return verify_sm100_suppo
 cudaError_t launch_verify_sm100(const gdn_shape_t &s, const float *S0, const void *q, const void *k,
                                 const void *v, const void *g, const void *beta, const int32_t *parent,
                                 const int32_t *node_offsets, void *o, const PlanPtrs &plan,
-                                int32_t *status_dev, cudaStream_t stream)
+                                int32_t *status_dev, cudaStream_t stream, bool behind_commit)
 {
     if (s.n_seq == 0 || s.total_nodes == 0) return cudaSuccess;
     VerifyPlainParams p = make_params(s, S0, q, k, v, g, beta, node_offsets, o, plan, status_dev);
     p.parent = parent;
+    p.state_late = behind_commit ? 1 : 0;
     if (!verify_sm100_single_group(s)) return launch_plain<true>(s, p, stream);
     return launch_plain<false>(s, p, stream);
 }

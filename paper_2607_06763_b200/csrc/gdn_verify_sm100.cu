@@ -1287,6 +1287,16 @@ VerifyFastParams make_params(const gdn_shape_t &s, const float *S0, const void *
 
 }  // namespace
 
+// Few units: the commit kernel and, behind it, the verification, which works out everything but the product with the state
+// meanwhile -- the two run side by side on different SMs as long as there are enough of them.  Measured (us, 64 nodes, path
+// of 7; this kernel / two kernels): 32 units 13.5 / 11.7, 64 units 13.7 / 11.9, 80 units 13.6 / 14.8, 128 units 14.0 / 15.0.
+static bool as_two_kernels(const gdn_shape_t &s)
+{
+    static PerDevice seen;
+    int sms = 0;
+    return device_sms(seen, nullptr, 0, &sms) == cudaSuccess && s.n_seq * s.h_v <= sms / 2;
+}
+
 cudaError_t launch_commit_verify_sm100_padded(const gdn_shape_t &s, int n_trees, bool raw_gates, float *S,
                                               int prev_t_pad, const void *k_prev, const void *v_prev,
                                               const void *g_prev, const void *beta_prev, const int32_t *parent_prev,
@@ -1297,6 +1307,14 @@ cudaError_t launch_commit_verify_sm100_padded(const gdn_shape_t &s, int n_trees,
                                               cudaStream_t stream)
 {
     if (s.n_seq == 0 || s.total_nodes == 0) return cudaSuccess;
+    if (as_two_kernels(s)) {
+        gdn_shape_t ps = s;   // the commit reads the slots of the previous step
+        ps.max_tree_nodes = prev_t_pad;
+        const cudaError_t e = launch_commit_padded(ps, n_trees, raw_gates, S, k_prev, v_prev, g_prev, beta_prev, parent_prev,
+                                                   n_nodes_prev, path, path_len, status_dev, stream);
+        if (e != cudaSuccess) return e;
+        return launch_verify_sm100_padded(s, n_trees, raw_gates, S, q, k, v, g, beta, parent, n_nodes, o, status_dev, stream, true);
+    }
     VerifyFastParams p = make_params(s, S, q, k, v, g, beta, nullptr, o, PlanPtrs{}, status_dev);
     p.parent = parent;
     p.t_pad = s.max_tree_nodes; p.n_trees = n_trees; p.n_nodes = n_nodes; p.raw_gates = raw_gates ? 1 : 0;
@@ -1318,6 +1336,12 @@ cudaError_t launch_commit_verify_sm100(const gdn_shape_t &s, float *S, const voi
                                        cudaStream_t stream)
 {
     if (s.n_seq == 0 || s.total_nodes == 0) return cudaSuccess;
+    if (as_two_kernels(s)) {
+        const cudaError_t e = launch_commit_generic(s, S, k_prev, v_prev, g_prev, beta_prev, parent_prev, node_offsets_prev, path,
+                                                    path_offsets, status_dev, stream);
+        if (e != cudaSuccess) return e;
+        return launch_verify_sm100(s, S, q, k, v, g, beta, parent, node_offsets, o, PlanPtrs{}, status_dev, stream, true);
+    }
     VerifyFastParams p = make_params(s, S, q, k, v, g, beta, node_offsets, o, PlanPtrs{}, status_dev);
     p.parent = parent;
     p.S_rw = S;

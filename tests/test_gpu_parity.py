@@ -732,6 +732,49 @@ def test_commit_tile_kernel_forms_of_large_calls(tl, slots):
     assert bool((dc.S0[3] == before[3]).all()) and bool((dc.S0[0] == before[0]).all())
 
 
+@pytest.mark.parametrize("slots", [1, 18, 19])
+def test_fused_step_on_both_sides_of_the_two_kernel_rule(tl, slots):
+    """4 heads per slot: 72 units run as two kernels, 76 as one (148 SMs).  Every input is overwritten by the kernels right
+    in front of the call, three times over; slot 0 has an empty new tree, the last slots a rejected and an empty path."""
+    import torch
+    import paper_2607_06763_b200 as gdn
+    from oracle import gdn_oracle as orc
+    rng = np.random.default_rng(53)
+    sizes = [0] + [1 + (7 * i) % 64 for i in range(1, slots)]
+    trees = [synth.tree_geo(rng, T) if T > 1 else np.full(T, -1, np.int32) for T in sizes]
+    paths = [np.arange((3 * i) % 17, dtype=np.int32) for i in range(1, slots + 1)]
+    paths_ok = list(paths)
+    if slots > 2:
+        paths[-1], paths_ok[-1], paths[-2], paths_ok[-2] = np.array([0, 2], np.int32), *[np.zeros(0, np.int32)] * 3
+    make_prev = lambda seed, ps: synth.random_case(seed, [synth.tree_chain(16)] * slots, 2, 4, 128, 128, synth.BF16, synth.F32, paths=ps)
+    prevs = [make_prev(60 + i, paths) for i in range(3)]
+    news = [synth.random_case(70 + i, trees, 2, 4, 128, 128, synth.BF16, synth.F32) for i in range(3)]
+    dps, dns = [tl.DeviceCase(w) for w in prevs], [tl.DeviceCase(w) for w in news]
+    dp, dn = tl.DeviceCase(prevs[2]), tl.DeviceCase(news[2])
+    got = []
+    torch.cuda.synchronize()
+    for i in range(3):
+        for name in ("S0", "k", "v", "g", "beta"):
+            getattr(dp, name).copy_(getattr(dps[i], name))
+        for name in ("q", "k", "v", "g", "beta"):
+            getattr(dn, name).copy_(getattr(dns[i], name))
+        rc = gdn.gdn_tree_commit_verify(dn.shape, dp.S0, dp.k, dp.v, dp.g, dp.beta, dp.parent, dp.node_offsets, dp.path,
+                                        dp.path_offsets, dn.q, dn.k, dn.v, dn.g, dn.beta, dn.parent, dn.node_offsets, dn.o,
+                                        dn.ws, dn.ws_bytes, dn.status, torch.cuda.current_stream())
+        assert rc == 0, gdn.gdn_status_string(rc)
+        got.append((dp.S0.clone(), dn.o.clone()))
+    assert dn.device_status() == (-9 if slots > 2 else 0)
+    for i, (S, o) in enumerate(got):
+        S_ref = tl.oracle_commit(make_prev(60 + i, paths_ok))
+        tl.assert_state_close(S.cpu().numpy().astype(np.float64), S_ref, what=f"fused, {slots} slots, S")
+        if slots > 2:
+            assert bool((S[-2:] == dps[i].S0[-2:]).all())
+        if news[i].q.size:
+            w = news[i]
+            o_ref = orc.verify(S_ref, *(w.f64(n) for n in ("q", "k", "v", "g", "beta")), w.parent, w.node_offsets, w.scale)
+            tl.assert_close_per_head(o.cpu().numpy().astype(np.float64), o_ref, w.node_offsets, f"fused, {slots} slots, o")
+
+
 def test_fused_call_on_large_trees(tl):
     """Trees beyond one CTA tile: the fused entry point runs the commit tile kernel and the grouped verify kernel back
     to back; results as for the small-tree kernel."""
