@@ -5,12 +5,12 @@
 // With S' = alpha S (decay first), Eq. 7 reads S <- S' - beta k (k^T S') + beta k v^T, i.e. per
 // value component c (one contiguous row of the [d_v][d_k] tile):
 //     s_c <- alpha s_c + k * beta (v_c - alpha (k . s_c)).
-// One CTA per (tree, value head); thread (c, s) owns 32 floats of row c (quarter s of the key
-// dimension, interleaved in 16-byte pieces so that the four lanes of a row read 64 contiguous
-// bytes) and k . s_c is reduced over the four lanes with warp shuffles.  The path nodes' k rows
-// are fetched once into shared memory; the state is read once and written once.  The state loads
-// are issued before anything else so that the path checks and the k-row staging run under their
-// latency, and the kernel keeps to 64 registers so that two CTAs (32 warps) share an SM.
+// General form: one CTA per (tree, value head); eight lanes hold four rows, an eighth of the key dimension each (16-byte
+// pieces, 128 contiguous bytes per row and load), and k . s_c of the four is reduced over them with shuffles.  The path
+// nodes' k and v rows are fetched once into shared memory; the state is read once and written once.  The state loads are
+// issued before anything else so that the path checks and the row staging run under their latency.  With four lanes per
+// row and one row per thread each k piece served one row only and shared memory bounded the steps: 8 trees, 32 heads of
+// 128 x 128, path of 5, fp32: 14.3 -> 8.6 us.
 #include "gdn_fragments.cuh"
 #include "gdn_internal.cuh"
 #include "gdn_plan.cuh"
@@ -19,10 +19,11 @@ namespace gdn {
 
 namespace {
 
-constexpr int CM_THREADS = 512;
-constexpr int CM_SPLIT = 4;
+constexpr int CM_THREADS = 256;
+constexpr int CM_SPLIT = 8;
+constexpr int CM_ROWS = 4;
 constexpr int CM_DK = GDN_MAX_HEAD_DIM;
-constexpr int CM_REGS = CM_DK / CM_SPLIT;
+static_assert(CM_THREADS / CM_SPLIT * CM_ROWS == GDN_MAX_HEAD_DIM, "a row of the state for every value component");
 
 struct CommitParams {
     int h_qk, h_v, d_k, d_v, max_depth;
@@ -62,16 +63,16 @@ cudaError_t launch_overlapped(void (*kernel)(KernelArgs...), int grid, int threa
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+constexpr size_t commit_generic_smem(int max_depth) { return sizeof(float) * (2 * (size_t)CM_DK + 2) * max_depth; }
+
 template <typename TIn>
 __global__ void __launch_bounds__(CM_THREADS, 2) commit_generic_kernel(const CommitParams p)
 {
     extern __shared__ __align__(16) float cm_smem[];
     float (*ks)[CM_DK] = reinterpret_cast<float (*)[CM_DK]>(cm_smem);   // [L][CM_DK]
-    float *alpha_s = cm_smem + (size_t)p.max_depth * CM_DK;             // [L]
+    float (*vs)[CM_DK] = ks + p.max_depth;                              // [L][CM_DK]
+    float *alpha_s = cm_smem + 2 * (size_t)p.max_depth * CM_DK;         // [L]
     float *beta_s = alpha_s + p.max_depth;                              // [L]
-    int *path_s = reinterpret_cast<int *>(beta_s + p.max_depth);        // [L] node ids
-    int *par_s = path_s + p.max_depth;                                  // [L] their parents
-    __shared__ int path_bad;
 
     wait_for_previous_kernel();
     const int b = blockIdx.x / p.h_v, h = blockIdx.x % p.h_v;
@@ -80,98 +81,103 @@ __global__ void __launch_bounds__(CM_THREADS, 2) commit_generic_kernel(const Com
     if (L == 0) return;   // nothing accepted from this tree: state untouched
     const int base = p.node_offsets[b];
     const int T = p.node_offsets[b + 1] - base;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31;
     const int d_k = p.d_k, d_v = p.d_v;
     const bool shape_ok = L > 0 && L <= p.max_depth && T > 0 && p0 >= 0;
 
     const int hk = h / (p.h_v / p.h_qk);
-    const int c = tid / CM_SPLIT, s = tid % CM_SPLIT;
-    const bool comp_on = c < d_v;
+    const int s = tid % CM_SPLIT, c = tid / CM_SPLIT * CM_ROWS;
     const TIn *k = static_cast<const TIn *>(p.k), *v = static_cast<const TIn *>(p.v);
     const TIn *g = static_cast<const TIn *>(p.g), *beta = static_cast<const TIn *>(p.beta);
 
-    // The state slice goes first: its latency covers the path checks and the k-row staging below.
-    float *row = p.S + ((size_t)(b * p.h_v + h) * d_v + (comp_on ? c : 0)) * d_k;
-    float sreg[CM_REGS];
+    // The state goes first: its latency covers the path checks and the row staging below.
+    float *rows = p.S + ((size_t)(b * p.h_v + h) * d_v + c) * d_k;
+    float2 x[CM_ROWS][8];   // row c + r, key positions 32 j + 4 s + e (zero beyond d_k / d_v)
 #pragma unroll
-    for (int j = 0; j < CM_REGS / 4; ++j) {
-        const int r = 16 * j + 4 * s;
-        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (shape_ok && comp_on && r < d_k) x = *reinterpret_cast<const float4 *>(row + r);
-        sreg[4 * j + 0] = x.x; sreg[4 * j + 1] = x.y; sreg[4 * j + 2] = x.z; sreg[4 * j + 3] = x.w;
-    }
-
-    // The accepted path must be a chain from a root inside this tree: every thread t < L fetches
-    // its entry (and that node's parent) in parallel, thread 0 then checks the chain.
-    if (shape_ok && tid < L) {
-        const int n = p.path[p0 + tid];
-        path_s[tid] = n;
-        par_s[tid] = (p.parent && n >= 0 && n < T) ? p.parent[base + n] : -2;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        int bad = !shape_ok;
-        for (int t = 0; !bad && t < L; ++t) {
-            const int n = path_s[t];
-            if (n < 0 || n >= T) bad = 1;
-            else if (p.parent) bad = par_s[t] != (t ? path_s[t - 1] : -1);
-            else if (t && n <= path_s[t - 1]) bad = 1;   // without parent[] only the topological order can be checked
+    for (int r = 0; r < CM_ROWS; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int at = 32 * j + 4 * s;
+            float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (shape_ok && c + r < d_v && at < d_k) y = *reinterpret_cast<const float4 *>(rows + (size_t)r * d_k + at);
+            x[r][2 * j] = make_float2(y.x, y.y);
+            x[r][2 * j + 1] = make_float2(y.z, y.w);
         }
-        path_bad = bad;
-        if (bad) report_status(p.status_dev, GDN_ERR_PATH);
-    }
-    __syncthreads();
-    if (path_bad) return;
 
-    // k rows of the path (fp32, zero padded to CM_DK) and the per-step scalars
-    for (int idx = tid; idx < L * CM_DK; idx += CM_THREADS) {
-        const int t = idx / CM_DK, r = idx % CM_DK;
-        const size_t n = (size_t)base + path_s[t];
-        ks[t][r] = r < d_k ? load_as_float(k + (n * p.h_qk + hk) * d_k + r) : 0.f;
+    // The path's rows (fp32, zero padded to CM_DK) and per-step scalars: every thread reads the path entry whose row piece
+    // it fetches, an entry outside the tree is skipped here and reported by the check.
+    bool bad = !shape_ok;
+    if (shape_ok) {
+#pragma unroll 2
+        for (int idx = tid; idx < L * CM_DK; idx += CM_THREADS) {
+            const int t = idx / CM_DK, r = idx % CM_DK, nt = p.path[p0 + t];
+            if (nt < 0 || nt >= T) continue;
+            const size_t n = (size_t)base + nt;
+            ks[t][r] = r < d_k ? load_as_float(k + (n * p.h_qk + hk) * d_k + r) : 0.f;
+            vs[t][r] = r < d_v ? load_as_float(v + (n * p.h_v + h) * d_v + r) : 0.f;
+        }
+        if (tid < L) {
+            // thread t: entry t must be the child of entry t - 1 (entry 0: a root)
+            const int nt = p.path[p0 + tid], up = tid ? p.path[p0 + tid - 1] : -1;
+            if (nt < 0 || nt >= T) bad = true;
+            else {
+                // (without parent[] only the topological order can be checked)
+                bad = p.parent ? p.parent[base + nt] != up : tid && nt <= up;
+                alpha_s[tid] = expf(load_as_float(g + ((size_t)base + nt) * p.h_v + h));
+                beta_s[tid] = load_as_float(beta + ((size_t)base + nt) * p.h_v + h);
+            }
+        }
     }
-    if (tid < L) {
-        const size_t n = (size_t)base + path_s[tid];
-        alpha_s[tid] = expf(load_as_float(g + n * p.h_v + h));
-        beta_s[tid] = load_as_float(beta + n * p.h_v + h);
+    if (__syncthreads_or(bad)) {
+        if (tid == 0) report_status(p.status_dev, GDN_ERR_PATH);
+        return;
     }
-    float vc = comp_on ? load_as_float(v + (((size_t)base + path_s[0]) * p.h_v + h) * d_v + c) : 0.f;
-    __syncthreads();
 
+    const bool b2 = (s & 4) != 0, b1 = (s & 2) != 0;
+    const int mine = (b2 ? 2 : 0) + (b1 ? 1 : 0);   // the row whose k.s this lane ends up with
+#pragma unroll 1
     for (int t = 0; t < L; ++t) {
-        float vnext = 0.f;   // next step's v[c], fetched while this step computes
-        if (comp_on && t + 1 < L)
-            vnext = load_as_float(v + (((size_t)base + path_s[t + 1]) * p.h_v + h) * d_v + c);
-        float dot = 0.f;
+        float2 kf[8];
 #pragma unroll
-        for (int j = 0; j < CM_REGS / 4; ++j) {
-            const float4 kx = *reinterpret_cast<const float4 *>(&ks[t][16 * j + 4 * s]);
-            dot = fmaf(kx.x, sreg[4 * j + 0], dot); dot = fmaf(kx.y, sreg[4 * j + 1], dot);
-            dot = fmaf(kx.z, sreg[4 * j + 2], dot); dot = fmaf(kx.w, sreg[4 * j + 3], dot);
+        for (int j = 0; j < 4; ++j) {
+            const float4 kx = *reinterpret_cast<const float4 *>(&ks[t][32 * j + 4 * s]);
+            kf[2 * j] = make_float2(kx.x, kx.y);
+            kf[2 * j + 1] = make_float2(kx.z, kx.w);
         }
-        dot += __shfl_xor_sync(0xffffffffu, dot, 1);
-        dot += __shfl_xor_sync(0xffffffffu, dot, 2);
+        float dot[CM_ROWS];
+#pragma unroll
+        for (int r = 0; r < CM_ROWS; ++r) {
+            float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc = __ffma2_rn(kf[j], x[r][j], acc);
+            dot[r] = acc.x + acc.y;
+        }
+        // the four rows folded into one another over the eight lanes; lanes 0, 2, 4, 6 of them end up with rows 0, 1, 2, 3
+        const float e0 = (b2 ? dot[2] : dot[0]) + __shfl_xor_sync(0xffffffffu, b2 ? dot[0] : dot[2], 4);
+        const float e1 = (b2 ? dot[3] : dot[1]) + __shfl_xor_sync(0xffffffffu, b2 ? dot[1] : dot[3], 4);
+        float d = (b1 ? e1 : e0) + __shfl_xor_sync(0xffffffffu, b1 ? e0 : e1, 2);
+        d += __shfl_xor_sync(0xffffffffu, d, 1);
         const float alpha = alpha_s[t];
-        const float w = beta_s[t] * (vc - alpha * dot);
+        const float w_mine = beta_s[t] * (vs[t][c + mine] - alpha * d);
+        const float2 a2 = make_float2(alpha, alpha);
 #pragma unroll
-        for (int j = 0; j < CM_REGS / 4; ++j) {
-            const float4 kx = *reinterpret_cast<const float4 *>(&ks[t][16 * j + 4 * s]);
-            sreg[4 * j + 0] = fmaf(kx.x, w, alpha * sreg[4 * j + 0]);
-            sreg[4 * j + 1] = fmaf(kx.y, w, alpha * sreg[4 * j + 1]);
-            sreg[4 * j + 2] = fmaf(kx.z, w, alpha * sreg[4 * j + 2]);
-            sreg[4 * j + 3] = fmaf(kx.w, w, alpha * sreg[4 * j + 3]);
+        for (int r = 0; r < CM_ROWS; ++r) {
+            const float w = __shfl_sync(0xffffffffu, w_mine, (lane & ~7) | (2 * r));
+            const float2 w2 = make_float2(w, w);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) x[r][j] = __ffma2_rn(kf[j], w2, __fmul2_rn(a2, x[r][j]));
         }
-        vc = vnext;
     }
 
-    if (comp_on) {
 #pragma unroll
-        for (int j = 0; j < CM_REGS / 4; ++j) {
-            const int r = 16 * j + 4 * s;
-            if (r < d_k)
-                *reinterpret_cast<float4 *>(row + r) =
-                    make_float4(sreg[4 * j + 0], sreg[4 * j + 1], sreg[4 * j + 2], sreg[4 * j + 3]);
+    for (int r = 0; r < CM_ROWS; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int at = 32 * j + 4 * s;
+            if (c + r < d_v && at < d_k)
+                *reinterpret_cast<float4 *>(rows + (size_t)r * d_k + at) =
+                    make_float4(x[r][2 * j].x, x[r][2 * j].y, x[r][2 * j + 1].x, x[r][2 * j + 1].y);
         }
-    }
 }
 
 // Fast forms for d_k = d_v = 128, bf16 inputs, paths of at most 16 nodes: one CTA of 256 threads per (tree, value head);
@@ -483,9 +489,13 @@ cudaError_t launch_commit_generic(const gdn_shape_t &s, float *S, const void *k,
                    parent, node_offsets, path, path_offsets, status_dev, 0, 0, 0, 0, nullptr, nullptr};
     if (s.d_k == GDN_TILE_D && s.d_v == GDN_TILE_D && s.in_dtype == GDN_BF16 && s.max_depth <= CF_MD)
         return launch_tile128(p, grid, stream);
-    const size_t smem = sizeof(float) * ((size_t)s.max_depth * CM_DK + 4 * (size_t)s.max_depth);   // at most 33 KB
-    return launch_overlapped(s.in_dtype == GDN_BF16 ? commit_generic_kernel<__nv_bfloat16> : commit_generic_kernel<float>, grid,
-                             CM_THREADS, smem, stream, p);
+    static PerDevice seen[2];
+    const auto kernel = s.in_dtype == GDN_BF16 ? commit_generic_kernel<__nv_bfloat16> : commit_generic_kernel<float>;
+    int sms = 0;
+    const cudaError_t e = device_sms(seen[s.in_dtype == GDN_BF16], reinterpret_cast<const void *>(kernel),
+                                     commit_generic_smem(GDN_MAX_DEPTH_CAP), &sms);
+    if (e != cudaSuccess) return e;
+    return launch_overlapped(kernel, grid, CM_THREADS, commit_generic_smem(s.max_depth), stream, p);
 }
 
 bool commit_tile128_supported(const gdn_shape_t &s) { return commit_padded_supported(s); }

@@ -181,19 +181,23 @@ __global__ void __launch_bounds__(VG_THREADS, 1) verify_generic_kernel(const Ver
 // X(l, t) = beta_l dec(l, t) (k_l.k_t) and y_it = dec(i, t) (q_i.k_t) along the root path of node i, row i of
 // Z = Y (I + X)^-1 is a back-substitution over that path alone, and
 //     o_i = S0^T q'_i + sum_t scale z_it beta_t v_t,      q'_i = scale (a_i q_i - sum_t z_it beta_t a_t k_t).
-// One CTA per (tree, value head, block of VS_NODES nodes); the tree metadata is derived from parent[] by every CTA (64
-// nodes: a walk of at most max_depth steps per thread), so no plan kernel runs in front.  Bound by FMA issue in the state
-// product (two rows of 32 key positions per thread against one read of q': 64 FMA per 8 shared-memory loads) and by
-// latency for small batches.  Against the kernel above, which visits the nodes of a tree one after the other: 8 trees of
-// 9..64 nodes, 32 heads of 128 components, fp32, verification and commit
-// 228 -> 79 us (the commit is 15 of them); one tree of 8 nodes, 4 heads of 32 components 26.6 -> 17.0 us.
+// One CTA per (tree, value head, run of blocks of VS_NODES nodes); the tree metadata is derived from parent[] by every CTA
+// (64 nodes: a walk of at most max_depth steps per thread), so no plan kernel runs in front.  Bound by shared memory
+// bandwidth (16-byte loads: the k rows in the dots, k and v rows in q' and outputs, q' in the state product, where eight
+// lanes hold four state rows so that a piece of q' serves four of them) and by latency for small batches.  Against the
+// kernel above, which visits the nodes of a tree one after the other: 8 trees of 9..64 nodes, 32 heads of 128 components,
+// fp32, verification alone: 61 us with one block per CTA, one dot per warp at a time, two rows per thread and v rows read
+// where they are used, 29 us in this form; verification and commit 230 -> 42 us; one tree of 8 nodes, 4 heads of 32
+// components 27.0 -> 10.4 us.
 constexpr int VS_THREADS = 256;
 constexpr int VS_TREE = 64;      // largest tree
-constexpr int VS_NODES = 16;     // nodes per CTA
-constexpr int VS_SPLIT = 4;      // lanes sharing two value components
+constexpr int VS_NODES = 16;     // nodes per block
+constexpr int VS_SPLIT = 8;      // lanes sharing four value components
+constexpr int VS_VROW = VG_DK + 4;   // floats of a staged v row: the eight lanes read one piece of eight different rows
 
 struct VerifySmallParams {
-    int h_qk, h_v, d_k, d_v, max_depth, max_tree_nodes, total_nodes, n_seq, n_blocks;
+    int h_qk, h_v, d_k, d_v, max_depth, max_tree_nodes, total_nodes, n_seq;
+    int n_parts, part_nodes;   // CTAs per (tree, head); nodes of each, a multiple of VS_NODES
     float scale;
     const float *S0;
     const void *q, *k, *v, *g, *beta;
@@ -202,21 +206,49 @@ struct VerifySmallParams {
     int32_t *status_dev;
 };
 
-template <typename T> __device__ __forceinline__ float4 load4_as_float(const T *p);
-template <> __device__ __forceinline__ float4 load4_as_float<float>(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
-template <> __device__ __forceinline__ float4 load4_as_float<__nv_bfloat16>(const __nv_bfloat16 *p)
+__device__ __forceinline__ float4 load4_as_float(const __nv_bfloat16 *p)
 {
     const uint2 w = __ldg(reinterpret_cast<const uint2 *>(p));
     return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xFFFF0000u), __uint_as_float(w.y << 16),
                        __uint_as_float(w.y & 0xFFFF0000u));
 }
 
+// Rows 0 .. rows - 1 of one head (d components, `stride` apart in memory) as fp32 into dst; fp32 rows by cp.async.
+template <typename T, int ROW>
+__device__ __forceinline__ void stage_rows(float (*dst)[ROW], const T *src, size_t stride, int rows, int d, int tid)
+{
+    if (d % 4 == 0) {
+#pragma unroll 4
+        for (int idx = tid; idx < rows * 32; idx += VS_THREADS) {
+            const int t = idx >> 5, r = (idx & 31) * 4;
+            if (r >= d) continue;
+            if constexpr (sizeof(T) == 4)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+                             ::"r"((uint32_t)__cvta_generic_to_shared(&dst[t][r])), "l"(src + t * stride + r) : "memory");
+            else
+                *reinterpret_cast<float4 *>(&dst[t][r]) = load4_as_float(src + t * stride + r);
+        }
+    } else {
+#pragma unroll 4
+        for (int idx = tid; idx < rows * VG_DK; idx += VS_THREADS) {
+            const int t = idx / VG_DK, r = idx % VG_DK;
+            if (r >= d) continue;
+            if constexpr (sizeof(T) == 4)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;"
+                             ::"r"((uint32_t)__cvta_generic_to_shared(&dst[t][r])), "l"(src + t * stride + r) : "memory");
+            else
+                dst[t][r] = load_as_float(src + t * stride + r);
+        }
+    }
+}
+
 struct VerifySmallSmem {
-    float ks[VS_TREE][VG_DK];              // k rows of the nodes this block needs
-    float qp[VS_NODES][VG_DK];             // q'
+    float ks[VS_TREE][VG_DK];              // k rows of the nodes up to the CTA's last
+    float vs[VS_TREE][VS_VROW];            // their v rows
+    float qp[2][VS_NODES][VG_DK];          // q rows of a block, then its q'
     float x[VS_TREE][VS_TREE];             // decays, then X(l, .): entry j belongs to the j-th node up the root path of l
-    float y[VS_NODES][VS_TREE];            // y, then the weights of the k rows; same order
-    float zv[VS_NODES][VS_TREE];           // weights of the v rows
+    float y[VS_NODES][2 * VS_TREE];        // y, then the weights of the k rows, same order; from VS_TREE on those of the v
+                                           // rows; then the v rows' part of the outputs
     float a[VS_TREE], beta[VS_TREE], g[VS_TREE];
     unsigned long long mask[VS_TREE];      // nodes on the root path
     int par[VS_TREE];
@@ -230,8 +262,8 @@ __global__ void __launch_bounds__(VS_THREADS, 2) verify_generic_small_kernel(con
     extern __shared__ __align__(16) uint8_t vs_smem[];
     VerifySmallSmem &sm = *reinterpret_cast<VerifySmallSmem *>(vs_smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int blk = blockIdx.x % p.n_blocks, bh = blockIdx.x / p.n_blocks, b = bh / p.h_v, h = bh % p.h_v;
-    const int hk = h / (p.h_v / p.h_qk), i0 = blk * VS_NODES;
+    const int part = blockIdx.x % p.n_parts, bh = blockIdx.x / p.n_parts, b = bh / p.h_v, h = bh % p.h_v;
+    const int hk = h / (p.h_v / p.h_qk), i_lo = part * p.part_nodes;
     const int d_k = p.d_k, d_v = p.d_v;
     const TIn *q = static_cast<const TIn *>(p.q), *k = static_cast<const TIn *>(p.k);
     const TIn *v = static_cast<const TIn *>(p.v), *g = static_cast<const TIn *>(p.g), *beta = static_cast<const TIn *>(p.beta);
@@ -247,21 +279,29 @@ __global__ void __launch_bounds__(VS_THREADS, 2) verify_generic_small_kernel(con
         if (tid == 0) report_status(p.status_dev, GDN_ERR_TREE);
         return;
     }
-    if (i0 >= T) return;
+    if (i_lo >= T) return;
+    const int i_hi = min(i_lo + p.part_nodes, T);
     if (tid < T) {
         sm.par[tid] = p.parent[base + tid];
         sm.g[tid] = load_as_float(g + (size_t)(base + tid) * p.h_v + h);
         sm.beta[tid] = load_as_float(beta + (size_t)(base + tid) * p.h_v + h);
     }
-    // State slice: rows c, c + 1; sreg[r][8 m + e] holds key position 16 j + 4 s + e, m = j / 2 (zero beyond d_k / d_v).
-    const int c = (tid / VS_SPLIT) * 2, s = tid % VS_SPLIT;
-    float2 sreg[2][VG_DK / VS_SPLIT / 2];
+    // Rows of the nodes up to the CTA's last (an ancestor has a smaller index) and the first block's q rows, then the state:
+    // all of it is under way while the root paths are walked.
+    const TIn *q_head = q + ((size_t)base * p.h_qk + hk) * d_k;
+    const size_t q_stride = (size_t)p.h_qk * d_k;
+    stage_rows(sm.ks, k + ((size_t)base * p.h_qk + hk) * d_k, q_stride, i_hi, d_k, tid);
+    stage_rows(sm.qp[0], q_head + i_lo * q_stride, q_stride, min(VS_NODES, i_hi - i_lo), d_k, tid);
+    stage_rows(sm.vs, v + ((size_t)base * p.h_v + h) * d_v, (size_t)p.h_v * d_v, i_hi, d_v, tid);
+    // State: rows c .. c + 3; sreg[r][2 j], [2 j + 1] hold key positions 32 j + 4 s + e (zero beyond d_k / d_v).
+    const int c = (tid / VS_SPLIT) * 4, s = tid % VS_SPLIT;
+    float2 sreg[4][8];
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
+    for (int r = 0; r < 4; ++r) {
         const float *row = p.S0 + ((size_t)(b * p.h_v + h) * d_v + (c + r < d_v ? c + r : 0)) * d_k;
 #pragma unroll
-        for (int j = 0; j < VG_DK / 16; ++j) {
-            const int at = 16 * j + 4 * s;
+        for (int j = 0; j < 4; ++j) {
+            const int at = 32 * j + 4 * s;
             float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
             if (c + r < d_v && at < d_k) x = __ldg(reinterpret_cast<const float4 *>(row + at));
             sreg[r][2 * j] = make_float2(x.x, x.y);
@@ -293,174 +333,226 @@ __global__ void __launch_bounds__(VS_THREADS, 2) verify_generic_small_kernel(con
         sm.a[tid] = expf(sfx);
     }
     if (err) report_status(p.status_dev, err);
+    asm volatile("cp.async.wait_all;" ::: "memory");
     if (__syncthreads_or(err != 0)) return;
-    const int nn = min(VS_NODES, T - i0);
-    unsigned long long need = 0;   // the block's nodes and their ancestors
-    for (int i = 0; i < nn; ++i) need |= sm.mask[i0 + i];
+    unsigned long long need = 0;   // the CTA's nodes and their ancestors
+    for (int i = i_lo; i < i_hi; ++i) need |= sm.mask[i];
     const int vecs = d_k / 4;
-    for (int idx = tid; idx < T * 32; idx += VS_THREADS) {
-        const int t = idx >> 5, r = idx & 31;
-        if (((need >> t) & 1) && r < vecs)
-            *reinterpret_cast<float4 *>(&sm.ks[t][4 * r]) = load4_as_float(k + ((size_t)(base + t) * p.h_qk + hk) * d_k + 4 * r);
-    }
-    __syncthreads();
 
-    // X and y: a warp per node, its lanes four key positions each
-    for (int l = warp; l < T; l += VS_THREADS / 32) {
-        if (!((need >> l) & 1)) continue;
-        const bool own = l >= i0 && l < i0 + nn;
-        float4 kl = make_float4(0.f, 0.f, 0.f, 0.f), ql = kl;
-        if (lane < vecs) {
-            kl = *reinterpret_cast<const float4 *>(&sm.ks[l][4 * lane]);
-            if (own) ql = load4_as_float(q + ((size_t)(base + l) * p.h_qk + hk) * d_k + 4 * lane);
-        }
-        const int d = sm.depth[l];
-        const float be = sm.beta[l];
-#pragma unroll 2
-        for (int j = own ? 0 : 1; j < d; ++j) {
-            float4 kt = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (lane < vecs) kt = *reinterpret_cast<const float4 *>(&sm.ks[sm.up[l][j]][4 * lane]);
-            float kk = fmaf(kl.x, kt.x, fmaf(kl.y, kt.y, fmaf(kl.z, kt.z, kl.w * kt.w)));
-            float qk = fmaf(ql.x, kt.x, fmaf(ql.y, kt.y, fmaf(ql.z, kt.z, ql.w * kt.w)));
-            // lanes 0..15 end up with kk, lanes 16..31 with qk
-            const float other = __shfl_xor_sync(0xffffffffu, lane & 16 ? kk : qk, 16);
-            float w = (lane & 16 ? qk : kk) + other;
-#pragma unroll
-            for (int m = 8; m > 0; m >>= 1) w += __shfl_xor_sync(0xffffffffu, w, m);
-            const float dec = sm.x[l][j];
-            __syncwarp();
-            if (lane == 0) sm.x[l][j] = be * dec * w;   // (entry 0, the node itself, is never read)
-            if (lane == 16 && own) sm.y[l - i0][j] = dec * w;
-        }
-    }
-    __syncthreads();
-
-    // z by back-substitution: 16 lanes per node, lane ln owning the entries ln, ln + 16, ... ; once z_j is final it is
-    // subtracted, times X(up_j, .), from the entries further up
-    {
-        const int i = tid >> 4, ln = tid & 15, n = i0 + i;
-        const int d = i < nn ? sm.depth[n] : 0;
-        const int d_warp = __reduce_max_sync(0xffffffffu, d);
-        float z[VS_TREE / 16];
-#pragma unroll
-        for (int e = 0; e < VS_TREE / 16; ++e) z[e] = ln + 16 * e < d ? sm.y[i][ln + 16 * e] : 0.f;
-#pragma unroll
-        for (int e = 0; e < VS_TREE / 16; ++e) {
-            if (16 * e >= d_warp - 1) break;
+    const int l8 = lane & 7;
+    // Block by block in ascending order, so that an ancestor's X is there; the buffer of the block after the next barrier
+    // takes the q rows of the block to come.
 #pragma unroll 1
-            for (int l = 0; l < 16; ++l) {
-                const int j = 16 * e + l;
-                if (j >= d_warp - 1) break;
-                const float zj = __shfl_sync(0xffffffffu, z[e], (lane & 16) | l);
-                if (j < d - 1) {
-                    const float *xr = sm.x[sm.up[n][j]];
+    for (int i0 = i_lo, buf = 0; i0 < i_hi; i0 += VS_NODES, buf ^= 1) {
+        const int nn = min(VS_NODES, i_hi - i0);
+        // X and y: a warp per node, eight lanes per path entry, four entries at a time; the first block also takes the
+        // ancestors in front of the CTA's nodes
+        for (int l = (i0 == i_lo ? 0 : i0) + warp; l < i0 + nn; l += VS_THREADS / 32) {
+            if (!((need >> l) & 1)) continue;
+            const bool own = l >= i0;
+            float4 kl[4], ql[4];
 #pragma unroll
-                    for (int f = e; f < VS_TREE / 16; ++f) {
-                        const int t = ln + 16 * f;
-                        if (t > j && t < d) z[f] = fmaf(-zj, xr[t - j], z[f]);
+            for (int m = 0; m < 4; ++m) {
+                const int r = l8 + 8 * m;
+                kl[m] = ql[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (r < vecs) {
+                    kl[m] = *reinterpret_cast<const float4 *>(&sm.ks[l][4 * r]);
+                    if (own) ql[m] = *reinterpret_cast<const float4 *>(&sm.qp[buf][l - i0][4 * r]);
+                }
+            }
+            const int d = sm.depth[l];
+            const float be = sm.beta[l];
+            for (int j0 = own ? 0 : 1; j0 < d; j0 += 8) {
+                float w[2], dec[2];
+                int j[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    j[e] = j0 + 4 * e + (lane >> 3);
+                    w[e] = dec[e] = 0.f;
+                    if (j0 + 4 * e >= d) break;
+                    const float *kr = sm.ks[j[e] < d ? sm.up[l][j[e]] : l];
+                    dec[e] = j[e] < d ? sm.x[l][j[e]] : 0.f;
+                    float4 k4 = make_float4(0.f, 0.f, 0.f, 0.f), q4 = k4;
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) {
+                        const int r = l8 + 8 * m;
+                        float4 kt = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (r < vecs) kt = *reinterpret_cast<const float4 *>(kr + 4 * r);
+                        k4 = make_float4(fmaf(kl[m].x, kt.x, k4.x), fmaf(kl[m].y, kt.y, k4.y), fmaf(kl[m].z, kt.z, k4.z),
+                                         fmaf(kl[m].w, kt.w, k4.w));
+                        q4 = make_float4(fmaf(ql[m].x, kt.x, q4.x), fmaf(ql[m].y, kt.y, q4.y), fmaf(ql[m].z, kt.z, q4.z),
+                                         fmaf(ql[m].w, kt.w, q4.w));
                     }
+                    // lanes 0..3 of the eight end up with k.k, lanes 4..7 with q.k
+                    const float kk = (k4.x + k4.y) + (k4.z + k4.w), qk = (q4.x + q4.y) + (q4.z + q4.w);
+                    w[e] = (lane & 4 ? qk : kk) + __shfl_xor_sync(0xffffffffu, lane & 4 ? kk : qk, 4);
+                }
+#pragma unroll
+                for (int e = 0; e < 2; ++e) w[e] += __shfl_xor_sync(0xffffffffu, w[e], 2);
+#pragma unroll
+                for (int e = 0; e < 2; ++e) w[e] += __shfl_xor_sync(0xffffffffu, w[e], 1);
+                __syncwarp();
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    if (j[e] < d && l8 == 0) sm.x[l][j[e]] = be * dec[e] * w[e];   // (entry 0, the node itself, is never read)
+                    if (j[e] < d && l8 == 4 && own) sm.y[l - i0][j[e]] = dec[e] * w[e];
                 }
             }
         }
-#pragma unroll
-        for (int e = 0; e < VS_TREE / 16; ++e) {
-            const int t = ln + 16 * e;
-            if (t < d) {
-                const int m = sm.up[n][t];
-                const float w = p.scale * z[e] * sm.beta[m];
-                sm.zv[i][t] = w;
-                sm.y[i][t] = w * sm.a[m];
-            }
-        }
-    }
-    __syncthreads();
+        __syncthreads();
+        if (i0 + VS_NODES < i_hi)
+            stage_rows(sm.qp[buf ^ 1], q_head + (i0 + VS_NODES) * q_stride, q_stride, min(VS_NODES, i_hi - i0 - VS_NODES), d_k, tid);
 
-    // q': 16 lanes per node, eight key positions each
-    {
-        const int i = tid >> 4, ln = tid & 15, n = i0 + i;
-        if (i < nn) {
-            const int d = sm.depth[n];
-            const float sa = p.scale * sm.a[n];
+        // z by back-substitution: 16 lanes per node, lane ln owning the entries ln, ln + 16, ... ; once z_j is final it is
+        // subtracted, times X(up_j, .), from the entries further up
+        {
+            const int i = tid >> 4, ln = tid & 15, n = i0 + i;
+            const int d = i < nn ? sm.depth[n] : 0;
+            const int d_warp = __reduce_max_sync(0xffffffffu, d);
+            float z[VS_TREE / 16];
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                const int r = half * 64 + ln * 4;
-                float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (r < d_k) {
-                    w = load4_as_float(q + ((size_t)(base + n) * p.h_qk + hk) * d_k + r);
-                    w = make_float4(sa * w.x, sa * w.y, sa * w.z, sa * w.w);
-                    for (int t = 0; t < d; ++t) {
-                        const float cf = -sm.y[i][t];
-                        const float4 kt = *reinterpret_cast<const float4 *>(&sm.ks[sm.up[n][t]][r]);
-                        w = make_float4(fmaf(cf, kt.x, w.x), fmaf(cf, kt.y, w.y), fmaf(cf, kt.z, w.z), fmaf(cf, kt.w, w.w));
+            for (int e = 0; e < VS_TREE / 16; ++e) z[e] = ln + 16 * e < d ? sm.y[i][ln + 16 * e] : 0.f;
+#pragma unroll
+            for (int e = 0; e < VS_TREE / 16; ++e) {
+                if (16 * e >= d_warp - 1) break;
+#pragma unroll 1
+                for (int l = 0; l < 16; ++l) {
+                    const int j = 16 * e + l;
+                    if (j >= d_warp - 1) break;
+                    const float zj = __shfl_sync(0xffffffffu, z[e], (lane & 16) | l);
+                    if (j < d - 1) {
+                        const float *xr = sm.x[sm.up[n][j]];
+#pragma unroll
+                        for (int f = e; f < VS_TREE / 16; ++f) {
+                            const int t = ln + 16 * f;
+                            if (t > j && t < d) z[f] = fmaf(-zj, xr[t - j], z[f]);
+                        }
                     }
                 }
-                *reinterpret_cast<float4 *>(&sm.qp[i][r]) = w;
+            }
+#pragma unroll
+            for (int e = 0; e < VS_TREE / 16; ++e) {
+                const int t = ln + 16 * e;
+                if (t < d) {
+                    const int m = sm.up[n][t];
+                    const float w = p.scale * z[e] * sm.beta[m];
+                    sm.y[i][VS_TREE + t] = w;
+                    sm.y[i][t] = w * sm.a[m];
+                }
             }
         }
-    }
-    __syncthreads();
+        __syncthreads();
 
-    // outputs, four nodes at a time: the four lanes of a row pair share key positions and path entries; the eight sums
-    // (four nodes x two rows) are folded into one another so that lane s ends up with those of node s
-#pragma unroll 1
-    for (int ib = 0; ib < nn; ib += 4) {
-        float acc[4][2];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int i = ib + u;
-            float2 s0 = make_float2(0.f, 0.f), s1 = s0;
+        // q' over the q rows, and the v rows' part of the outputs over the weights: 16 lanes per node, eight key positions and
+        // eight components each
+        {
+            const int i = tid >> 4, ln = tid & 15, n = i0 + i;
             if (i < nn) {
+                const int d = sm.depth[n];
+                const float sa = p.scale * sm.a[n];
+                float4 w[2], ov[2];
 #pragma unroll
-                for (int j = 0; j < VG_DK / 16; ++j) {
-                    const float4 x = *reinterpret_cast<const float4 *>(&sm.qp[i][16 * j + 4 * s]);
-                    s0 = __ffma2_rn(sreg[0][2 * j], make_float2(x.x, x.y), s0);
-                    s1 = __ffma2_rn(sreg[1][2 * j], make_float2(x.x, x.y), s1);
-                    s0 = __ffma2_rn(sreg[0][2 * j + 1], make_float2(x.z, x.w), s0);
-                    s1 = __ffma2_rn(sreg[1][2 * j + 1], make_float2(x.z, x.w), s1);
-                }
-                const int d = sm.depth[i0 + i];
-                if (c < d_v) {
-                    const int c1 = c + 1 < d_v ? c + 1 : c;
-#pragma unroll 2
-                    for (int t = s; t < d; t += VS_SPLIT) {
-                        const TIn *vr = v + ((size_t)(base + sm.up[i0 + i][t]) * p.h_v + h) * d_v;
-                        const float w = sm.zv[i][t];
-                        s0.x = fmaf(w, load_as_float(vr + c), s0.x);
-                        s1.x = fmaf(w, load_as_float(vr + c1), s1.x);
+                for (int half = 0; half < 2; ++half) {
+                    const int r = half * 64 + ln * 4;
+                    w[half] = ov[half] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (r < d_k) {
+                        const float4 x = *reinterpret_cast<const float4 *>(&sm.qp[buf][i][r]);
+                        w[half] = make_float4(sa * x.x, sa * x.y, sa * x.z, sa * x.w);
                     }
                 }
+#pragma unroll 2
+                for (int t = 0; t < d; ++t) {
+                    const float cf = -sm.y[i][t], cv = sm.y[i][VS_TREE + t];
+                    const int m = sm.up[n][t];
+                    const float *kr = sm.ks[m], *vr = sm.vs[m];
+#pragma unroll
+                    for (int half = 0; half < 2; ++half) {
+                        const int r = half * 64 + ln * 4;
+                        if (r < d_k) {
+                            const float4 kt = *reinterpret_cast<const float4 *>(&kr[r]);
+                            w[half] = make_float4(fmaf(cf, kt.x, w[half].x), fmaf(cf, kt.y, w[half].y), fmaf(cf, kt.z, w[half].z),
+                                                  fmaf(cf, kt.w, w[half].w));
+                        }
+                        const float4 vt = *reinterpret_cast<const float4 *>(&vr[r]);   // (components beyond d_v are not stored)
+                        ov[half] = make_float4(fmaf(cv, vt.x, ov[half].x), fmaf(cv, vt.y, ov[half].y), fmaf(cv, vt.z, ov[half].z),
+                                               fmaf(cv, vt.w, ov[half].w));
+                    }
+                }
+                __syncwarp(0xffffu << (lane & 16));   // the node's weights have been read
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    *reinterpret_cast<float4 *>(&sm.qp[buf][i][half * 64 + ln * 4]) = w[half];
+                    *reinterpret_cast<float4 *>(&sm.y[i][half * 64 + ln * 4]) = ov[half];
+                }
             }
-            acc[u][0] = s0.x + s0.y;
-            acc[u][1] = s1.x + s1.y;
         }
-        float half_sum[2][2], out[2];
-        const bool odd = (s & 1) != 0, high = (s & 2) != 0;
+        __syncthreads();
+
+        // outputs, four nodes at a time: the eight lanes of four rows share key positions and path entries; the sixteen sums
+        // (four nodes x four rows) are folded into one another so that lane s ends up with two rows of node s >> 1
+#pragma unroll 1
+        for (int ib = 0; ib < nn; ib += 4) {
+            float acc[4][4];
 #pragma unroll
-        for (int u = 0; u < 2; ++u)
+            for (int u = 0; u < 4; ++u) {
+                float2 sum[4];   // (of no use from node nn on)
 #pragma unroll
-            for (int r = 0; r < 2; ++r)   // keep nodes u * 2 + (s & 1)
-                half_sum[u][r] = (odd ? acc[2 * u + 1][r] : acc[2 * u][r]) +
-                                 __shfl_xor_sync(0xffffffffu, odd ? acc[2 * u][r] : acc[2 * u + 1][r], 1);
+                for (int r = 0; r < 4; ++r) sum[r] = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int r = 0; r < 2; ++r)
-            out[r] = (high ? half_sum[1][r] : half_sum[0][r]) + __shfl_xor_sync(0xffffffffu, high ? half_sum[0][r] : half_sum[1][r], 2);
-        if (ib + s < nn) {
-            TOut *dst = o + ((size_t)(base + i0 + ib + s) * p.h_v + h) * d_v + c;
-            if (c < d_v) store_from_float(dst, out[0]);
-            if (c + 1 < d_v) store_from_float(dst + 1, out[1]);
+                for (int j = 0; j < 4; ++j) {
+                    const float4 x = *reinterpret_cast<const float4 *>(&sm.qp[buf][ib + u][32 * j + 4 * s]);
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        sum[r] = __ffma2_rn(sreg[r][2 * j], make_float2(x.x, x.y), sum[r]);
+                        sum[r] = __ffma2_rn(sreg[r][2 * j + 1], make_float2(x.z, x.w), sum[r]);
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < 4; ++r) acc[u][r] = sum[r].x + sum[r].y;
+            }
+            const bool b2 = (s & 4) != 0, b1 = (s & 2) != 0, b0 = (s & 1) != 0;
+            float f2[2][4], f1[4], out[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+#pragma unroll
+                for (int r = 0; r < 4; ++r)   // keep nodes 2 (s >> 2) + u
+                    f2[u][r] = (b2 ? acc[2 + u][r] : acc[u][r]) + __shfl_xor_sync(0xffffffffu, b2 ? acc[u][r] : acc[2 + u][r], 4);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) f1[r] = (b1 ? f2[1][r] : f2[0][r]) + __shfl_xor_sync(0xffffffffu, b1 ? f2[0][r] : f2[1][r], 2);
+#pragma unroll
+            for (int r = 0; r < 2; ++r) out[r] = (b0 ? f1[2 + r] : f1[r]) + __shfl_xor_sync(0xffffffffu, b0 ? f1[r] : f1[2 + r], 1);
+            const int i = ib + (s >> 1), c2 = c + 2 * (s & 1);
+            if (i < nn) {
+                TOut *dst = o + ((size_t)(base + i0 + i) * p.h_v + h) * d_v + c2;
+                const float2 ov = *reinterpret_cast<const float2 *>(&sm.y[i][c2]);
+                if (c2 < d_v) store_from_float(dst, out[0] + ov.x);
+                if (c2 + 1 < d_v) store_from_float(dst + 1, out[1] + ov.y);
+            }
         }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();   // the next block's q rows are there; y, zv and this block's q' have been read
     }
 }
 
 template <typename TIn, typename TOut>
-cudaError_t launch_small_typed(const VerifySmallParams &p, cudaStream_t stream)
+cudaError_t launch_small_typed(VerifySmallParams p, cudaStream_t stream)
 {
     static PerDevice seen;
-    const int grid = p.n_seq * p.h_v * p.n_blocks;
     int sms = 0;
     const cudaError_t e = device_sms(seen, reinterpret_cast<const void *>(verify_generic_small_kernel<TIn, TOut>),
                                      sizeof(VerifySmallSmem), &sms);
     if (e != cudaSuccess) return e;
+    // Blocks per CTA: as few as let all CTAs be resident at once, so that small calls spread over the SMs; a CTA reads rows
+    // and state once for all of its blocks.  No more than three: a fourth leaves the largest trees as the tail of the call,
+    // as CTAs of their own the last blocks fill in behind the small trees (8 trees of 10..54 nodes, 32 heads, fp32; 1 / 2 / 3 /
+    // 4 blocks per CTA: 35.0 / 34.8 / 29.4 / 34.4 us).
+    const int blocks = (p.max_tree_nodes + VS_NODES - 1) / VS_NODES;
+    const long long heads = (long long)p.n_seq * p.h_v;
+    int per = 1;
+    while (per < min(blocks, 3) && heads * ((blocks + per - 1) / per) > 2 * sms) ++per;
+    p.part_nodes = per * VS_NODES;
+    p.n_parts = (blocks + per - 1) / per;
+    const long long grid = heads * p.n_parts;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(VS_THREADS);
@@ -502,7 +594,7 @@ cudaError_t launch_verify_generic_small(const gdn_shape_t &s, const float *S0, c
 {
     if (s.n_seq == 0 || s.total_nodes == 0) return cudaSuccess;
     const VerifySmallParams p{s.h_qk, s.h_v, s.d_k, s.d_v, s.max_depth, s.max_tree_nodes, s.total_nodes, s.n_seq,
-                              (s.max_tree_nodes + VS_NODES - 1) / VS_NODES, s.scale, S0, q, k, v, g, beta, parent,
+                              0, 0, s.scale, S0, q, k, v, g, beta, parent,
                               node_offsets, o, status_dev};
     const bool in_bf = s.in_dtype == GDN_BF16, out_bf = s.out_dtype == GDN_BF16;
     if (in_bf && out_bf) return launch_small_typed<__nv_bfloat16, __nv_bfloat16>(p, stream);

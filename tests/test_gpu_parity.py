@@ -111,9 +111,11 @@ def test_edge_shapes(tl, name, dims):
 
 
 @pytest.mark.parametrize("dims", [(2, 6, 128, 127, synth.F32, synth.F32), (1, 2, 4, 1, synth.F32, synth.F32),
-                                  (2, 2, 100, 65, synth.BF16, synth.BF16)])
+                                  (2, 2, 100, 65, synth.BF16, synth.BF16), (1, 20, 36, 40, synth.F32, synth.F32),
+                                  (2, 24, 64, 33, synth.BF16, synth.F32)])
 def test_general_path_node_blocks(tl, dims):
-    """General path on trees around its block of 16 nodes, with root paths of up to 64 nodes (tolerance: fp32 sums)."""
+    """General path on trees around its block of 16 nodes, one, two and four blocks per CTA, with root paths of up to 64
+    nodes (tolerance: fp32 sums)."""
     h_qk, h_v, d_k, d_v, idt, odt = dims
     rng = np.random.default_rng(71)
     trees = [synth.tree_geo(rng, T) for T in (1, 15, 16, 17, 33, 63)] + [synth.tree_chain(64)]
