@@ -450,12 +450,11 @@ template <int CTAS> __global__ void __launch_bounds__(CF_THREADS, CTAS) commit_t
 // The fused call on trees of more than 64 nodes: the plans of the NEW trees do not depend on the commit of the previous
 // step's paths, so they are built by the first n_seq CTAs of the same grid instead of by a launch of their own in
 // between (one launch and one dependency hop less in front of the verify kernel).
-static_assert(PLAN_THREADS == CF_THREADS, "the plan CTAs and the commit CTAs share a block size");
 template <int CTAS> __global__ void __launch_bounds__(CF_THREADS, CTAS) commit_plan_kernel(const CommitParams p, const PlanArgs a)
 {
     if ((int)blockIdx.x < a.n_seq) {
         wait_for_previous_kernel();
-        plan_tree(a, (int)blockIdx.x);
+        plan_tree<CF_THREADS>(a, (int)blockIdx.x);
     } else
         commit_unit<CTAS>(p, (int)blockIdx.x - a.n_seq);
 }

@@ -18,7 +18,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_kernel(const PlanArgs a)
     // may be launched early in turn; it waits for this grid to finish before it reads anything written here.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
-    plan_tree(a, (int)blockIdx.x);
+    plan_tree<PLAN_THREADS>(a, (int)blockIdx.x);
 }
 
 }  // namespace
