@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
     const uint32_t mbar_kq = mbar_g + 24, mbar_v = mbar_g + 32;
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-    // The asynchronous work is issued by one elected lane each of four warps: warp 0 C and V^T.z', warp 1 the last product,
+    // The asynchronous work is issued by one elected lane each of four warps: warp 0 C, warp 1 V^T.z' and the last product,
     // warp 2 the Gram block of the unit to come, warp 3 the TMA loads; warps 2 and 3 also keep the tree tables (thread
     // 64 + i: node i).
     constexpr int W_MMA_C = 0, W_MMA_O = 1, W_MMA_G = 2, W_TMA = 3;
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
     if (warp == 0) tmem_alloc(sbase + SP_TMEM, TM_COLS);
     if (tid == 32) {
         mbar_init(mbar_g, 1);
-        mbar_init(mbar_c, 1);
+        mbar_init(mbar_c, 2);   // C and V^T.z'
         mbar_init(mbar_o, 1);
         mbar_init(mbar_kq, GROUPED ? VP_THREADS : 1);   // gathered rows: every thread arrives once its copies have landed
         mbar_init(mbar_v, GROUPED ? VP_THREADS : 1);
@@ -373,10 +373,11 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
 
     // ------------------------------------------------------------------------------------ tree tables
     // Thread 64 + i keeps node i.  tables_load() asks for its parent and gates (registers), tables_put() stages parent and
-    // log decay in shared memory, and behind a barrier tables_walk() climbs from the node to its root, shifting each id
+    // log decay in shared memory, and behind a barrier tables_build() climbs from the node to its root, shifting each id
     // into a 16-byte row from below (the root ends up in byte 0), collecting the ancestor mask and the path sum of g.  A
-    // tree with a bad parent[] or a root path of more than max_depth nodes is reported and runs as a tree of no nodes.
-    // GROUPED: parents in virtual indices from the plan.
+    // tree with a bad parent[] or a root path of more than max_depth nodes is reported and runs as a tree of no nodes.  A
+    // climb is a chain of shared-memory loads: the units of a tree share the rows (and the verdict) of its first one, and
+    // GROUPED takes them, in virtual indices, from the plan; what is left is the sum of g over the row.
     signed char *par_s = reinterpret_cast<signed char *>(smem + SP_PAR);
     float *g_s = reinterpret_cast<float *>(smem + SP_G);
     volatile int *bad_s = reinterpret_cast<volatile int *>(smem + SP_BAD);
@@ -388,7 +389,7 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
             nr.beta = __ldg(reinterpret_cast<const unsigned short *>(p.beta) + n);
         }
     };
-    auto tables_load = [&](const Unit &un, NodeRaw &nr) {
+    auto tables_load = [&](const Unit &un, NodeRaw &nr, const bool same_tree) {
         nr.par = -1;
         nr.node = 0;
         nr.g = nr.beta = 0;
@@ -396,38 +397,72 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
             nr.node = tnode;
             if constexpr (GROUPED) {
                 nr.node = vnode_of(un, tnode);
-                if (un.ident) {
-                    const int d = p.depth[un.pb + tnode];
-                    if (d > 1) nr.par = p.anc8[(size_t)(un.pb + tnode) * 16 + d - 2];
-                } else if (tnode < un.n_prefix) {   // an ancestor of the group's first node: its path is 0..tnode
-                    nr.par = tnode - 1;
-                } else {
-                    const int r = un.pb + un.g0 + tnode - un.n_prefix, d = p.dfs_depth[r];
-                    if (d > 1) nr.par = p.dfs_anc8[(size_t)r * 16 + d - 2];
+                if (!un.ident && tnode < un.n_prefix) {   // an ancestor of the group's first node: its path is 0..tnode
+                    const uint32_t ids[4] = {0x03020100u, 0x07060504u, 0x0B0A0908u, 0x0F0E0D0Cu};
+                    uint32_t w[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int n = min(max(tnode + 1 - 4 * e, 0), 4);
+                        w[e] = n == 4 ? ids[e] : ids[e] | 0xFFFFFFFFu << (8 * n);
+                    }
+                    *reinterpret_cast<uint4 *>(smem + SP_ANC + tnode * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+                } else {   // (the rows of the unit before have been read)
+                    cp_async_16(sbase + SP_ANC + tnode * 16, un.ident ? p.anc8 + (size_t)(un.pb + tnode) * 16
+                                                                      : p.dfs_anc8 + (size_t)(un.pb + un.g0 + tnode - un.n_prefix) * 16, true);
+                    asm volatile("cp.async.commit_group;" ::: "memory");
                 }
             } else {
-                nr.par = __ldg(p.parent + un.par0 + tnode);
+                if (!same_tree) nr.par = __ldg(p.parent + un.par0 + tnode);
                 gates_load(un, nr);
             }
         }
     };
     bool my_bad = false;
-    auto tables_put = [&](const Unit &un, const NodeRaw &nr) {
+    auto tables_put = [&](const Unit &un, const NodeRaw &nr, const bool same_tree) {
         if (tbl_thread) {
-            int pv = nr.par;
-            my_bad = tnode < un.T && (pv < -1 || pv >= tnode);
-            if (my_bad) pv = -1;
-            par_s[tnode] = (signed char)pv;
+            if (!GROUPED && !same_tree) {
+                int pv = nr.par;
+                my_bad = tnode < un.T && (pv < -1 || pv >= tnode);
+                if (my_bad) pv = -1;
+                par_s[tnode] = (signed char)pv;
+            }
             g_s[tnode] = gate_log_decay(nr.g, PADDED && p.raw_gates);
             if constexpr (GROUPED) vnode_s[tnode] = (uint16_t)nr.node;
         }
-        if (tid == 0) *bad_s = 0;
+        if (tid == 0 && !same_tree) *bad_s = 0;
     };
-    auto tables_walk = [&](const Unit &un, const NodeRaw &nr) {
-        if (tbl_thread) {
+    auto tables_build = [&](const Unit &un, const NodeRaw &nr, const bool same_tree) {
+        if (!tbl_thread) return;
+        float G = 0.f;
+        if (GROUPED || same_tree) {
+            if constexpr (GROUPED) asm volatile("cp.async.wait_group 0;" ::: "memory");   // (the row copies are in no group)
+            uint4 path = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
+            if (tnode < un.T) path = *reinterpret_cast<const uint4 *>(smem + SP_ANC + tnode * 16);
+            const uint32_t w[4] = {path.x, path.y, path.z, path.w};
+            uint32_t mlo = 0, mhi = 0;
+            float sum[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if (!__any_sync(0xffffffffu, w[e] != 0xFFFFFFFFu)) break;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const uint32_t id = (w[e] >> (8 * c)) & 0xFFu;
+                    const float gv = g_s[id & 63u];
+                    if (id != 0xFFu) sum[c] += gv;
+                    if constexpr (GROUPED) {
+                        if (id < 32u) mlo |= 1u << id;
+                        else if (id < 64u) mhi |= 1u << (id - 32u);
+                    }
+                }
+            }
+            G = (sum[0] + sum[1]) + (sum[2] + sum[3]);
+            if constexpr (GROUPED) {
+                if (tnode >= un.T) *reinterpret_cast<uint4 *>(smem + SP_ANC + tnode * 16) = path;
+                *reinterpret_cast<uint2 *>(smem + SP_AMASK + tnode * 8) = make_uint2(mlo, mhi);
+            }
+        } else {
             int d = 0, err = my_bad ? GDN_ERR_TREE : 0, c = tnode < un.T && !err ? tnode : -1;
             uint32_t w0 = 0xFFFFFFFFu, w1 = 0xFFFFFFFFu, w2 = 0xFFFFFFFFu, w3 = 0xFFFFFFFFu, mlo = 0, mhi = 0;
-            float G = 0.f;
 #pragma unroll 1
             while (c >= 0) {
                 if (++d > p.max_depth) { err = GDN_ERR_DEPTH; break; }
@@ -448,9 +483,9 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
             }
             *reinterpret_cast<uint4 *>(smem + SP_ANC + tnode * 16) = make_uint4(w0, w1, w2, w3);
             *reinterpret_cast<uint2 *>(smem + SP_AMASK + tnode * 8) = make_uint2(mlo, mhi);
-            *reinterpret_cast<float2 *>(smem + SP_GB + tnode * 8) = make_float2(G, gate_beta(nr.beta, PADDED && p.raw_gates));
-            reinterpret_cast<float *>(smem + SP_SA)[tnode] = p.scale * __expf(G);
         }
+        *reinterpret_cast<float2 *>(smem + SP_GB + tnode * 8) = make_float2(G, gate_beta(nr.beta, PADDED && p.raw_gates));
+        reinterpret_cast<float *>(smem + SP_SA)[tnode] = p.scale * __expf(G);
     };
 
     // ------------------------------------------------------------------------------------ first unit
@@ -463,9 +498,9 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
             issue_kq(un);
             issue_v(un);
         }
-        tables_load(un, nr);
+        tables_load(un, nr, false);
         if constexpr (GROUPED) gates_load(un, nr);
-        tables_put(un, nr);
+        tables_put(un, nr, false);
     }
     __syncthreads();
     if (have) {
@@ -473,7 +508,7 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
             issue_kq(un);
             issue_v(un);
         }
-        tables_walk(un, nr);
+        tables_build(un, nr, false);
         issue_gram(un.T, 0);
         rows_parity = 1;
     }
@@ -625,11 +660,8 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
         tc_fence_after();
         // (4) C = -sa w.K (nodes on the lanes) and O = V^T.z' (value components on the lanes)
         if (warp == W_MMA_C && elect_one()) {
-            constexpr uint32_t id_c = idesc_bf16(64, 64) | (1u << 16);                         // B: rows along K (nodes)
-            const uint32_t id_v = idesc_bf16(128, 0) | (1u << 15) | (uint32_t)(nk * 2) << 17;   // A: rows along K (nodes)
-            const uint64_t w_hi = smem_desc_sw128(sbase + SP_WZ), z_hi = w_hi + 1024;
-            const uint64_t k0 = smem_desc_sw128(sbase + SP_KQ);
-            const uint64_t v0 = smem_desc_sw128(sbase + SP_V) + (511ull << 16);   // halves 8 KB apart
+            constexpr uint32_t id_c = idesc_bf16(64, 64) | (1u << 16);   // B: rows along K (nodes)
+            const uint64_t w_hi = smem_desc_sw128(sbase + SP_WZ), k0 = smem_desc_sw128(sbase + SP_KQ);
 #pragma unroll 1
             for (int ks = 0; ks < nk; ++ks) {
 #pragma unroll
@@ -637,18 +669,40 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
                     const uint32_t acc = (ks | part) != 0;
                     umma_bf16(tmem + TM_GC, w_hi + (uint64_t)(part * 512 + ks * 2), k0 + (uint64_t)(ks * 128), id_c, acc);
                     umma_bf16(tmem + TM_GC + (16u << 16), w_hi + (uint64_t)(part * 512 + ks * 2), k0 + (uint64_t)(1024 + ks * 128), id_c, acc);
-                    umma_bf16(tmem + TM_O, v0 + (uint64_t)(ks * 128), z_hi + (uint64_t)(part * 512 + ks * 2), id_v, acc);
                 }
             }
+            umma_commit(mbar_c);
+        } else if (warp == W_MMA_O && elect_one()) {
+            const uint32_t id_v = idesc_bf16(128, 0) | (1u << 15) | (uint32_t)(nk * 2) << 17;   // A: rows along K (nodes)
+            const uint64_t z_hi = smem_desc_sw128(sbase + SP_WZ) + 1024;
+            const uint64_t v0 = smem_desc_sw128(sbase + SP_V) + (511ull << 16);   // halves 8 KB apart
+#pragma unroll 1
+            for (int ks = 0; ks < nk; ++ks)
+#pragma unroll
+                for (int part = 0; part < 2; ++part)
+                    umma_bf16(tmem + TM_O, v0 + (uint64_t)(ks * 128), z_hi + (uint64_t)(part * 512 + ks * 2), id_v, (ks | part) != 0);
             umma_commit(mbar_c);
         }
         // the next unit: its place and its tables (registers)
         const bool have_n = pull(nx);
         const bool next_rows = have_n && (GROUPED || nx.b != un.b || hk_of(nx.h) != hk_of(un.h));
+        const bool same_tree = !GROUPED && have_n && (PADDED ? tree_of(nx.b) == tree_of(un.b) : nx.b == un.b);
         if (have_n) {
-            tables_load(nx, nr);
-            if (tid < 4 && (!GROUPED || nx.fresh))   // ... and its state tile into L2
+            tables_load(nx, nr, same_tree);
+            if (tid < 4 && (!GROUPED || nx.fresh))   // ... and its state tile and, not gathered, its rows into L2
                 prefetch_l2_bulk(p.S0 + (size_t)(nx.b * p.h_v + nx.h) * VP_D * VP_D + (size_t)tid * 4096, 16384);
+            if (!GROUPED && tbl_thread && tnode < nx.T) {
+                const size_t n = (size_t)(nx.base + tnode);
+                auto prefetch_row = [](const __nv_bfloat16 *r) {
+                    asm volatile("prefetch.global.L2 [%0];\n\tprefetch.global.L2 [%0 + 128];" ::"l"(r));
+                };
+                prefetch_row(p.v + (n * p.h_v + nx.h) * VP_D);
+                if (next_rows) {
+                    const size_t hk = (size_t)hk_of(nx.h);
+                    prefetch_row(p.k + (n * p.h_qk + hk) * VP_D);
+                    prefetch_row(p.q + (n * p.h_qk + hk) * VP_D);
+                }
+            }
         }
         if (state_late) {
             wait_for_previous_kernel();
@@ -718,7 +772,7 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
             for (int e = 0; e < VP_T / ROWS_STEP; ++e) out_ids[e] = vnode_s[tid / CHUNKS + e * ROWS_STEP];
             __syncthreads();
         }
-        if (have_n) tables_put(nx, nr);
+        if (have_n) tables_put(nx, nr, same_tree);
         fence_proxy_async();
         tc_fence_before();
         __syncthreads();
@@ -740,7 +794,7 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
         if (have_n) {
             if (next_rows) issue_kq(nx);
             issue_v(nx);
-            tables_walk(nx, nr);
+            tables_build(nx, nr, same_tree);
         }
         if (!mbar_wait_bounded(mbar_o, par)) *flag = 1;
         tc_fence_after();
