@@ -18,9 +18,9 @@
 // memory: the tile goes there from registers without passing through shared memory.
 //
 // Measured against the kernel that formed S0^T k and S0^T q and a right-hand side per node (same two CTAs per SM): 48
-// slots x 32 heads, 64-node tree, verification then commit as two calls 110.0 -> 95.7 us; 256-node trees, fused call
-// (commit kernel + this one) 324 -> 284 us; 32 ragged trees of 16..256 nodes 132 -> 123 us; one layer of 512 nodes 25.7 ->
-// 24.6 us.
+// slots x 32 heads, 64-node tree, verification then commit as two calls 110 -> 84 us (the commit from 48 to 43 of it);
+// 256-node trees, fused call (commit kernel + this one) 324 -> 263 us; 32 ragged trees of 16..256 nodes 132 -> 121 us; one
+// layer of 512 nodes, plan included, 29.7 -> 24.7 us.
 //
 // What bounds it: the chain of a unit (Gram -> lists -> back-substitution -> C -> q' -> output product -> rows), not memory
 // and not the tensor pipe; so the unit has as few instructions and barriers as could be found, two CTAs share an SM and
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
     const int u_first = (int)((long long)p.n_units * cta / (int)gridDim.x);   // (not GROUPED)
     if constexpr (!GROUPED) {
         if (tid < 4) prefetch_l2_bulk(p.S0 + (size_t)u_first * VP_D * VP_D + (size_t)tid * 4096, 16384);
-        if (tid >= 128 && tid < 128 + VP_T && tid - 128 < p.max_tree_nodes) {
+        if (!p.state_late && tid >= 128 && tid < 128 + VP_T && tid - 128 < p.max_tree_nodes) {
             const int ub = u_first / p.h_v, uh = u_first % p.h_v, uhk = uh / (p.h_v / p.h_qk);
             const int row = (PADDED ? ub * p.t_pad : __ldg(p.node_offsets + ub)) + tid - 128;
             if (row >= 0 && row < p.total_nodes) {
@@ -170,7 +170,8 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
         }
     }
     // state_late: the kernel in front is the commit of the same call, which itself has waited for everything before it and
-    // writes nothing but the state; only the first use of a state tile waits for it.
+    // writes nothing but the state; only the first use of a state tile waits for it (and the rows are loaded right away:
+    // prefetches would only stand in front of the loads, one layer 9.4 -> 11.7 us).
     bool state_late = !GROUPED && p.state_late;
     auto wait_for_previous_kernel = [&]() {
         asm volatile("griddepcontrol.wait;" ::: "memory");
