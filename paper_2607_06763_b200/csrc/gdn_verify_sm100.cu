@@ -1,6 +1,5 @@
 // Commit of the previous step's paths and tree verification in one kernel (gdn_verify_plain.cu: verification alone) for
-// sm_100a: d_k = d_v = 128, bf16 inputs, root paths of at most 16 nodes, at most 64 nodes
-// per unit of work (larger trees are cut into ancestor-closed groups, each a unit of its own).  It evaluates the
+// sm_100a: d_k = d_v = 128, bf16 inputs, root paths of at most 16 nodes, trees of at most 64 nodes.  It evaluates the
 // triangular form of Section 3.4.1 (Eq. 9-11) restricted to real ancestors, with the W S0 term folded into the
 // right-hand side as in Section 3.4.2, and turns all of the per-component work into dense contractions on the
 // 5th-generation tensor cores (tcgen05.mma, bf16 operands, fp32 accumulators in tensor memory):
@@ -20,9 +19,13 @@
 //
 // Operand orientation: d_v on the TMEM lanes, nodes on the TMEM columns, so every thread of a warp owns one value
 // component.  256 threads, about 112 KB of shared memory and 256 TMEM columns per CTA, so two CTAs share an SM.
-// One persistent kernel: a software pipeline across the units of a CTA, TMA tiles on mbarriers for trees that fit
-// one unit (optionally with the commit of the previous step fused in front), row gathers through the plan's node
-// table for the groups of larger trees.
+// One persistent kernel: a software pipeline across the units of a CTA, TMA tiles on mbarriers, the commit of the previous
+// step in front of each unit's verification, on the same registers.
+//
+// What bounds it: the chain of a unit together with the FMA of the replay (about 364 cycles per step and SM), not memory;
+// the state crosses HBM once each way.  48 slots x 32 heads, 64 nodes, path of 7: 84.5 us (43 of memory traffic).  Of the
+// forms tried for it -- one CTA per SM with specialised warps, the replay as matrix products on the fragments, the commit
+// and verify kernels back to back (86.6 us; 72 against 84 at a path of 1) -- none is faster over the path lengths.
 #include "gdn_internal.cuh"
 #include "gdn_replay.cuh"
 #include "gdn_tc.cuh"
@@ -67,18 +70,16 @@ constexpr int SM_TMEM = SM_MBAR + 40;            // u32
 constexpr int SM_FLAG = SM_TMEM + 4;             // u32 (timeout flag)
 constexpr int SM_PAR = SM_FLAG + 4;              // s8 [64] parent[] of the tree whose tables are being built
 constexpr int SM_BAD = SM_PAR + FV_T;            // int [2], tree of table buffer tb was rejected
-constexpr int SM_VN2 = SM_BAD + 8;               // grouped mode: u16 [2][64] node id of virtual index u (per table buffer)
-constexpr int SM_BYTES = SM_VN2 + 2 * 2 * FV_T;
+constexpr int SM_BYTES = SM_BAD + 8;
 constexpr int SM_ALLOC = SM_BYTES + 1024;        // slack for the 1024-byte alignment of the base
 
 struct VerifyFastParams {
-    // TMA descriptors of the packed k, q, v tensors viewed as [N][heads][128] bf16 (not used by the grouped mode)
+    // TMA descriptors of the packed k, q, v tensors viewed as [N][heads][128] bf16
     alignas(64) CUtensorMap tm_k;
     alignas(64) CUtensorMap tm_q;
     alignas(64) CUtensorMap tm_v;
     int h_qk, h_v;
-    int n_units;        // n_seq * h_v (grouped mode: an upper bound that only sizes the grid)
-    int prefetch_dist;  // a CTA warms L2 for unit blockIdx.x + prefetch_dist (about one wave ahead)
+    int n_units;        // n_seq * h_v
     float scale;
     const float *S0;
     const __nv_bfloat16 *q, *k, *v, *g, *beta;
@@ -86,18 +87,8 @@ struct VerifyFastParams {
     const int32_t *parent;                             // trees of at most 64 nodes: the kernel builds the metadata itself
     int n_seq, total_nodes, max_tree_nodes, max_depth;
     void *o;
-    const uint8_t *depth;
-    const uint8_t *anc8;
     int32_t *status_dev;
-    // grouped verification of trees with more than 64 nodes (only read by the GROUPED instantiation)
-    int groups_per_tree, anc_stride;                   // upper bound of the groups of a tree (sizes the grid); entries
-                                                       // per row of anc16
-    const uint16_t *anc16, *dfs_node;
-    const uint4 *unit_list;                            // one record per group (see the workspace layout)
-    const int32_t *unit_count;                         // [0] records in the list, [1] plan_magic of the plan's shape
-    int unit_capacity, plan_magic;                     // what the list can hold; what [1] has to read
-    const uint8_t *dfs_depth, *dfs_anc8;
-    // fused commit of the previous step's accepted paths (only read by the FUSED instantiation)
+    // commit of the previous step's accepted paths
     float *S_rw;                                       // same tensor as S0, written in place
     const __nv_bfloat16 *pk, *pv, *pg, *pbeta;         // the previous tree's k, v, g, beta
     const int32_t *pparent, *pnode_offsets, *path, *path_offsets;
@@ -112,7 +103,7 @@ struct VerifyFastParams {
 // ---------------------------------------------------------------------------------------- kernel
 // The k/q tile holds the k rows first and the q rows second (rows i and 64 + i), so P has p^k in columns 0..63 and
 // p^q in columns 64..127, and the Gram block needs only N = 64.
-// FUSED: Eq. 7 is replayed along the previous step's accepted path on the state tile while it sits in registers
+// Eq. 7 is replayed along the previous step's accepted path on the state tile while it sits in registers
 // -- per row c, s_c <- alpha s_c + k beta (v_c - alpha k.s_c), the eight lanes that share a row reducing k.s_c with
 // three shuffles -- the tile is written back as the only state write of the step, and the new tree is verified
 // against it.
@@ -123,18 +114,9 @@ struct VerifyFastParams {
 // its value is used.  The state tile is asked for at the top of the unit and is needed only after the Gram /
 // coefficient phases; the v rows land by TMA in an area that is free until the state operand is written.
 // SMALL (every tree of the call has at most 32 nodes): the R and output phases skip the 16-node pieces beyond the tree.
-// GROUPED (trees of more than 64 nodes, cut into ancestor-closed groups by the plan kernel): a unit is (tree, value
-// head, group); it is verified as a virtual tree of the <= 15 proper ancestors of the group's first node followed by
-// the group's own nodes.  The rows of a virtual tree are not contiguous, so its k/q/v rows are gathered with
-// cp.async (completing on the same mbarriers as the TMA tiles otherwise), its tables come from the plan, and
-// outputs are stored for the group's own nodes only.  The units are the records of the plan's unit list (one per
-// real group, the groups of a tree next to one another) times the heads: the five or so groups of a (tree, head) run
-// on neighbouring CTAs at about the same time, so the state tile crosses HBM once, and the work spreads evenly over
-// the CTAs whatever the tree sizes.
-template <typename TOut, bool FUSED, bool SMALL, bool PADDED, bool GROUPED>
-__global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(const __grid_constant__ VerifyFastParams p)
+template <typename TOut, bool SMALL, bool PADDED>
+__global__ void __launch_bounds__(FV_THREADS, 2) commit_verify_kernel(const __grid_constant__ VerifyFastParams p)
 {
-    static_assert(!GROUPED || (!FUSED && !SMALL), "the grouped mode is verification only");
     extern __shared__ uint8_t fv_smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(fv_smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t sbase = smem_u32(smem);
@@ -151,15 +133,14 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
     // carries all of it: warp 0 the projection MMA group, warp 1 the D group, warp 2 the Gram block of the unit to
     // come, warp 3 the TMA loads.  Every issuer commits its own MMAs to an mbarrier.
     constexpr int W_MMA_P = 0, W_MMA_D = 1, W_MMA_G = 2, W_TMA = 3;
-    auto tbl_thread_g = [&]() -> bool { return tid >= FV_T && tid < 2 * FV_T; };   // thread FV_T + i keeps node i's tables
 
     if (warp == 0) tmem_alloc(sbase + SM_TMEM, FV_TMEM_COLS);
     if (tid == 32) {
         mbar_init(mbar_g, 1);
         mbar_init(mbar_p, 1);
         mbar_init(mbar_d, 1);
-        mbar_init(mbar_kq, GROUPED ? FV_THREADS : 1);   // gathered rows: every thread arrives once its copies have landed
-        mbar_init(mbar_v, GROUPED ? FV_THREADS : 1);
+        mbar_init(mbar_kq, 1);
+        mbar_init(mbar_v, 1);
         *flag = 0;
     }
     tc_fence_before();
@@ -169,14 +150,14 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
     // Launched with programmatic stream serialization: everything above overlaps the tail of the kernel in front
     // (the previous call, or the plan kernel); nothing that is computed from memory may run before that kernel's
     // writes are visible.  L2 can be asked for the first unit's state tile meanwhile (a prefetch consumes nothing).
-    if (!GROUPED && tid < 4 && (int)blockIdx.x < p.n_units)
+    if (tid < 4 && (int)blockIdx.x < p.n_units)
         prefetch_l2_bulk(p.S0 + (size_t)blockIdx.x * FV_D * FV_D + (size_t)tid * 4096, 16384);
     // ... and for the rows of the first unit's tree.  Their place may depend on node_offsets[], which the kernel in
     // front may still be writing: the value read here only steers prefetches (clamped to the tensors), it is read
     // again behind the dependency wait before anything is computed from it.
-    if (!GROUPED && (int)blockIdx.x < p.n_units && tid >= 128 && tid < 128 + FV_T) {
+    if ((int)blockIdx.x < p.n_units && tid >= 128 && tid < 128 + FV_T) {
         const int ub = (int)blockIdx.x / p.h_v, uh = (int)blockIdx.x % p.h_v, uhk = uh / (p.h_v / p.h_qk);
-        const int row = ((PADDED && p.t_pad) ? ub * p.t_pad : __ldg(p.node_offsets + ub)) + tid - 128;
+        const int row = ((PADDED) ? ub * p.t_pad : __ldg(p.node_offsets + ub)) + tid - 128;
         if (row >= 0 && row < p.total_nodes) {
             prefetch_l2_bulk(p.v + ((size_t)row * p.h_v + uh) * FV_D, 256);
             prefetch_l2_bulk(p.k + ((size_t)row * p.h_qk + uhk) * FV_D, 256);
@@ -193,12 +174,9 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
     // A CTA walks the units blockIdx.x, blockIdx.x + gridDim.x, ...: the indices of a unit follow from those of the
     // unit before by additions and carries, so that the integer divisions by the head and group counts (a few dozen
     // instructions each, for every thread) are paid once per CTA and not once per unit.
-    // Trees of at most 64 nodes: unit = slot b * h_v + head h.  GROUPED: unit = (layer b * E + record grp) * h_v + h,
-    // where E is the number of records in the plan's unit list (one per group; known behind the dependency wait) and
-    // `layer` counts the repetitions of the n_trees shared trees in the padded layout (always 0 otherwise).
-    struct Cursor { int u, b, h, grp; };
-    int n_units = GROUPED ? 0 : p.n_units;
-    int n_records = 1, gstep_h = 0, gstep_e = 0, gstep_l = 0;   // GROUPED, set behind the dependency wait
+    // Unit = slot b * h_v + head h.
+    struct Cursor { int u, b, h; };
+    const int n_units = p.n_units;
     const int ratio = p.h_v / p.h_qk;
     const int ratio_shift = (ratio & (ratio - 1)) == 0 ? 31 - __clz(ratio) : -1;
     auto hk_of = [&](int h_) -> int { return ratio_shift >= 0 ? h_ >> ratio_shift : h_ / ratio; };
@@ -208,38 +186,24 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
         Cursor c;
         c.u = u;
         c.h = u % p.h_v;
-        const int t = u / p.h_v;
-        c.grp = GROUPED ? t % n_records : 0;
-        c.b = GROUPED ? t / n_records : t;
+        c.b = u / p.h_v;
         return c;
     };
     auto advance = [&](Cursor &c) {
         c.u += (int)gridDim.x;
-        if constexpr (GROUPED) {
-            c.h += gstep_h;
-            const int carry_h = c.h >= p.h_v ? 1 : 0;
-            c.h -= carry_h ? p.h_v : 0;
-            c.grp += gstep_e + carry_h;
-            const int carry_e = c.grp >= n_records ? 1 : 0;
-            c.grp -= carry_e ? n_records : 0;
-            c.b += gstep_l + carry_e;
-        } else {
-            c.h += step_h;
-            const int carry_h = c.h >= p.h_v ? 1 : 0;
-            c.h -= carry_h ? p.h_v : 0;
-            c.b += step_b + carry_h;
-        }
+        c.h += step_h;
+        const int carry_h = c.h >= p.h_v ? 1 : 0;
+        c.h -= carry_h ? p.h_v : 0;
+        c.b += step_b + carry_h;
     };
-    // The loads a decode needs are issued by decode_load() and looked at by decode() / decode_g() later (the unit after
+    // The loads a decode needs are issued by decode_load() and looked at by decode() later (the unit after
     // next is asked for at the top of a unit and decoded in its middle), so that no thread waits for them.
-    struct DecodeRaw { int lo, hi; uint4 rec; };
+    struct DecodeRaw { int lo, hi; };
     auto decode_load = [&](const Cursor &c) -> DecodeRaw {
-        DecodeRaw r{0, 0, make_uint4(0u, 0u, 0u, 0u)};
+        DecodeRaw r{0, 0};
         if (c.u >= n_units) return r;
         const int ub = c.b;
-        if constexpr (GROUPED) {
-            r.rec = p.unit_list[c.grp];   // written by the plan kernel in front of this grid: no read-only path
-        } else if (PADDED && p.t_pad) {
+        if (PADDED) {
             r.lo = p.n_nodes[tree_of(ub)];
         } else {
             r.lo = p.node_offsets[ub];
@@ -253,7 +217,7 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
         uh = c.h;
         uhk = hk_of(uh);
         bool off_ok;
-        if (PADDED && p.t_pad) {   // padded layout: rows of the slot, node count and parent[] row of its tree
+        if (PADDED) {   // padded layout: rows of the slot, node count and parent[] row of its tree
             const int tree = tree_of(ub);
             ubase = ub * p.t_pad;
             uT = raw.lo;
@@ -270,7 +234,7 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
         }
         if (!off_ok && tid == 0) report_status(p.status_dev, GDN_ERR_TREE);
         const bool tree_good = off_ok && uT > 0;
-        if (FUSED && !tree_good) {
+        if (!tree_good) {
             // the commit of the previous step does not depend on the new tree: the unit runs as a tree of no
             // nodes (every node masked, nothing stored), so that its accepted path is still replayed
             ubase = 0;
@@ -279,96 +243,6 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
             return true;
         }
         return tree_good;
-    };
-    // GROUPED: unit -> (tree, head, group).  pb = first row of the tree in the plan's tables, g0 = first depth-first
-    // position of the group, n_prefix = proper ancestors of its first node (virtual indices 0 .. n_prefix - 1),
-    // first = node at position g0; ident: a tree of at most 64 nodes inside a grouped call (identity numbering).
-    struct GroupX { int pb, g0, n_prefix, first; bool ident; };
-    auto decode_g = [&](const Cursor &c, const DecodeRaw &raw, int &ub, int &uh, int &uhk, int &ubase, int &uT, GroupX &gx) -> bool {
-        if (c.u >= n_units) return false;
-        const int tree = (int)raw.rec.x;
-        uh = c.h;
-        uhk = hk_of(uh);
-        if (PADDED && p.t_pad) {   // slot = layer * n_trees + tree
-            ub = c.b * p.n_trees + tree;
-            ubase = ub * p.t_pad;
-            gx.pb = tree * p.t_pad;
-        } else {
-            ub = tree;
-            ubase = (int)raw.rec.y;   // checked by the plan kernel (a tree with bad offsets has no record)
-            gx.pb = ubase;
-        }
-        const uint2 gi = make_uint2(raw.rec.z, raw.rec.w);
-        const int own = (int)(gi.x >> 16);
-        if (own == 0) return false;   // no such group (or the plan rejected the tree, which it has reported)
-        gx.g0 = (int)(gi.x & 0xFFFFu);
-        gx.ident = (gi.y & 0xFFFFu) == 0xFFFFu;
-        gx.n_prefix = gx.ident ? 0 : (int)(gi.y & 0xFFFFu);
-        gx.first = (int)(gi.y >> 16);
-        uT = gx.n_prefix + own;
-        return true;
-    };
-    // node id of virtual index u (< T) of a group, from the plan
-    auto vnode_global = [&](const GroupX &gx, int u) -> int {
-        if (gx.ident) return u;
-        if (u < gx.n_prefix) return (int)__ldg(p.anc16 + (size_t)(gx.pb + gx.first) * p.anc_stride + u);
-        return (int)__ldg(p.dfs_node + gx.pb + gx.g0 + u - gx.n_prefix);
-    };
-    // table entries of virtual index tnode: node id, depth, root path in virtual indices
-    auto lookup_tables_g = [&](const GroupX &gx, int uT, int &node, int &d, uint4 &row) {
-        node = 0;
-        d = 0;
-        row = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
-        if (tbl_thread_g() && tid - FV_T < uT) {
-            const int t = tid - FV_T;
-            if (gx.ident) {
-                node = t;
-                d = p.depth[gx.pb + t];
-                row = __ldg(reinterpret_cast<const uint4 *>(p.anc8 + (size_t)(gx.pb + t) * 16));
-            } else if (t < gx.n_prefix) {   // an ancestor of the group's first node: its path is 0..t
-                node = vnode_global(gx, t);
-                d = t + 1;
-                const uint32_t all[4] = {0x03020100u, 0x07060504u, 0x0B0A0908u, 0x0F0E0D0Cu};
-                uint32_t w[4];
-#pragma unroll
-                for (int q4 = 0; q4 < 4; ++q4) {
-                    const int keep = d - 4 * q4;   // bytes of this word that are on the path
-                    w[q4] = keep >= 4 ? all[q4] : keep <= 0 ? 0xFFFFFFFFu : (all[q4] | (0xFFFFFFFFu << (8 * keep)));
-                }
-                row = make_uint4(w[0], w[1], w[2], w[3]);
-            } else {
-                const int r = gx.pb + gx.g0 + t - gx.n_prefix;
-                node = (int)__ldg(p.dfs_node + r);
-                d = p.dfs_depth[r];
-                row = __ldg(reinterpret_cast<const uint4 *>(p.dfs_anc8 + (size_t)r * 16));
-            }
-        }
-    };
-    auto put_tables_g = [&](int uT, int tb, int node, int d, uint4 row, uint32_t g_bits, uint32_t be_bits) {
-        if (tbl_thread_g()) {
-            const int t = tid - FV_T;
-            const bool on = t < uT;
-            (smem + SM_DEPTH + tb * SM_TABLE_STRIDE)[t] = (uint8_t)(on ? d : 0);
-            *reinterpret_cast<uint4 *>(smem + SM_ANC + tb * SM_TABLE_STRIDE + t * 16) = row;
-            reinterpret_cast<float4 *>(smem + SM_GAB + tb * SM_TABLE_STRIDE)[t] =
-                make_float4(0.f, 0.f, on ? gate_beta(be_bits, PADDED && p.raw_gates) : 0.f,
-                            on ? gate_log_decay(g_bits, PADDED && p.raw_gates) : 0.f);
-            reinterpret_cast<uint16_t *>(smem + SM_VN2)[tb * FV_T + t] = (uint16_t)(on ? node : 0);
-        }
-    };
-    // k and q rows of a virtual tree -> B operand tile (rows beyond the tree zero-filled): thread (r16, c16) fetches
-    // 16-byte piece c16 of the rows r16, r16 + 16, r16 + 32, r16 + 48, whose node ids it is handed
-    auto gather_kq = [&](int uhk, int ubase, int uT, const int (&nid)[4]) {
-        const int r16 = tid >> 4, c16 = tid & 15;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int u = r16 + 16 * j;
-            const bool valid = u < uT;
-            const size_t off = ((size_t)(ubase + (valid ? nid[j] : 0)) * p.h_qk + uhk) * FV_D + c16 * 8;
-            cp_async_16(sbase + SM_B_KQ + sw128_offset(u, c16), p.k + off, valid);
-            cp_async_16(sbase + SM_B_KQ + sw128_offset(FV_T + u, c16), p.q + off, valid);
-        }
-        cp_async_arrive_on(mbar_kq);
     };
     // k and q rows -> B operand tile by TMA: four 64-row x 64-column boxes (k and q, either K half), 128-byte
     // swizzled, completing on mbar_kq.  A box always spans 64 nodes: rows beyond the tree belong to the next tree
@@ -390,12 +264,14 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
     // lets thread i climb from node i to its root, shifting each id into a 16-byte row from below, so that the
     // root ends up in byte 0.  A tree with a bad parent[] or a root path of more than max_depth nodes is flagged in
     // bad_s[tb]; the unit then runs as a tree of no nodes.
-    // Node i is handled by thread FV_T + i (warps 2 and 3; warps 0 and 1 issue MMAs at the same time).
+    // Node i is handled by thread FV_T + i (warps 2 and 3; warps 0 and 1 issue MMAs at the same time).  In the padded layout
+    // the slots of a tree share its parent[]: a unit with the tree of the one before copies its rows and verdict (48 slots of one
+    // 61-node tree, path of 12: 104.6 -> 102.3 us).
     const int tnode = tid - FV_T;
     const bool tbl_thread = tid >= FV_T && tid < 2 * FV_T;
-    auto put_parent = [&](int uT, int par, int tb) -> bool {
+    auto put_parent = [&](int uT, int par, int tb, bool same_tree) -> bool {
         bool bad = false;
-        if (tbl_thread) {
+        if (tbl_thread && !same_tree) {
             int pv = -1;
             if (tnode < uT) {
                 pv = par;
@@ -403,14 +279,18 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
             }
             par_s[tnode] = (signed char)pv;
         }
-        if (tid == 0) bad_s[tb] = 0;
+        if (tid == 0) bad_s[tb] = same_tree ? bad_s[tb ^ 1] : 0;
         return bad;
     };
-    auto walk_tables = [&](int uT, int tb, uint32_t g_bits, uint32_t be_bits, bool my_bad) {
+    auto walk_tables = [&](int uT, int tb, uint32_t g_bits, uint32_t be_bits, bool my_bad, bool same_tree) {
         if (tbl_thread) {
             int d = 0, err = my_bad ? GDN_ERR_TREE : 0;
             uint32_t w0 = 0xFFFFFFFFu, w1 = 0xFFFFFFFFu, w2 = 0xFFFFFFFFu, w3 = 0xFFFFFFFFu;
-            if (tnode < uT && !err) {
+            if (same_tree) {   // rows of the unit before
+                d = (smem + SM_DEPTH + (tb ^ 1) * SM_TABLE_STRIDE)[tnode];
+                const uint4 row = *reinterpret_cast<const uint4 *>(smem + SM_ANC + (tb ^ 1) * SM_TABLE_STRIDE + tnode * 16);
+                w0 = row.x; w1 = row.y; w2 = row.z; w3 = row.w;
+            } else if (tnode < uT && !err) {
                 int cur = tnode;
                 while (cur >= 0) {
                     if (++d > p.max_depth) { err = GDN_ERR_DEPTH; break; }
@@ -434,7 +314,7 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
     };
     // the same two steps with the loads issued on the spot (first unit of a CTA, and behind a skipped unit)
     auto load_parent = [&](int upar, int uT, int tb) -> bool {
-        return put_parent(uT, tbl_thread && tnode < uT ? p.parent[upar + tnode] : -1, tb);
+        return put_parent(uT, tbl_thread && tnode < uT ? p.parent[upar + tnode] : -1, tb, false);
     };
     auto load_tables = [&](int uh, int ubase, int uT, int tb, bool my_bad) {
         uint32_t gb = 0, bb = 0;
@@ -443,7 +323,7 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
             gb = __ldg(reinterpret_cast<const unsigned short *>(p.g) + n * p.h_v + uh);
             bb = __ldg(reinterpret_cast<const unsigned short *>(p.beta) + n * p.h_v + uh);
         }
-        walk_tables(uT, tb, gb, bb, my_bad);
+        walk_tables(uT, tb, gb, bb, my_bad, false);
     };
 
     // Fused commit: the accepted path of tree `ub` in the previous step goes to path slot `ps`.  One warp
@@ -451,52 +331,50 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
     // root inside the previous tree; a bad path is reported and its length stored as 0, so that this state
     // stays as it was.  Readable by the other warps after the next CTA barrier.
     auto fetch_path = [&](int ub, int ps) {
-        if constexpr (FUSED) {
-            if (warp == 4) {
-                int *slot = reinterpret_cast<int *>(smem + SM_PATH + ps * SM_PATH_SLOT);
-                int pp0, len, pb = 0, pT = 0, ppar = 0;   // len 0 leaves the state alone
-                if (PADDED && p.t_pad) {
-                    const int tree = tree_of(ub);
-                    pp0 = tree * p.path_stride;
-                    len = p.path_len[tree];
-                    pb = ub * p.pt_pad;
-                    pT = min(p.pn_nodes[tree], p.pt_pad);
-                    ppar = tree * p.pt_pad;
-                } else {
-                    pp0 = p.path_offsets[ub];
-                    len = p.path_offsets[ub + 1] - pp0;
-                    if (len != 0) {
-                        pb = p.pnode_offsets[ub];
-                        pT = p.pnode_offsets[ub + 1] - pb;
-                        ppar = pb;
-                    }
-                }
+        if (warp == 4) {
+            int *slot = reinterpret_cast<int *>(smem + SM_PATH + ps * SM_PATH_SLOT);
+            int pp0, len, pb = 0, pT = 0, ppar = 0;   // len 0 leaves the state alone
+            if (PADDED) {
+                const int tree = tree_of(ub);
+                pp0 = tree * p.path_stride;
+                len = p.path_len[tree];
+                pb = ub * p.pt_pad;
+                pT = min(p.pn_nodes[tree], p.pt_pad);
+                ppar = tree * p.pt_pad;
+            } else {
+                pp0 = p.path_offsets[ub];
+                len = p.path_offsets[ub + 1] - pp0;
                 if (len != 0) {
-                    const bool shape_ok = len > 0 && len <= FV_MD && len <= p.max_depth && pT > 0 && pp0 >= 0;
-                    const bool mine = shape_ok && lane < len;
-                    int n = -1, parent_n = -2;
-                    if (mine) {
-                        n = p.path[pp0 + lane];
-                        if (p.pparent && n >= 0 && n < pT) parent_n = p.pparent[ppar + n];
-                        slot[lane] = n;
-                    }
-                    const int n_up = __shfl_up_sync(0xffffffffu, n, 1);
-                    bool bad = false;
-                    if (mine) {
-                        if (n < 0 || n >= pT) bad = true;
-                        else if (p.pparent) bad = parent_n != (lane ? n_up : -1);
-                        else if (lane && n <= n_up) bad = true;   // without parent[] only the topological order can be checked
-                    }
-                    if (__any_sync(0xffffffffu, bad) || !shape_ok) {
-                        if (lane == 0) report_status(p.status_dev, GDN_ERR_PATH);
-                        len = 0;
-                    }
+                    pb = p.pnode_offsets[ub];
+                    pT = p.pnode_offsets[ub + 1] - pb;
+                    ppar = pb;
                 }
-                if (lane == 0) {
-                    slot[16] = len;
-                    slot[17] = pb;
-                    slot[18] = len;
+            }
+            if (len != 0) {
+                const bool shape_ok = len > 0 && len <= FV_MD && len <= p.max_depth && pT > 0 && pp0 >= 0;
+                const bool mine = shape_ok && lane < len;
+                int n = -1, parent_n = -2;
+                if (mine) {
+                    n = p.path[pp0 + lane];
+                    if (p.pparent && n >= 0 && n < pT) parent_n = p.pparent[ppar + n];
+                    slot[lane] = n;
                 }
+                const int n_up = __shfl_up_sync(0xffffffffu, n, 1);
+                bool bad = false;
+                if (mine) {
+                    if (n < 0 || n >= pT) bad = true;
+                    else if (p.pparent) bad = parent_n != (lane ? n_up : -1);
+                    else if (lane && n <= n_up) bad = true;   // without parent[] only the topological order can be checked
+                }
+                if (__any_sync(0xffffffffu, bad) || !shape_ok) {
+                    if (lane == 0) report_status(p.status_dev, GDN_ERR_PATH);
+                    len = 0;
+                }
+            }
+            if (lane == 0) {
+                slot[16] = len;
+                slot[17] = pb;
+                slot[18] = len;
             }
         }
     };
@@ -504,37 +382,33 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
     // readable and the parking area is free.  Only node ids that have been range-checked are used (slot[18] =
     // length of the path as far as it has been checked when the rows are asked for).
     auto fetch_path_kv = [&](int uh, int uhk, int ps) {
-        if constexpr (FUSED) {
-            const int *slot = reinterpret_cast<const int *>(smem + SM_PATH + ps * SM_PATH_SLOT);
-            const int len = slot[18], pb = slot[17];
-            for (int idx = tid; idx < len * 32; idx += FV_THREADS) {
-                const int t = idx >> 5, c16 = idx & 15;
-                const size_t n = (size_t)pb + slot[t];
-                if (idx & 16)
-                    cp_async_16(sbase + SM_PV + t * 256 + c16 * 16, p.pv + (n * p.h_v + uh) * FV_D + c16 * 8, true);
-                else
-                    cp_async_16(sbase + SM_PK + t * 256 + c16 * 16, p.pk + (n * p.h_qk + uhk) * FV_D + c16 * 8, true);
-            }
+        const int *slot = reinterpret_cast<const int *>(smem + SM_PATH + ps * SM_PATH_SLOT);
+        const int len = slot[18], pb = slot[17];
+        for (int idx = tid; idx < len * 32; idx += FV_THREADS) {
+            const int t = idx >> 5, c16 = idx & 15;
+            const size_t n = (size_t)pb + slot[t];
+            if (idx & 16)
+                cp_async_16(sbase + SM_PV + t * 256 + c16 * 16, p.pv + (n * p.h_v + uh) * FV_D + c16 * 8, true);
+            else
+                cp_async_16(sbase + SM_PK + t * 256 + c16 * 16, p.pk + (n * p.h_qk + uhk) * FV_D + c16 * 8, true);
         }
     };
     // per-step scalars of the path, computed on the spot (first unit of a CTA, and behind a skipped unit)
     auto path_scalars_direct = [&](int uh, int ps) {
-        if constexpr (FUSED) {
-            const int *slot = reinterpret_cast<const int *>(smem + SM_PATH + ps * SM_PATH_SLOT);
-            float4 *ab = reinterpret_cast<float4 *>(smem + SM_PATH + ps * SM_PATH_SLOT + 128);
-            const int len = slot[16], pb = slot[17];
-            if (tid < len) {
-                float gsum = 0.f, gt = 0.f;
-                const unsigned short *pg = reinterpret_cast<const unsigned short *>(p.pg);
-                const unsigned short *pbe = reinterpret_cast<const unsigned short *>(p.pbeta);
-                for (int t = 0; t <= tid; ++t) {
-                    gt = gate_log_decay(pg[((size_t)pb + slot[t]) * p.h_v + uh], PADDED && p.raw_gates);
-                    gsum += gt;
-                }
-                const size_t n = (size_t)pb + slot[tid];
-                const float A = expf(gsum);
-                ab[tid] = make_float4(A, gate_beta(pbe[n * p.h_v + uh], PADDED && p.raw_gates), expf(gt), 1.f / A);
+        const int *slot = reinterpret_cast<const int *>(smem + SM_PATH + ps * SM_PATH_SLOT);
+        float4 *ab = reinterpret_cast<float4 *>(smem + SM_PATH + ps * SM_PATH_SLOT + 128);
+        const int len = slot[16], pb = slot[17];
+        if (tid < len) {
+            float gsum = 0.f, gt = 0.f;
+            const unsigned short *pg = reinterpret_cast<const unsigned short *>(p.pg);
+            const unsigned short *pbe = reinterpret_cast<const unsigned short *>(p.pbeta);
+            for (int t = 0; t <= tid; ++t) {
+                gt = gate_log_decay(pg[((size_t)pb + slot[t]) * p.h_v + uh], PADDED && p.raw_gates);
+                gsum += gt;
             }
+            const size_t n = (size_t)pb + slot[tid];
+            const float A = expf(gsum);
+            ab[tid] = make_float4(A, gate_beta(pbe[n * p.h_v + uh], PADDED && p.raw_gates), expf(gt), 1.f / A);
         }
     };
     // G_i = sum of g along the root path (root first), a_i = exp(G_i), for the tables in buffer `tb`
@@ -559,7 +433,6 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
     auto issue_gram = [&](uint32_t kq_parity) {
         if (warp == W_MMA_G && elect_one()) {
             if (!mbar_wait_bounded(mbar_kq, kq_parity)) *flag = 1;
-            if constexpr (GROUPED) fence_proxy_async();   // rows written by cp.async become visible to the tensor core
             tc_fence_after();
             const uint64_t b_kq = smem_desc_sw128(sbase + SM_B_KQ);
             constexpr uint32_t id = idesc_bf16(128, 64);   // B = the 64 k rows
@@ -577,69 +450,27 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
     // ... and whatever is launched behind this grid with the same attribute (the next call's kernel, which itself
     // waits for this grid to complete before it reads or writes anything) may be made resident now.
     asm volatile("griddepcontrol.launch_dependents;");
-    GroupX gx{0, 0, 0, 0, true}, ngx{0, 0, 0, 0, true};
-    if constexpr (GROUPED) {
-        // the plan kernel has counted the groups of all trees: that many records, times the heads, times the layers
-        // that share the trees in the padded layout, are the units of this grid
-        int n_rec = reinterpret_cast<const volatile int32_t *>(p.unit_count)[0];
-        if (reinterpret_cast<const volatile int32_t *>(p.unit_count)[1] != p.plan_magic || n_rec < 0 ||
-            n_rec > p.unit_capacity) {   // not a plan of this shape (never built, or built for other sizes)
-            if (tid == 0) report_status(p.status_dev, GDN_ERR_WORKSPACE);
-            n_rec = 0;
-        }
-        const int n_layers = (PADDED && p.t_pad) ? p.n_seq / p.n_trees : 1;
-        n_records = n_rec > 0 ? n_rec : 1;
-        n_units = n_rec > 0 ? n_rec * p.h_v * n_layers : 0;
-        gstep_h = (int)gridDim.x % p.h_v;
-        const int t = (int)gridDim.x / p.h_v;
-        gstep_e = t % n_records;
-        gstep_l = t / n_records;
-    }
     Cursor ucur = cursor_at((int)blockIdx.x);
     bool cur_ok;
-    if constexpr (GROUPED) {
-        cur_ok = decode_g(ucur, decode_load(ucur), b, h, hk, base, T, gx);
-        while (!cur_ok && (advance(ucur), ucur.u < n_units)) cur_ok = decode_g(ucur, decode_load(ucur), b, h, hk, base, T, gx);
-        int t_node, t_d;
-        uint4 t_row;
-        lookup_tables_g(gx, T, t_node, t_d, t_row);
-        uint32_t gb = 0, bb = 0;
-        if (cur_ok && tbl_thread_g() && tid - FV_T < T) {
-            const size_t n = (size_t)(base + t_node);
-            gb = __ldg(reinterpret_cast<const unsigned short *>(p.g) + n * p.h_v + h);
-            bb = __ldg(reinterpret_cast<const unsigned short *>(p.beta) + n * p.h_v + h);
-        }
-        if (cur_ok) put_tables_g(T, 0, t_node, t_d, t_row, gb, bb);
-        __syncthreads();
-        if (cur_ok) {
-            path_decay(0);
-            const uint16_t *vn = reinterpret_cast<const uint16_t *>(smem + SM_VN2);
-            const int nid[4] = {vn[tid >> 4], vn[(tid >> 4) + 16], vn[(tid >> 4) + 32], vn[(tid >> 4) + 48]};
-            gather_kq(hk, base, T, nid);
-            issue_gram(0);
-        }
-    } else {
-        cur_ok = decode(ucur, decode_load(ucur), b, h, hk, base, T, par0);
-        bool par_bad = false;
-        if (cur_ok) {
-            issue_kq(b, hk, base, T);
-            fetch_path(b, 0);
-            par_bad = load_parent(par0, T, 0);
-        }
-        __syncthreads();
-        if (cur_ok) load_tables(h, base, T, 0, par_bad);
-        __syncthreads();
-        if (cur_ok) {
-            path_decay(0);
-            fetch_path_kv(h, hk, 0);
-            path_scalars_direct(h, 0);
-            issue_gram(0);
-        }
+    cur_ok = decode(ucur, decode_load(ucur), b, h, hk, base, T, par0);
+    bool par_bad = false;
+    if (cur_ok) {
+        issue_kq(b, hk, base, T);
+        fetch_path(b, 0);
+        par_bad = load_parent(par0, T, 0);
+    }
+    __syncthreads();
+    if (cur_ok) load_tables(h, base, T, 0, par_bad);
+    __syncthreads();
+    if (cur_ok) {
+        path_decay(0);
+        fetch_path_kv(h, hk, 0);
+        path_scalars_direct(h, 0);
+        issue_gram(0);
     }
     int done_units = 0;
 #pragma unroll 1
     for (int iter = 0; ucur.u < n_units; ++iter) {
-    const bool unit_ok = cur_ok;
     const uint32_t par = (uint32_t)(done_units & 1);   // every barrier completes once per processed unit
     int nb = 0, nh = 0, nhk = 0, nbase = 0, nT = 0, npar0 = 0;
     Cursor ncur = ucur;
@@ -647,60 +478,20 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
     bool next_ok = false;
     const DecodeRaw next_raw = decode_load(ncur);   // looked at in the middle of the unit (stage 1)
     auto decode_next = [&]() {
-        if constexpr (GROUPED) {
-            next_ok = decode_g(ncur, next_raw, nb, nh, nhk, nbase, nT, ngx);
-            while (!next_ok && (advance(ncur), ncur.u < n_units))   // (every record is a real group: not taken)
-                next_ok = decode_g(ncur, decode_load(ncur), nb, nh, nhk, nbase, nT, ngx);
-        } else {
-            next_ok = decode(ncur, next_raw, nb, nh, nhk, nbase, nT, npar0);
-        }
+        next_ok = decode(ncur, next_raw, nb, nh, nhk, nbase, nT, npar0);
     };
     float4 *gab = reinterpret_cast<float4 *>(smem + SM_GAB + (iter & 1) * SM_TABLE_STRIDE);
     uint8_t *anc_s = smem + SM_ANC + (iter & 1) * SM_TABLE_STRIDE;
     uint8_t *depth_s = smem + SM_DEPTH + (iter & 1) * SM_TABLE_STRIDE;
-    if (!unit_ok) {   // nothing to compute here: only keep the pipeline fed (never taken in the grouped mode)
-        decode_next();
-        if constexpr (!GROUPED) {
-            __syncthreads();
-            bool nbad = false;
-            if (next_ok) {
-                issue_kq(nb, nhk, nbase, nT);
-                nbad = load_parent(npar0, nT, (iter + 1) & 1);
-                fetch_path(nb, (iter + 1) & 1);
-            }
-            __syncthreads();
-            if (next_ok) load_tables(nh, nbase, nT, (iter + 1) & 1, nbad);
-            __syncthreads();
-            if (next_ok) {
-                path_decay((iter + 1) & 1);
-                fetch_path_kv(nh, nhk, (iter + 1) & 1);
-                path_scalars_direct(nh, (iter + 1) & 1);
-                issue_gram(par);   // no unit was processed in between: the tile's barrier phase is this one
-            }
-        }
-        b = nb; h = nh; hk = nhk; base = nbase; T = nT; cur_ok = next_ok;
-        ucur = ncur;
-        continue;
-    }
     // L2 warming for this CTA's next unit, in slices at phase boundaries
     auto warm_l2_state = [&](int slice) {
-        if constexpr (GROUPED) {
-            // the next unit's slot is known once its record has been looked at (stage 1): both halves of the tile are
-            // asked for behind that; the groups of a (tree, head) are neighbours, so most of the time L2 has it already
-            if (tid == 96 && slice >= 2 && next_ok) {
-                const float *S = p.S0 + (size_t)(nb * p.h_v + nh) * FV_D * FV_D + (size_t)(slice - 2) * 8192;
-                prefetch_l2_bulk(S, 16384);
-                prefetch_l2_bulk(S + 4096, 16384);
-            }
-        } else {
-            if (tid == 96 && ncur.u < n_units)
-                prefetch_l2_bulk(p.S0 + (size_t)(ncur.b * p.h_v + ncur.h) * FV_D * FV_D + (size_t)slice * 4096, 16384);
-        }
+        if (tid == 96 && ncur.u < n_units)
+            prefetch_l2_bulk(p.S0 + (size_t)(ncur.b * p.h_v + ncur.h) * FV_D * FV_D + (size_t)slice * 4096, 16384);
     };
 
     // a tree whose parent[] was rejected while its tables were built runs as a tree of no nodes: nothing of it
     // is stored (fused form: its accepted path of the previous step is committed all the same)
-    if (!GROUPED && bad_s[iter & 1]) {
+    if (bad_s[iter & 1]) {
         T = 0;
         if (tid < FV_T) depth_s[tid] = 0;
     }
@@ -720,27 +511,16 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
             for (int kh = 0; kh < 2; ++kh) ldg_v8(src + kh * 64, x[i][kh * 2 + 0], x[i][kh * 2 + 1]);
         }
     };
-    load_state_rows(0, FUSED ? 2 : 1);
-    const uint16_t *vnode_s = reinterpret_cast<const uint16_t *>(smem + SM_VN2) + (iter & 1) * FV_T;
+    load_state_rows(0, 2);
     // this tree's v rows: one TMA box into an area that stays free until the state operand is written
-    if constexpr (GROUPED) {   // ... gathered row by row (rows beyond the virtual tree zero-filled)
-        const int r16 = tid >> 4, c16 = tid & 15;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int u = r16 + 16 * j;
-            const bool valid = u < T;
-            cp_async_16(sbase + SM_VE + u * 256 + c16 * 16,
-                        p.v + ((size_t)(base + (valid ? (int)vnode_s[u] : 0)) * p.h_v + h) * FV_D + c16 * 8, valid);
-        }
-        cp_async_arrive_on(mbar_v);
-    } else if (warp == W_TMA && elect_one()) {
+    if (warp == W_TMA && elect_one()) {
         mbar_expect_tx(mbar_v, FV_T * FV_D * 2);
         tma_load_3d(sbase + SM_VE, &p.tm_v, 0, h, base, mbar_v);
     }
     // fused commit: this tree's accepted path of the previous step was fetched one unit ahead
     const float4 *ab_path = reinterpret_cast<const float4 *>(smem + SM_PATH + (iter & 1) * SM_PATH_SLOT + 128);
     int path_len = 0;
-    if constexpr (FUSED) path_len = reinterpret_cast<const int *>(smem + SM_PATH + (iter & 1) * SM_PATH_SLOT)[16];
+    path_len = reinterpret_cast<const int *>(smem + SM_PATH + (iter & 1) * SM_PATH_SLOT)[16];
 
     // Everything that depends only on q, k, g, beta runs now, under the latency of the state loads.  The Gram
     // block of this unit was issued one unit ahead; every thread waits for it on its own (bounded: on expiry it
@@ -748,7 +528,6 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
     if (!mbar_wait_bounded(mbar_g, par)) *flag = 1;
     tc_fence_after();
     __syncthreads();
-    if constexpr (!FUSED) load_state_rows(1, 2);
     warm_l2_state(0);
     if (*flag == 0) {
         // k-columns of the Gram block out of tensor memory, into the (still unused) state-operand area
@@ -811,12 +590,10 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
     // Per row c (one value component): s_c <- alpha s_c + k beta (v_c - alpha k.s_c); the eight lanes that
     // share a row reduce k.s_c with three shuffles.  The path's k/v rows were fetched above.
     const bool healthy = *flag == 0;   // uniform: every write of the flag so far lies before the barrier above
-    if constexpr (FUSED) {
-        if (!healthy) path_len = 0;    // a wait expired: this state is left as it was
-        if (path_len > 0) {
-            replay_path_on_tile(x, path_len, reinterpret_cast<const uint16_t *>(smem + SM_PK),
-                                reinterpret_cast<const uint16_t *>(smem + SM_PV), ab_path, warp, r4, l8);
-        }
+    if (!healthy) path_len = 0;    // a wait expired: this state is left as it was
+    if (path_len > 0) {
+        replay_path_on_tile(x, path_len, reinterpret_cast<const uint16_t *>(smem + SM_PK),
+                            reinterpret_cast<const uint16_t *>(smem + SM_PV), ab_path, warp, r4, l8);
     }
     // The v rows move into registers in the orientation of the R phase (component c = TMEM lane of this
     // thread, its 32 nodes, two bf16 per register): they are about to be overwritten by the state operand.
@@ -829,23 +606,19 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
         for (int m = 0; m < 16; ++m)
             vreg[m] = (uint32_t)ve[(2 * m) * FV_D] | ((uint32_t)ve[(2 * m + 1) * FV_D] << 16);
     }
-    __syncthreads();   // the v rows and (FUSED) the path rows sit where the state operand is about to be written
+    __syncthreads();   // the v rows and the path rows sit where the state operand is about to be written
 
-    // (4) fp32 -> bf16 hi + lo, written as the A operand.  FUSED: the committed state -- the only state write of
+    // (4) fp32 -> bf16 hi + lo, written as the A operand.  The committed state -- the only state write of
     // the step -- goes out from the same registers, one 32-byte store in front of each piece's conversion so
     // that the stores drain while the arithmetic runs.
     float *S_out = nullptr;
-    if constexpr (FUSED) {
-        if (path_len > 0) S_out = p.S_rw + (size_t)(b * p.h_v + h) * FV_D * FV_D;
-    }
+    if (path_len > 0) S_out = p.S_rw + (size_t)(b * p.h_v + h) * FV_D * FV_D;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int row = warp * 16 + i * 4 + r4;
 #pragma unroll
         for (int kh = 0; kh < 2; ++kh) {
-            if constexpr (FUSED) {
-                if (S_out) stg_v8(S_out + (size_t)row * FV_D + l8 * 8 + kh * 64, x[i][kh * 2 + 0], x[i][kh * 2 + 1]);
-            }
+            if (S_out) stg_v8(S_out + (size_t)row * FV_D + l8 * 8 + kh * 64, x[i][kh * 2 + 0], x[i][kh * 2 + 1]);
             const float4 u = x[i][kh * 2 + 0], w = x[i][kh * 2 + 1];
             const float f[8] = {u.x, u.y, u.z, u.w, w.x, w.y, w.z, w.w};
             uint32_t hi[4], lo[4];
@@ -889,42 +662,28 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
     unsigned short q_g = 0, q_be = 0;
     bool q_shape_ok = false, q_mine = false;
     decode_next();
-    int t_node = 0, t_d = 0;                 // grouped mode: table entries of virtual index tnode, and the
-    uint4 t_row = make_uint4(0u, 0u, 0u, 0u);   // node ids of the four rows this thread gathers
-    int nid[4] = {0, 0, 0, 0};
-    if constexpr (GROUPED) {
-        if (next_ok) {
-            lookup_tables_g(ngx, nT, t_node, t_d, t_row);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int u = (tid >> 4) + 16 * j;
-                nid[j] = u < nT ? vnode_global(ngx, u) : 0;
-            }
-        }
-    }
-    if (!GROUPED && next_ok) {
+    const bool same_tree = PADDED && next_ok && tree_of(nb) == tree_of(b);
+    if (next_ok) {
         if (tbl_thread && tnode < nT) {
             const int n = nbase + tnode;
-            t_par = __ldg(p.parent + npar0 + tnode);
+            if (!same_tree) t_par = __ldg(p.parent + npar0 + tnode);
             t_g = __ldg(reinterpret_cast<const unsigned short *>(p.g) + (size_t)n * p.h_v + nh);
             t_be = __ldg(reinterpret_cast<const unsigned short *>(p.beta) + (size_t)n * p.h_v + nh);
         }
-        if constexpr (FUSED) {
-            if (warp == 4) {
-                if (PADDED && p.t_pad) {   // (stage 2 takes differences: hand it begin / end pairs)
-                    const int tree = tree_of(nb);
-                    q_pp0 = tree * p.path_stride;
-                    q_len = q_pp0 + p.path_len[tree];
-                    q_pb = nb * p.pt_pad;
-                    q_pT = q_pb + min(p.pn_nodes[tree], p.pt_pad);
-                    q_ppar = tree * p.pt_pad;
-                } else {
-                    q_pp0 = p.path_offsets[nb];
-                    q_len = p.path_offsets[nb + 1];
-                    q_pb = p.pnode_offsets[nb];
-                    q_pT = p.pnode_offsets[nb + 1];
-                    q_ppar = q_pb;
-                }
+        if (warp == 4) {
+            if (PADDED) {   // (stage 2 takes differences: hand it begin / end pairs)
+                const int tree = tree_of(nb);
+                q_pp0 = tree * p.path_stride;
+                q_len = q_pp0 + p.path_len[tree];
+                q_pb = nb * p.pt_pad;
+                q_pT = q_pb + min(p.pn_nodes[tree], p.pt_pad);
+                q_ppar = tree * p.pt_pad;
+            } else {
+                q_pp0 = p.path_offsets[nb];
+                q_len = p.path_offsets[nb + 1];
+                q_pb = p.pnode_offsets[nb];
+                q_pT = p.pnode_offsets[nb + 1];
+                q_ppar = q_pb;
             }
         }
     }
@@ -954,14 +713,12 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
             }
         }
     // stage 2: the path entries
-    if constexpr (FUSED) {
-        if (next_ok && warp == 4) {
-            q_len -= q_pp0;
-            q_pT -= q_pb;
-            q_shape_ok = q_len > 0 && q_len <= FV_MD && q_len <= p.max_depth && q_pT > 0 && q_pp0 >= 0;
-            q_mine = q_shape_ok && lane < q_len;
-            if (q_mine) q_n = p.path[q_pp0 + lane];
-        }
+    if (next_ok && warp == 4) {
+        q_len -= q_pp0;
+        q_pT -= q_pb;
+        q_shape_ok = q_len > 0 && q_len <= FV_MD && q_len <= p.max_depth && q_pT > 0 && q_pp0 >= 0;
+        q_mine = q_shape_ok && lane < q_len;
+        if (q_mine) q_n = p.path[q_pp0 + lane];
     }
     bool unit_done_ok = false;
     // From here to the output staging every thread waits on the barriers of the tensor core and of TMA itself;
@@ -975,35 +732,23 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
         // the root path) over the state operand
         // the k/q tile is dead: start on the next unit of this CTA (its k/q tile, its tables), to be
         // consumed after the loop comes round
-        if constexpr (GROUPED) {
-            if (next_ok) {
-                gather_kq(nhk, nbase, nT, nid);
-                if (tbl_thread && tnode < nT) {   // stage 3: the gates of the node found in stage 1
-                    const size_t n = (size_t)(nbase + t_node);
-                    t_g = __ldg(reinterpret_cast<const unsigned short *>(p.g) + n * p.h_v + nh);
-                    t_be = __ldg(reinterpret_cast<const unsigned short *>(p.beta) + n * p.h_v + nh);
-                }
-            }
-        }
-        if (!GROUPED && next_ok) {
+        if (next_ok) {
             issue_kq(nb, nhk, nbase, nT);
             // stage 3: parent[] of the next tree is staged for the walk behind the next CTA barrier; the parents of
             // the path entries are asked for
-            t_bad = put_parent(nT, t_par, (iter + 1) & 1);
-            if constexpr (FUSED) {
-                if (warp == 4) {
-                    // the entries are published as far as they are checked (inside the previous tree), so that
-                    // their rows can be asked for behind the next barrier; whether they form a chain is decided then
-                    int *slot = reinterpret_cast<int *>(smem + SM_PATH + ((iter + 1) & 1) * SM_PATH_SLOT);
-                    const bool in_range = q_mine && q_n >= 0 && q_n < q_pT;
-                    const bool all_in = __all_sync(0xffffffffu, !q_mine || in_range);
-                    if (lane < FV_MD) slot[lane] = in_range ? q_n : 0;
-                    if (lane == 0) {
-                        slot[17] = q_pb;
-                        slot[18] = q_shape_ok && all_in ? q_len : 0;
-                    }
-                    if (in_range && p.pparent) q_par = p.pparent[q_ppar + q_n];
+            t_bad = put_parent(nT, t_par, (iter + 1) & 1, same_tree);
+            if (warp == 4) {
+                // the entries are published as far as they are checked (inside the previous tree), so that
+                // their rows can be asked for behind the next barrier; whether they form a chain is decided then
+                int *slot = reinterpret_cast<int *>(smem + SM_PATH + ((iter + 1) & 1) * SM_PATH_SLOT);
+                const bool in_range = q_mine && q_n >= 0 && q_n < q_pT;
+                const bool all_in = __all_sync(0xffffffffu, !q_mine || in_range);
+                if (lane < FV_MD) slot[lane] = in_range ? q_n : 0;
+                if (lane == 0) {
+                    slot[17] = q_pb;
+                    slot[18] = q_shape_ok && all_in ? q_len : 0;
                 }
+                if (in_range && p.pparent) q_par = p.pparent[q_ppar + q_n];
             }
         }
         {
@@ -1101,38 +846,32 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
         }
         // stage 4: the path is checked (a chain from a root inside the previous tree) and published; the
         // per-step scalars of its nodes are asked for
-        if constexpr (FUSED) {
-            if (next_ok && warp == 4) {
-                int *slot = reinterpret_cast<int *>(smem + SM_PATH + ((iter + 1) & 1) * SM_PATH_SLOT);
-                const int n_up = __shfl_up_sync(0xffffffffu, q_n, 1);
-                bool bad = false;
-                if (q_mine) {
-                    if (q_n < 0 || q_n >= q_pT) bad = true;
-                    else if (p.pparent) bad = q_par != (lane ? n_up : -1);
-                    else if (lane && q_n <= n_up) bad = true;
-                }
-                if (q_len != 0 && (__any_sync(0xffffffffu, bad) || !q_shape_ok)) {
-                    if (lane == 0) report_status(p.status_dev, GDN_ERR_PATH);
-                    q_len = 0;
-                }
-                if (lane == 0) {
-                    slot[16] = q_len;
-                    slot[17] = q_pb;
-                }
-                if (lane < q_len) {
-                    const size_t n = (size_t)q_pb + q_n;
-                    q_g = __ldg(reinterpret_cast<const unsigned short *>(p.pg) + n * p.h_v + nh);
-                    q_be = __ldg(reinterpret_cast<const unsigned short *>(p.pbeta) + n * p.h_v + nh);
-                }
+        if (next_ok && warp == 4) {
+            int *slot = reinterpret_cast<int *>(smem + SM_PATH + ((iter + 1) & 1) * SM_PATH_SLOT);
+            const int n_up = __shfl_up_sync(0xffffffffu, q_n, 1);
+            bool bad = false;
+            if (q_mine) {
+                if (q_n < 0 || q_n >= q_pT) bad = true;
+                else if (p.pparent) bad = q_par != (lane ? n_up : -1);
+                else if (lane && q_n <= n_up) bad = true;
+            }
+            if (q_len != 0 && (__any_sync(0xffffffffu, bad) || !q_shape_ok)) {
+                if (lane == 0) report_status(p.status_dev, GDN_ERR_PATH);
+                q_len = 0;
+            }
+            if (lane == 0) {
+                slot[16] = q_len;
+                slot[17] = q_pb;
+            }
+            if (lane < q_len) {
+                const size_t n = (size_t)q_pb + q_n;
+                q_g = __ldg(reinterpret_cast<const unsigned short *>(p.pg) + n * p.h_v + nh);
+                q_be = __ldg(reinterpret_cast<const unsigned short *>(p.pbeta) + n * p.h_v + nh);
             }
         }
 
         // stage 5, while the tensor core works: the next unit's tables (depth, root paths) from the staged parent[]
-        if constexpr (GROUPED) {
-            if (next_ok) put_tables_g(nT, (iter + 1) & 1, t_node, t_d, t_row, t_g, t_be);
-        } else {
-            if (next_ok) walk_tables(nT, (iter + 1) & 1, t_g, t_be, t_bad);
-        }
+        if (next_ok) walk_tables(nT, (iter + 1) & 1, t_g, t_be, t_bad, same_tree);
         if (!mbar_wait_bounded(mbar_d, par)) *flag = 1;
         tc_fence_after();
 
@@ -1168,20 +907,19 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
         // they land in is free)
         if (next_ok) path_decay((iter + 1) & 1);
         if (next_ok) fetch_path_kv(nh, nhk, (iter + 1) & 1);
-        if constexpr (FUSED) {   // ... and the scalars of that path (asked for a phase ago)
-            if (next_ok && warp == 4) {   // lane t: decay of the path up to and including step t by a prefix sum
-                const float gt = lane < q_len ? gate_log_decay(q_g, PADDED && p.raw_gates) : 0.f;
-                float gsum = gt;
+        // ... and the scalars of that path (asked for a phase ago)
+        if (next_ok && warp == 4) {   // lane t: decay of the path up to and including step t by a prefix sum
+            const float gt = lane < q_len ? gate_log_decay(q_g, PADDED && p.raw_gates) : 0.f;
+            float gsum = gt;
 #pragma unroll
-                for (int off = 1; off < FV_MD; off <<= 1) {
-                    const float up = __shfl_up_sync(0xffffffffu, gsum, off);
-                    if (lane >= off) gsum += up;
-                }
-                if (lane < q_len) {
-                    const float A = expf(gsum);
-                    reinterpret_cast<float4 *>(smem + SM_PATH + ((iter + 1) & 1) * SM_PATH_SLOT + 128)[lane] =
-                        make_float4(A, gate_beta(q_be, PADDED && p.raw_gates), expf(gt), 1.f / A);
-                }
+            for (int off = 1; off < FV_MD; off <<= 1) {
+                const float up = __shfl_up_sync(0xffffffffu, gsum, off);
+                if (lane >= off) gsum += up;
+            }
+            if (lane < q_len) {
+                const float A = expf(gsum);
+                reinterpret_cast<float4 *>(smem + SM_PATH + ((iter + 1) & 1) * SM_PATH_SLOT + 128)[lane] =
+                    make_float4(A, gate_beta(q_be, PADDED && p.raw_gates), expf(gt), 1.f / A);
             }
         }
         unit_done_ok = *flag == 0;
@@ -1191,12 +929,7 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
             for (int idx = tid; idx < T * ROW_CHUNKS; idx += FV_THREADS) {
                 const int i = idx / ROW_CHUNKS, ck = idx % ROW_CHUNKS;
                 const uint4 val = *reinterpret_cast<const uint4 *>(smem + SM_RT_HI + (size_t)i * FV_D * sizeof(TOut) + ck * 16);
-                if constexpr (GROUPED) {   // the ancestors in front of a group belong to other groups' outputs
-                    if (i >= gx.n_prefix)
-                        *reinterpret_cast<uint4 *>(o + (((size_t)(base + vnode_s[i]) * p.h_v + h) * FV_D) * sizeof(TOut) + ck * 16) = val;
-                } else {
-                    *reinterpret_cast<uint4 *>(o + (((size_t)(base + i) * p.h_v + h) * FV_D) * sizeof(TOut) + ck * 16) = val;
-                }
+                *reinterpret_cast<uint4 *>(o + (((size_t)(base + i) * p.h_v + h) * FV_D) * sizeof(TOut) + ck * 16) = val;
             }
         }
     }
@@ -1204,7 +937,6 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
     if (!unit_done_ok) break;   // a bounded wait expired: stop, report, release
     if (next_ok) issue_gram((uint32_t)(done_units & 1));   // the next unit's Gram block, as soon as its tile is there
     b = nb; h = nh; hk = nhk; base = nbase; T = nT; cur_ok = next_ok;
-    gx = ngx;
     ucur = ncur;
     }   // unit loop
 
@@ -1215,39 +947,24 @@ __global__ void __launch_bounds__(FV_THREADS, 2) verify_sm100_persistent_kernel(
     if (warp == 0) tmem_dealloc(tmem, FV_TMEM_COLS);
 }
 
-template <typename TOut, bool FUSED, bool GROUPED>
-cudaError_t launch_fast_typed(const gdn_shape_t &s, const VerifyFastParams &p, cudaStream_t stream)
+template <typename TOut> cudaError_t launch_typed(const gdn_shape_t &s, const VerifyFastParams &p, cudaStream_t stream)
 {
     // persistent CTAs, two per SM, pipelined across units
     VerifyFastParams pt = p;
-    const bool padded = p.t_pad != 0;   // the padded layout and the on-chip gate activations share an instantiation
-    void (*kernel)(const VerifyFastParams);
-    if constexpr (GROUPED) {
-        // trees of more than 64 nodes: a unit is one ancestor-closed group of a (tree, head), taken from the plan's
-        // unit list (its length is read on the device; this bound only sizes the grid); rows are gathered
-        pt.n_units = p.n_units * p.groups_per_tree;
-        kernel = padded ? verify_sm100_persistent_kernel<TOut, false, false, true, true>
-                        : verify_sm100_persistent_kernel<TOut, false, false, false, true>;
-    } else {
-        // trees that fit one CTA: TMA tiles of the packed row tensors
-        if (!make_row_tensor_map(&pt.tm_k, p.k, s.total_nodes, s.h_qk, 64, FV_T, true) ||
-            !make_row_tensor_map(&pt.tm_q, p.q, s.total_nodes, s.h_qk, 64, FV_T, true) ||
-            !make_row_tensor_map(&pt.tm_v, p.v, s.total_nodes, s.h_v, FV_D, FV_T, false))
-            return cudaErrorNotSupported;
-        const bool small = s.max_tree_nodes <= 32;
-        kernel = small ? verify_sm100_persistent_kernel<TOut, FUSED, true, false, false>
-                       : verify_sm100_persistent_kernel<TOut, FUSED, false, false, false>;
-        if (padded)
-            kernel = small ? verify_sm100_persistent_kernel<TOut, FUSED, true, true, false>
-                           : verify_sm100_persistent_kernel<TOut, FUSED, false, true, false>;
-    }
+    const bool padded = p.t_pad != 0, small = s.max_tree_nodes <= 32;
+    if (!make_row_tensor_map(&pt.tm_k, p.k, s.total_nodes, s.h_qk, 64, FV_T, true) ||
+        !make_row_tensor_map(&pt.tm_q, p.q, s.total_nodes, s.h_qk, 64, FV_T, true) ||
+        !make_row_tensor_map(&pt.tm_v, p.v, s.total_nodes, s.h_v, FV_D, FV_T, false))
+        return cudaErrorNotSupported;
+    // the padded layout and the on-chip gate activations share an instantiation
+    void (*kernel)(const VerifyFastParams) = small ? padded ? commit_verify_kernel<TOut, true, true> : commit_verify_kernel<TOut, true, false>
+                                                   : padded ? commit_verify_kernel<TOut, false, true> : commit_verify_kernel<TOut, false, false>;
     static PerDevice seen[4];
     int sms = 0;
-    const cudaError_t e = device_sms(seen[(padded ? 2 : 0) + (s.max_tree_nodes <= 32 ? 1 : 0)], reinterpret_cast<const void *>(kernel),
+    const cudaError_t e = device_sms(seen[2 * padded + small], reinterpret_cast<const void *>(kernel),
                                      SM_ALLOC, &sms);
     if (e != cudaSuccess) return e;
-    pt.prefetch_dist = 2 * sms;
-    const int grid = pt.n_units < pt.prefetch_dist ? pt.n_units : pt.prefetch_dist;
+    const int grid = pt.n_units < 2 * sms ? pt.n_units : 2 * sms;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(FV_THREADS);
@@ -1263,7 +980,7 @@ cudaError_t launch_fast_typed(const gdn_shape_t &s, const VerifyFastParams &p, c
 
 VerifyFastParams make_params(const gdn_shape_t &s, const float *S0, const void *q, const void *k, const void *v,
                              const void *g, const void *beta, const int32_t *node_offsets, void *o,
-                             const PlanPtrs &plan, int32_t *status_dev)
+                             int32_t *status_dev)
 {
     VerifyFastParams p{};
     p.h_qk = s.h_qk; p.h_v = s.h_v; p.n_units = s.n_seq * s.h_v; p.scale = s.scale;
@@ -1273,23 +990,16 @@ VerifyFastParams make_params(const gdn_shape_t &s, const float *S0, const void *
     p.beta = static_cast<const __nv_bfloat16 *>(beta);
     p.node_offsets = node_offsets; p.o = o;
     p.n_seq = s.n_seq; p.total_nodes = s.total_nodes; p.max_tree_nodes = s.max_tree_nodes; p.max_depth = s.max_depth;
-    p.depth = plan.depth; p.anc8 = plan.anc8; p.status_dev = status_dev;
-    // upper bound of the groups of a tree (the real ones are in the plan's unit list)
-    p.groups_per_tree = s.max_tree_nodes <= FV_T ? 1 : (s.max_tree_nodes + GDN_GROUP_MIN_NODES - 1) / GDN_GROUP_MIN_NODES;
-    p.anc_stride = s.max_depth;
-    p.anc16 = plan.anc; p.dfs_node = plan.dfs_node; p.dfs_depth = plan.dfs_depth; p.dfs_anc8 = plan.dfs_anc8;
-    p.unit_list = plan.unit_list;
-    p.unit_count = plan.unit_count;
-    p.unit_capacity = (int)unit_list_capacity(s);
-    p.plan_magic = plan_magic(s.n_seq, s.max_tree_nodes, s.max_depth);
+    p.status_dev = status_dev;
     return p;
 }
 
 }  // namespace
 
 // Few units: the commit kernel and, behind it, the verification, which works out everything but the product with the state
-// meanwhile -- the two run side by side on different SMs as long as there are enough of them.  Measured (us, 64 nodes, path
-// of 7; this kernel / two kernels): 32 units 13.5 / 11.7, 64 units 13.7 / 11.9, 80 units 13.6 / 14.8, 128 units 14.0 / 15.0.
+// meanwhile -- the two run side by side on SMs of their own as long as there are enough of them.  Measured (us, 64 nodes;
+// this kernel / two kernels), path of 7: 32 units 13.3 / 9.5, 64 units 13.5 / 9.7, 128 units 13.9 / 13.0; path of 1: 64 units
+// 11.3 / 9.9, 128 units 11.6 / 12.3 (the path lengths are on the device, so the line lies where both gain).
 static bool as_two_kernels(const gdn_shape_t &s)
 {
     static PerDevice seen;
@@ -1315,7 +1025,7 @@ cudaError_t launch_commit_verify_sm100_padded(const gdn_shape_t &s, int n_trees,
         if (e != cudaSuccess) return e;
         return launch_verify_sm100_padded(s, n_trees, raw_gates, S, q, k, v, g, beta, parent, n_nodes, o, status_dev, stream, true);
     }
-    VerifyFastParams p = make_params(s, S, q, k, v, g, beta, nullptr, o, PlanPtrs{}, status_dev);
+    VerifyFastParams p = make_params(s, S, q, k, v, g, beta, nullptr, o, status_dev);
     p.parent = parent;
     p.t_pad = s.max_tree_nodes; p.n_trees = n_trees; p.n_nodes = n_nodes; p.raw_gates = raw_gates ? 1 : 0;
     p.S_rw = S;
@@ -1323,8 +1033,8 @@ cudaError_t launch_commit_verify_sm100_padded(const gdn_shape_t &s, int n_trees,
     p.pg = static_cast<const __nv_bfloat16 *>(g_prev); p.pbeta = static_cast<const __nv_bfloat16 *>(beta_prev);
     p.pparent = parent_prev; p.path = path;
     p.pt_pad = prev_t_pad; p.pn_nodes = n_nodes_prev; p.path_len = path_len; p.path_stride = s.max_depth;
-    if (s.out_dtype == GDN_BF16) return launch_fast_typed<__nv_bfloat16, true, false>(s, p, stream);
-    return launch_fast_typed<float, true, false>(s, p, stream);
+    if (s.out_dtype == GDN_BF16) return launch_typed<__nv_bfloat16>(s, p, stream);
+    return launch_typed<float>(s, p, stream);
 }
 
 cudaError_t launch_commit_verify_sm100(const gdn_shape_t &s, float *S, const void *k_prev, const void *v_prev,
@@ -1342,14 +1052,14 @@ cudaError_t launch_commit_verify_sm100(const gdn_shape_t &s, float *S, const voi
         if (e != cudaSuccess) return e;
         return launch_verify_sm100(s, S, q, k, v, g, beta, parent, node_offsets, o, PlanPtrs{}, status_dev, stream, true);
     }
-    VerifyFastParams p = make_params(s, S, q, k, v, g, beta, node_offsets, o, PlanPtrs{}, status_dev);
+    VerifyFastParams p = make_params(s, S, q, k, v, g, beta, node_offsets, o, status_dev);
     p.parent = parent;
     p.S_rw = S;
     p.pk = static_cast<const __nv_bfloat16 *>(k_prev); p.pv = static_cast<const __nv_bfloat16 *>(v_prev);
     p.pg = static_cast<const __nv_bfloat16 *>(g_prev); p.pbeta = static_cast<const __nv_bfloat16 *>(beta_prev);
     p.pparent = parent_prev; p.pnode_offsets = node_offsets_prev; p.path = path; p.path_offsets = path_offsets;
-    if (s.out_dtype == GDN_BF16) return launch_fast_typed<__nv_bfloat16, true, false>(s, p, stream);
-    return launch_fast_typed<float, true, false>(s, p, stream);
+    if (s.out_dtype == GDN_BF16) return launch_typed<__nv_bfloat16>(s, p, stream);
+    return launch_typed<float>(s, p, stream);
 }
 
 

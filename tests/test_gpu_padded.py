@@ -105,6 +105,33 @@ def test_commit_verify_padded(tl, raw_gates):
     _assert_outputs(tl, dn, _oracle_verify(new, S_ref), f"commit_verify_padded raw={raw_gates}")
 
 
+@pytest.mark.parametrize("n_trees,rejected", [(1, None), (1, 0), (2, None), (2, 1)])
+def test_commit_verify_padded_shares_tables_between_units(tl, n_trees, rejected):
+    """640 units, several per CTA, whose trees repeat or alternate; a rejected tree is reported, nothing of its slots is
+    stored, and their accepted paths are committed all the same."""
+    import paper_2607_06763_b200 as gdn
+    rng = np.random.default_rng(805)
+    prev = synth.padded_case(830, _trees(rng, (16, 9)[:n_trees]), 20 // n_trees, 16, False, h_qk=16, h_v=32)
+    new = synth.padded_case(831, _trees(rng, (13, 16)[:n_trees]), 20 // n_trees, 16, False, h_qk=16, h_v=32)
+    dp, dn = PaddedDevice(prev), PaddedDevice(new)
+    if rejected is not None:
+        dn.parent[rejected, 5] = 9
+    S = dp.S0.clone()
+    rc = gdn.gdn_tree_commit_verify_padded(dn.shape, n_trees, False, S, prev.t_pad, dp.k, dp.v, dp.g_in, dp.beta_in,
+                                           dp.parent, dp.n_nodes, dp.path, dp.path_len, dn.q, dn.k, dn.v, dn.g_in,
+                                           dn.beta_in, dn.parent, dn.n_nodes, dn.o, dn.status)
+    assert rc == 0 and dn.status_value() == (0 if rejected is None else -7)
+    S_ref = _oracle_commit(prev, prev.S0.astype(np.float64))
+    tl.assert_state_close(S.cpu().numpy().astype(np.float64), S_ref, what="state")
+    o, ref = dn.o_host(), _oracle_verify(new, S_ref)
+    for s in range(new.n_slots):
+        t = s % n_trees
+        n = 0 if t == rejected else int(new.n_nodes[t])
+        if n:
+            tl.assert_close_per_head(o[s, :n], ref[s, :n], np.array([0, n]), f"slot {s}", bf16_out=True)
+        assert np.all(o[s, n:] == 7.0)
+
+
 def test_commit_verify_padded_with_nothing_to_commit(tl):
     """All path lengths zero: a plain verification, every state untouched."""
     import paper_2607_06763_b200 as gdn
