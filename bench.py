@@ -562,13 +562,16 @@ def main():
         if args.impl == "recurrent":
             kernel_name, launches_per_step, dom_bytes, dom_ms = "verify_recurrent_kernel", 1, vbytes, ms_per_step
         elif single_cta_trees:
-            kernel_name = "verify_sm100_persistent_kernel<fused commit>" if fused else "verify_sm100_persistent_kernel"
+            kernel_name = "commit_verify_kernel" if fused else "verify_plain_kernel"
             launches_per_step = {"fused": 1, "separate": 2, "verify": 1}[args.mode]
+            sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
+            if fused and w.n_seq * w.h_v <= sms // 2:   # few units: commit and verify kernels side by side
+                kernel_name, launches_per_step = "commit_tile128_kernel + verify_plain_kernel", 2
             dom_bytes = sbytes if fused else vbytes
             dom_ms = ms_per_step if args.mode != "separate" else split[0]
         else:   # larger trees: tree plan + the verify kernel in its grouped mode; the fused call builds the plan in
                 # extra CTAs of the commit kernel's grid (two launches), the padded layout plans in a call of its own
-            kernel_name = "verify_sm100_persistent_kernel<grouped>"
+            kernel_name = "verify_plain_kernel<grouped>"
             launches_per_step = {"fused": 3 if args.layout == "padded" else 2, "separate": 3, "verify": 2}[args.mode]
             dom_bytes = vbytes
             dom_ms = None if args.mode == "fused" else (ms_per_step if args.mode == "verify" else split[0])
