@@ -47,19 +47,23 @@ __device__ __forceinline__ void wait_for_previous_kernel()
     asm volatile("griddepcontrol.launch_dependents;");
 }
 
+// max_shared: on SMs set up for the most shared memory, so that a verification launched behind can move in beside the grid.
 template <typename... KernelArgs, typename... Args>
-cudaError_t launch_overlapped(void (*kernel)(KernelArgs...), int grid, int threads, size_t smem, cudaStream_t stream, Args... args)
+cudaError_t launch_overlapped(void (*kernel)(KernelArgs...), int grid, int threads, size_t smem, bool max_shared, cudaStream_t stream,
+                              Args... args)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[1].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = max_shared ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
@@ -180,11 +184,15 @@ __global__ void __launch_bounds__(CM_THREADS, 2) commit_generic_kernel(const Com
         }
 }
 
-// Fast forms for d_k = d_v = 128, bf16 inputs, paths of at most 16 nodes: one CTA of 256 threads per (tree, value head);
+// Fast forms for d_k = d_v = 128, bf16 inputs, paths of at most 16 nodes: CTAs of 256 threads, one per (tree, value head);
 // the state loads go first, the path is fetched and checked by one warp with shuffles, its k/v rows arrive by cp.async.
-// Two forms of the arithmetic, chosen by how many CTAs the call has for how many SMs (commit_form):
+// Two forms of the arithmetic and, for few tiles, a split of the tile, chosen by how many tiles the call has for how many SMs
+// (commit_form):
 //   step by step (commit_replay_unit): 64 state registers per thread, two CTAs per SM; the shortest chain, the better one
 //     while all CTAs of the call are resident at once that way;
+//   step by step with 32 rows of the tile per CTA, one per thread: a step is as short as its reduction then.  32 tiles, path of
+//     1 / 7 / 12: 4.1 / 5.7 / 6.8 -> 3.1 / 3.9 / 4.6 us, followed by a verification 11.5 / 13.0 / 14.4 -> 11.6 / 11.7 / 12.9 us (only
+//     with the carve-out of launch_overlapped: 14.5 without); at 64 tiles the pair gets slower (11.7 / 13.2 -> 12.7 / 13.4);
 //   as matrix products (commit_fragment_unit, gdn_fragments.cuh): 32 state registers, the tile read twice, the second time
 //     out of L2; three or four CTAs per SM, so that the loads of some run under the arithmetic of others.
 // Measured (us; 32 heads per slot, path of 7; two by two / three / four per SM): 4 slots 8.2 / 8.9 / 9.3, 8 slots 10.6 /
@@ -203,8 +211,10 @@ __device__ __forceinline__ void cf_cp_async_4(uint32_t dst, const void *src, boo
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
 }
 
-__device__ __forceinline__ void commit_replay_unit(const CommitParams &p, const int unit)
+// PARTS: the tile's rows split over that many CTAs.
+template <int PARTS> __device__ __forceinline__ void commit_replay_unit(const CommitParams &p, const int unit, const int part)
 {
+    constexpr int ROWS = 4 / PARTS;   // per thread
     __shared__ __align__(16) uint16_t pk_s[CF_MD * GDN_TILE_D];
     __shared__ __align__(16) uint16_t pv_s[CF_MD * GDN_TILE_D];
     __shared__ __align__(16) float4 ab_s[CF_MD];
@@ -213,9 +223,10 @@ __device__ __forceinline__ void commit_replay_unit(const CommitParams &p, const 
     const int b = unit / p.h_v, h = unit % p.h_v;
     const int hk = h / (p.h_v / p.h_qk);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid < 4)   // L2 may be asked for the tile meanwhile (a prefetch consumes nothing)
+    const int row0 = part * (GDN_TILE_D / PARTS) + warp * 4 * ROWS;   // of this warp
+    if (tid < ROWS)   // L2 may be asked for the tile meanwhile (a prefetch consumes nothing)
         asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;"
-                     ::"l"(p.S + (size_t)unit * GDN_TILE_D * GDN_TILE_D + (size_t)tid * 4096), "r"(16384) : "memory");
+                     ::"l"(p.S + (size_t)unit * GDN_TILE_D * GDN_TILE_D + (size_t)(part * ROWS + tid) * 4096), "r"(16384) : "memory");
     wait_for_previous_kernel();
     const int r4 = lane >> 3, l8 = lane & 7;
     const int tree = p.t_pad ? b % p.n_trees : b;
@@ -225,10 +236,10 @@ __device__ __forceinline__ void commit_replay_unit(const CommitParams &p, const 
 
     // the state tile first: its latency covers the path fetch below
     float *S = p.S + (size_t)(b * p.h_v + h) * GDN_TILE_D * GDN_TILE_D;
-    float4 x[4][4];
+    float4 x[ROWS][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float *src = S + (size_t)(warp * 16 + i * 4 + r4) * GDN_TILE_D + l8 * 8;
+    for (int i = 0; i < ROWS; ++i) {
+        const float *src = S + (size_t)(row0 + i * 4 + r4) * GDN_TILE_D + l8 * 8;
 #pragma unroll
         for (int kh = 0; kh < 2; ++kh) ldg_v8(src + kh * 64, x[i][kh * 2 + 0], x[i][kh * 2 + 1]);
     }
@@ -299,11 +310,11 @@ __device__ __forceinline__ void commit_replay_unit(const CommitParams &p, const 
     len = len_s;
     if (len == 0) return;   // rejected path: this state stays as it was
 
-    replay_path_on_tile(x, len, pk_s, pv_s, ab_s, warp, r4, l8);
+    replay_path_on_tile(x, len, pk_s, pv_s, ab_s, row0, r4, l8);
 
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        float *dst = S + (size_t)(warp * 16 + i * 4 + r4) * GDN_TILE_D + l8 * 8;
+    for (int i = 0; i < ROWS; ++i) {
+        float *dst = S + (size_t)(row0 + i * 4 + r4) * GDN_TILE_D + l8 * 8;
 #pragma unroll
         for (int kh = 0; kh < 2; ++kh) stg_v8(dst + kh * 64, x[i][kh * 2 + 0], x[i][kh * 2 + 1]);
     }
@@ -435,14 +446,15 @@ __device__ __forceinline__ void commit_fragment_unit(const CommitParams &p, cons
         }
 }
 
-// CTAS: CTAs per SM (2: step by step, otherwise as matrix products)
-template <int CTAS> __device__ __forceinline__ void commit_unit(const CommitParams &p, const int unit)
+// CTAS: CTAs per SM (1, 2: step by step, 1: a quarter of a tile per CTA; otherwise as matrix products)
+template <int CTAS> __device__ __forceinline__ void commit_unit(const CommitParams &p, const int i)
 {
-    if constexpr (CTAS == 2) commit_replay_unit(p, unit);
-    else commit_fragment_unit(p, unit);
+    if constexpr (CTAS == 1) commit_replay_unit<4>(p, i >> 2, i & 3);
+    else if constexpr (CTAS == 2) commit_replay_unit<1>(p, i, 0);
+    else commit_fragment_unit(p, i);
 }
 
-template <int CTAS> __global__ void __launch_bounds__(CF_THREADS, CTAS) commit_tile128_kernel(const CommitParams p)
+template <int CTAS> __global__ void __launch_bounds__(CF_THREADS, CTAS == 1 ? 4 : CTAS) commit_tile128_kernel(const CommitParams p)
 {
     commit_unit<CTAS>(p, (int)blockIdx.x);
 }
@@ -450,7 +462,7 @@ template <int CTAS> __global__ void __launch_bounds__(CF_THREADS, CTAS) commit_t
 // The fused call on trees of more than 64 nodes: the plans of the NEW trees do not depend on the commit of the previous
 // step's paths, so they are built by the first n_seq CTAs of the same grid instead of by a launch of their own in
 // between (one launch and one dependency hop less in front of the verify kernel).
-template <int CTAS> __global__ void __launch_bounds__(CF_THREADS, CTAS) commit_plan_kernel(const CommitParams p, const PlanArgs a)
+template <int CTAS> __global__ void __launch_bounds__(CF_THREADS, CTAS == 1 ? 2 : CTAS) commit_plan_kernel(const CommitParams p, const PlanArgs a)
 {
     if ((int)blockIdx.x < a.n_seq) {
         wait_for_previous_kernel();
@@ -459,20 +471,24 @@ template <int CTAS> __global__ void __launch_bounds__(CF_THREADS, CTAS) commit_p
         commit_unit<CTAS>(p, (int)blockIdx.x - a.n_seq);
 }
 
-// CTAs per SM for a call of `units` tiles: the fewest with which they are all resident at once.
+// Form for a call of `units` tiles: a quarter of a tile per CTA while those have SMs of their own, otherwise the fewest CTAs
+// per SM with which they are all resident at once.
 int commit_form(int units)
 {
     static PerDevice seen;
     int sms = 0;
     if (device_sms(seen, nullptr, 0, &sms) != cudaSuccess) return 2;
-    return units <= 2 * sms ? 2 : units <= 3 * sms ? 3 : 4;
+    return 4 * units <= sms ? 1 : units <= 2 * sms ? 2 : units <= 3 * sms ? 3 : 4;
 }
 
 cudaError_t launch_tile128(const CommitParams &p, int units, cudaStream_t stream)
 {
     const int form = commit_form(units);
-    return launch_overlapped(form == 2 ? commit_tile128_kernel<2> : form == 3 ? commit_tile128_kernel<3> : commit_tile128_kernel<4>,
-                             units, CF_THREADS, 0, stream, p);
+    return launch_overlapped(form == 1   ? commit_tile128_kernel<1>
+                             : form == 2 ? commit_tile128_kernel<2>
+                             : form == 3 ? commit_tile128_kernel<3>
+                                         : commit_tile128_kernel<4>,
+                             form == 1 ? 4 * units : units, CF_THREADS, 0, form == 1, stream, p);
 }
 
 }  // namespace
@@ -494,7 +510,7 @@ cudaError_t launch_commit_generic(const gdn_shape_t &s, float *S, const void *k,
     const cudaError_t e = device_sms(seen[s.in_dtype == GDN_BF16], reinterpret_cast<const void *>(kernel),
                                      commit_generic_smem(GDN_MAX_DEPTH_CAP), &sms);
     if (e != cudaSuccess) return e;
-    return launch_overlapped(kernel, grid, CM_THREADS, commit_generic_smem(s.max_depth), stream, p);
+    return launch_overlapped(kernel, grid, CM_THREADS, commit_generic_smem(s.max_depth), false, stream, p);
 }
 
 bool commit_tile128_supported(const gdn_shape_t &s) { return commit_padded_supported(s); }
@@ -513,9 +529,13 @@ cudaError_t launch_commit_plan(const gdn_shape_t &s, float *S, const void *k, co
     }
     CommitParams p{s.h_qk, s.h_v, s.d_k, s.d_v, s.max_depth, S, k, v, g, beta, parent_prev, node_offsets_prev, path,
                    path_offsets, status_dev, 0, 0, 0, 0, nullptr, nullptr};
-    const int grid = s.n_seq + s.n_seq * s.h_v, form = commit_form(s.n_seq * s.h_v);
-    return launch_overlapped(form == 2 ? commit_plan_kernel<2> : form == 3 ? commit_plan_kernel<3> : commit_plan_kernel<4>, grid,
-                             CF_THREADS, 0, stream, p, plan_args(s, parent, node_offsets, nullptr, plan, status_dev));
+    const int units = s.n_seq * s.h_v, form = commit_form(units);
+    return launch_overlapped(form == 1   ? commit_plan_kernel<1>
+                             : form == 2 ? commit_plan_kernel<2>
+                             : form == 3 ? commit_plan_kernel<3>
+                                         : commit_plan_kernel<4>,
+                             s.n_seq + (form == 1 ? 4 * units : units), CF_THREADS, 0, form == 1, stream, p,
+                             plan_args(s, parent, node_offsets, nullptr, plan, status_dev));
 }
 
 bool commit_padded_supported(const gdn_shape_t &s)

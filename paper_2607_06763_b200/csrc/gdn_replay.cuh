@@ -32,8 +32,10 @@ __device__ __forceinline__ void stg_v8(float *p, const float4 &a, const float4 &
 // k.s_c by shuffles (the four rows of a thread folded into one butterfly), the four rows of a thread advance together.
 //   pks, pvs : the path's k and v rows in shared memory, bf16 [L][128]
 //   ab_path  : per step (A_t = decay of the path up to and including step t, beta_t, alpha_t, 1 / A_t)
-__device__ __forceinline__ void replay_path_on_tile(float4 (&x)[4][4], int L, const uint16_t *pks, const uint16_t *pvs,
-                                                    const float4 *ab_path, int warp, int r4, int l8)
+// ROWS < 4: a warp owns 4 ROWS rows from row0 on (a thread row0 + 4 i + r4, i < ROWS).
+template <int ROWS>
+__device__ __forceinline__ void replay_path_on_tile(float4 (&x)[ROWS][4], int L, const uint16_t *pks, const uint16_t *pvs,
+                                                    const float4 *ab_path, int row0, int r4, int l8)
 {
     // Scaled form: with A_t = alpha_1 .. alpha_t and s~ = s / A_t a step is s~ += k beta_t (v / A_t - k.s~)
     // (the decay costs nothing), and s = A_L s~ at the end.  It is taken unless the path decays below 2^-80:
@@ -56,12 +58,12 @@ __device__ __forceinline__ void replay_path_on_tile(float4 (&x)[4][4], int L, co
         const float4 ab = ab_path[t];   // (A_t, beta_t, alpha_t, 1 / A_t)
         // the four rows of this thread advance together: four independent FMA chains, then their
         // shuffle reductions back to back, then the four updates
-        float dot[4];
+        float dot[ROWS];
         float2 kf2[8];   // the same values as packed pairs for the two-wide fp32 FMA
 #pragma unroll
         for (int e = 0; e < 8; ++e) kf2[e] = make_float2(kf[2 * e], kf[2 * e + 1]);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < ROWS; ++i) {
             float2 acc = make_float2(0.f, 0.f);
 #pragma unroll
             for (int q4 = 0; q4 < 4; ++q4) {
@@ -73,31 +75,42 @@ __device__ __forceinline__ void replay_path_on_tile(float4 (&x)[4][4], int L, co
         // Reduction over the eight lanes of a row group with the four rows folded as it goes: after the exchange
         // with lane ^ 1 a lane keeps two rows, after lane ^ 2 one, after lane ^ 4 it holds the complete k.s of row
         // my_i (4 shuffles instead of 12); it forms w of that row alone and the four w come back by shuffles.
-        const bool b0 = (l8 & 1) != 0, b1 = (l8 & 2) != 0;
-        const int my_i = (b0 ? 2 : 0) + (b1 ? 1 : 0);
-        float a0, a1;
-        {
-            const float s0 = b0 ? dot[0] : dot[2], s1 = b0 ? dot[1] : dot[3];
-            const float r0 = __shfl_xor_sync(0xffffffffu, s0, 1), r1 = __shfl_xor_sync(0xffffffffu, s1, 1);
-            a0 = (b0 ? dot[2] : dot[0]) + r0;
-            a1 = (b0 ? dot[3] : dot[1]) + r1;
+        float wv[ROWS];
+        if constexpr (ROWS == 4) {
+            const bool b0 = (l8 & 1) != 0, b1 = (l8 & 2) != 0;
+            const int my_i = (b0 ? 2 : 0) + (b1 ? 1 : 0);
+            float a0, a1;
+            {
+                const float s0 = b0 ? dot[0] : dot[2], s1 = b0 ? dot[1] : dot[3];
+                const float r0 = __shfl_xor_sync(0xffffffffu, s0, 1), r1 = __shfl_xor_sync(0xffffffffu, s1, 1);
+                a0 = (b0 ? dot[2] : dot[0]) + r0;
+                a1 = (b0 ? dot[3] : dot[1]) + r1;
+            }
+            float d1 = (b1 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, b1 ? a0 : a1, 2);
+            d1 += __shfl_xor_sync(0xffffffffu, d1, 4);
+            const int my_row = row0 + my_i * 4 + r4;
+            const float vc = __uint_as_float((uint32_t)pvs[t * GDN_TILE_D + my_row] << 16);
+            // scaled form: x holds s / A_t and w = beta_t (v / A_t - k.s~); plain form: w = beta_t (v - alpha_t k.s)
+            const float w_mine = scaled ? ab.y * fmaf(vc, ab.w, -d1) : ab.y * (vc - ab.z * d1);
+            const int g8 = (r4 << 3);   // first lane of this row group
+            wv[0] = __shfl_sync(0xffffffffu, w_mine, g8 | 0);
+            wv[1] = __shfl_sync(0xffffffffu, w_mine, g8 | 2);
+            wv[2] = __shfl_sync(0xffffffffu, w_mine, g8 | 1);
+            wv[3] = __shfl_sync(0xffffffffu, w_mine, g8 | 3);
+        } else {
+#pragma unroll
+            for (int i = 0; i < ROWS; ++i) {
+                float d = dot[i];
+#pragma unroll
+                for (int m = 1; m < 8; m <<= 1) d += __shfl_xor_sync(0xffffffffu, d, m);
+                const float vc = __uint_as_float((uint32_t)pvs[t * GDN_TILE_D + row0 + i * 4 + r4] << 16);
+                wv[i] = scaled ? ab.y * fmaf(vc, ab.w, -d) : ab.y * (vc - ab.z * d);
+            }
         }
-        float d1 = (b1 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, b1 ? a0 : a1, 2);
-        d1 += __shfl_xor_sync(0xffffffffu, d1, 4);
-        const int my_row = warp * 16 + my_i * 4 + r4;
-        const float vc = __uint_as_float((uint32_t)pvs[t * GDN_TILE_D + my_row] << 16);
-        // scaled form: x holds s / A_t and w = beta_t (v / A_t - k.s~); plain form: w = beta_t (v - alpha_t k.s)
-        const float w_mine = scaled ? ab.y * fmaf(vc, ab.w, -d1) : ab.y * (vc - ab.z * d1);
-        const int g8 = (r4 << 3);   // first lane of this row group
-        float wv[4];
-        wv[0] = __shfl_sync(0xffffffffu, w_mine, g8 | 0);
-        wv[1] = __shfl_sync(0xffffffffu, w_mine, g8 | 2);
-        wv[2] = __shfl_sync(0xffffffffu, w_mine, g8 | 1);
-        wv[3] = __shfl_sync(0xffffffffu, w_mine, g8 | 3);
         if (scaled) {
             // s~ += k w, one packed FMA per pair
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < ROWS; ++i) {
                 const float2 w2 = make_float2(wv[i], wv[i]);
 #pragma unroll
                 for (int q4 = 0; q4 < 4; ++q4) {
@@ -108,7 +121,7 @@ __device__ __forceinline__ void replay_path_on_tile(float4 (&x)[4][4], int L, co
             }
         } else {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < ROWS; ++i) {
                 const float2 w2 = make_float2(wv[i], wv[i]), a2 = make_float2(ab.z, ab.z);
 #pragma unroll
                 for (int q4 = 0; q4 < 4; ++q4) {
@@ -122,7 +135,7 @@ __device__ __forceinline__ void replay_path_on_tile(float4 (&x)[4][4], int L, co
     if (scaled) {   // back to s = A_L s~
         const float aL = ab_path[L - 1].x;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < ROWS; ++i)
 #pragma unroll
             for (int q4 = 0; q4 < 4; ++q4)
                 x[i][q4] = make_float4(aL * x[i][q4].x, aL * x[i][q4].y, aL * x[i][q4].z, aL * x[i][q4].w);

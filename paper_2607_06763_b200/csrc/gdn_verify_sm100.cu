@@ -593,7 +593,7 @@ __global__ void __launch_bounds__(FV_THREADS, 2) commit_verify_kernel(const __gr
     if (!healthy) path_len = 0;    // a wait expired: this state is left as it was
     if (path_len > 0) {
         replay_path_on_tile(x, path_len, reinterpret_cast<const uint16_t *>(smem + SM_PK),
-                            reinterpret_cast<const uint16_t *>(smem + SM_PV), ab_path, warp, r4, l8);
+                            reinterpret_cast<const uint16_t *>(smem + SM_PV), ab_path, warp * 16, r4, l8);
     }
     // The v rows move into registers in the orientation of the R phase (component c = TMEM lane of this
     // thread, its 32 nodes, two bf16 per register): they are about to be overwritten by the state operand.
