@@ -372,7 +372,7 @@ __device__ __forceinline__ void commit_fragment_unit(const CommitParams &p, cons
                                v + ((size_t)(pb + nt) * p.h_v + h) * GDN_TILE_D + c16 * 8);
         }
     }
-    float G = 0.f, be = 0.f;   // of step `lane` (warp 0)
+    float gt = 0.f, be = 0.f;   // of step `lane` (warp 0)
     if (warp == 0) {
         // lane t: entry t of the path and that node's parent; the path must be a chain from a root inside the tree
         const int ppar = p.t_pad ? tree * p.t_pad : pb;   // first entry of the tree in parent[]
@@ -383,7 +383,7 @@ __device__ __forceinline__ void commit_fragment_unit(const CommitParams &p, cons
             if (n >= 0 && n < pT) {
                 if (p.parent) parent_n = p.parent[ppar + n];
                 const size_t i = (size_t)(pb + n) * p.h_v + h;
-                G = gate_log_decay(static_cast<const unsigned short *>(p.g)[i], p.raw_gates != 0);
+                gt = gate_log_decay(static_cast<const unsigned short *>(p.g)[i], p.raw_gates != 0);
                 be = gate_beta(static_cast<const unsigned short *>(p.beta)[i], p.raw_gates != 0);
             }
         }
@@ -398,14 +398,16 @@ __device__ __forceinline__ void commit_fragment_unit(const CommitParams &p, cons
             if (lane == 0) report_status(p.status_dev, GDN_ERR_PATH);
             len = 0;
         }
-        // sums of g along the path over the lanes, and the per-step scalars
+        // sums of g along the path over the lanes (up to and including step t, and behind it), and the per-step scalars
+        float G = gt;
 #pragma unroll
         for (int off = 1; off < CF_MD; off <<= 1) {
             const float up = __shfl_up_sync(0xffffffffu, G, off);
             if (lane >= off) G += up;
         }
         const float G_L = __shfl_sync(0xffffffffu, G, max(len - 1, 0));
-        if (lane < len) scal_s[lane] = make_float4(be, be * expf(G), expf(G_L - G), 0.f);
+        const float behind = DecayWindows(gt).sum(max(len - 1, 0), max(len - 1 - lane, 0));
+        if (lane < len) scal_s[lane] = make_float4(be, be * expf(G), expf(behind), 0.f);
         if (lane == 0) {
             len_s = len;
             decay_s = expf(G_L);
@@ -417,7 +419,7 @@ __device__ __forceinline__ void commit_fragment_unit(const CommitParams &p, cons
     if (len == 0) return;   // rejected path: this state stays as it was
     const bool two = len > 8;
     const uint32_t operand = path_operand(pk, lane);
-    if (warp == 0 && len > 1) path_coupling(pk, len, G, be, couple_s, lane);
+    if (warp == 0 && len > 1) path_coupling(pk, len, gt, be, couple_s, lane);
     PathUpdate up;
     {
         PathProducts a;

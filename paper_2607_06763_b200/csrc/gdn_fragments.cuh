@@ -84,8 +84,10 @@ __device__ __forceinline__ void store_chunk(float *dst, int jj, const float (&x)
 }
 
 // An accepted path in shared memory: k rows in the permuted order (zero up to the next multiple of eight rows), v rows
-// bf16 [..][128], and per step t: scal (beta_t, beta_t A_t, E_t, .) with A_t = exp(G_t), E_t = exp(G_L - G_t), G = sum of g
-// along the path; coupling[u][t] = beta_t exp(G_t - G_u) k_t.k_u for t > u, 0 otherwise (row stride 16).
+// bf16 [..][128], and per step t: scal (beta_t, beta_t A_t, E_t, .) with A_t = exp(sum of g up to and including step t), E_t =
+// exp(sum of g behind step t); coupling[u][t] = beta_t exp(sum of g behind step u up to and including t) k_t.k_u for t > u, 0
+// otherwise (row stride 16).  Every sum runs over just the steps it names: as a difference of two sums from the root it would
+// lose the weak decays behind a strong one (-3000 on the path: 1.2e-4 off), and be no number behind g = -inf (alpha = 0).
 struct PathTile {
     const uint16_t *pv;
     const float4 *scal;
@@ -93,8 +95,8 @@ struct PathTile {
 };
 
 // S <- S after L steps (1 <= L <= 16).  With u_t = beta_t (v_t - A_t k_t.S) - sum_{u < t} coupling_ut u_u (the triangular
-// form of Section 3.4.1 on the path alone), S_L = A_L S + sum_t E_t u_t k_t^T; every factor is at most 1, so nothing can
-// overflow whatever the decays.  The products run on bf16 operands that are exact (k) or three-term splits (S, E u), i.e.
+// form of Section 3.4.1 on the path alone), S_L = A_L S + sum_t E_t u_t k_t^T; every decay factor is in 0..1 whatever the
+// decays.  The products run on bf16 operands that are exact (k) or three-term splits (S, E u), i.e.
 // at fp32 precision.  The tile passes through the registers twice: once for the products, once for the update.
 struct PathProducts {     // steps 2 l4, 2 l4 + 1 (+ 8 in the second entry) of rows g (entries 0, 1) and g + 8 (2, 3)
     float z[2][4], rest[2][4];   // the mid and lo terms go to accumulators of their own (shorter chains)
@@ -194,9 +196,35 @@ __device__ __forceinline__ void path_update_chunk(float (&x)[4][4], int jj, bool
     }
 }
 
-// The coupling table of a path whose k rows are in shared memory, by one warp (lane t: G_t, beta_t of step t; rows beyond
+// Sums of g over runs of steps, by one warp whose lane t holds g of step t (0 beyond the path): w[j] is the sum of the 2^j
+// steps up to and including step t.
+struct DecayWindows {
+    float w[4];
+    __device__ __forceinline__ explicit DecayWindows(float g)
+    {
+        w[0] = g;
+#pragma unroll
+        for (int j = 1; j < 4; ++j) w[j] = w[j - 1] + __shfl_up_sync(0xffffffffu, w[j - 1], 1 << (j - 1));
+    }
+    // the n steps up to and including step t (0 <= n <= 15, n <= t + 1; all lanes call)
+    __device__ __forceinline__ float sum(int t, int n) const
+    {
+        float s = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float x = __shfl_sync(0xffffffffu, w[j], t);
+            if ((n >> j) & 1) {
+                s += x;
+                t -= 1 << j;
+            }
+        }
+        return s;
+    }
+};
+
+// The coupling table of a path whose k rows are in shared memory, by one warp (lane t: g_t, beta_t of step t; rows beyond
 // L up to the next multiple of eight are zero).
-__device__ __forceinline__ void path_coupling(uint32_t pk, int L, float G, float beta, float *coupling, int lane)
+__device__ __forceinline__ void path_coupling(uint32_t pk, int L, float g_t, float beta, float *coupling, int lane)
 {
     const int g = lane >> 2, l4 = lane & 3;
     const bool two = L > 8;
@@ -214,19 +242,25 @@ __device__ __forceinline__ void path_coupling(uint32_t pk, int L, float G, float
         mma_16816(k[c & 1][0], a, a[0], a[2]);
         if (two) mma_16816(k[c & 1][1], a, a[1], a[3]);
     }
+    const DecayWindows windows(g_t);
 #pragma unroll
     for (int r = 0; r < 2; ++r) {   // t = g + 8 r
+        if (r == 1 && !two) break;
         const int t = g + 8 * r;
-        const float Gt = __shfl_sync(0xffffffffu, G, t), bt = __shfl_sync(0xffffffffu, beta, t);
+        const float bt = __shfl_sync(0xffffffffu, beta, t);
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int u = 8 * i + 2 * l4 + e;
-                const float Gu = __shfl_sync(0xffffffffu, G, u);
-                if ((two || (r == 0 && i == 0)) && u < L)
-                    coupling[u * 16 + t] = t > u && t < L ? bt * expf(Gt - Gu) * (k[0][i][2 * r + e] + k[1][i][2 * r + e]) : 0.f;
+        for (int i = 0; i < 2; ++i) {
+            const int u = 8 * i + 2 * l4;   // ... and u + 1
+            float d0 = 0.f, d1 = 0.f;   // decays behind u, behind u + 1
+            if (i <= r) {               // (otherwise t < u)
+                const float near = windows.sum(t, max(t - u - 1, 0));
+                d0 = expf(near + __shfl_sync(0xffffffffu, g_t, u + 1));
+                d1 = expf(near);
             }
+            if (!two && i == 1) continue;
+            if (u < L) coupling[u * 16 + t] = t > u && t < L ? bt * d0 * (k[0][i][2 * r] + k[1][i][2 * r]) : 0.f;
+            if (u + 1 < L) coupling[(u + 1) * 16 + t] = t > u + 1 && t < L ? bt * d1 * (k[0][i][2 * r + 1] + k[1][i][2 * r + 1]) : 0.f;
+        }
     }
 }
 

@@ -734,6 +734,23 @@ def test_commit_tile_kernel_forms_of_large_calls(tl, slots):
     assert bool((dc.S0[3] == before[3]).all()) and bool((dc.S0[0] == before[0]).all())
 
 
+@pytest.mark.parametrize("at", [0, 3, 9])
+@pytest.mark.parametrize("g_strong", [-3000.0, -30000.0, -np.inf])
+@pytest.mark.parametrize("slots", [2, 10, 17])
+def test_commit_behind_a_strong_decay(tl, slots, g_strong, at):
+    """One strong decay (alpha = 0 at the last) on a path of weak ones, in every form of the tile commit: the steps behind it
+    keep their precision.  A difference of two sums that both contain it would be off by its last place (1.2e-4 at -3000, 2e-3
+    at -30000), or not a number."""
+    trees = [synth.tree_chain(16)] * slots
+    paths = [np.arange(7 if i % 2 else 16, dtype=np.int32) for i in range(slots)]
+    w = synth.random_case(48, trees, 2, 32, 128, 128, synth.BF16, synth.BF16, paths=paths)
+    w.g[:] = synth.f32_to_bf16_bits(np.float32([-0.0101]))[0]
+    w.g[at::16] = synth.f32_to_bf16_bits(np.float32([g_strong]))[0]
+    dc = tl.DeviceCase(w)
+    assert dc.commit() == 0 and dc.device_status() == 0
+    tl.assert_state_close(dc.S0.cpu().numpy().astype(np.float64), tl.oracle_commit(w), what=f"commit behind g = {g_strong}")
+
+
 @pytest.mark.parametrize("slots", [1, 18, 19])
 def test_fused_step_on_both_sides_of_the_two_kernel_rule(tl, slots):
     """4 heads per slot: 72 units run as two kernels, 76 as one (148 SMs).  Every input is overwritten by the kernels right
