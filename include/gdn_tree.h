@@ -12,7 +12,9 @@
  *
  * Conventions common to every entry point
  *   - Pointers marked [device] are CUDA device pointers on the current
- *     device, contiguous, row-major, 16-byte aligned; pointers marked [host]
+ *     device, contiguous, row-major, 16-byte aligned (the padded entry points
+ *     want the state 32-byte aligned; elsewhere a state off a 32-byte boundary
+ *     is taken by the general kernels); pointers marked [host]
  *     are ordinary host pointers.  The caller owns every buffer.  The library
  *     allocates no memory and keeps no state between calls.
  *   - Work is enqueued on `cuda_stream` (a cudaStream_t passed as void*,
@@ -58,7 +60,7 @@ enum gdn_status {
     GDN_ERR_NULL = -1,        /* a required pointer is NULL                                   */
     GDN_ERR_SHAPE = -2,       /* a size is out of range or inconsistent                       */
     GDN_ERR_DTYPE = -3,       /* unknown in_dtype / out_dtype                                 */
-    GDN_ERR_ALIGN = -4,       /* a pointer is not 16-byte aligned                             */
+    GDN_ERR_ALIGN = -4,       /* a pointer is not aligned as required                         */
     GDN_ERR_UNSUPPORTED = -5, /* valid request that this build cannot run                     */
     GDN_ERR_CUDA = -6,        /* a CUDA runtime call failed (launch, copy, attribute)         */
     GDN_ERR_TREE = -7,        /* parent[] / node_offsets[] do not describe a topological forest */

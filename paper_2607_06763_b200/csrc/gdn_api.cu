@@ -11,6 +11,9 @@ using namespace gdn;
 namespace {
 
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+// The kernels for 128 components and bf16 inputs move the state in 32-byte accesses.  Callers may pass any 16-byte aligned
+// state: one off a 32-byte boundary goes to the general kernels, or, where there are none (padded layout), is refused.
+inline bool aligned32(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0; }
 inline bool aligned256(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 255u) == 0; }
 inline size_t dtype_size(int dt) { return dt == GDN_BF16 ? 2 : 4; }
 
@@ -180,14 +183,15 @@ extern "C" int gdn_tree_verify(const gdn_shape_t *shape, const float *S0, const 
     const WorkspaceLayout lay = workspace_layout(s);
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const PlanPtrs plan = plan_ptrs(workspace, lay);
+    const bool tensor_cores = verify_sm100_supported(s) && aligned32(S0);
     // trees of at most 64 nodes: the kernels build the tree metadata themselves
-    if (!verify_sm100_supported(s) && verify_generic_small_supported(s))
+    if (!tensor_cores && verify_generic_small_supported(s))
         return launch_verify_generic_small(s, S0, q, k, v, g, beta, parent, node_offsets, o, status_dev, stream) == cudaSuccess
                    ? GDN_OK : GDN_ERR_CUDA;
-    if (!verify_sm100_single_group(s) &&
+    if (!(tensor_cores && verify_sm100_single_group(s)) &&
         launch_plan(s, parent, node_offsets, nullptr, plan, status_dev, stream) != cudaSuccess)
         return GDN_ERR_CUDA;
-    const cudaError_t e = verify_sm100_supported(s)
+    const cudaError_t e = tensor_cores
                               ? launch_verify_sm100(s, S0, q, k, v, g, beta, parent, node_offsets, o, plan, status_dev, stream)
                               : launch_verify_generic(s, S0, q, k, v, g, beta, node_offsets, o, plan, stream);
     if (e != cudaSuccess) return GDN_ERR_CUDA;
@@ -224,6 +228,7 @@ extern "C" int gdn_tree_verify_padded(const gdn_shape_t *shape, int32_t n_trees,
         !aligned16(o) || (reinterpret_cast<uintptr_t>(parent) & 3u) || (reinterpret_cast<uintptr_t>(n_nodes) & 3u) ||
         (reinterpret_cast<uintptr_t>(status_dev) & 3u))
         return GDN_ERR_ALIGN;
+    if (!aligned32(S0)) return GDN_ERR_ALIGN;
     if (launch_verify_sm100_padded(s, n_trees, raw_gates != 0, S0, q, k, v, g, beta, parent, n_nodes, o, status_dev,
                                    static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
         return GDN_ERR_CUDA;
@@ -255,6 +260,7 @@ extern "C" int gdn_tree_commit_verify_padded(const gdn_shape_t *shape, int32_t n
         (reinterpret_cast<uintptr_t>(parent) & 3u) || (reinterpret_cast<uintptr_t>(n_nodes) & 3u) ||
         (reinterpret_cast<uintptr_t>(status_dev) & 3u))
         return GDN_ERR_ALIGN;
+    if (!aligned32(S)) return GDN_ERR_ALIGN;
     if (launch_commit_verify_sm100_padded(s, n_trees, raw_gates != 0, S, prev_t_pad, k_prev, v_prev, g_prev, beta_prev,
                                           parent_prev, n_nodes_prev, path, path_len, q, k, v, g, beta, parent, n_nodes,
                                           o, status_dev, static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
@@ -332,6 +338,7 @@ extern "C" int gdn_tree_verify_planned(const gdn_shape_t *shape, int32_t n_trees
         return GDN_ERR_ALIGN;
     const WorkspaceLayout lay = workspace_layout(plan_shape(s, n_trees));
     if (plan_bytes < lay.total) return GDN_ERR_WORKSPACE;
+    if (!aligned32(S0)) return GDN_ERR_ALIGN;
     if (launch_verify_sm100_planned(s, n_trees, raw_gates != 0, S0, q, k, v, g, beta,
                                     plan_ptrs(const_cast<void *>(plan), lay), o, status_dev,
                                     static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
@@ -357,6 +364,7 @@ extern "C" int gdn_tree_commit_padded(const gdn_shape_t *shape, int32_t n_trees,
         (reinterpret_cast<uintptr_t>(path) & 3u) || (reinterpret_cast<uintptr_t>(path_len) & 3u) ||
         (reinterpret_cast<uintptr_t>(status_dev) & 3u))
         return GDN_ERR_ALIGN;
+    if (!aligned32(S)) return GDN_ERR_ALIGN;
     if (launch_commit_padded(s, n_trees, raw_gates != 0, S, k, v, g, beta, parent, n_nodes, path, path_len, status_dev,
                              static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
         return GDN_ERR_CUDA;
@@ -414,7 +422,7 @@ extern "C" int gdn_tree_commit_verify(const gdn_shape_t *shape, float *S, const 
     const gdn_shape_t &s = *shape;
     if (s.n_seq == 0) return GDN_OK;
     if (!S || !node_offsets_prev || !path_offsets || !status_dev) return GDN_ERR_NULL;
-    if (!verify_sm100_single_group(s) || s.total_nodes == 0) {
+    if (!verify_sm100_single_group(s) || s.total_nodes == 0 || !aligned32(S)) {
         // general shapes: the two kernels back to back on the stream (the shape's node counts are
         // not used by commit, so the new tree's shape serves for the previous tree as well).  Both
         // halves are checked before the first launch: a refused call must leave the state as it was.
@@ -426,7 +434,7 @@ extern "C" int gdn_tree_commit_verify(const gdn_shape_t *shape, float *S, const 
                                    status_dev);
             if (rc != GDN_OK) return rc;
         }
-        if (s.total_nodes > 0 && verify_sm100_supported(s) && commit_tile128_supported(s)) {
+        if (s.total_nodes > 0 && verify_sm100_supported(s) && commit_tile128_supported(s) && aligned32(S)) {
             // trees of more than 64 nodes on the tensor-core path: the plan of the new trees does not depend on the
             // commit, so it is built by extra CTAs of the commit grid; then the verify kernel in its grouped mode
             const WorkspaceLayout lay = workspace_layout(s);

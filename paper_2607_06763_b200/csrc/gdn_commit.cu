@@ -504,7 +504,7 @@ cudaError_t launch_commit_generic(const gdn_shape_t &s, float *S, const void *k,
     if (grid == 0) return cudaSuccess;
     CommitParams p{s.h_qk, s.h_v, s.d_k, s.d_v, s.max_depth, S, k, v, g, beta,
                    parent, node_offsets, path, path_offsets, status_dev, 0, 0, 0, 0, nullptr, nullptr};
-    if (s.d_k == GDN_TILE_D && s.d_v == GDN_TILE_D && s.in_dtype == GDN_BF16 && s.max_depth <= CF_MD)
+    if (commit_tile128_supported(s) && (reinterpret_cast<uintptr_t>(S) & 31u) == 0)   // 32-byte accesses of the state
         return launch_tile128(p, grid, stream);
     static PerDevice seen[2];
     const auto kernel = s.in_dtype == GDN_BF16 ? commit_generic_kernel<__nv_bfloat16> : commit_generic_kernel<float>;

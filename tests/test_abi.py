@@ -155,6 +155,17 @@ def test_entry_points_reject_bad_arguments_before_touching_cuda(lib):
                                None, None, 0, None) == 0
 
 
+def test_padded_entry_points_refuse_a_state_off_a_32_byte_boundary(lib):
+    """Their kernels read and write the state in 32-byte accesses: 16 mod 32 is refused before any CUDA call."""
+    s = gdn.GdnShape(4, 16, 32, 128, 128, 1, 1, 16, 4 * 64, 64, 0.0883883)
+    a, plan = 1 << 20, _FakeBuf(1 << 24)
+    off = a + 16
+    assert gdn.gdn_tree_verify_padded(s, 2, 0, off, a, a, a, a, a, a, a, a, a) == -4
+    assert gdn.gdn_tree_commit_verify_padded(s, 2, 0, off, 64, *[a] * 18) == -4
+    assert gdn.gdn_tree_verify_planned(s, 2, 0, off, a, a, a, a, a, plan, a, a) == -4
+    assert gdn.gdn_tree_commit_padded(s, 2, 0, off, *[a] * 9) == -4
+
+
 def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     from paper_2607_06763_b200 import binding
     monkeypatch.setattr(binding, "_lib", None)

@@ -794,6 +794,40 @@ def test_fused_step_on_both_sides_of_the_two_kernel_rule(tl, slots):
             tl.assert_close_per_head(o.cpu().numpy().astype(np.float64), o_ref, w.node_offsets, f"fused, {slots} slots, o")
 
 
+@pytest.mark.parametrize("sizes", [(64, 1, 33), (20, 130), (64,) * 19, (300,)])
+def test_state_off_a_32_byte_boundary(tl, sizes):
+    """A state at 16 mod 32 bytes, which the ragged entry points accept: verification, commit and fused call on the general
+    kernels, against the oracle.  The words around the state stay as they are."""
+    import torch
+    import paper_2607_06763_b200 as gdn
+    rng = np.random.default_rng(211)
+    make = lambda seed: synth.random_case(seed, [synth.tree_geo(rng, T) if T > 1 else np.full(1, -1, np.int32) for T in sizes],
+                                          2, 4, 128, 128, synth.BF16, synth.F32)
+    prev, new = make(212), make(213)
+    dp, dn = tl.DeviceCase(prev), tl.DeviceCase(new)
+    buf = torch.full((dp.S0.numel() + 8,), 7.0, device="cuda")
+    S = buf[4:-4].view(dp.S0.shape)
+    assert S.data_ptr() % 32 == 16
+    S.copy_(dp.S0)
+    stream = torch.cuda.current_stream()
+    rc = gdn.gdn_tree_verify(dp.shape, S, dp.q, dp.k, dp.v, dp.g, dp.beta, dp.parent, dp.node_offsets, dp.o, dp.ws,
+                             dp.ws_bytes, dp.status, stream)
+    assert rc == 0 and dp.device_status() == 0 and bool((S == dp.S0).all())
+    tl.assert_close_per_head(dp.o_host(), tl.oracle_verify(prev), prev.node_offsets, "verify")
+    assert dp.commit(S=S, stream=stream) == 0 and dp.device_status() == 0
+    S1 = tl.oracle_commit(prev)
+    tl.assert_state_close(S.cpu().numpy().astype(np.float64), S1, what="commit")
+    S.copy_(dp.S0)
+    rc = gdn.gdn_tree_commit_verify(dn.shape, S, dp.k, dp.v, dp.g, dp.beta, dp.parent, dp.node_offsets, dp.path, dp.path_offsets,
+                                    dn.q, dn.k, dn.v, dn.g, dn.beta, dn.parent, dn.node_offsets, dn.o, dn.ws, dn.ws_bytes,
+                                    dn.status, stream)
+    assert rc == 0 and dn.device_status() == 0
+    tl.assert_state_close(S.cpu().numpy().astype(np.float64), S1, what="fused commit")
+    ref = tl.oracle_verify(dataclass_replace_S0(new, S1))
+    tl.assert_close_per_head(dn.o_host(), ref, new.node_offsets, "fused verify")
+    assert bool((buf[:4] == 7.0).all()) and bool((buf[-4:] == 7.0).all())
+
+
 def test_fused_call_on_large_trees(tl):
     """Trees beyond one CTA tile: the fused entry point runs the commit tile kernel and the grouped verify kernel back
     to back; results as for the small-tree kernel."""
