@@ -22,7 +22,9 @@
  *     synchronise; the *_host entry points synchronise the stream before
  *     returning.
  *   - Return value: GDN_OK or a negative gdn_status decided on the host
- *     before anything is launched (nothing is launched on error).
+ *     before anything is launched (nothing is launched on error, except that
+ *     GDN_ERR_CUDA may also mean that a launch itself failed: what the same
+ *     call had launched in front of it runs).
  *     Data-dependent faults that only the device can see (a bad parent[],
  *     a root path longer than max_depth, a path that is not a root chain)
  *     are reported by writing a negative gdn_status into *status_dev with
@@ -243,8 +245,11 @@ int gdn_tree_commit(const gdn_shape_t *shape, float *S, const void *k, const voi
  *     S[b] <- Eq. 7 replayed over the accepted path of the PREVIOUS tree of b   (as gdn_tree_commit)
  *     o    <- verification of the NEW tree of b against that advanced state     (as gdn_tree_verify)
  * so every state tile is read from memory once and written once per step.  The results are those
- * of gdn_tree_commit followed by gdn_tree_verify (same tolerances; on the tensor-core path it is
- * one kernel, otherwise the two kernels are launched back to back).
+ * of gdn_tree_commit followed by gdn_tree_verify (same tolerances).  Trees of at most 64 nodes on
+ * the tensor-core path run as one kernel when there are more (tree, value head) pairs than half the
+ * SMs; otherwise the commit and the verify kernel are launched one behind the other, the commit
+ * once everything of the verification that can fail short of its launch is done: if that launch
+ * fails all the same (GDN_ERR_CUDA), the state has been advanced.
  *   shape        : describes the NEW tree (total_nodes, max_tree_nodes) and the common head shapes
  *   S            : [device] in: committed state before the previous step, out: state after it
  *   k_prev, v_prev, g_prev, beta_prev, parent_prev (may be NULL), node_offsets_prev :

@@ -169,6 +169,30 @@ extern "C" int gdn_tree_validate_host(const gdn_shape_t *shape, const int32_t *p
     return worst;
 }
 
+namespace {
+
+// gdn_tree_verify behind its checks; commit (optional): launched right in front of the verify kernel.
+int verify_checked(const gdn_shape_t &s, const float *S0, const void *q, const void *k, const void *v, const void *g,
+                   const void *beta, const int32_t *parent, const int32_t *node_offsets, void *o, void *workspace,
+                   int32_t *status_dev, cudaStream_t stream, LaunchInFront commit)
+{
+    const PlanPtrs plan = plan_ptrs(workspace, workspace_layout(s));
+    const bool tensor_cores = verify_sm100_supported(s) && aligned32(S0);
+    // trees of at most 64 nodes: the kernels build the tree metadata themselves
+    if (!tensor_cores && verify_generic_small_supported(s))
+        return launch_verify_generic_small(s, S0, q, k, v, g, beta, parent, node_offsets, o, status_dev, stream, commit) == cudaSuccess
+                   ? GDN_OK : GDN_ERR_CUDA;
+    if (!(tensor_cores && verify_sm100_single_group(s)) &&
+        launch_plan(s, parent, node_offsets, nullptr, plan, status_dev, stream) != cudaSuccess)
+        return GDN_ERR_CUDA;
+    const cudaError_t e = tensor_cores
+                              ? launch_verify_sm100(s, S0, q, k, v, g, beta, parent, node_offsets, o, plan, status_dev, stream, commit)
+                              : launch_verify_generic(s, S0, q, k, v, g, beta, node_offsets, o, plan, stream, commit);
+    return e == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
+}
+
+}  // namespace
+
 extern "C" int gdn_tree_verify(const gdn_shape_t *shape, const float *S0, const void *q, const void *k,
                                const void *v, const void *g, const void *beta, const int32_t *parent,
                                const int32_t *node_offsets, void *o, void *workspace,
@@ -180,22 +204,8 @@ extern "C" int gdn_tree_verify(const gdn_shape_t *shape, const float *S0, const 
     if (s.n_seq == 0 || s.total_nodes == 0) return GDN_OK;
     rc = check_verify_args(s, S0, q, k, v, g, beta, parent, node_offsets, o, workspace, workspace_bytes, status_dev);
     if (rc != GDN_OK) return rc;
-    const WorkspaceLayout lay = workspace_layout(s);
-    cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    const PlanPtrs plan = plan_ptrs(workspace, lay);
-    const bool tensor_cores = verify_sm100_supported(s) && aligned32(S0);
-    // trees of at most 64 nodes: the kernels build the tree metadata themselves
-    if (!tensor_cores && verify_generic_small_supported(s))
-        return launch_verify_generic_small(s, S0, q, k, v, g, beta, parent, node_offsets, o, status_dev, stream) == cudaSuccess
-                   ? GDN_OK : GDN_ERR_CUDA;
-    if (!(tensor_cores && verify_sm100_single_group(s)) &&
-        launch_plan(s, parent, node_offsets, nullptr, plan, status_dev, stream) != cudaSuccess)
-        return GDN_ERR_CUDA;
-    const cudaError_t e = tensor_cores
-                              ? launch_verify_sm100(s, S0, q, k, v, g, beta, parent, node_offsets, o, plan, status_dev, stream)
-                              : launch_verify_generic(s, S0, q, k, v, g, beta, node_offsets, o, plan, stream);
-    if (e != cudaSuccess) return GDN_ERR_CUDA;
-    return GDN_OK;
+    return verify_checked(s, S0, q, k, v, g, beta, parent, node_offsets, o, workspace, status_dev,
+                          static_cast<cudaStream_t>(cuda_stream), {});
 }
 
 namespace {
@@ -434,25 +444,26 @@ extern "C" int gdn_tree_commit_verify(const gdn_shape_t *shape, float *S, const 
                                    status_dev);
             if (rc != GDN_OK) return rc;
         }
-        if (s.total_nodes > 0 && verify_sm100_supported(s) && commit_tile128_supported(s) && aligned32(S)) {
+        if (s.total_nodes == 0)
+            return gdn_tree_commit(shape, S, k_prev, v_prev, g_prev, beta_prev, parent_prev, node_offsets_prev, path,
+                                   path_offsets, status_dev, cuda_stream);
+        cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+        if (verify_sm100_supported(s) && commit_tile128_supported(s) && aligned32(S)) {
             // trees of more than 64 nodes on the tensor-core path: the plan of the new trees does not depend on the
             // commit, so it is built by extra CTAs of the commit grid; then the verify kernel in its grouped mode
-            const WorkspaceLayout lay = workspace_layout(s);
-            const PlanPtrs plan = plan_ptrs(workspace, lay);
-            cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-            if (launch_commit_plan(s, S, k_prev, v_prev, g_prev, beta_prev, parent_prev, node_offsets_prev, path,
-                                   path_offsets, parent, node_offsets, plan, status_dev, stream) != cudaSuccess)
-                return GDN_ERR_CUDA;
-            if (launch_verify_sm100(s, S, q, k, v, g, beta, parent, node_offsets, o, plan, status_dev, stream) !=
-                cudaSuccess)
-                return GDN_ERR_CUDA;
-            return GDN_OK;
+            const PlanPtrs plan = plan_ptrs(workspace, workspace_layout(s));
+            const auto commit = [&] {
+                return launch_commit_plan(s, S, k_prev, v_prev, g_prev, beta_prev, parent_prev, node_offsets_prev, path,
+                                          path_offsets, parent, node_offsets, plan, status_dev, stream);
+            };
+            return launch_verify_sm100(s, S, q, k, v, g, beta, parent, node_offsets, o, plan, status_dev, stream,
+                                       in_front(commit)) == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
         }
-        rc = gdn_tree_commit(shape, S, k_prev, v_prev, g_prev, beta_prev, parent_prev, node_offsets_prev, path,
-                             path_offsets, status_dev, cuda_stream);
-        if (rc != GDN_OK) return rc;
-        return gdn_tree_verify(shape, S, q, k, v, g, beta, parent, node_offsets, o, workspace, workspace_bytes,
-                               status_dev, cuda_stream);
+        const auto commit = [&] {
+            return launch_commit_generic(s, S, k_prev, v_prev, g_prev, beta_prev, parent_prev, node_offsets_prev, path,
+                                         path_offsets, status_dev, stream);
+        };
+        return verify_checked(s, S, q, k, v, g, beta, parent, node_offsets, o, workspace, status_dev, stream, in_front(commit));
     }
     if (!k_prev || !v_prev || !g_prev || !beta_prev || !path) return GDN_ERR_NULL;
     if (!q || !k || !v || !g || !beta || !parent || !node_offsets || !o) return GDN_ERR_NULL;

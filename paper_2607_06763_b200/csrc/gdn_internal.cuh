@@ -125,6 +125,20 @@ inline cudaError_t device_sms(PerDevice &seen, const void *kernel, size_t smem, 
     return e;
 }
 
+// A launch that goes to the stream right in front of another kernel's, once everything of that kernel that can fail short of
+// its launch (tensor maps, attributes) has been done: the commit, which writes the state in place, in front of the
+// verification of a fused call.
+struct LaunchInFront {
+    cudaError_t (*launch)(const void *);
+    const void *args;
+    explicit operator bool() const { return launch != nullptr; }
+    cudaError_t operator()() const { return launch(args); }
+};
+template <typename F> LaunchInFront in_front(const F &f)   // (f outlives the call that is given the result)
+{
+    return {[](const void *x) { return (*static_cast<const F *>(x))(); }, &f};
+}
+
 // Host launchers (each returns the cudaError_t of its launch).
 // node_offsets == nullptr: padded layout, s.n_seq trees of s.max_tree_nodes rows each (parent [n_seq][rows], the node
 // counts in n_nodes [n_seq]); otherwise ragged packing and n_nodes is not read.
@@ -134,15 +148,17 @@ cudaError_t launch_plan(const gdn_shape_t &s, const int32_t *parent, const int32
 cudaError_t launch_verify_generic(const gdn_shape_t &s, const float *S0, const void *q, const void *k,
                                   const void *v, const void *g, const void *beta,
                                   const int32_t *node_offsets, void *o, const PlanPtrs &plan,
-                                  cudaStream_t stream);
+                                  cudaStream_t stream, LaunchInFront commit);
 
 // The same for trees of at most 64 nodes, which need no plan: the metadata is derived from parent[] on chip.
 bool verify_generic_small_supported(const gdn_shape_t &s);
 cudaError_t launch_verify_generic_small(const gdn_shape_t &s, const float *S0, const void *q, const void *k,
                                         const void *v, const void *g, const void *beta, const int32_t *parent,
-                                        const int32_t *node_offsets, void *o, int32_t *status_dev, cudaStream_t stream);
+                                        const int32_t *node_offsets, void *o, int32_t *status_dev, cudaStream_t stream,
+                                        LaunchInFront commit);
 
-// Tensor-core fast path (d_k = d_v = 128, bf16 inputs, trees <= 64 nodes, root paths <= 16 nodes).
+// Tensor-core path (d_k = d_v = 128, bf16 inputs, trees of at most GDN_GROUPED_MAX_NODES nodes, root paths of at most 16).
+// commit (optional): launched right in front, writes the state and, for trees of more than 64 nodes, the plan.
 bool verify_sm100_supported(const gdn_shape_t &s);
 bool verify_sm100_single_group(const gdn_shape_t &s);   // every tree fits one CTA (<= 64 nodes): fusable with commit
 // Trees of at most 64 nodes: the kernel builds the tree metadata itself from parent[] (`plan` is not read);
@@ -150,11 +166,10 @@ bool verify_sm100_single_group(const gdn_shape_t &s);   // every tree fits one C
 cudaError_t launch_verify_sm100(const gdn_shape_t &s, const float *S0, const void *q, const void *k,
                                 const void *v, const void *g, const void *beta, const int32_t *parent,
                                 const int32_t *node_offsets, void *o, const PlanPtrs &plan,
-                                int32_t *status_dev, cudaStream_t stream, bool behind_commit = false);
+                                int32_t *status_dev, cudaStream_t stream, LaunchInFront commit = {});
 
-// Same kernel with the commit of the previous step's accepted paths fused in front of the verify:
-// the state tile is read once, advanced along the path (Eq. 7), written back, and the new tree is
-// verified against the advanced state.
+// The commit of the previous step's accepted paths, then the verification of the new trees (at most 64 nodes) against the
+// advanced state: one kernel that reads and writes the state once or, for few units, the two kernels side by side.
 cudaError_t launch_commit_verify_sm100(const gdn_shape_t &s, float *S, const void *k_prev, const void *v_prev,
                                        const void *g_prev, const void *beta_prev, const int32_t *parent_prev,
                                        const int32_t *node_offsets_prev, const int32_t *path,
@@ -163,14 +178,14 @@ cudaError_t launch_commit_verify_sm100(const gdn_shape_t &s, float *S, const voi
                                        const int32_t *node_offsets, void *o, int32_t *status_dev,
                                        cudaStream_t stream);
 
-// Padded layout of Section 3.4.2 on the persistent tensor-core kernel (s.max_tree_nodes = rows per slot, s.total_nodes =
+// Padded layout of Section 3.4.2 on the tensor-core kernels (s.max_tree_nodes = rows per slot, s.total_nodes =
 // n_seq * rows per slot, trees of at most 64 nodes): slot b carries tree b % n_trees; parent [n_trees][t_pad], n_nodes
 // [n_trees]; raw_gates: g / beta are raw gate inputs.  The fused form takes the previous step in the same layout
 // (prev_t_pad rows per slot) and one accepted path per tree: path [n_trees][max_depth], path_len [n_trees].
 cudaError_t launch_verify_sm100_padded(const gdn_shape_t &s, int n_trees, bool raw_gates, const float *S0,
                                        const void *q, const void *k, const void *v, const void *g, const void *beta,
                                        const int32_t *parent, const int32_t *n_nodes, void *o, int32_t *status_dev,
-                                       cudaStream_t stream, bool behind_commit = false);
+                                       cudaStream_t stream, LaunchInFront commit = {});
 cudaError_t launch_commit_verify_sm100_padded(const gdn_shape_t &s, int n_trees, bool raw_gates, float *S,
                                               int prev_t_pad, const void *k_prev, const void *v_prev,
                                               const void *g_prev, const void *beta_prev, const int32_t *parent_prev,

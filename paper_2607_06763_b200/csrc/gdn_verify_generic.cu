@@ -535,12 +535,13 @@ __global__ void __launch_bounds__(VS_THREADS, 2) verify_generic_small_kernel(con
 }
 
 template <typename TIn, typename TOut>
-cudaError_t launch_small_typed(VerifySmallParams p, cudaStream_t stream)
+cudaError_t launch_small_typed(VerifySmallParams p, cudaStream_t stream, LaunchInFront commit)
 {
     static PerDevice seen;
     int sms = 0;
-    const cudaError_t e = device_sms(seen, reinterpret_cast<const void *>(verify_generic_small_kernel<TIn, TOut>),
-                                     sizeof(VerifySmallSmem), &sms);
+    cudaError_t e = device_sms(seen, reinterpret_cast<const void *>(verify_generic_small_kernel<TIn, TOut>),
+                               sizeof(VerifySmallSmem), &sms);
+    if (e == cudaSuccess && commit) e = commit();
     if (e != cudaSuccess) return e;
     // Blocks per CTA: as few as let all CTAs be resident at once, so that small calls spread over the SMs; a CTA reads rows
     // and state once for all of its blocks.  No more than three: a fourth leaves the largest trees as the tail of the call,
@@ -567,13 +568,14 @@ cudaError_t launch_small_typed(VerifySmallParams p, cudaStream_t stream)
 }
 
 template <typename TIn, typename TOut>
-cudaError_t launch_typed(const gdn_shape_t &s, const VerifyGenericParams &p, cudaStream_t stream)
+cudaError_t launch_typed(const gdn_shape_t &s, const VerifyGenericParams &p, cudaStream_t stream, LaunchInFront commit)
 {
     const int grid = s.n_seq * s.h_v;
     if (grid == 0 || s.total_nodes == 0) return cudaSuccess;
     const size_t smem = sizeof(float) * (2 * VG_CHUNK * VG_DK + 2 * VG_CHUNK * (size_t)s.max_depth + 2 * VG_CHUNK);
     cudaError_t e = cudaFuncSetAttribute(verify_generic_kernel<TIn, TOut>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess && commit) e = commit();
     if (e != cudaSuccess) return e;
     verify_generic_kernel<TIn, TOut><<<grid, VG_THREADS, smem, stream>>>(p);
     return cudaGetLastError();
@@ -590,31 +592,32 @@ bool verify_generic_small_supported(const gdn_shape_t &s)
 
 cudaError_t launch_verify_generic_small(const gdn_shape_t &s, const float *S0, const void *q, const void *k,
                                         const void *v, const void *g, const void *beta, const int32_t *parent,
-                                        const int32_t *node_offsets, void *o, int32_t *status_dev, cudaStream_t stream)
+                                        const int32_t *node_offsets, void *o, int32_t *status_dev, cudaStream_t stream,
+                                        LaunchInFront commit)
 {
     if (s.n_seq == 0 || s.total_nodes == 0) return cudaSuccess;
     const VerifySmallParams p{s.h_qk, s.h_v, s.d_k, s.d_v, s.max_depth, s.max_tree_nodes, s.total_nodes, s.n_seq,
                               0, 0, s.scale, S0, q, k, v, g, beta, parent,
                               node_offsets, o, status_dev};
     const bool in_bf = s.in_dtype == GDN_BF16, out_bf = s.out_dtype == GDN_BF16;
-    if (in_bf && out_bf) return launch_small_typed<__nv_bfloat16, __nv_bfloat16>(p, stream);
-    if (in_bf) return launch_small_typed<__nv_bfloat16, float>(p, stream);
-    if (out_bf) return launch_small_typed<float, __nv_bfloat16>(p, stream);
-    return launch_small_typed<float, float>(p, stream);
+    if (in_bf && out_bf) return launch_small_typed<__nv_bfloat16, __nv_bfloat16>(p, stream, commit);
+    if (in_bf) return launch_small_typed<__nv_bfloat16, float>(p, stream, commit);
+    if (out_bf) return launch_small_typed<float, __nv_bfloat16>(p, stream, commit);
+    return launch_small_typed<float, float>(p, stream, commit);
 }
 
 cudaError_t launch_verify_generic(const gdn_shape_t &s, const float *S0, const void *q, const void *k,
                                   const void *v, const void *g, const void *beta,
                                   const int32_t *node_offsets, void *o, const PlanPtrs &plan,
-                                  cudaStream_t stream)
+                                  cudaStream_t stream, LaunchInFront commit)
 {
     VerifyGenericParams p{s.h_qk, s.h_v, s.d_k, s.d_v, s.max_depth, s.scale, S0, q, k, v, g, beta,
                           node_offsets, o, plan.tree_ok, plan.depth, plan.anc, plan.utilde};
     const bool in_bf = s.in_dtype == GDN_BF16, out_bf = s.out_dtype == GDN_BF16;
-    if (in_bf && out_bf) return launch_typed<__nv_bfloat16, __nv_bfloat16>(s, p, stream);
-    if (in_bf) return launch_typed<__nv_bfloat16, float>(s, p, stream);
-    if (out_bf) return launch_typed<float, __nv_bfloat16>(s, p, stream);
-    return launch_typed<float, float>(s, p, stream);
+    if (in_bf && out_bf) return launch_typed<__nv_bfloat16, __nv_bfloat16>(s, p, stream, commit);
+    if (in_bf) return launch_typed<__nv_bfloat16, float>(s, p, stream, commit);
+    if (out_bf) return launch_typed<float, __nv_bfloat16>(s, p, stream, commit);
+    return launch_typed<float, float>(s, p, stream, commit);
 }
 
 }  // namespace gdn

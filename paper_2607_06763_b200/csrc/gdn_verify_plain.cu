@@ -869,11 +869,12 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
     if (warp == 0) tmem_dealloc(tmem, TM_COLS);
 }
 
-template <typename TOut, bool PADDED, bool GROUPED> cudaError_t launch_kernel(const VerifyPlainParams &p, cudaStream_t stream)
+template <typename TOut, bool PADDED, bool GROUPED> cudaError_t launch_kernel(const VerifyPlainParams &p, LaunchInFront commit, cudaStream_t stream)
 {
     static PerDevice seen;
     int sms = 0;
-    const cudaError_t e = device_sms(seen, reinterpret_cast<const void *>(verify_plain_kernel<TOut, PADDED, GROUPED>), SP_ALLOC, &sms);
+    cudaError_t e = device_sms(seen, reinterpret_cast<const void *>(verify_plain_kernel<TOut, PADDED, GROUPED>), SP_ALLOC, &sms);
+    if (e == cudaSuccess && commit) e = commit();
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(p.n_units < 2 * sms ? p.n_units : 2 * sms));   // persistent CTAs, two per SM
@@ -888,8 +889,9 @@ template <typename TOut, bool PADDED, bool GROUPED> cudaError_t launch_kernel(co
     return cudaLaunchKernelEx(&cfg, verify_plain_kernel<TOut, PADDED, GROUPED>, p);
 }
 
-template <bool GROUPED> cudaError_t launch_plain(const gdn_shape_t &s, VerifyPlainParams &p, cudaStream_t stream)
+template <bool GROUPED> cudaError_t launch_plain(const gdn_shape_t &s, VerifyPlainParams &p, LaunchInFront commit, cudaStream_t stream)
 {
+    p.state_late = !GROUPED && commit ? 1 : 0;   // (grouped: the kernel in front writes the plan as well)
     if constexpr (GROUPED) {
         // trees of more than 64 nodes: a unit is one ancestor-closed group of a (tree, head), taken from the plan's
         // unit list (its length is read on the device; this bound only sizes the grid); rows are gathered
@@ -903,8 +905,8 @@ template <bool GROUPED> cudaError_t launch_plain(const gdn_shape_t &s, VerifyPla
     }
     // the padded layout and the on-chip gate activations share an instantiation
     if (s.out_dtype == GDN_BF16)
-        return p.t_pad != 0 ? launch_kernel<__nv_bfloat16, true, GROUPED>(p, stream) : launch_kernel<__nv_bfloat16, false, GROUPED>(p, stream);
-    return p.t_pad != 0 ? launch_kernel<float, true, GROUPED>(p, stream) : launch_kernel<float, false, GROUPED>(p, stream);
+        return p.t_pad != 0 ? launch_kernel<__nv_bfloat16, true, GROUPED>(p, commit, stream) : launch_kernel<__nv_bfloat16, false, GROUPED>(p, commit, stream);
+    return p.t_pad != 0 ? launch_kernel<float, true, GROUPED>(p, commit, stream) : launch_kernel<float, false, GROUPED>(p, commit, stream);
 }
 
 VerifyPlainParams make_params(const gdn_shape_t &s, const float *S0, const void *q, const void *k, const void *v,
@@ -938,14 +940,13 @@ VerifyPlainParams make_params(const gdn_shape_t &s, const float *S0, const void 
 cudaError_t launch_verify_sm100_padded(const gdn_shape_t &s, int n_trees, bool raw_gates, const float *S0,
                                        const void *q, const void *k, const void *v, const void *g, const void *beta,
                                        const int32_t *parent, const int32_t *n_nodes, void *o, int32_t *status_dev,
-                                       cudaStream_t stream, bool behind_commit)
+                                       cudaStream_t stream, LaunchInFront commit)
 {
     if (s.n_seq == 0 || s.total_nodes == 0) return cudaSuccess;
     VerifyPlainParams p = make_params(s, S0, q, k, v, g, beta, nullptr, o, PlanPtrs{}, status_dev);
-    p.state_late = behind_commit ? 1 : 0;
     p.parent = parent;
     p.t_pad = s.max_tree_nodes; p.n_trees = n_trees; p.n_nodes = n_nodes; p.raw_gates = raw_gates ? 1 : 0;
-    return launch_plain<false>(s, p, stream);
+    return launch_plain<false>(s, p, commit, stream);
 }
 
 cudaError_t launch_verify_sm100_planned(const gdn_shape_t &s, int n_trees, bool raw_gates, const float *S0,
@@ -960,7 +961,7 @@ cudaError_t launch_verify_sm100_planned(const gdn_shape_t &s, int n_trees, bool 
     ps.total_nodes = n_trees * s.max_tree_nodes;
     p.unit_capacity = (int)unit_list_capacity(ps);
     p.plan_magic = plan_magic(n_trees, s.max_tree_nodes, s.max_depth);
-    return launch_plain<true>(s, p, stream);
+    return launch_plain<true>(s, p, {}, stream);
 }
 
 bool verify_sm100_supported(const gdn_shape_t &s)
@@ -974,14 +975,13 @@ bool verify_sm100_single_group(const gdn_shape_t &s) { return verify_sm100_suppo
 cudaError_t launch_verify_sm100(const gdn_shape_t &s, const float *S0, const void *q, const void *k,
                                 const void *v, const void *g, const void *beta, const int32_t *parent,
                                 const int32_t *node_offsets, void *o, const PlanPtrs &plan,
-                                int32_t *status_dev, cudaStream_t stream, bool behind_commit)
+                                int32_t *status_dev, cudaStream_t stream, LaunchInFront commit)
 {
     if (s.n_seq == 0 || s.total_nodes == 0) return cudaSuccess;
     VerifyPlainParams p = make_params(s, S0, q, k, v, g, beta, node_offsets, o, plan, status_dev);
     p.parent = parent;
-    p.state_late = behind_commit ? 1 : 0;
-    if (!verify_sm100_single_group(s)) return launch_plain<true>(s, p, stream);
-    return launch_plain<false>(s, p, stream);
+    if (!verify_sm100_single_group(s)) return launch_plain<true>(s, p, commit, stream);
+    return launch_plain<false>(s, p, commit, stream);
 }
 
 }  // namespace gdn

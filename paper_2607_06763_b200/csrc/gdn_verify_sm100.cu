@@ -1020,10 +1020,12 @@ cudaError_t launch_commit_verify_sm100_padded(const gdn_shape_t &s, int n_trees,
     if (as_two_kernels(s)) {
         gdn_shape_t ps = s;   // the commit reads the slots of the previous step
         ps.max_tree_nodes = prev_t_pad;
-        const cudaError_t e = launch_commit_padded(ps, n_trees, raw_gates, S, k_prev, v_prev, g_prev, beta_prev, parent_prev,
-                                                   n_nodes_prev, path, path_len, status_dev, stream);
-        if (e != cudaSuccess) return e;
-        return launch_verify_sm100_padded(s, n_trees, raw_gates, S, q, k, v, g, beta, parent, n_nodes, o, status_dev, stream, true);
+        const auto commit = [&] {
+            return launch_commit_padded(ps, n_trees, raw_gates, S, k_prev, v_prev, g_prev, beta_prev, parent_prev, n_nodes_prev,
+                                        path, path_len, status_dev, stream);
+        };
+        return launch_verify_sm100_padded(s, n_trees, raw_gates, S, q, k, v, g, beta, parent, n_nodes, o, status_dev, stream,
+                                          in_front(commit));
     }
     VerifyFastParams p = make_params(s, S, q, k, v, g, beta, nullptr, o, status_dev);
     p.parent = parent;
@@ -1047,10 +1049,11 @@ cudaError_t launch_commit_verify_sm100(const gdn_shape_t &s, float *S, const voi
 {
     if (s.n_seq == 0 || s.total_nodes == 0) return cudaSuccess;
     if (as_two_kernels(s)) {
-        const cudaError_t e = launch_commit_generic(s, S, k_prev, v_prev, g_prev, beta_prev, parent_prev, node_offsets_prev, path,
-                                                    path_offsets, status_dev, stream);
-        if (e != cudaSuccess) return e;
-        return launch_verify_sm100(s, S, q, k, v, g, beta, parent, node_offsets, o, PlanPtrs{}, status_dev, stream, true);
+        const auto commit = [&] {
+            return launch_commit_generic(s, S, k_prev, v_prev, g_prev, beta_prev, parent_prev, node_offsets_prev, path,
+                                         path_offsets, status_dev, stream);
+        };
+        return launch_verify_sm100(s, S, q, k, v, g, beta, parent, node_offsets, o, PlanPtrs{}, status_dev, stream, in_front(commit));
     }
     VerifyFastParams p = make_params(s, S, q, k, v, g, beta, node_offsets, o, status_dev);
     p.parent = parent;

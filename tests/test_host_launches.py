@@ -1,0 +1,99 @@
+"""What the entry points launch, and in which order, without a GPU: the library's objects linked with ``fake_cudart.c`` in
+place of the CUDA runtime.  No kernel runs."""
+import ctypes
+import os
+import re
+import shutil
+import subprocess
+
+import pytest
+
+import paper_2607_06763_b200 as gdn
+from paper_2607_06763_b200 import binding, build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+A = 1 << 20   # an address that is aligned for everything; nothing is read there
+
+
+@pytest.fixture(scope="module")
+def fake_path(tmp_path_factory):
+    d = str(tmp_path_factory.mktemp("fake"))
+    build.build_library()   # (the argument marshaller)
+    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+    flags = ["-gencode", "arch=compute_100a,code=compute_100a", "-O1", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler",
+             "-fno-gnu-unique", "-I", os.path.join(build._ROOT, "include"), "-I", build.CSRC]
+    objects = [os.path.join(d, os.path.basename(s)[:-3] + ".o") for s in build.sources()]
+    jobs = [subprocess.Popen([nvcc] + flags + ["-c", "-o", o, s]) for s, o in zip(build.sources(), objects)]
+    assert [j.wait() for j in jobs] == [0] * len(jobs)
+    fake = os.path.join(d, "fake.o")
+    subprocess.check_call(["gcc", "-O1", "-fPIC", "-c", "-o", fake, os.path.join(HERE, "fake_cudart.c")])
+    path = os.path.join(d, "libgdn_fake.so")
+    subprocess.check_call(["g++", "-shared", "-Wl,-Bsymbolic", "-Wl,-z,defs", "-o", path] + objects + [fake])
+    return path
+
+
+class Fake:
+    """A copy of the library of its own: everything a process keeps is as at its start."""
+    n = 0
+
+    def __init__(self, path):
+        Fake.n += 1
+        copy = f"{path}.{Fake.n}"
+        shutil.copy(path, copy)
+        self.lib = ctypes.CDLL(copy)
+        self.lib.fake_log.restype = ctypes.c_char_p
+        self.reset()
+
+    def reset(self, fail_call=-1):
+        self.lib.fake_reset(fail_call)
+
+    def call(self, name, *args):
+        return binding._call(ctypes.cast(getattr(self.lib, name), ctypes.c_void_p).value, *args)
+
+    def launches(self):
+        return re.findall(r"\d((?:commit|verify|plan)_[a-z0-9_]*?kernel)(?=[EI])", self.lib.fake_log().decode())   # (mangled names)
+
+
+def _shape(n_seq, T, in_dtype=1, d=128, h_v=32):
+    return gdn.GdnShape(n_seq, h_v // 2, h_v, d, d, in_dtype, 1, 16, n_seq * T, T, 0.0883883)
+
+
+def _fused(fake, s, S=A):
+    ws = fake.lib.gdn_tree_workspace_bytes(ctypes.byref(s))
+    return fake.call("gdn_tree_commit_verify", s, S, *[A] * 15, A, A, ws, A, 0)
+
+
+def _fused_padded(fake, s, S=A):
+    return fake.call("gdn_tree_commit_verify_padded", s, 1, 0, S, s.max_tree_nodes, *[A] * 17, A, 0)
+
+
+FUSED = [
+    (_fused, _shape(1, 64), A, ["commit_tile128_kernel", "verify_plain_kernel"]),
+    (_fused_padded, _shape(1, 64), A, ["commit_tile128_kernel", "verify_plain_kernel"]),
+    (_fused, _shape(48, 64), A, ["commit_verify_kernel"]),
+    (_fused_padded, _shape(48, 64), A, ["commit_verify_kernel"]),
+    (_fused, _shape(4, 256), A, ["commit_plan_kernel", "verify_plain_kernel"]),
+    (_fused, _shape(4, 64, in_dtype=0), A, ["commit_generic_kernel", "verify_generic_small_kernel"]),
+    (_fused, _shape(4, 100, d=64), A, ["plan_kernel", "commit_generic_kernel", "verify_generic_kernel"]),
+    # a state off a 32-byte boundary
+    (_fused, _shape(1, 64), A + 16, ["commit_generic_kernel", "verify_generic_small_kernel"]),
+    (_fused, _shape(48, 256), A + 16, ["plan_kernel", "commit_generic_kernel", "verify_generic_kernel"]),
+]
+
+
+@pytest.mark.parametrize("call,shape,S,kernels", FUSED, ids=range(len(FUSED)))
+def test_fused_call_commits_only_once_the_verification_is_prepared(fake_path, call, shape, S, kernels):
+    """The commit advances the state in place: where a CUDA call of the host path fails, short of a launch, the call must not
+    have touched the state (or have gone through by another route: queries that only choose between routes)."""
+    fake = Fake(fake_path)
+    assert call(fake, shape, S) == 0 and fake.launches() == kernels
+    n = fake.lib.fake_calls()
+    assert n > 0
+    for k in range(n):
+        fresh = Fake(fake_path)
+        fresh.reset(k)
+        rc = call(fresh, shape, S)
+        if rc == 0:
+            assert fresh.launches() in (kernels, ["commit_verify_kernel"])
+        else:
+            assert rc == -6 and not any("commit" in x for x in fresh.launches()), f"call {k} of {n} failed behind the commit"
