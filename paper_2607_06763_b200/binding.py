@@ -154,7 +154,8 @@ def _call(address, *args) -> int:
     """Replaced by the C marshaller (``csrc/gdn_call.c``) on the first call; loading it here keeps the import of the
     package possible before the build."""
     global _call
-    from ._gdn_call import call
+    from ._gdn_call import call, set_shape_type
+    set_shape_type(GdnShape)
     _call = call
     return call(address, *args)
 

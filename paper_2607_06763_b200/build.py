@@ -1,5 +1,5 @@
-"""Builds ``libgdn_tree.so`` (``csrc/*.cu``, nvcc for sm_100a) and ``_gdn_call.so`` (``csrc/gdn_call.c``, the binding's argument
-marshalling) in-tree; no GPU needed to compile."""
+"""Builds ``libgdn_tree.so`` (``csrc/*.cu``, nvcc for sm_100a) and the extension module ``_gdn_call`` (``csrc/gdn_call.c``, the
+binding's argument marshalling) in-tree; no GPU needed to compile."""
 from __future__ import annotations
 
 import glob
@@ -13,7 +13,7 @@ _ROOT = os.path.dirname(_HERE)
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libgdn_tree.so")
 CALL_SRC = os.path.join(CSRC, "gdn_call.c")
-CALL_LIB = os.path.join(_HERE, "_gdn_call.so")
+CALL_LIB = os.path.join(_HERE, "_gdn_call" + sysconfig.get_config_var("EXT_SUFFIX"))   # one for each Python's ABI
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
     "-Xcompiler", "-fPIC", "--shared", "-I", os.path.join(_ROOT, "include"), "-I", CSRC,

@@ -1,42 +1,62 @@
-/* Argument marshalling of binding.py in C: call(address, args...) converts every argument to the 64-bit value that the C
- * ABI of gdn_tree.h passes for it -- None and numbers as they are, torch tensors by data_ptr(), the shape struct and numpy
- * arrays by the address of their buffer -- and calls the function.  All parameters of the ABI are pointers or integers,
- * which the calling convention treats alike.  The arguments of gdn_tree_verify take 1.2 us this way, 4.2 us through
+/* Argument marshalling of binding.py in C: call(address, shape, args...) converts every argument to the 64-bit value that the
+ * C ABI of gdn_tree.h passes for it -- None and integers as they are, the shape struct by its address, torch tensors by
+ * data_ptr(), numpy arrays by ctypes.data, nothing else -- and calls the function.  All parameters of the ABI are pointers or
+ * integers, which the calling convention treats alike.  The arguments of gdn_tree_verify take 1.2 us this way, 4.2 us through
  * ctypes; a verification of one layer, which the host bounds, 7.8 us against 10.7 us. */
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <stdint.h>
 
 enum { MAX_ARGS = 24 };
-static PyObject *s_data_ptr;
+static PyObject *s_data_ptr, *s_ctypes, *s_data;
+static PyObject *shape_type;   /* GdnShape, a ctypes.Structure */
+
+static int value_of(PyObject *x, uint64_t *out)
+{
+    *out = PyLong_AsUnsignedLongLongMask(x);
+    return *out == (uint64_t)-1 && PyErr_Occurred() ? -1 : 0;
+}
+
+static int shape_of(PyObject *x, uint64_t *out)
+{
+    Py_buffer view;
+    const int is_shape = shape_type ? PyObject_IsInstance(x, shape_type) : 0;
+    if (is_shape < 0) return -1;
+    if (!is_shape) {
+        PyErr_Format(PyExc_TypeError, "the shape is a GdnShape, not %R", (PyObject *)Py_TYPE(x));
+        return -1;
+    }
+    if (PyObject_GetBuffer(x, &view, PyBUF_STRIDED_RO) != 0) return -1;
+    *out = (uint64_t)(uintptr_t)view.buf;
+    PyBuffer_Release(&view);   /* (the caller holds the object for the time of the call) */
+    return 0;
+}
 
 static int address_of(PyObject *x, uint64_t *out)
 {
-    PyObject *v = NULL;
+    PyObject *v;
+    int rc;
     if (x == Py_None) {
         *out = 0;
         return 0;
     }
-    if (PyLong_Check(x)) {
-        *out = PyLong_AsUnsignedLongLongMask(x);
-        return *out == (uint64_t)-1 && PyErr_Occurred() ? -1 : 0;
-    }
-    if (PyObject_CheckBuffer(x)) {
-        Py_buffer view;
-        if (PyObject_GetBuffer(x, &view, PyBUF_STRIDED_RO) != 0) return -1;
-        *out = (uint64_t)(uintptr_t)view.buf;
-        PyBuffer_Release(&view);   /* (the caller holds the object for the time of the call) */
-        return 0;
-    }
+    if (PyLong_Check(x)) return value_of(x, out);
     v = PyObject_CallMethodNoArgs(x, s_data_ptr);
-    if (!v) {
-        if (PyErr_ExceptionMatches(PyExc_AttributeError))
+    if (!v && PyErr_ExceptionMatches(PyExc_AttributeError)) {
+        PyObject *c;
+        PyErr_Clear();
+        c = PyObject_GetAttr(x, s_ctypes);   /* numpy arrays have it; scalars, bytes and ctypes objects do not */
+        if (c) {
+            v = PyObject_GetAttr(c, s_data);
+            Py_DECREF(c);
+        } else if (PyErr_ExceptionMatches(PyExc_AttributeError)) {
             PyErr_Format(PyExc_TypeError, "cannot take the address of %R", (PyObject *)Py_TYPE(x));
-        return -1;
+        }
     }
-    *out = PyLong_AsUnsignedLongLongMask(v);
+    if (!v) return -1;
+    rc = value_of(v, out);
     Py_DECREF(v);
-    return *out == (uint64_t)-1 && PyErr_Occurred() ? -1 : 0;
+    return rc;
 }
 
 typedef int (*abi_fn)(uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t,
@@ -48,12 +68,12 @@ static PyObject *call(PyObject *self, PyObject *const *args, Py_ssize_t n)
     uint64_t a[MAX_ARGS + 1] = {0};
     int rc;
     (void)self;
-    if (n < 1 || n > MAX_ARGS + 1) {
-        PyErr_SetString(PyExc_TypeError, "call(address, up to 24 arguments)");
+    if (n < 2 || n > MAX_ARGS + 1) {
+        PyErr_SetString(PyExc_TypeError, "call(address, shape, up to 23 arguments)");
         return NULL;
     }
     for (Py_ssize_t i = 0; i < n; ++i)
-        if (address_of(args[i], &a[i]) != 0) return NULL;
+        if ((i == 1 ? shape_of(args[i], &a[i]) : address_of(args[i], &a[i])) != 0) return NULL;
     /* the *_host entry points synchronise: other Python threads run meanwhile, as they do under ctypes */
     Py_BEGIN_ALLOW_THREADS
     rc = ((abi_fn)(uintptr_t)a[0])(a[1], a[2], a[3], a[4], a[5], a[6], a[7], a[8], a[9], a[10], a[11], a[12], a[13], a[14],
@@ -62,11 +82,23 @@ static PyObject *call(PyObject *self, PyObject *const *args, Py_ssize_t n)
     return PyLong_FromLong(rc);
 }
 
-static PyMethodDef methods[] = {{"call", (PyCFunction)(void (*)(void))call, METH_FASTCALL, NULL}, {NULL, NULL, 0, NULL}};
+static PyObject *set_shape_type(PyObject *self, PyObject *type)
+{
+    (void)self;
+    Py_INCREF(type);
+    Py_XSETREF(shape_type, type);
+    Py_RETURN_NONE;
+}
+
+static PyMethodDef methods[] = {{"call", (PyCFunction)(void (*)(void))call, METH_FASTCALL, NULL},
+                                {"set_shape_type", set_shape_type, METH_O, NULL},
+                                {NULL, NULL, 0, NULL}};
 static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_gdn_call", NULL, -1, methods, NULL, NULL, NULL, NULL};
 
 PyMODINIT_FUNC PyInit__gdn_call(void)
 {
     s_data_ptr = PyUnicode_InternFromString("data_ptr");
-    return s_data_ptr ? PyModule_Create(&module) : NULL;
+    s_ctypes = PyUnicode_InternFromString("ctypes");
+    s_data = PyUnicode_InternFromString("data");
+    return s_data_ptr && s_ctypes && s_data ? PyModule_Create(&module) : NULL;
 }

@@ -166,6 +166,35 @@ def test_padded_entry_points_refuse_a_state_off_a_32_byte_boundary(lib):
     assert gdn.gdn_tree_commit_padded(s, 2, 0, off, *[a] * 9) == -4
 
 
+def test_argument_conversion(lib):
+    """What the binding passes for each kind of argument, and what it refuses (a callback stands in for the library)."""
+    from paper_2607_06763_b200 import binding
+    seen = []
+    proto = ctypes.CFUNCTYPE(ctypes.c_int, *[ctypes.c_uint64] * 3)
+    fn = proto(lambda *a: seen.append(a) or -5)
+    address = ctypes.cast(fn, ctypes.c_void_p).value
+    s, a, t = gdn.GdnShape(), np.zeros(8, np.float32), _FakeBuf(0)
+    call = lambda *args: binding._call(address, *args)
+    for given, passed in ((None, 0), (7, 7), (True, 1), (-1, (1 << 64) - 1), ((1 << 63) + 5, (1 << 63) + 5), (t, 1 << 20),
+                          (a, a.ctypes.data), (a[::2], a.ctypes.data), (a[3:], a.ctypes.data + 12)):
+        assert call(s, given, 3) == -5 and seen.pop() == (ctypes.addressof(s), passed, 3)
+    for refused in (np.int64(1 << 40), np.uint64(1 << 40), np.float32(1), ctypes.c_void_p(1 << 40), ctypes.c_int(3), b"abcd",
+                    bytearray(8), memoryview(b"abcd"), s, 1.5, "x", [1], object()):
+        with pytest.raises(TypeError, match="cannot take the address"):
+            call(s, refused, 3)
+    for no_shape in (None, 0, a, ctypes.c_int(3), b"abcd", t):
+        with pytest.raises(TypeError, match="GdnShape"):
+            call(no_shape, 1, 2)
+
+    class Fails:
+        def data_ptr(self):
+            raise RuntimeError("no storage")
+
+    with pytest.raises(RuntimeError, match="no storage"):
+        call(s, Fails(), 3)
+    assert not seen
+
+
 def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     from paper_2607_06763_b200 import binding
     monkeypatch.setattr(binding, "_lib", None)
