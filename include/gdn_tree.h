@@ -16,7 +16,9 @@
  *     want the state 32-byte aligned; elsewhere a state off a 32-byte boundary
  *     is taken by the general kernels); pointers marked [host]
  *     are ordinary host pointers.  The caller owns every buffer.  The library
- *     allocates no memory and keeps no state between calls.
+ *     allocates no memory and keeps nothing of a call for the next one; what it
+ *     remembers is which kernels have had their shared memory limit raised in
+ *     the current CUDA context, and the number of its SMs.
  *   - Work is enqueued on `cuda_stream` (a cudaStream_t passed as void*,
  *     NULL = the legacy default stream).  The [device] entry points never
  *     synchronise; the *_host entry points synchronise the stream before

@@ -477,7 +477,7 @@ template <int CTAS> __global__ void __launch_bounds__(CF_THREADS, CTAS == 1 ? 2 
 // per SM with which they are all resident at once.
 int commit_form(int units)
 {
-    static PerDevice seen;
+    static PerContext seen;
     int sms = 0;
     if (device_sms(seen, nullptr, 0, &sms) != cudaSuccess) return 2;
     return 4 * units <= sms ? 1 : units <= 2 * sms ? 2 : units <= 3 * sms ? 3 : 4;
@@ -506,7 +506,7 @@ cudaError_t launch_commit_generic(const gdn_shape_t &s, float *S, const void *k,
                    parent, node_offsets, path, path_offsets, status_dev, 0, 0, 0, 0, nullptr, nullptr};
     if (commit_tile128_supported(s) && (reinterpret_cast<uintptr_t>(S) & 31u) == 0)   // 32-byte accesses of the state
         return launch_tile128(p, grid, stream);
-    static PerDevice seen[2];
+    static PerContext seen[2];
     const auto kernel = s.in_dtype == GDN_BF16 ? commit_generic_kernel<__nv_bfloat16> : commit_generic_kernel<float>;
     int sms = 0;
     const cudaError_t e = device_sms(seen[s.in_dtype == GDN_BF16], reinterpret_cast<const void *>(kernel),

@@ -2,6 +2,7 @@
 // Nothing here is part of the public ABI (that is include/gdn_tree.h).
 #pragma once
 
+#include <cuda.h>   // driver types (functions are resolved at run time, no libcuda link)
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -107,21 +108,43 @@ inline PlanPtrs plan_ptrs(void *workspace, const WorkspaceLayout &w)
             reinterpret_cast<float *>(b + w.utilde)};
 }
 
-// What a launcher needs of the current device, asked for once per device and kernel (the runtime calls cost about a
-// microsecond each): the number of SMs, and the kernel's dynamic shared memory limit raised to `smem` bytes.
-struct PerDevice {
-    std::atomic<int> sms[64];   // 0 = not asked yet
-};
-inline cudaError_t device_sms(PerDevice &seen, const void *kernel, size_t smem, int *sms)
+// What a launcher needs of the current device: the number of SMs, and the kernel's dynamic shared memory limit raised to
+// `smem` bytes.  The runtime calls cost about a microsecond each, so that the answers are kept, for the context they were asked
+// for in: a new one (after cudaDeviceReset, for instance) has limits of its own.  A context is known by its id, which no other
+// one of the process ever has.
+inline bool current_context(unsigned long long *id)   // id >= 1; false: no context yet, or none that can be asked
 {
+    using GetId = CUresult (*)(CUcontext, unsigned long long *);
+    static const GetId get = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        return cudaGetDriverEntryPoint("cuCtxGetId", &f, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess
+                   ? reinterpret_cast<GetId>(f) : nullptr;
+    }();
+    if (!get || get(nullptr, id) != CUDA_SUCCESS) return false;
+    ++*id;
+    return true;
+}
+struct PerContext {
+    std::atomic<unsigned long long> known[64];   // by context id mod 64: id << 16 | SMs, 0 = nothing yet
+};
+inline cudaError_t device_sms(PerContext &seen, const void *kernel, size_t smem, int *sms)
+{
+    unsigned long long id = 0;
+    const bool keep = current_context(&id) && id >> 48 == 0;
+    std::atomic<unsigned long long> &slot = seen.known[id & 63];
+    if (keep) {
+        const unsigned long long was = slot.load(std::memory_order_acquire);
+        if (was >> 16 == id) {
+            *sms = (int)(was & 0xFFFFu);
+            return cudaSuccess;
+        }
+    }
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    *sms = dev < 64 ? seen.sms[dev].load(std::memory_order_acquire) : 0;
-    if (*sms != 0) return cudaSuccess;
-    e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess && kernel) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess && dev < 64) seen.sms[dev].store(*sms, std::memory_order_release);
+    if (e == cudaSuccess && keep) slot.store(id << 16 | (unsigned)*sms, std::memory_order_release);
     return e;
 }
 

@@ -537,7 +537,7 @@ __global__ void __launch_bounds__(VS_THREADS, 2) verify_generic_small_kernel(con
 template <typename TIn, typename TOut>
 cudaError_t launch_small_typed(VerifySmallParams p, cudaStream_t stream, LaunchInFront commit)
 {
-    static PerDevice seen;
+    static PerContext seen;
     int sms = 0;
     cudaError_t e = device_sms(seen, reinterpret_cast<const void *>(verify_generic_small_kernel<TIn, TOut>),
                                sizeof(VerifySmallSmem), &sms);

@@ -871,7 +871,7 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
 
 template <typename TOut, bool PADDED, bool GROUPED> cudaError_t launch_kernel(const VerifyPlainParams &p, LaunchInFront commit, cudaStream_t stream)
 {
-    static PerDevice seen;
+    static PerContext seen;
     int sms = 0;
     cudaError_t e = device_sms(seen, reinterpret_cast<const void *>(verify_plain_kernel<TOut, PADDED, GROUPED>), SP_ALLOC, &sms);
     if (e == cudaSuccess && commit) e = commit();

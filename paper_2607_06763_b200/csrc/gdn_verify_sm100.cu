@@ -959,7 +959,7 @@ template <typename TOut> cudaError_t launch_typed(const gdn_shape_t &s, const Ve
     // the padded layout and the on-chip gate activations share an instantiation
     void (*kernel)(const VerifyFastParams) = small ? padded ? commit_verify_kernel<TOut, true, true> : commit_verify_kernel<TOut, true, false>
                                                    : padded ? commit_verify_kernel<TOut, false, true> : commit_verify_kernel<TOut, false, false>;
-    static PerDevice seen[4];
+    static PerContext seen[4];
     int sms = 0;
     const cudaError_t e = device_sms(seen[2 * padded + small], reinterpret_cast<const void *>(kernel),
                                      SM_ALLOC, &sms);
@@ -1002,7 +1002,7 @@ VerifyFastParams make_params(const gdn_shape_t &s, const float *S0, const void *
 // 11.3 / 9.9, 128 units 11.6 / 12.3 (the path lengths are on the device, so the line lies where both gain).
 static bool as_two_kernels(const gdn_shape_t &s)
 {
-    static PerDevice seen;
+    static PerContext seen;
     int sms = 0;
     return device_sms(seen, nullptr, 0, &sms) == cudaSuccess && s.n_seq * s.h_v <= sms / 2;
 }

@@ -1,5 +1,6 @@
 /* The parts of the CUDA runtime that the host side of libgdn_tree.so calls, for tests without a GPU: nothing runs, every
- * kernel launch is written to a log, and any other call can be made to fail.  Linked with the library's objects in place of
+ * kernel launch is written to a log, and any other call can be made to fail.  A kernel's shared memory limit counts in the
+ * context it was raised in.  Linked with the library's objects in place of
  * the runtime (test_host_launches.py). */
 #include <stddef.h>
 #include <stdio.h>
@@ -14,6 +15,11 @@ static char log_text[1 << 14];   /* names of the launched kernels, one per line 
 static int calls;                /* calls other than launches so far */
 static int fail_at = -1;         /* number of the call that fails */
 
+static unsigned long long context;                                                  /* id of the current one */
+static struct { const void *host; unsigned long long context; int bytes; } limits[256];   /* raised so far */
+static int n_limits;
+
+void fake_context(unsigned long long id) { context = id; }
 void fake_reset(int fail_call) { log_text[0] = 0; calls = 0; fail_at = fail_call; }
 const char *fake_log(void) { return log_text; }
 int fake_calls(void) { return calls; }
@@ -69,13 +75,28 @@ int cudaLaunchKernel(const void *f, dim3_t grid, dim3_t block, void **args, size
     (void)grid; (void)block; (void)args; (void)smem; (void)stream;
     return launched(f);
 }
-int cudaLaunchKernelExC(const launch_config *cfg, const void *f, void **args) { (void)cfg; (void)args; return launched(f); }
+int cudaLaunchKernelExC(const launch_config *cfg, const void *f, void **args)
+{
+    size_t limit = 48 << 10;
+    (void)args;
+    for (int i = 0; i < n_limits; ++i)
+        if (limits[i].host == f && limits[i].context == context) limit = (size_t)limits[i].bytes;
+    return cfg->smem > limit ? INVALID_VALUE : launched(f);
+}
 int cudaGetLastError(void) { return SUCCESS; }
 
 /* everything else */
 int cudaGetDevice(int *dev) { *dev = 0; return call_result(); }
 int cudaDeviceGetAttribute(int *value, int attr, int dev) { (void)attr; (void)dev; *value = 148; return call_result(); }
-int cudaFuncSetAttribute(const void *f, int attr, int value) { (void)f; (void)attr; (void)value; return call_result(); }
+int cudaFuncSetAttribute(const void *f, int attr, int value)
+{
+    if (attr == 8 && n_limits < 256) {   /* cudaFuncAttributeMaxDynamicSharedMemorySize */
+        limits[n_limits].host = f;
+        limits[n_limits].context = context;
+        limits[n_limits++].bytes = value;
+    }
+    return call_result();
+}
 int cudaMemsetAsync(void *p, int v, size_t n, void *s) { (void)p; (void)v; (void)n; (void)s; return call_result(); }
 int cudaMemcpyAsync(void *d, const void *p, size_t n, int k, void *s) { (void)d; (void)p; (void)n; (void)k; (void)s; return call_result(); }
 int cudaGetSymbolAddress(void **p, const void *symbol) { *p = (void *)symbol; return call_result(); }
@@ -86,10 +107,11 @@ int cudaEventCreateWithFlags(void **e, unsigned f) { (void)f; *e = NULL; return 
 int cudaEventRecord(void *e, void *s) { (void)e; (void)s; return call_result(); }
 
 static int encode_tiled(void) { return call_result(); }   /* cuTensorMapEncodeTiled: arguments not looked at */
+static int ctx_get_id(void *ctx, unsigned long long *id) { (void)ctx; *id = context; return SUCCESS; }   /* cuCtxGetId */
 int cudaGetDriverEntryPoint(const char *name, void **f, unsigned long long flags, int *found)
 {
     (void)flags;
-    *f = strcmp(name, "cuTensorMapEncodeTiled") == 0 ? (void *)encode_tiled : NULL;
+    *f = strcmp(name, "cuTensorMapEncodeTiled") == 0 ? (void *)encode_tiled : strcmp(name, "cuCtxGetId") == 0 ? (void *)ctx_get_id : NULL;
     *found = *f ? 0 : 1;
     return call_result();
 }

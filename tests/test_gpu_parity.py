@@ -945,3 +945,14 @@ def test_recurrent_comparator_rejects_a_broken_branch(tl):
     assert gdn.gdn_tree_verify_recurrent(dc.shape, dc.S0, dc.q, dc.k, dc.v, dc.g, dc.beta, dc.parent, dc.node_offsets,
                                          dc.o, dc.status) == 0
     assert dc.device_status() == -8 and bool((dc.o == 7.0).all())
+
+
+def test_calls_in_a_second_context(tl):
+    """The library in driver contexts of a child process's own, one after the other and side by side: what it keeps about one
+    (raised shared memory limits) must not be taken for the next."""
+    import os
+    import subprocess
+    import sys
+    child = os.path.join(os.path.dirname(os.path.abspath(__file__)), "context_child.py")
+    r = subprocess.run([sys.executable, child], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr

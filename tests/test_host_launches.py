@@ -97,3 +97,13 @@ def test_fused_call_commits_only_once_the_verification_is_prepared(fake_path, ca
             assert fresh.launches() in (kernels, ["commit_verify_kernel"])
         else:
             assert rc == -6 and not any("commit" in x for x in fresh.launches()), f"call {k} of {n} failed behind the commit"
+
+
+@pytest.mark.parametrize("call,shape,S,kernels", FUSED, ids=range(len(FUSED)))
+def test_shared_memory_limits_are_raised_in_every_context(fake_path, call, shape, S, kernels):
+    """Limits raised in one context do not count in another one (after cudaDeviceReset, say): every launch has its own."""
+    fake = Fake(fake_path)
+    for context in (3, 3, 4, 3, 0):
+        fake.lib.fake_context(ctypes.c_ulonglong(context))
+        fake.reset()
+        assert call(fake, shape, S) == 0 and fake.launches() == kernels, f"context {context}"
