@@ -334,7 +334,7 @@ int gdn_tree_commit_verify_host(const gdn_shape_t *shape, float *S_h, int32_t pr
  *   - Limit: gdn_tree_workspace_bytes(shape) must not exceed GDN_STATIC_SCRATCH_BYTES (about
  *     one layer of 32 value heads x 128 with a tree of up to ~250 nodes); larger problems get
  *     GDN_ERR_WORKSPACE and nothing is launched.
- *   - The first call on each device does one-time set-up with that device current: the CUDA
+ *   - The first call in each context of a device does one-time set-up: the CUDA
  *     runtime loads the library's device code (which is when the array itself comes into being),
  *     the array's device address is resolved, the kernels' shared-memory attributes are set and the
  *     driver entry point for tensor maps is looked up.  Make that first call before starting any

@@ -18,22 +18,27 @@ namespace {
 // not a device address: it must go through cudaGetSymbolAddress before a kernel can be given it.
 static __device__ __align__(256) unsigned char g_static_scratch[GDN_STATIC_SCRATCH_BYTES];
 
-constexpr int kMaxDevices = 64;
 std::mutex g_setup_mutex;
-void *g_scratch_addr[kMaxDevices] = {};   // device address of g_static_scratch, per device ordinal
+struct { unsigned long long context; void *addr; } g_scratch[64];   // device address of g_static_scratch, by context id mod 64
 
-// Device address of the scratch array on the current device (resolved once per device).
-int scratch_for_current_device(void **out)
+// Device address of the scratch array in the current context (resolved once for each: another context, after cudaDeviceReset
+// for instance, has an array of its own).
+int scratch_for_current_context(void **out)
 {
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return GDN_ERR_CUDA;
+    unsigned long long id = 0;
+    const bool known = gdn::current_context(&id);
     std::lock_guard<std::mutex> lock(g_setup_mutex);
-    if (!g_scratch_addr[dev]) {
+    auto &slot = g_scratch[id & 63];
+    if (!known || slot.context != id) {
         void *ptr = nullptr;
         if (cudaGetSymbolAddress(&ptr, g_static_scratch) != cudaSuccess || !ptr) return GDN_ERR_CUDA;
-        g_scratch_addr[dev] = ptr;
+        if (!known) {
+            *out = ptr;
+            return GDN_OK;
+        }
+        slot = {id, ptr};
     }
-    *out = g_scratch_addr[dev];
+    *out = slot.addr;
     return GDN_OK;
 }
 
@@ -50,7 +55,7 @@ extern "C" int gdn_tree_verify_static(const gdn_shape_t *shape, const float *S0,
                                cuda_stream);
     if (need > GDN_STATIC_SCRATCH_BYTES) return GDN_ERR_WORKSPACE;   // problem too large for the fixed scratch
     void *scratch = nullptr;
-    const int rc = scratch_for_current_device(&scratch);
+    const int rc = scratch_for_current_context(&scratch);
     if (rc != GDN_OK) return rc;
     return gdn_tree_verify(shape, S0, q, k, v, g, beta, parent, node_offsets, o, scratch,
                            GDN_STATIC_SCRATCH_BYTES, status_dev, cuda_stream);

@@ -11,7 +11,7 @@ enum { SUCCESS = 0, INVALID_VALUE = 1, UNKNOWN = 999 };
 static struct { const void *host; const char *name; } kernels[256];
 static int n_kernels;
 
-static char log_text[1 << 14];   /* names of the launched kernels, one per line */
+static char log_text[1 << 14];   /* names of the launched kernels and of a few other calls, one per line */
 static int calls;                /* calls other than launches so far */
 static int fail_at = -1;         /* number of the call that fails */
 
@@ -26,13 +26,18 @@ int fake_calls(void) { return calls; }
 
 static int call_result(void) { return calls++ == fail_at ? UNKNOWN : SUCCESS; }
 
+static void note(const char *line)
+{
+    const size_t n = strlen(log_text);
+    snprintf(log_text + n, sizeof log_text - n, "%s\n", line);
+}
+
 static int launched(const void *host)
 {
     const char *name = "?";
     for (int i = 0; i < n_kernels; ++i)
         if (kernels[i].host == host) name = kernels[i].name;
-    const size_t n = strlen(log_text);
-    snprintf(log_text + n, sizeof log_text - n, "%s\n", name);
+    note(name);
     return SUCCESS;
 }
 
@@ -99,7 +104,7 @@ int cudaFuncSetAttribute(const void *f, int attr, int value)
 }
 int cudaMemsetAsync(void *p, int v, size_t n, void *s) { (void)p; (void)v; (void)n; (void)s; return call_result(); }
 int cudaMemcpyAsync(void *d, const void *p, size_t n, int k, void *s) { (void)d; (void)p; (void)n; (void)k; (void)s; return call_result(); }
-int cudaGetSymbolAddress(void **p, const void *symbol) { *p = (void *)symbol; return call_result(); }
+int cudaGetSymbolAddress(void **p, const void *symbol) { *p = (void *)symbol; note("cudaGetSymbolAddress"); return call_result(); }
 int cudaStreamCreateWithFlags(void **s, unsigned f) { (void)f; *s = NULL; return call_result(); }
 int cudaStreamSynchronize(void *s) { (void)s; return call_result(); }
 int cudaStreamWaitEvent(void *s, void *e, unsigned f) { (void)s; (void)e; (void)f; return call_result(); }

@@ -50,6 +50,9 @@ class Fake:
     def call(self, name, *args):
         return binding._call(ctypes.cast(getattr(self.lib, name), ctypes.c_void_p).value, *args)
 
+    def count(self, name):
+        return self.lib.fake_log().decode().split().count(name)
+
     def launches(self):
         return re.findall(r"\d((?:commit|verify|plan)_[a-z0-9_]*?kernel)(?=[EI])", self.lib.fake_log().decode())   # (mangled names)
 
@@ -107,3 +110,13 @@ def test_shared_memory_limits_are_raised_in_every_context(fake_path, call, shape
         fake.lib.fake_context(ctypes.c_ulonglong(context))
         fake.reset()
         assert call(fake, shape, S) == 0 and fake.launches() == kernels, f"context {context}"
+
+
+def test_static_scratch_is_found_in_every_context(fake_path):
+    """The address of the library's scratch array belongs to a context: it is asked for in each, and once."""
+    fake, s = Fake(fake_path), _shape(1, 100, d=32, h_v=4)
+    for context, asked in ((3, 1), (3, 0), (4, 1), (4, 0), (5, 1)):
+        fake.lib.fake_context(ctypes.c_ulonglong(context))
+        fake.reset()
+        assert fake.call("gdn_tree_verify_static", s, *[A] * 10, 0) == 0
+        assert fake.launches() == ["plan_kernel", "verify_generic_kernel"] and fake.count("cudaGetSymbolAddress") == asked
