@@ -304,8 +304,8 @@ int gdn_tree_commit_host(const gdn_shape_t *shape, float *S_h, const void *k_h, 
  * With two or more sequences the call is pipelined: the batch is cut into up to six groups of
  * sequences, and the copies up of one group, the kernels of the group before it and the copies down
  * of the group before that run at the same time (both directions of the host link busy).  The
- * copies run on two helper streams that the library creates on first use for each device and keeps
- * (the one exception to "keeps no state"); `cuda_stream` is synchronised before returning, as for
+ * copies run on two helper streams that the library creates on first use in each context and keeps
+ * for as long as that lives; `cuda_stream` is synchronised before returning, as for
  * the other host variants, and nothing is left in flight.  Host buffers should be pinned: with
  * pageable memory the copies are staged synchronously and nothing overlaps.
  */

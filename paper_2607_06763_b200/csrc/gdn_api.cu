@@ -1,6 +1,7 @@
 // C-ABI entry points of libgdn_tree.so: argument validation, workspace carving, kernel launches,
 // and the host-buffer variants.  See include/gdn_tree.h for the contract of every function.
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <vector>
 
@@ -595,8 +596,8 @@ extern "C" int gdn_tree_commit_host(const gdn_shape_t *shape, float *S_h, const 
 
 namespace {
 
-// Helper streams and events of the pipelined host-buffer call, created on first use for each device and kept for
-// the life of the process (the one piece of state the library keeps besides the static scratch array).
+// Helper streams and events of the pipelined host-buffer call, created on first use in each context and kept for as long as the
+// process lives (they go with their context).
 constexpr int HOST_PIPE_GROUPS = 6;
 struct HostPipe {
     bool ready = false;
@@ -604,14 +605,20 @@ struct HostPipe {
     cudaEvent_t start = nullptr, done = nullptr, in[HOST_PIPE_GROUPS] = {}, k[HOST_PIPE_GROUPS] = {};
 };
 std::mutex g_pipe_mutex;
-HostPipe g_pipe[64];
+std::map<unsigned long long, HostPipe> g_pipes;   // by context id (see current_context)
 
 HostPipe *host_pipe()
 {
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    unsigned long long id = 0;
+    if (!current_context(&id)) return nullptr;   // (the call has used the runtime before: there is one)
     std::lock_guard<std::mutex> lock(g_pipe_mutex);
-    HostPipe &p = g_pipe[dev];
+    HostPipe *found = nullptr;
+    try {
+        found = &g_pipes[id];
+    } catch (...) {   // (out of memory: the call runs unpipelined)
+        return nullptr;
+    }
+    HostPipe &p = *found;
     if (!p.ready) {
         bool ok = cudaStreamCreateWithFlags(&p.s_in, cudaStreamNonBlocking) == cudaSuccess &&
                   cudaStreamCreateWithFlags(&p.s_out, cudaStreamNonBlocking) == cudaSuccess &&

@@ -105,7 +105,7 @@ int cudaFuncSetAttribute(const void *f, int attr, int value)
 int cudaMemsetAsync(void *p, int v, size_t n, void *s) { (void)p; (void)v; (void)n; (void)s; return call_result(); }
 int cudaMemcpyAsync(void *d, const void *p, size_t n, int k, void *s) { (void)d; (void)p; (void)n; (void)k; (void)s; return call_result(); }
 int cudaGetSymbolAddress(void **p, const void *symbol) { *p = (void *)symbol; note("cudaGetSymbolAddress"); return call_result(); }
-int cudaStreamCreateWithFlags(void **s, unsigned f) { (void)f; *s = NULL; return call_result(); }
+int cudaStreamCreateWithFlags(void **s, unsigned f) { (void)f; *s = NULL; note("cudaStreamCreate"); return call_result(); }
 int cudaStreamSynchronize(void *s) { (void)s; return call_result(); }
 int cudaStreamWaitEvent(void *s, void *e, unsigned f) { (void)s; (void)e; (void)f; return call_result(); }
 int cudaEventCreateWithFlags(void **e, unsigned f) { (void)f; *e = NULL; return call_result(); }

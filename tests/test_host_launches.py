@@ -6,6 +6,7 @@ import re
 import shutil
 import subprocess
 
+import numpy as np
 import pytest
 
 import paper_2607_06763_b200 as gdn
@@ -120,3 +121,22 @@ def test_static_scratch_is_found_in_every_context(fake_path):
         fake.reset()
         assert fake.call("gdn_tree_verify_static", s, *[A] * 10, 0) == 0
         assert fake.launches() == ["plan_kernel", "verify_generic_kernel"] and fake.count("cudaGetSymbolAddress") == asked
+
+
+def _fused_host(fake, s):
+    """gdn_tree_commit_verify_host of trees of max_tree_nodes nodes, paths of one node (the arrays read on the host are real)."""
+    nodes = np.arange(s.n_seq + 1, dtype=np.int32) * s.max_tree_nodes
+    paths = np.arange(s.n_seq + 1, dtype=np.int32)
+    arena = fake.lib.gdn_tree_commit_verify_host_arena_bytes(ctypes.byref(s), s.total_nodes, s.n_seq)
+    return fake.call("gdn_tree_commit_verify_host", s, A, s.total_nodes, *[A] * 5, nodes, A, paths, s.n_seq, *[A] * 6, nodes, A, A,
+                     arena, 0)
+
+
+def test_host_buffer_pipeline_has_streams_in_every_context(fake_path):
+    """The helper streams and events of the pipelined call belong to a context: each has its own, made once."""
+    fake, s = Fake(fake_path), _shape(4, 64)
+    for context, made in ((3, 2), (3, 0), (4, 2), (3, 0), (4, 0)):
+        fake.lib.fake_context(ctypes.c_ulonglong(context))
+        fake.reset()
+        assert _fused_host(fake, s) == 0
+        assert fake.launches() == ["commit_tile128_kernel", "verify_plain_kernel"] * 4 and fake.count("cudaStreamCreate") == made
