@@ -305,7 +305,7 @@ int gdn_tree_commit_host(const gdn_shape_t *shape, float *S_h, const void *k_h, 
  * sequences, and the copies up of one group, the kernels of the group before it and the copies down
  * of the group before that run at the same time (both directions of the host link busy).  The
  * copies run on two helper streams that the library creates on first use in each context and keeps
- * for as long as that lives; `cuda_stream` is synchronised before returning, as for
+ * for as long as that lives (calls of several threads take turns on them); `cuda_stream` is synchronised before returning, as for
  * the other host variants, and nothing is left in flight.  Host buffers should be pinned: with
  * pageable memory the copies are staged synchronously and nothing overlaps.
  */

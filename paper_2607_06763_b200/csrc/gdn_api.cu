@@ -600,6 +600,8 @@ namespace {
 // process lives (they go with their context).
 constexpr int HOST_PIPE_GROUPS = 6;
 struct HostPipe {
+    std::mutex turn;   // held by the call that uses them: an event recorded by one call must not be recorded by another one
+                       // before it has been waited for (the call ends with a synchronisation anyway)
     bool ready = false;
     cudaStream_t s_in = nullptr, s_out = nullptr;
     cudaEvent_t start = nullptr, done = nullptr, in[HOST_PIPE_GROUPS] = {}, k[HOST_PIPE_GROUPS] = {};
@@ -702,6 +704,7 @@ extern "C" int gdn_tree_commit_verify_host(const gdn_shape_t *shape, float *S_h,
     const bool sliceable = ((size_t)s.h_v * dtype_size(s.in_dtype)) % 16 == 0;
     HostPipe *pipe = (sliceable && s.n_seq >= 2 && s.total_nodes > 0 && total_path_len > 0) ? host_pipe() : nullptr;
     if (pipe) {
+        std::lock_guard<std::mutex> turn(pipe->turn);
         // Pipelined form: the layer slots / sequences are cut into groups; the copies up of group i+1 (helper stream
         // s_in), the kernels of group i (the caller's stream) and the copies down of group i-1 (helper stream s_out)
         // run at the same time, so that both directions of the host link are busy.  Each group is a call of its own

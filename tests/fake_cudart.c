@@ -2,9 +2,12 @@
  * kernel launch is written to a log, and any other call can be made to fail.  A kernel's shared memory limit counts in the
  * context it was raised in.  Linked with the library's objects in place of
  * the runtime (test_host_launches.py). */
+#define _GNU_SOURCE
+#include <pthread.h>
 #include <stddef.h>
 #include <stdio.h>
 #include <string.h>
+#include <unistd.h>
 
 enum { SUCCESS = 0, INVALID_VALUE = 1, UNKNOWN = 999 };
 
@@ -28,8 +31,11 @@ static int call_result(void) { return calls++ == fail_at ? UNKNOWN : SUCCESS; }
 
 static void note(const char *line)
 {
+    static pthread_mutex_t lock = PTHREAD_MUTEX_INITIALIZER;
+    pthread_mutex_lock(&lock);
     const size_t n = strlen(log_text);
     snprintf(log_text + n, sizeof log_text - n, "%s\n", line);
+    pthread_mutex_unlock(&lock);
 }
 
 static int launched(const void *host)
@@ -109,7 +115,15 @@ int cudaStreamCreateWithFlags(void **s, unsigned f) { (void)f; *s = NULL; note("
 int cudaStreamSynchronize(void *s) { (void)s; return call_result(); }
 int cudaStreamWaitEvent(void *s, void *e, unsigned f) { (void)s; (void)e; (void)f; return call_result(); }
 int cudaEventCreateWithFlags(void **e, unsigned f) { (void)f; *e = NULL; return call_result(); }
-int cudaEventRecord(void *e, void *s) { (void)e; (void)s; return call_result(); }
+int cudaEventRecord(void *e, void *s)
+{
+    char line[32];
+    (void)e; (void)s;
+    snprintf(line, sizeof line, "record:%d", (int)gettid());
+    note(line);
+    usleep(500);   /* another thread's turn, if it may have one */
+    return call_result();
+}
 
 static int encode_tiled(void) { return call_result(); }   /* cuTensorMapEncodeTiled: arguments not looked at */
 static int ctx_get_id(void *ctx, unsigned long long *id) { (void)ctx; *id = context; return SUCCESS; }   /* cuCtxGetId */

@@ -5,6 +5,7 @@ import os
 import re
 import shutil
 import subprocess
+import threading
 
 import numpy as np
 import pytest
@@ -140,3 +141,17 @@ def test_host_buffer_pipeline_has_streams_in_every_context(fake_path):
         fake.reset()
         assert _fused_host(fake, s) == 0
         assert fake.launches() == ["commit_tile128_kernel", "verify_plain_kernel"] * 4 and fake.count("cudaStreamCreate") == made
+
+
+def test_host_buffer_pipeline_is_one_thread_at_a_time(fake_path):
+    """The calls of a context share its helper streams and events: an event that one thread has recorded is waited for by the
+    same thread before another one records it again."""
+    fake, s, rcs = Fake(fake_path), _shape(6, 64), []
+    threads = [threading.Thread(target=lambda: rcs.append(_fused_host(fake, s))) for _ in range(3)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    who = [x for x in fake.lib.fake_log().decode().split() if x.startswith("record:")]
+    assert rcs == [0] * 3 and len(who) == 3 * (2 + 2 * 6)
+    assert sum(a != b for a, b in zip(who, who[1:])) == 2, "calls of several threads ran into one another"
