@@ -293,7 +293,8 @@ __global__ void __launch_bounds__(VS_THREADS, 2) verify_generic_small_kernel(con
     stage_rows(sm.ks, k + ((size_t)base * p.h_qk + hk) * d_k, q_stride, i_hi, d_k, tid);
     stage_rows(sm.qp[0], q_head + i_lo * q_stride, q_stride, min(VS_NODES, i_hi - i_lo), d_k, tid);
     stage_rows(sm.vs, v + ((size_t)base * p.h_v + h) * d_v, (size_t)p.h_v * d_v, i_hi, d_v, tid);
-    // State: rows c .. c + 3; sreg[r][2 j], [2 j + 1] hold key positions 32 j + 4 s + e (zero beyond d_k / d_v).
+    // State: rows c .. c + 3; sreg[r][2 j], [2 j + 1] hold key positions 32 j + 4 s + e (zero beyond d_k / d_v).  Not through the
+    // read-only path: the commit in front may still be writing the state while this grid moves in.
     const int c = (tid / VS_SPLIT) * 4, s = tid % VS_SPLIT;
     float2 sreg[4][8];
 #pragma unroll
@@ -303,7 +304,7 @@ __global__ void __launch_bounds__(VS_THREADS, 2) verify_generic_small_kernel(con
         for (int j = 0; j < 4; ++j) {
             const int at = 32 * j + 4 * s;
             float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (c + r < d_v && at < d_k) x = __ldg(reinterpret_cast<const float4 *>(row + at));
+            if (c + r < d_v && at < d_k) x = *reinterpret_cast<const float4 *>(row + at);
             sreg[r][2 * j] = make_float2(x.x, x.y);
             sreg[r][2 * j + 1] = make_float2(x.z, x.w);
         }

@@ -153,13 +153,13 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
     // previous call, or the plan kernel); nothing that is computed from memory may run before that kernel's writes are
     // visible.  L2 can be asked for the first unit's state tile and rows meanwhile (a prefetch consumes nothing): where
     // the rows are may depend on node_offsets[], which the kernel in front may still be writing, so the value read here
-    // only steers prefetches (clamped to the tensors).
+    // only steers prefetches (clamped to the tensors), and comes from L2: nothing of it stays in L1 for the read that counts.
     const int u_first = (int)((long long)p.n_units * cta / (int)gridDim.x);   // (not GROUPED)
     if constexpr (!GROUPED) {
         if (tid < 4) prefetch_l2_bulk(p.S0 + (size_t)u_first * VP_D * VP_D + (size_t)tid * 4096, 16384);
         if (!p.state_late && tid >= 128 && tid < 128 + VP_T && tid - 128 < p.max_tree_nodes) {
             const int ub = u_first / p.h_v, uh = u_first % p.h_v, uhk = uh / (p.h_v / p.h_qk);
-            const int row = (PADDED ? ub * p.t_pad : __ldg(p.node_offsets + ub)) + tid - 128;
+            const int row = (PADDED ? ub * p.t_pad : __ldcg(p.node_offsets + ub)) + tid - 128;
             if (row >= 0 && row < p.total_nodes) {
                 prefetch_l2_bulk(p.v + ((size_t)row * p.h_v + uh) * VP_D, 256);
                 prefetch_l2_bulk(p.k + ((size_t)row * p.h_qk + uhk) * VP_D, 256);
@@ -311,11 +311,11 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
     };
 
     // ------------------------------------------------------------------------------------ rows
-    // node id of virtual index u (< T) of a group, from the plan
+    // node id of virtual index u (< T) of a group, from the plan (written by the kernel in front: no read-only path)
     auto vnode_of = [&](const Unit &un, int u) -> int {
         if (un.ident) return u;
-        if (u < un.n_prefix) return (int)__ldg(p.anc16 + (size_t)(un.pb + un.first) * p.anc_stride + u);
-        return (int)__ldg(p.dfs_node + un.pb + un.g0 + u - un.n_prefix);
+        if (u < un.n_prefix) return (int)p.anc16[(size_t)(un.pb + un.first) * p.anc_stride + u];
+        return (int)p.dfs_node[un.pb + un.g0 + u - un.n_prefix];
     };
     uint16_t *vnode_s = reinterpret_cast<uint16_t *>(smem + SP_VN);   // node ids of the unit whose rows are asked for next
     // k/q rows (rows 0..63 = k, 64..127 = q) by TMA: four boxes, 128-byte swizzled.  A box always spans box_rows rows: rows

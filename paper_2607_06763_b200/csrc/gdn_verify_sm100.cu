@@ -153,11 +153,12 @@ __global__ void __launch_bounds__(FV_THREADS, 2) commit_verify_kernel(const __gr
     if (tid < 4 && (int)blockIdx.x < p.n_units)
         prefetch_l2_bulk(p.S0 + (size_t)blockIdx.x * FV_D * FV_D + (size_t)tid * 4096, 16384);
     // ... and for the rows of the first unit's tree.  Their place may depend on node_offsets[], which the kernel in
-    // front may still be writing: the value read here only steers prefetches (clamped to the tensors), it is read
-    // again behind the dependency wait before anything is computed from it.
+    // front may still be writing: the value read here only steers prefetches (clamped to the tensors) and comes from
+    // L2, so that nothing of it stays in L1; it is read again behind the dependency wait before anything is computed
+    // from it.
     if ((int)blockIdx.x < p.n_units && tid >= 128 && tid < 128 + FV_T) {
         const int ub = (int)blockIdx.x / p.h_v, uh = (int)blockIdx.x % p.h_v, uhk = uh / (p.h_v / p.h_qk);
-        const int row = ((PADDED) ? ub * p.t_pad : __ldg(p.node_offsets + ub)) + tid - 128;
+        const int row = ((PADDED) ? ub * p.t_pad : __ldcg(p.node_offsets + ub)) + tid - 128;
         if (row >= 0 && row < p.total_nodes) {
             prefetch_l2_bulk(p.v + ((size_t)row * p.h_v + uh) * FV_D, 256);
             prefetch_l2_bulk(p.k + ((size_t)row * p.h_qk + uhk) * FV_D, 256);

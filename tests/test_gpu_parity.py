@@ -794,6 +794,37 @@ def test_fused_step_on_both_sides_of_the_two_kernel_rule(tl, slots):
             tl.assert_close_per_head(o.cpu().numpy().astype(np.float64), o_ref, w.node_offsets, f"fused, {slots} slots, o")
 
 
+@pytest.mark.parametrize("in_dtype,sizes", [(synth.F32, (40, 9, 64)), (synth.BF16, (300, 20)), (synth.BF16, (40, 9, 64))])
+def test_verify_and_commit_in_turn_without_a_wait(tl, in_dtype, sizes):
+    """Kernels of this library move in while the one in front still runs, here with the state, the trees and the workspace
+    that the ones before have just read: every verification has to see what is written in between."""
+    import torch
+    from oracle import gdn_oracle as orc
+    rng = np.random.default_rng(231)
+    make = lambda seed: synth.random_case(seed, [synth.tree_geo(rng, T) for T in sizes], 2, 4, 128, 128, in_dtype, synth.F32)
+    ws, got = [make(232 + i) for i in range(4)], []
+    src = [tl.DeviceCase(w) for w in ws]
+    dc = tl.DeviceCase(ws[0])
+    dc.path = torch.zeros(16 * len(sizes), dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    for i in range(8):
+        if i % 2 == 0:   # another tree and other rows in the same buffers
+            for name in ("q", "k", "v", "g", "beta", "parent", "path_offsets"):
+                getattr(dc, name).copy_(getattr(src[i // 2], name))
+            dc.path[: ws[i // 2].path.size].copy_(src[i // 2].path[: ws[i // 2].path.size])
+        assert dc.verify(torch.cuda.current_stream()) == 0 and dc.commit(stream=torch.cuda.current_stream()) == 0
+        got.append((dc.o.clone(), dc.S0.clone()))
+    assert dc.device_status() == 0
+    S = ws[0].f64("S0")
+    for i, (o, S1) in enumerate(got):
+        w = ws[i // 2]
+        rows = [w.f64(n) for n in ("q", "k", "v", "g", "beta")]
+        o_ref = orc.verify(S, *rows, w.parent, w.node_offsets, w.scale)
+        S = orc.commit(S, *rows[1:], w.parent, w.node_offsets, w.path, w.path_offsets)
+        tl.assert_close_per_head(o.cpu().numpy().astype(np.float64), o_ref, w.node_offsets, f"pass {i}")
+        tl.assert_state_close(S1.cpu().numpy().astype(np.float64), S, what=f"state behind pass {i}")
+
+
 @pytest.mark.parametrize("sizes", [(64, 1, 33), (20, 130), (64,) * 19, (300,)])
 def test_state_off_a_32_byte_boundary(tl, sizes):
     """A state at 16 mod 32 bytes, which the ragged entry points accept: verification, commit and fused call on the general
