@@ -57,9 +57,9 @@ constexpr int SP_KAPPA = 81920;                  // fp32 [64][16] kappa(i, t): t
 constexpr int SP_GAMMA = 86016;                  // fp32 [64][16] gamma(i, t), i itself included; same places
 constexpr int SP_ANC = 90112;                    // u8 [64][16] root path, root first, node itself last (0xFF = unused)
 constexpr int SP_AMASK = 91136;                  // u64 [64]: ancestors of i and i itself as bits (0 beyond the tree)
-constexpr int SP_GB = 91648;                     // float2 [64]: (G_i, beta_i)
+constexpr int SP_BETA = 91648;                   // float [64]: beta_i
 constexpr int SP_SA = 92160;                     // float [64]: scale exp(G_i)
-constexpr int SP_G = 92416;                      // float [64]: g of the unit whose tables are being built
+constexpr int SP_G = 92416;                      // float [64]: g_i; from step (6) on of the next unit
 constexpr int SP_PAR = 92672;                    // s8 [64]: its parents
 constexpr int SP_VN = 92736;                     // u16 [64]: grouped mode, node id of virtual index u
 constexpr int SP_BAD = 92864;                    // int: the unit's tree was rejected (nothing of it is stored)
@@ -485,7 +485,7 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
             *reinterpret_cast<uint4 *>(smem + SP_ANC + tnode * 16) = make_uint4(w0, w1, w2, w3);
             *reinterpret_cast<uint2 *>(smem + SP_AMASK + tnode * 8) = make_uint2(mlo, mhi);
         }
-        *reinterpret_cast<float2 *>(smem + SP_GB + tnode * 8) = make_float2(G, gate_beta(nr.beta, PADDED && p.raw_gates));
+        reinterpret_cast<float *>(smem + SP_BETA)[tnode] = gate_beta(nr.beta, PADDED && p.raw_gates);
         reinterpret_cast<float *>(smem + SP_SA)[tnode] = p.scale * __expf(G);
     };
 
@@ -589,19 +589,19 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
             const uint32_t idw[4] = {path.x, path.y, path.z, path.w};
             const uint32_t mine = *reinterpret_cast<const uint32_t *>(smem + SP_ANC + zi * 16 + sq * 4);
             const float *kappa = reinterpret_cast<const float *>(smem + SP_KAPPA);
-            const float2 *gb_s = reinterpret_cast<const float2 *>(smem + SP_GB);
-            float z[4], bt[4], et[4];   // of this lane's path nodes: beta, scale exp(G_i - G)
-            const float Gi = gb_s[zi].x;
+            const float *beta_s = reinterpret_cast<const float *>(smem + SP_BETA);
+            float z[4], bt[4], et[4];   // of this lane's path nodes: beta, scale exp(sum of g behind the node, down to node i)
+            float gl[4];
             {
                 const float4 g4 = *reinterpret_cast<const float4 *>(smem + SP_GAMMA + zi * 64 + ((sq ^ ((zi >> 1) & 3)) << 4));
                 const float gv[4] = {g4.x, g4.y, g4.z, g4.w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const float2 gb = gb_s[(mine >> (8 * e)) & 63u];
+                    const uint32_t id = (mine >> (8 * e)) & 63u;
                     const bool on = sq * 4 + e < d;
                     z[e] = on ? gv[e] : 0.f;
-                    bt[e] = on ? gb.y : 0.f;
-                    et[e] = p.scale * __expf(Gi - gb.x);
+                    bt[e] = on ? beta_s[id] : 0.f;
+                    gl[e] = on ? g_s[id] : 0.f;
                 }
             }
             const int dmax = __reduce_max_sync(0xffffffffu, d);
@@ -617,6 +617,17 @@ __global__ void __launch_bounds__(VP_THREADS, 2) verify_plain_kernel(const __gri
                         for (int e = 0; e < 4; ++e)
                             if (sq * 4 + e < l) z[e] = fmaf(-wl, xv[e], z[e]);
                     }
+                }
+            }
+            // (sums over just those nodes: G_i - G would lose the weak decays behind a strong one, and alpha = 0)
+            {
+                const float all = (gl[0] + gl[1]) + (gl[2] + gl[3]), next = __shfl_xor_sync(0xffffffffu, all, 1);
+                const float other = __shfl_xor_sync(0xffffffffu, all + next, 2);
+                float behind = ((sq & 1) ? 0.f : next) + ((sq & 2) ? 0.f : other);
+#pragma unroll
+                for (int e = 3; e >= 0; --e) {
+                    et[e] = p.scale * __expf(behind);
+                    behind += gl[e];
                 }
             }
             // (3) -sa w and z' into their operand tiles (zero off the root path)

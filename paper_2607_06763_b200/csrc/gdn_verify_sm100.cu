@@ -55,7 +55,7 @@ constexpr int SM_Z_LO = 57344;                   // Z lo
 constexpr int SM_X = 98304;                      // fp32 [64][16]  X(i, t-th path node)
 constexpr int SM_Y = SM_X + 4096;                // fp32 [64][16]  Y(i, t-th path node), node itself included
 constexpr int SM_ANC = SM_Y + 4096;              // u8   [64][16]  root-path node ids (0xFF = unused)
-constexpr int SM_GAB = SM_ANC + 1024;            // float4 [64]: (G_i = log a_i, a_i, beta_i, g_i)
+constexpr int SM_GAB = SM_ANC + 1024;            // float4 [64]: (., a_i, beta_i, g_i)
 constexpr int SM_DEPTH = SM_GAB + 1024;          // u8 [64] (0 beyond T)
 constexpr int SM_PATH = SM_DEPTH + FV_T;         // fused commit, two slots of 384 B: int [16] path node ids, int length (0 = no
                                                  // replay), int first node of the tree; at +128 float4 [16] (A_t = decay of the
@@ -412,22 +412,22 @@ __global__ void __launch_bounds__(FV_THREADS, 2) commit_verify_kernel(const __gr
             ab[tid] = make_float4(A, gate_beta(pbe[n * p.h_v + uh], PADDED && p.raw_gates), expf(gt), 1.f / A);
         }
     };
-    // G_i = sum of g along the root path (root first), a_i = exp(G_i), for the tables in buffer `tb`
+    // a_i = exp(sum of g along the root path), and for every path node the sum of g behind it, down to node i, in the place of
+    // its Y (free by now; a difference of two sums from the root would lose the weak decays behind a strong one, and alpha = 0),
+    // for the tables in buffer `tb`
     auto path_decay = [&](int tb) {   // four threads per node, four path positions each
         float4 *gab_t = reinterpret_cast<float4 *>(smem + SM_GAB + tb * SM_TABLE_STRIDE);
         const int i = tid >> 2, s4 = tid & 3;
         const int d = (smem + SM_DEPTH + tb * SM_TABLE_STRIDE)[i];
         const uint32_t ids = *reinterpret_cast<const uint32_t *>(smem + SM_ANC + tb * SM_TABLE_STRIDE + i * FV_MD + s4 * 4);
-        float G = 0.f;
+        float gl[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-            if (s4 * 4 + e < d) G += gab_t[(ids >> (8 * e)) & 0xFFu].w;
-        G += __shfl_xor_sync(0xffffffffu, G, 1);
-        G += __shfl_xor_sync(0xffffffffu, G, 2);
-        if (s4 == 0) {
-            gab_t[i].x = G;
-            gab_t[i].y = d ? __expf(G) : 0.f;
-        }
+        for (int e = 0; e < 4; ++e) gl[e] = s4 * 4 + e < d ? gab_t[(ids >> (8 * e)) & 0xFFu].w : 0.f;
+        const float all = (gl[0] + gl[1]) + (gl[2] + gl[3]), next = __shfl_xor_sync(0xffffffffu, all, 1);
+        const float other = __shfl_xor_sync(0xffffffffu, all + next, 2);
+        const float b3 = ((s4 & 1) ? 0.f : next) + ((s4 & 2) ? 0.f : other), b2 = b3 + gl[3], b1 = b2 + gl[2], b0 = b1 + gl[1];
+        *reinterpret_cast<float4 *>(ys + i * FV_MD + s4 * 4) = make_float4(b0, b1, b2, b3);
+        if (s4 == 0) gab_t[i].y = d ? __expf(all + next + other) : 0.f;
     };
     // Gram = [k;q].k^T of the tile in the k/q operand area, into TMEM columns 192..255, which nothing else uses:
     // issued by one thread as soon as the tile has landed, one unit ahead of its use.
@@ -553,7 +553,7 @@ __global__ void __launch_bounds__(FV_THREADS, 2) commit_verify_kernel(const __gr
         tc_fence_before();
         __syncthreads();
         warm_l2_state(1);
-        // X and Y for real ancestors only; the decay ratio a_i / a_j is exp(G_i - G_j)
+        // X and Y for real ancestors only; the decay from node j down to node i is the exponential of what stands in Y's place
         // (SMALL: nodes 32.. do not exist; their rows of X and Y are never looked at)
         {
             constexpr int NU = SMALL ? 2 : 4;
@@ -567,9 +567,8 @@ __global__ void __launch_bounds__(FV_THREADS, 2) commit_verify_kernel(const __gr
                 on[u] = t < d;
                 onx[u] = t < d - 1;
                 const int j = on[u] ? anc_s[idx] : 0;
-                const float4 gi = gab[i];
-                gdiff[u] = gi.x - gab[j].x;
-                bi[u] = gi.z;
+                gdiff[u] = ys[idx];
+                bi[u] = gab[i].z;
                 const int jpos = (((j >> 2) ^ (i & 15)) << 2) | (j & 3);   // rows i and 64 + i share i & 15
                 gq[u] = gram[(64 + i) * 64 + jpos];   // row 64 + i: q_i
                 gk[u] = gram[i * 64 + jpos];          // row i: k_i

@@ -751,6 +751,30 @@ def test_commit_behind_a_strong_decay(tl, slots, g_strong, at):
     tl.assert_state_close(dc.S0.cpu().numpy().astype(np.float64), tl.oracle_commit(w), what=f"commit behind g = {g_strong}")
 
 
+@pytest.mark.parametrize("at", [0, 2])
+@pytest.mark.parametrize("g_strong", [-3000.0, -30000.0, -np.inf])
+@pytest.mark.parametrize("kind,slots,T", [("verify", 2, 60), ("verify", 2, 200), ("fused", 2, 60), ("fused", 20, 60),
+                                          ("fused", 2, 200)])
+def test_verify_behind_a_strong_decay(tl, kind, slots, T, g_strong, at):
+    """The same for the verification, alone and fused, of trees within one tile and of larger ones: node `at` of every tree
+    has the strong decay, and the outputs of the nodes below it keep their precision."""
+    import paper_2607_06763_b200 as gdn
+    rng = np.random.default_rng(49)
+    trees = [synth.tree_geo(rng, T) if i % 2 else synth.tree_bestfirst(rng, T, concentration=0.1) for i in range(slots)]
+    w = synth.random_case(50, trees, 2, 4, 128, 128, synth.BF16, synth.F32, paths=[np.zeros(0, np.int32)] * slots)
+    w.g[:] = synth.f32_to_bf16_bits(np.float32([-0.0101]))[0]
+    w.g[at::T] = synth.f32_to_bf16_bits(np.float32([g_strong]))[0]
+    dc = tl.DeviceCase(w)
+    if kind == "verify":
+        assert dc.verify() == 0
+    else:
+        assert gdn.gdn_tree_commit_verify(dc.shape, dc.S0, dc.k, dc.v, dc.g, dc.beta, dc.parent, dc.node_offsets, dc.path,
+                                          dc.path_offsets, dc.q, dc.k, dc.v, dc.g, dc.beta, dc.parent, dc.node_offsets, dc.o,
+                                          dc.ws, dc.ws_bytes, dc.status) == 0
+    assert dc.device_status() == 0
+    tl.assert_close_per_head(dc.o_host(), tl.oracle_verify(w), w.node_offsets, f"{kind} behind g = {g_strong}")
+
+
 @pytest.mark.parametrize("slots", [1, 18, 19])
 def test_fused_step_on_both_sides_of_the_two_kernel_rule(tl, slots):
     """4 heads per slot: 72 units run as two kernels, 76 as one (148 SMs).  Every input is overwritten by the kernels right
