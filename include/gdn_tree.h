@@ -45,7 +45,11 @@
  *                               parent[i] < i (topological numbering, Section 3.4.1)
  *       node_offsets[n_seq+1] int32, node_offsets[0] = 0 (ragged packing of trees)
  *     Value head h uses key head h / (h_v / h_qk).  L2-normalising q and k
- *     and the gate activations are the caller's business.
+ *     and the gate activations are the caller's business.  Keys of another
+ *     length are taken too, as long as the weights of the undecayed delta
+ *     rule along a root path stay within fp32: they grow by at most
+ *     max(1, beta |k|^2 - 1) from node to node, so that beta |k|^2 <= 128 is
+ *     safe for paths of 16 nodes whatever the keys and decays.
  */
 #ifndef GDN_TREE_H_
 #define GDN_TREE_H_

@@ -775,13 +775,41 @@ def test_verify_behind_a_strong_decay(tl, kind, slots, T, g_strong, at):
     tl.assert_close_per_head(dc.o_host(), tl.oracle_verify(w), w.node_offsets, f"{kind} behind g = {g_strong}")
 
 
-@pytest.mark.parametrize("slots", [1, 18, 19])
-def test_fused_step_on_both_sides_of_the_two_kernel_rule(tl, slots):
-    """4 heads per slot: 72 units run as two kernels, 76 as one (148 SMs).  Every input is overwritten by the kernels right
+@pytest.mark.parametrize("b", [2, 8, 128])
+@pytest.mark.parametrize("kind,slots,T", [("verify", 2, 60), ("verify", 2, 200), ("fused", 20, 60)])
+def test_verify_with_keys_of_any_length(tl, kind, slots, T, b):
+    """Keys that are not normalised: beta |k|^2 = b at every node, nearly parallel, under decays of 1 / (b - 1), so that the state
+    neither grows nor vanishes down a path.  The verification solves without the decays, where a weight grows up to (b - 1)^15
+    over 16 nodes: 127^15 = 3.6e31 at the limit that the header names."""
+    import paper_2607_06763_b200 as gdn
+    rng = np.random.default_rng(51)
+    trees = [synth.tree_bestfirst(rng, T, concentration=0.1) for _ in range(slots)]
+    w = synth.random_case(52, trees, 2, 4, 128, 128, synth.BF16, synth.F32, paths=[np.zeros(0, np.int32)] * slots)
+    k = rng.standard_normal((1, 2, 128)) + 0.02 * rng.standard_normal((w.total_nodes, 2, 128))
+    k /= np.linalg.norm(k, axis=-1, keepdims=True)
+    w.k = synth.store(np.float32(k * np.sqrt(2.0 * b)), synth.BF16)
+    w.beta = synth.store(np.full(w.beta.shape, 0.5, np.float32), synth.BF16)
+    w.g = synth.store(np.full(w.g.shape, -np.log(max(b - 1, 1.5)), np.float32), synth.BF16)
+    dc = tl.DeviceCase(w)
+    if kind == "verify":
+        assert dc.verify() == 0
+    else:
+        assert gdn.gdn_tree_commit_verify(dc.shape, dc.S0, dc.k, dc.v, dc.g, dc.beta, dc.parent, dc.node_offsets, dc.path,
+                                          dc.path_offsets, dc.q, dc.k, dc.v, dc.g, dc.beta, dc.parent, dc.node_offsets, dc.o,
+                                          dc.ws, dc.ws_bytes, dc.status) == 0
+    assert dc.device_status() == 0
+    tl.assert_close_per_head(dc.o_host(), tl.oracle_verify(w), w.node_offsets, f"{kind}, beta |k|^2 = {b}")
+
+
+@pytest.mark.parametrize("side", ["one_slot", "last_as_two_kernels", "first_as_one"])
+def test_fused_step_on_both_sides_of_the_two_kernel_rule(tl, side):
+    """4 heads per slot: as many units as half the SMs run as two kernels, one slot more as one.  Every input is overwritten by the kernels right
     in front of the call, three times over; slot 0 has an empty new tree, the last slots a rejected and an empty path."""
     import torch
     import paper_2607_06763_b200 as gdn
     from oracle import gdn_oracle as orc
+    half = torch.cuda.get_device_properties(0).multi_processor_count // 2
+    slots = {"one_slot": 1, "last_as_two_kernels": half // 4, "first_as_one": half // 4 + 1}[side]
     rng = np.random.default_rng(53)
     sizes = [0] + [1 + (7 * i) % 64 for i in range(1, slots)]
     trees = [synth.tree_geo(rng, T) if T > 1 else np.full(T, -1, np.int32) for T in sizes]
