@@ -195,9 +195,11 @@ __global__ void __launch_bounds__(CM_THREADS, 2) commit_generic_kernel(const Com
 //     with the carve-out of launch_overlapped: 14.5 without); at 64 tiles the pair gets slower (11.7 / 13.2 -> 12.7 / 13.4);
 //   as matrix products (commit_fragment_unit, gdn_fragments.cuh): 32 state registers, the tile read twice, the second time
 //     out of L2; three or four CTAs per SM, so that the loads of some run under the arithmetic of others.
-// Measured (us; 32 heads per slot, path of 7; two by two / three / four per SM): 4 slots 8.2 / 8.9 / 9.3, 8 slots 10.6 /
-// 13.3 / 12.7, 12 slots 16.6 / 13.4 / 16.0, 14 slots 18.4 / 18.4 / 16.6, 32 slots 36.2 / 33.9 / 31.1, 48 slots 49.5 /
-// 45.8 / 43.0 (path of 12: 56.8 / 50.7 / 49.1; HBM alone: 31).
+// Measured (us; 32 heads per slot, path of 7; two by two / three / four per SM): 4 slots 6.5 / 6.9 / 7.2, 8 slots 9.8 / 11.4 /
+// 10.3, 12 slots 15.4 / 12.9 / 14.7, 14 slots 17.2 / 17.9 / 16.0, 32 slots 33.2 / 31.2 / 29.5, 48 slots 46.9 / 43.1 / 40.6 (path of
+// 1: 37.7 / 39.9 / 38.0, of 12: 57.4 / 52.2 / 54.3, of 16: 64.2 / 54.0 / 55.7; HBM alone: 31).
+// Error of the state against 64 bits, in the norm, step by step / as matrix products: path of 1 5.5e-8 / 4.5e-8, of 7 6.7e-8 /
+// 6.2e-8, of 16 6.6e-8 / 6.3e-8.
 constexpr int CF_THREADS = 256;
 constexpr int CF_MD = 16;
 
@@ -320,6 +322,39 @@ template <int PARTS> __device__ __forceinline__ void commit_replay_unit(const Co
     }
 }
 
+// The two passes of the tile through the registers (all threads; a barrier in between, for the coupling table).  x: chunks 0, 1.
+template <int TILES>
+__device__ __forceinline__ void commit_tile_passes(float *S, float (&x)[2][4][4], int len, uint32_t operand, const PathTile &path, int row,
+                                                   int lane, const float &decay_s)
+{
+    PathUpdate<TILES> up;
+    {
+        PathProducts<TILES> a;
+#pragma unroll
+        for (int i = 0; i < TILES; ++i)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) a.z[i][e] = a.rest[i][e] = 0.f;
+#pragma unroll 1
+        for (int j = 0; j < 4; j += 2)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                path_products_chunk(x[i], j + i, operand, a);
+                load_chunk(S, (j + i + 2) & 3, x[i]);   // (the first two again, for the update)
+            }
+        __syncthreads();   // the coupling table
+        path_solve(a, len, path, row, lane, up);
+    }
+    const float A_L = decay_s;
+#pragma unroll 1
+    for (int j = 0; j < 4; j += 2)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            path_update_chunk(x[i], j + i, operand, A_L, up);
+            store_chunk(S, j + i, x[i]);
+            if (j == 0) load_chunk(S, i + 2, x[i]);
+        }
+}
+
 __device__ __forceinline__ void commit_fragment_unit(const CommitParams &p, const int unit)
 {
     __shared__ __align__(16) uint8_t pk_s[CF_MD * GDN_PK_STRIDE];
@@ -417,35 +452,10 @@ __device__ __forceinline__ void commit_fragment_unit(const CommitParams &p, cons
     __syncthreads();
     len = len_s;
     if (len == 0) return;   // rejected path: this state stays as it was
-    const bool two = len > 8;
-    const uint32_t operand = path_operand(pk, lane);
     if (warp == 0 && len > 1) path_coupling(pk, len, gt, be, couple_s, lane);
-    PathUpdate up;
-    {
-        PathProducts a;
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) a.z[i][e] = a.rest[i][e] = 0.f;
-#pragma unroll 1
-        for (int j = 0; j < 4; j += 2)
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                path_products_chunk(x[i], j + i, two, operand, a);
-                load_chunk(S, (j + i + 2) & 3, x[i]);   // (the first two again, for the update)
-            }
-        __syncthreads();   // the coupling table
-        path_solve(a, len, PathTile{pv_s, scal_s, couple_s}, row, lane, up);
-    }
-    const float A_L = decay_s;
-#pragma unroll 1
-    for (int j = 0; j < 4; j += 2)
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            path_update_chunk(x[i], j + i, two, operand, A_L, up);
-            store_chunk(S, j + i, x[i]);
-            if (j == 0) load_chunk(S, i + 2, x[i]);
-        }
+    const PathTile path{pv_s, scal_s, couple_s};
+    if (len <= 8) commit_tile_passes<1>(S, x, len, path_operand(pk, lane), path, row, lane, decay_s);
+    else commit_tile_passes<2>(S, x, len, path_operand(pk, lane), path, row, lane, decay_s);
 }
 
 // CTAS: CTAs per SM (1, 2: step by step, 1: a quarter of a tile per CTA; otherwise as matrix products)

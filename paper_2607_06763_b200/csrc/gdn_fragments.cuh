@@ -1,9 +1,9 @@
 // The commit (Eq. 7 along an accepted path, the delayed commit of Section 3.4) on a 128 x 128 fp32 state tile taken
 // through registers as accumulator fragments of the warp-level tensor-core instruction m16n8k16, so that both halves of
 // the work -- the products k_t.s of every step with the old state, and the rank-L update -- are matrix products on the
-// registers as they are.  Against the step-by-step replay (gdn_replay.cuh) the work per tile hardly grows with the length
-// of the path: 0.45 K + 0.09 K per step instead of 0.68 K per step cycles with two tiles per SM (7 steps: 4.0 K against
-// 4.8 K, 16 steps: 6.0 K against 10.5 K), and a tile needs 32 registers per thread instead of 64.
+// registers as they are.  Against the step-by-step replay (gdn_replay.cuh) the work per tile grows little with the length of
+// the path, and a tile needs 32 registers per thread instead of 64, so that four share an SM instead of two: 1536 tiles, path of
+// 1 / 7 / 12 / 16: 38.0 / 40.6 / 54.3 / 55.7 us against 37.7 / 46.9 / 57.4 / 64.2.
 //
 // Thread layout: a warp owns 16 rows (rows = value components, contiguous in memory along the key dimension), taken in
 // four chunks of 32 key positions; lane = 4 g + l4 holds of rows g and g + 8 the key positions 32 jj + 8 l4 + e (e = 0..7)
@@ -97,43 +97,45 @@ struct PathTile {
 // S <- S after L steps (1 <= L <= 16).  With u_t = beta_t (v_t - A_t k_t.S) - sum_{u < t} coupling_ut u_u (the triangular
 // form of Section 3.4.1 on the path alone), S_L = A_L S + sum_t E_t u_t k_t^T; every decay factor is in 0..1 whatever the
 // decays.  The products run on bf16 operands that are exact (k) or three-term splits (S, E u), i.e.
-// at fp32 precision.  The tile passes through the registers twice: once for the products, once for the update.
-struct PathProducts {     // steps 2 l4, 2 l4 + 1 (+ 8 in the second entry) of rows g (entries 0, 1) and g + 8 (2, 3)
-    float z[2][4], rest[2][4];   // the mid and lo terms go to accumulators of their own (shorter chains)
+// at fp32 precision; what is left of an error comes from the tensor core, which cuts off what it adds to an accumulator, and is
+// kept below that of the replay by short sums that meet one another with ordinary roundings (gdn_commit.cu has both errors).
+// The tile passes through the registers twice: once for the products, once for the update.
+// TILES: 8-step tiles of the path, 1 for L <= 8, 2 otherwise (code of their own: 64 registers are few).
+template <int TILES> struct PathProducts {     // steps 2 l4, 2 l4 + 1 (+ 8 in the second entry) of rows g (entries 0, 1) and g + 8 (2, 3)
+    float z[TILES][4], rest[TILES][4];   // the mid and lo terms go to accumulators of their own (shorter chains)
 };
 __device__ __forceinline__ uint32_t path_operand(uint32_t pk, int lane)
 {
     return pk + (uint32_t)(lane & 7) * GDN_PK_STRIDE + (uint32_t)(lane >> 3) * 16;
 }
-__device__ __forceinline__ void path_products_chunk(const float (&x)[4][4], int jj, bool two, uint32_t operand, PathProducts &a)
+template <int TILES>
+__device__ __forceinline__ void path_products_chunk(const float (&x)[4][4], int jj, uint32_t operand, PathProducts<TILES> &a)
 {
-    uint32_t b0[4], b1[4];
-    ldmatrix_x4(operand + jj * 64, b0);
-    if (two) ldmatrix_x4(operand + 8 * GDN_PK_STRIDE + jj * 64, b1);
+    uint32_t b[TILES][4];
+#pragma unroll
+    for (int i = 0; i < TILES; ++i) ldmatrix_x4(operand + i * 8 * GDN_PK_STRIDE + jj * 64, b[i]);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         uint32_t hi[4], mid[4], lo[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) split3_bf16(x[2 * h + (i >> 1)][2 * (i & 1)], x[2 * h + (i >> 1)][2 * (i & 1) + 1], hi[i], mid[i], lo[i]);
-        mma_16816(a.z[0], hi, b0[2 * h], b0[2 * h + 1]);
-        mma_16816(a.rest[0], mid, b0[2 * h], b0[2 * h + 1]);
-        mma_16816(a.rest[0], lo, b0[2 * h], b0[2 * h + 1]);
-        if (two) {
-            mma_16816(a.z[1], hi, b1[2 * h], b1[2 * h + 1]);
-            mma_16816(a.rest[1], mid, b1[2 * h], b1[2 * h + 1]);
-            mma_16816(a.rest[1], lo, b1[2 * h], b1[2 * h + 1]);
+#pragma unroll
+        for (int i = 0; i < TILES; ++i) {
+            mma_16816(a.z[i], hi, b[i][2 * h], b[i][2 * h + 1]);
+            mma_16816(a.rest[i], mid, b[i][2 * h], b[i][2 * h + 1]);
+            mma_16816(a.rest[i], lo, b[i][2 * h], b[i][2 * h + 1]);
         }
     }
 }
 // products -> E_t u_t in three bf16 terms, the other operand of the update.  row: this lane's first row
-struct PathUpdate { uint32_t hi[4], mid[4], lo[4]; };
-__device__ __forceinline__ void path_solve(PathProducts &a, int L, const PathTile &p, int row, int lane, PathUpdate &u)
+template <int TILES> struct PathUpdate { uint32_t hi[2 * TILES], mid[2 * TILES], lo[2 * TILES]; };
+template <int TILES>
+__device__ __forceinline__ void path_solve(PathProducts<TILES> &a, int L, const PathTile &p, int row, int lane, PathUpdate<TILES> &u)
 {
     const int l4 = lane & 3;
-    const bool two = L > 8;   // (warp-uniform)
-    float (&z)[2][4] = a.z;
+    float (&z)[TILES][4] = a.z, (&sum)[TILES][4] = a.rest;
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
+    for (int i = 0; i < TILES; ++i)
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             const int t = 8 * i + 2 * l4 + e;
@@ -143,56 +145,57 @@ __device__ __forceinline__ void path_solve(PathProducts &a, int L, const PathTil
             for (int r = 0; r < 2; ++r) {
                 const float v = on ? __uint_as_float((uint32_t)p.pv[t * GDN_TILE_D + row + 8 * r] << 16) : 0.f;
                 z[i][2 * r + e] = on ? fmaf(-sc.y, z[i][2 * r + e] + a.rest[i][2 * r + e], sc.x * v) : 0.f;
+                sum[i][2 * r + e] = 0.f;
             }
         }
-    // forward substitution: once u_t is final its four lanes subtract its share from the later steps (coupling is zero
-    // for the others)
-#pragma unroll 1
-    for (int t = 0; t < L - 1; ++t) {
-        const int src = (lane & ~3) | ((t & 7) >> 1);
-        const float2 c0 = *reinterpret_cast<const float2 *>(p.coupling + t * 16 + 2 * l4);
-        const float a0 = t & 8 ? z[1][0] : z[0][0], a1 = t & 8 ? z[1][1] : z[0][1];
-        const float a2 = t & 8 ? z[1][2] : z[0][2], a3 = t & 8 ? z[1][3] : z[0][3];
-        const float u0 = __shfl_sync(0xffffffffu, t & 1 ? a1 : a0, src), u1 = __shfl_sync(0xffffffffu, t & 1 ? a3 : a2, src);
-        z[0][0] = fmaf(-c0.x, u0, z[0][0]); z[0][1] = fmaf(-c0.y, u0, z[0][1]);
-        z[0][2] = fmaf(-c0.x, u1, z[0][2]); z[0][3] = fmaf(-c0.y, u1, z[0][3]);
-        if (two) {
-            const float2 c1 = *reinterpret_cast<const float2 *>(p.coupling + t * 16 + 8 + 2 * l4);
-            z[1][0] = fmaf(-c1.x, u0, z[1][0]); z[1][1] = fmaf(-c1.y, u0, z[1][1]);
-            z[1][2] = fmaf(-c1.x, u1, z[1][2]); z[1][3] = fmaf(-c1.y, u1, z[1][3]);
-        }
-    }
+    // forward substitution: once u_t is final its four lanes add its share to the sums that the later steps subtract (coupling
+    // is zero for the others); the sums are much smaller than u, and are rounded as such
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
+    for (int k = 0; k < TILES; ++k)   // steps of tile k, which later ones of it and of the tiles behind it depend on
+#pragma unroll 1
+        for (int t = 8 * k; t < min(L - 1, 8 * k + 8); ++t) {
+            const int src = (lane & ~3) | ((t & 7) >> 1);
+            const bool odd = (t & 1) != 0;
+            const float u0 = __shfl_sync(0xffffffffu, odd ? z[k][1] - sum[k][1] : z[k][0] - sum[k][0], src);
+            const float u1 = __shfl_sync(0xffffffffu, odd ? z[k][3] - sum[k][3] : z[k][2] - sum[k][2], src);
+#pragma unroll
+            for (int i = k; i < TILES; ++i) {
+                const float2 c = *reinterpret_cast<const float2 *>(p.coupling + t * 16 + 8 * i + 2 * l4);
+                sum[i][0] = fmaf(c.x, u0, sum[i][0]); sum[i][1] = fmaf(c.y, u0, sum[i][1]);
+                sum[i][2] = fmaf(c.x, u1, sum[i][2]); sum[i][3] = fmaf(c.y, u1, sum[i][3]);
+            }
+        }
+#pragma unroll
+    for (int i = 0; i < TILES; ++i) {
         const int t = 8 * i + 2 * l4;
         const float e0 = t < L ? p.scal[t].z : 0.f, e1 = t + 1 < L ? p.scal[t + 1].z : 0.f;
-        split3_bf16(t < L ? e0 * z[i][0] : 0.f, t + 1 < L ? e1 * z[i][1] : 0.f, u.hi[2 * i], u.mid[2 * i], u.lo[2 * i]);
-        split3_bf16(t < L ? e0 * z[i][2] : 0.f, t + 1 < L ? e1 * z[i][3] : 0.f, u.hi[2 * i + 1], u.mid[2 * i + 1], u.lo[2 * i + 1]);
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+            split3_bf16(t < L ? e0 * (z[i][2 * r] - sum[i][2 * r]) : 0.f, t + 1 < L ? e1 * (z[i][2 * r + 1] - sum[i][2 * r + 1]) : 0.f,
+                        u.hi[2 * i + r], u.mid[2 * i + r], u.lo[2 * i + r]);
     }
 }
-__device__ __forceinline__ void path_update_chunk(float (&x)[4][4], int jj, bool two, uint32_t operand, float A_L, const PathUpdate &u)
+// x <- A_L x + sum_t (E_t u_t) k_t^T, eight steps at a time.  The products of the hi terms have an accumulator of their own, those
+// of the mid and lo terms another; both meet the state with ordinary roundings, the large one last (the tensor core cuts off
+// what it adds).
+template <int TILES>
+__device__ __forceinline__ void path_update_chunk(float (&x)[4][4], int jj, uint32_t operand, float A_L, const PathUpdate<TILES> &u)
 {
 #pragma unroll
-    for (int n = 0; n < 4; ++n)
+    for (int i = 0; i < TILES; ++i) {
+        uint32_t b[4];
+        ldmatrix_x4_trans(operand + i * 8 * GDN_PK_STRIDE + jj * 64, b);
 #pragma unroll
-        for (int e = 0; e < 4; ++e) x[n][e] *= A_L;
-    uint32_t b0[4], b1[4];
-    ldmatrix_x4_trans(operand + jj * 64, b0);
-    if (two) {
-        ldmatrix_x4_trans(operand + 8 * GDN_PK_STRIDE + jj * 64, b1);
+        for (int q = 0; q < 4; ++q) {
+            float hi[4], rest[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) mma_16816(x[q], u.lo, b0[q], b1[q]);
+            for (int e = 0; e < 4; ++e) hi[e] = rest[e] = 0.f;
+            mma_1688(rest, u.lo[2 * i], u.lo[2 * i + 1], b[q]);
+            mma_1688(hi, u.hi[2 * i], u.hi[2 * i + 1], b[q]);
+            mma_1688(rest, u.mid[2 * i], u.mid[2 * i + 1], b[q]);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) mma_16816(x[q], u.mid, b0[q], b1[q]);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) mma_16816(x[q], u.hi, b0[q], b1[q]);
-    } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) mma_1688(x[q], u.lo[0], u.lo[1], b0[q]);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) mma_1688(x[q], u.mid[0], u.mid[1], b0[q]);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) mma_1688(x[q], u.hi[0], u.hi[1], b0[q]);
+            for (int e = 0; e < 4; ++e) x[q][e] = hi[e] + (i == 0 ? fmaf(A_L, x[q][e], rest[e]) : x[q][e] + rest[e]);
+        }
     }
 }
 
