@@ -405,14 +405,18 @@ __global__ void __launch_bounds__(VS_THREADS, 2) verify_generic_small_kernel(con
             stage_rows(sm.qp[buf ^ 1], q_head + (i0 + VS_NODES) * q_stride, q_stride, min(VS_NODES, i_hi - i0 - VS_NODES), d_k, tid);
 
         // z by back-substitution: 16 lanes per node, lane ln owning the entries ln, ln + 16, ... ; once z_j is final it is
-        // subtracted, times X(up_j, .), from the entries further up
+        // added, times X(up_j, .), to what the entries further up subtract (sums of their own: they are smaller than z, and are
+        // rounded as such)
         {
             const int i = tid >> 4, ln = tid & 15, n = i0 + i;
             const int d = i < nn ? sm.depth[n] : 0;
             const int d_warp = __reduce_max_sync(0xffffffffu, d);
-            float z[VS_TREE / 16];
+            float z[VS_TREE / 16], sub[VS_TREE / 16];
 #pragma unroll
-            for (int e = 0; e < VS_TREE / 16; ++e) z[e] = ln + 16 * e < d ? sm.y[i][ln + 16 * e] : 0.f;
+            for (int e = 0; e < VS_TREE / 16; ++e) {
+                z[e] = ln + 16 * e < d ? sm.y[i][ln + 16 * e] : 0.f;
+                sub[e] = 0.f;
+            }
 #pragma unroll
             for (int e = 0; e < VS_TREE / 16; ++e) {
                 if (16 * e >= d_warp - 1) break;
@@ -420,13 +424,13 @@ __global__ void __launch_bounds__(VS_THREADS, 2) verify_generic_small_kernel(con
                 for (int l = 0; l < 16; ++l) {
                     const int j = 16 * e + l;
                     if (j >= d_warp - 1) break;
-                    const float zj = __shfl_sync(0xffffffffu, z[e], (lane & 16) | l);
+                    const float zj = __shfl_sync(0xffffffffu, z[e] - sub[e], (lane & 16) | l);
                     if (j < d - 1) {
                         const float *xr = sm.x[sm.up[n][j]];
 #pragma unroll
                         for (int f = e; f < VS_TREE / 16; ++f) {
                             const int t = ln + 16 * f;
-                            if (t > j && t < d) z[f] = fmaf(-zj, xr[t - j], z[f]);
+                            if (t > j && t < d) sub[f] = fmaf(zj, xr[t - j], sub[f]);
                         }
                     }
                 }
@@ -436,7 +440,7 @@ __global__ void __launch_bounds__(VS_THREADS, 2) verify_generic_small_kernel(con
                 const int t = ln + 16 * e;
                 if (t < d) {
                     const int m = sm.up[n][t];
-                    const float w = p.scale * z[e] * sm.beta[m];
+                    const float w = p.scale * (z[e] - sub[e]) * sm.beta[m];
                     sm.y[i][VS_TREE + t] = w;
                     sm.y[i][t] = w * sm.a[m];
                 }
@@ -453,16 +457,10 @@ __global__ void __launch_bounds__(VS_THREADS, 2) verify_generic_small_kernel(con
                 const float sa = p.scale * sm.a[n];
                 float4 w[2], ov[2];
 #pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    const int r = half * 64 + ln * 4;
-                    w[half] = ov[half] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (r < d_k) {
-                        const float4 x = *reinterpret_cast<const float4 *>(&sm.qp[buf][i][r]);
-                        w[half] = make_float4(sa * x.x, sa * x.y, sa * x.z, sa * x.w);
-                    }
-                }
+                for (int half = 0; half < 2; ++half) w[half] = ov[half] = make_float4(0.f, 0.f, 0.f, 0.f);
+                // (from the root down, q last: the large terms come last)
 #pragma unroll 2
-                for (int t = 0; t < d; ++t) {
+                for (int t = d - 1; t >= 0; --t) {
                     const float cf = -sm.y[i][t], cv = sm.y[i][VS_TREE + t];
                     const int m = sm.up[n][t];
                     const float *kr = sm.ks[m], *vr = sm.vs[m];
@@ -477,6 +475,15 @@ __global__ void __launch_bounds__(VS_THREADS, 2) verify_generic_small_kernel(con
                         const float4 vt = *reinterpret_cast<const float4 *>(&vr[r]);   // (components beyond d_v are not stored)
                         ov[half] = make_float4(fmaf(cv, vt.x, ov[half].x), fmaf(cv, vt.y, ov[half].y), fmaf(cv, vt.z, ov[half].z),
                                                fmaf(cv, vt.w, ov[half].w));
+                    }
+                }
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    const int r = half * 64 + ln * 4;
+                    if (r < d_k) {
+                        const float4 x = *reinterpret_cast<const float4 *>(&sm.qp[buf][i][r]);
+                        w[half] = make_float4(fmaf(sa, x.x, w[half].x), fmaf(sa, x.y, w[half].y), fmaf(sa, x.z, w[half].z),
+                                              fmaf(sa, x.w, w[half].w));
                     }
                 }
                 __syncwarp(0xffffu << (lane & 16));   // the node's weights have been read

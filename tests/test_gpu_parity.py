@@ -131,6 +131,17 @@ def test_verify_shares_rows_and_state_between_units(tl, sizes, out_dtype):
     _check_full(tl, w, f"sizes {sizes}")
 
 
+@pytest.mark.parametrize("in_dtype,d,bound", [(synth.F32, 128, 1.05e-7), (synth.F32, 64, 0.95e-7), (synth.BF16, 64, 0.75e-7)])
+def test_general_path_is_as_exact_on_small_trees_as_on_large_ones(tl, in_dtype, d, bound):
+    """Deep trees of at most 64 nodes (the solve on the query side) against 64 bits: no further off than the node-by-node form that
+    larger trees take (0.97e-7, 0.91e-7, 0.68e-7 here), i.e. fp32 rounding of the last sums and little more."""
+    w = synth.random_case(71, [synth.tree_chain(40)] * 8, 4, 16, d, d, in_dtype, synth.F32, paths=[np.zeros(0, np.int32)] * 8)
+    dc = tl.DeviceCase(w, max_depth=64)
+    assert dc.verify() == 0 and dc.device_status() == 0
+    ref = tl.oracle_verify(w)
+    assert np.sqrt(((dc.o_host() - ref) ** 2).sum() / (ref ** 2).sum()) < bound
+
+
 def test_deep_chain_needs_larger_max_depth(tl):
     w = synth.random_case(5, [synth.tree_chain(40)], 1, 2, 64, 64, synth.F32, synth.F32,
                           paths=[np.arange(40, dtype=np.int32)])
