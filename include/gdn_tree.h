@@ -129,7 +129,7 @@ int gdn_tree_validate_host(const gdn_shape_t *shape, const int32_t *parent_h,
  *   S0, q, k, v, g, beta, parent, node_offsets : [device], read-only
  *   o            : [device], written for every node of every valid tree
  *   workspace    : [device], >= gdn_tree_workspace_bytes(shape) bytes, 256-byte aligned;
- *                  contents after the call: the tree metadata and u~ (reused by nothing else)
+ *                  contents after the call: whatever the kernels of this shape left there
  *   status_dev   : [device] one int32, see "Return value" above
  */
 int gdn_tree_verify(const gdn_shape_t *shape, const float *S0, const void *q, const void *k,

@@ -15,10 +15,11 @@ namespace gdn {
 
 // Layout of the caller-provided verify workspace (all offsets 256-byte aligned).
 //   tree_ok  int32 [n_seq]                 1 = tree passed the metadata checks
-//   depth    uint8 [N]                     nodes on the root path of node n (root = 1)
+//   depth    uint8 [N]                     nodes on the root path of node n (root = 1); read by the general kernel
 //   anc      uint16[N][max_depth]          local ids of the root path of n, root first, n itself last
 //   anc8     uint8 [N][16]                 the same list as bytes (filled when max_depth <= 16 and the
-//                                          tree has <= 256 nodes; unused entries are 0xFF)
+//                                          tree has <= 256 nodes; unused entries are 0xFF); read for trees of at most 64
+//                                          nodes in a grouped call
 // Grouped verification of trees with more than 64 nodes (filled when max_depth <= 16 and the tree has at
 // most GDN_GROUPED_MAX_NODES nodes).  "Position" = index in the depth-first pre-order of the tree (children
 // by increasing id).  The positions are cut into consecutive groups; a group together with the proper
@@ -27,7 +28,8 @@ namespace gdn {
 // group for the group's own nodes.  A group takes as many positions as the 64-node tile leaves after its prefix
 // (64 - n_prefix, i.e. at least GDN_GROUP_MIN_NODES).
 //   group_start uint16[n_seq][GDN_MAX_GROUPS + 1]  first position of group k of tree b; entries behind the
-//                                          last group hold the tree's size
+//                                          last group hold the tree's size (the unit list has what the kernels
+//                                          need of it: nothing reads it now, nor dfs_depth)
 //   unit_count int32 [2]                   number of groups over all trees (zeroed in front of the plan kernel), and
 //                                          a word that says for which shape the plan was built (plan_magic)
 //   unit_list uint32[..][4]                one record per group, the groups of a tree next to one another, the trees

@@ -94,9 +94,8 @@ struct VerifyPlainParams {
     // grouped verification of trees with more than 64 nodes (only read by the GROUPED instantiation)
     int groups_per_tree, anc_stride;                   // upper bound of the groups of a tree (sizes the grid); entries
                                                        // per row of anc16
-    const uint8_t *depth, *anc8;
+    const uint8_t *anc8, *dfs_anc8;
     const uint16_t *anc16, *dfs_node;
-    const uint8_t *dfs_depth, *dfs_anc8;
     const uint4 *unit_list;                            // one record per group (see the workspace layout)
     const int32_t *unit_count;                         // [0] records in the list, [1] plan_magic of the plan's shape
     int unit_capacity, plan_magic;                     // what the list can hold; what [1] has to read
@@ -939,8 +938,8 @@ VerifyPlainParams make_params(const gdn_shape_t &s, const float *S0, const void 
     // upper bound of the groups of a tree (the real ones are in the plan's unit list)
     p.groups_per_tree = s.max_tree_nodes <= VP_T ? 1 : (s.max_tree_nodes + GDN_GROUP_MIN_NODES - 1) / GDN_GROUP_MIN_NODES;
     p.anc_stride = s.max_depth;
-    p.depth = plan.depth; p.anc8 = plan.anc8;
-    p.anc16 = plan.anc; p.dfs_node = plan.dfs_node; p.dfs_depth = plan.dfs_depth; p.dfs_anc8 = plan.dfs_anc8;
+    p.anc8 = plan.anc8; p.dfs_anc8 = plan.dfs_anc8;
+    p.anc16 = plan.anc; p.dfs_node = plan.dfs_node;
     p.unit_list = plan.unit_list;
     p.unit_count = plan.unit_count;
     p.unit_capacity = (int)unit_list_capacity(s);
