@@ -5,7 +5,7 @@ import sys
 
 import numpy as np
 
-sys.path.insert(0, os.environ.get("GDN_ROOT", os.path.dirname(os.path.dirname(os.path.abspath(__file__)))))
+sys.path.insert(0, os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
 import paper_2607_06763_b200 as gdn  # noqa: E402
 from oracle import gdn_oracle as orc  # noqa: E402
 from paper_2607_06763_b200 import synth  # noqa: E402
