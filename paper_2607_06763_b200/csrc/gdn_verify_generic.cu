@@ -552,13 +552,17 @@ cudaError_t launch_small_typed(VerifySmallParams p, cudaStream_t stream, LaunchI
     if (e == cudaSuccess && commit) e = commit();
     if (e != cudaSuccess) return e;
     // Blocks per CTA: as few as let all CTAs be resident at once, so that small calls spread over the SMs; a CTA reads rows
-    // and state once for all of its blocks.  No more than three: a fourth leaves the largest trees as the tail of the call,
-    // as CTAs of their own the last blocks fill in behind the small trees (8 trees of 10..54 nodes, 32 heads, fp32; 1 / 2 / 3 /
-    // 4 blocks per CTA: 35.0 / 34.8 / 29.4 / 34.4 us).
+    // and state once for all of its blocks.  A batch of mixed sizes (mean below two thirds of the largest) stops at three: the last
+    // blocks of its few large trees, as CTAs of their own, fill in behind the small trees.  32 heads of 128 components, fp32, 3 / 4
+    // blocks per CTA (us): 8 trees of 10..54 nodes 29.1 / 33.5, of 28..61 28.6 / 32.3, 8 more of 9..64 28.4 / 34.7, 12 of 9..64 43.0 /
+    // 41.3, 32 of 16..64 111.9 / 104.1; but 8 trees of 64 nodes 49.6 / 38.4, of 50..64 49.5 / 37.1, 9 of 64 53.0 / 38.5, 16 of 64
+    // 85.1 / 76.1.
     const int blocks = (p.max_tree_nodes + VS_NODES - 1) / VS_NODES;
     const long long heads = (long long)p.n_seq * p.h_v;
+    const bool mixed = 3LL * p.total_nodes < 2LL * p.max_tree_nodes * p.n_seq;
+    const int most = mixed ? min(blocks, 3) : blocks;
     int per = 1;
-    while (per < min(blocks, 3) && heads * ((blocks + per - 1) / per) > 2 * sms) ++per;
+    while (per < most && heads * ((blocks + per - 1) / per) > 2 * sms) ++per;
     p.part_nodes = per * VS_NODES;
     p.n_parts = (blocks + per - 1) / per;
     const long long grid = heads * p.n_parts;

@@ -131,6 +131,15 @@ def test_verify_shares_rows_and_state_between_units(tl, sizes, out_dtype):
     _check_full(tl, w, f"sizes {sizes}")
 
 
+@pytest.mark.parametrize("sizes", [(64,) * 8, (64, 17, 33, 9, 40, 16, 5, 1), (64, 50, 33, 60, 48) * 3])
+def test_general_path_blocks_per_cta(tl, sizes):
+    """32 heads: trees of one size (four blocks of nodes per CTA), mixed ones (three and one), and more of them than are resident."""
+    rng = np.random.default_rng(72)
+    trees = [synth.tree_geo(rng, T) if T > 1 else np.full(1, -1, np.int32) for T in sizes]
+    w = synth.random_case(73, trees, 4, 32, 32, 32, synth.F32, synth.F32)
+    _check_full(tl, w, f"general path, {len(sizes)} trees")
+
+
 @pytest.mark.parametrize("in_dtype,d,bound", [(synth.F32, 128, 1.05e-7), (synth.F32, 64, 0.95e-7), (synth.BF16, 64, 0.75e-7)])
 def test_general_path_is_as_exact_on_small_trees_as_on_large_ones(tl, in_dtype, d, bound):
     """Deep trees of at most 64 nodes (the solve on the query side) against 64 bits: no further off than the node-by-node form that
