@@ -455,9 +455,13 @@ __global__ void __launch_bounds__(VS_THREADS, 2) verify_generic_small_kernel(con
             if (i < nn) {
                 const int d = sm.depth[n];
                 const float sa = p.scale * sm.a[n];
-                float4 w[2], ov[2];
+                float4 w[2], ov[2], x[2];
 #pragma unroll
-                for (int half = 0; half < 2; ++half) w[half] = ov[half] = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int half = 0; half < 2; ++half) {
+                    const int r = half * 64 + ln * 4;
+                    w[half] = ov[half] = x[half] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (r < d_k) x[half] = *reinterpret_cast<const float4 *>(&sm.qp[buf][i][r]);
+                }
                 // (from the root down, q last: the large terms come last)
 #pragma unroll 2
                 for (int t = d - 1; t >= 0; --t) {
@@ -478,14 +482,9 @@ __global__ void __launch_bounds__(VS_THREADS, 2) verify_generic_small_kernel(con
                     }
                 }
 #pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    const int r = half * 64 + ln * 4;
-                    if (r < d_k) {
-                        const float4 x = *reinterpret_cast<const float4 *>(&sm.qp[buf][i][r]);
-                        w[half] = make_float4(fmaf(sa, x.x, w[half].x), fmaf(sa, x.y, w[half].y), fmaf(sa, x.z, w[half].z),
-                                              fmaf(sa, x.w, w[half].w));
-                    }
-                }
+                for (int half = 0; half < 2; ++half)
+                    w[half] = make_float4(fmaf(sa, x[half].x, w[half].x), fmaf(sa, x[half].y, w[half].y), fmaf(sa, x[half].z, w[half].z),
+                                          fmaf(sa, x[half].w, w[half].w));
                 __syncwarp(0xffffu << (lane & 16));   // the node's weights have been read
 #pragma unroll
                 for (int half = 0; half < 2; ++half) {
