@@ -11,8 +11,7 @@
 // issued before anything else so that the path checks and the row staging run under their latency.  With four lanes per
 // row and one row per thread each k piece served one row only and shared memory bounded the steps: 8 trees, 32 heads of
 // 128 x 128, path of 5, fp32: 14.3 -> 8.6 us.
-#include "gdn_fragments.cuh"
-#include "gdn_internal.cuh"
+#include "gdn_path.cuh"
 #include "gdn_plan.cuh"
 
 namespace gdn {
@@ -24,28 +23,6 @@ constexpr int CM_SPLIT = 8;
 constexpr int CM_ROWS = 4;
 constexpr int CM_DK = GDN_MAX_HEAD_DIM;
 static_assert(CM_THREADS / CM_SPLIT * CM_ROWS == GDN_MAX_HEAD_DIM, "a row of the state for every value component");
-
-struct CommitParams {
-    int h_qk, h_v, d_k, d_v, max_depth;
-    float *S;
-    const void *k, *v, *g, *beta;
-    const int32_t *parent, *node_offsets, *path, *path_offsets;
-    int32_t *status_dev;
-    // padded layout (tile kernel only; t_pad = 0: ragged packing): slot b keeps its rows at b * t_pad and carries
-    // tree b % n_trees, whose parent[] row, node count and accepted path are shared by its slots
-    int t_pad, n_trees, path_stride, raw_gates;
-    const int32_t *n_nodes, *path_len;
-};
-
-// The commit kernels are launched with programmatic stream serialization: a grid may become resident under the tail of
-// the kernel in front of it and waits here before it reads or writes anything; the kernel behind it (a verification that
-// waits for this grid in turn) may be made resident as the last CTAs run.  48 layers of two calls each (121 nodes, 32
-// heads): 994 -> 850 us; verification and commit of 48 slots as two calls: 95.7 -> 92.3 us.
-__device__ __forceinline__ void wait_for_previous_kernel()
-{
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;");
-}
 
 // max_shared: on SMs set up for the most shared memory, so that a verification launched behind can move in beside the grid.
 template <typename... KernelArgs, typename... Args>
@@ -200,19 +177,6 @@ __global__ void __launch_bounds__(CM_THREADS, 2) commit_generic_kernel(const Com
 // 1: 37.7 / 39.9 / 38.0, of 12: 57.4 / 52.2 / 54.3, of 16: 64.2 / 54.0 / 55.7; HBM alone: 31).
 // Error of the state against 64 bits, in the norm, step by step / as matrix products: path of 1 5.5e-8 / 4.5e-8, of 7 6.7e-8 /
 // 6.2e-8, of 16 6.6e-8 / 6.3e-8.
-constexpr int CF_THREADS = 256;
-constexpr int CF_MD = 16;
-
-__device__ __forceinline__ void cf_cp_async_16(uint32_t dst, const void *src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cf_cp_async_4(uint32_t dst, const void *src, bool valid)   // zero-fills where not valid
-{
-    const int n = valid ? 4 : 0;
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
-}
-
 // PARTS: the tile's rows split over that many CTAs.
 template <int PARTS> __device__ __forceinline__ void commit_replay_unit(const CommitParams &p, const int unit, const int part)
 {
@@ -385,68 +349,13 @@ __device__ __forceinline__ void commit_fragment_unit(const CommitParams &p, cons
 
     const int pb = p.t_pad ? b * p.t_pad : p.node_offsets[b];
     const int pT = p.t_pad ? min(p.n_nodes[tree], p.t_pad) : p.node_offsets[b + 1] - pb;
-    const __nv_bfloat16 *k = static_cast<const __nv_bfloat16 *>(p.k), *v = static_cast<const __nv_bfloat16 *>(p.v);
     const bool shape_ok = len > 0 && len <= CF_MD && len <= p.max_depth && pT > 0 && pp0 >= 0;
     const uint32_t pk = (uint32_t)__cvta_generic_to_shared(pk_s);
-    // Every thread reads the path entry whose row piece it fetches (no hand-over through shared memory in front of the
-    // row fetch); an entry outside the tree is skipped here and reported by the check below.  k rows word by word into the
-    // fragment order, zero up to the next multiple of eight rows.
-    if (shape_ok) {
-#pragma unroll 2
-        for (int idx = tid; idx < ((len + 7) & ~7) * 64; idx += CF_THREADS) {
-            const int t = idx >> 6, w = idx & 63;
-            int nt = t < len ? p.path[pp0 + t] : 0;
-            const bool valid = t < len && nt >= 0 && nt < pT;
-            if (!valid) nt = 0;
-            cf_cp_async_4(pk + t * GDN_PK_STRIDE + path_row_word(w), k + ((size_t)(pb + nt) * p.h_qk + hk) * GDN_TILE_D + w * 2, valid);
-        }
-        if (tid < len * 16) {
-            const int t = tid >> 4, c16 = tid & 15, nt = p.path[pp0 + t];
-            if (nt >= 0 && nt < pT)
-                cf_cp_async_16((uint32_t)__cvta_generic_to_shared(pv_s + t * GDN_TILE_D + c16 * 8),
-                               v + ((size_t)(pb + nt) * p.h_v + h) * GDN_TILE_D + c16 * 8);
-        }
-    }
+    if (shape_ok) path_rows_fetch(p, pp0, len, pb, pT, h, hk, pk, pv_s, tid);
     float gt = 0.f, be = 0.f;   // of step `lane` (warp 0)
     if (warp == 0) {
-        // lane t: entry t of the path and that node's parent; the path must be a chain from a root inside the tree
-        const int ppar = p.t_pad ? tree * p.t_pad : pb;   // first entry of the tree in parent[]
-        const bool mine = shape_ok && lane < len;
-        int n = -1, parent_n = -2;
-        if (mine) {
-            n = p.path[pp0 + lane];
-            if (n >= 0 && n < pT) {
-                if (p.parent) parent_n = p.parent[ppar + n];
-                const size_t i = (size_t)(pb + n) * p.h_v + h;
-                gt = gate_log_decay(static_cast<const unsigned short *>(p.g)[i], p.raw_gates != 0);
-                be = gate_beta(static_cast<const unsigned short *>(p.beta)[i], p.raw_gates != 0);
-            }
-        }
-        const int n_up = __shfl_up_sync(0xffffffffu, n, 1);
-        bool bad = false;
-        if (mine) {
-            if (n < 0 || n >= pT) bad = true;
-            else if (p.parent) bad = parent_n != (lane ? n_up : -1);
-            else if (lane && n <= n_up) bad = true;   // without parent[] only the topological order can be checked
-        }
-        if (__any_sync(0xffffffffu, bad) || !shape_ok) {
-            if (lane == 0) report_status(p.status_dev, GDN_ERR_PATH);
-            len = 0;
-        }
-        // sums of g along the path over the lanes (up to and including step t, and behind it), and the per-step scalars
-        float G = gt;
-#pragma unroll
-        for (int off = 1; off < CF_MD; off <<= 1) {
-            const float up = __shfl_up_sync(0xffffffffu, G, off);
-            if (lane >= off) G += up;
-        }
-        const float G_L = __shfl_sync(0xffffffffu, G, max(len - 1, 0));
-        const float behind = DecayWindows(gt).sum(max(len - 1, 0), max(len - 1 - lane, 0));
-        if (lane < len) scal_s[lane] = make_float4(be, be * expf(G), expf(behind), 0.f);
-        if (lane == 0) {
-            len_s = len;
-            decay_s = expf(G_L);
-        }
+        len = path_check_and_scalars(p, pp0, shape_ok ? len : 0, pb, pT, p.t_pad ? tree * p.t_pad : pb, h, lane, gt, be, scal_s, decay_s);
+        if (lane == 0) len_s = len;
     }
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
     __syncthreads();

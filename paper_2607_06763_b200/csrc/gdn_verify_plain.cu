@@ -26,6 +26,7 @@
 // and not the tensor pipe; so the unit has as few instructions and barriers as could be found, two CTAs share an SM and
 // fill each other's waits, and a CTA takes neighbouring units, which have much in common.
 #include "gdn_internal.cuh"
+#include "gdn_path.cuh"
 #include "gdn_replay.cuh"
 #include "gdn_tc.cuh"
 
@@ -947,6 +948,17 @@ VerifyPlainParams make_params(const gdn_shape_t &s, const float *S0, const void 
     return p;
 }
 
+// The state of a verification alone, for the kernel of small trees (which writes it behind a commit only).
+CommitParams state_only(const gdn_shape_t &s, const float *S0, bool raw_gates, int32_t *status_dev)
+{
+    CommitParams c{};
+    c.h_qk = s.h_qk; c.h_v = s.h_v; c.d_k = s.d_k; c.d_v = s.d_v; c.max_depth = s.max_depth;
+    c.S = const_cast<float *>(S0);
+    c.status_dev = status_dev;
+    c.raw_gates = raw_gates ? 1 : 0;
+    return c;
+}
+
 }  // namespace
 
 // Padded layout, trees of at most 64 nodes.
@@ -956,6 +968,9 @@ cudaError_t launch_verify_sm100_padded(const gdn_shape_t &s, int n_trees, bool r
                                        cudaStream_t stream, LaunchInFront commit)
 {
     if (s.n_seq == 0 || s.total_nodes == 0) return cudaSuccess;
+    if (step_small_supported(s))
+        return launch_step_small(s, state_only(s, S0, raw_gates, status_dev), false, q, k, v, g, beta, parent, nullptr, n_trees, n_nodes, o,
+                                 stream, commit);
     VerifyPlainParams p = make_params(s, S0, q, k, v, g, beta, nullptr, o, PlanPtrs{}, status_dev);
     p.parent = parent;
     p.t_pad = s.max_tree_nodes; p.n_trees = n_trees; p.n_nodes = n_nodes; p.raw_gates = raw_gates ? 1 : 0;
@@ -991,6 +1006,9 @@ cudaError_t launch_verify_sm100(const gdn_shape_t &s, const float *S0, const voi
                                 int32_t *status_dev, cudaStream_t stream, LaunchInFront commit)
 {
     if (s.n_seq == 0 || s.total_nodes == 0) return cudaSuccess;
+    if (step_small_supported(s))
+        return launch_step_small(s, state_only(s, S0, false, status_dev), false, q, k, v, g, beta, parent, node_offsets, 1, nullptr, o,
+                                 stream, commit);
     VerifyPlainParams p = make_params(s, S0, q, k, v, g, beta, node_offsets, o, plan, status_dev);
     p.parent = parent;
     if (!verify_sm100_single_group(s)) return launch_plain<true>(s, p, commit, stream);

@@ -27,6 +27,7 @@
 // forms tried for it -- one CTA per SM with specialised warps, the replay as matrix products on the fragments, the commit
 // and verify kernels back to back (86.6 us; 72 against 84 at a path of 1) -- none is faster over the path lengths.
 #include "gdn_internal.cuh"
+#include "gdn_path.cuh"
 #include "gdn_replay.cuh"
 #include "gdn_tc.cuh"
 
@@ -1017,6 +1018,11 @@ cudaError_t launch_commit_verify_sm100_padded(const gdn_shape_t &s, int n_trees,
                                               cudaStream_t stream)
 {
     if (s.n_seq == 0 || s.total_nodes == 0) return cudaSuccess;
+    if (step_small_supported(s)) {
+        const CommitParams prev{s.h_qk, s.h_v, s.d_k, s.d_v, s.max_depth, S, k_prev, v_prev, g_prev, beta_prev, parent_prev, nullptr,
+                                path, nullptr, status_dev, prev_t_pad, n_trees, s.max_depth, raw_gates ? 1 : 0, n_nodes_prev, path_len};
+        return launch_step_small(s, prev, true, q, k, v, g, beta, parent, nullptr, n_trees, n_nodes, o, stream);
+    }
     if (as_two_kernels(s)) {
         gdn_shape_t ps = s;   // the commit reads the slots of the previous step
         ps.max_tree_nodes = prev_t_pad;
@@ -1048,6 +1054,11 @@ cudaError_t launch_commit_verify_sm100(const gdn_shape_t &s, float *S, const voi
                                        cudaStream_t stream)
 {
     if (s.n_seq == 0 || s.total_nodes == 0) return cudaSuccess;
+    if (step_small_supported(s)) {
+        const CommitParams prev{s.h_qk, s.h_v, s.d_k, s.d_v, s.max_depth, S, k_prev, v_prev, g_prev, beta_prev, parent_prev, node_offsets_prev,
+                                path, path_offsets, status_dev, 0, 0, 0, 0, nullptr, nullptr};
+        return launch_step_small(s, prev, true, q, k, v, g, beta, parent, node_offsets, 1, nullptr, o, stream);
+    }
     if (as_two_kernels(s)) {
         const auto commit = [&] {
             return launch_commit_generic(s, S, k_prev, v_prev, g_prev, beta_prev, parent_prev, node_offsets_prev, path,
