@@ -38,7 +38,14 @@ struct StepSmallParams {
 
 // CTAs per SM: what the registers give without spilling more than a few words (N = 16 alone at three instead of four: 36.2 us for
 // 64 chains of 16 nodes instead of 35.0; N = 32 alone at three instead of two: 12.7 us for 8 trees instead of 9.8).
-constexpr int ss_ctas(int n, bool commit) { return n == 16 ? (commit ? 3 : 4) : 2; }
+// A commit at four spills 64 words' worth, which paths of more than 8 nodes pay for (step of 64 chains of 16 nodes, paths of 16 / 7: 91.3 /
+// 80.9 at three, 96.8 / 75.5 at four), so that it runs at four where such paths are not to be expected (trees of at most 8 nodes: 48 of
+// them, path of 7, 61.0 / 57.6) or where that makes one wave of what would be two (16 trees of 16 nodes 27.9 / 23.4), but not where
+// three are enough (12 trees 17.0 / 21.3).
+inline bool commit_at_four(int max_tree_nodes, long long units, int sms)
+{
+    return units > 3LL * sms && (units <= 4LL * sms || max_tree_nodes <= 8);
+}
 
 // N: nodes a tree may have here (16 or 32).
 template <int N> struct StepSmallSmem {
@@ -121,8 +128,9 @@ __device__ __forceinline__ void state_passes(float *S, float (&x)[2][4][4], int 
         }
 }
 
-template <int N, typename TOut, bool COMMIT>
-__global__ void __launch_bounds__(SS_THREADS, ss_ctas(N, COMMIT)) verify_step_small_kernel(const StepSmallParams p)
+// CTAS: per SM.
+template <int N, typename TOut, bool COMMIT, int CTAS>
+__global__ void __launch_bounds__(SS_THREADS, CTAS) verify_step_small_kernel(const StepSmallParams p)
 {
     extern __shared__ __align__(16) uint8_t ss_smem[];
     using Smem = StepSmallSmem<N>;
@@ -411,11 +419,12 @@ __global__ void __launch_bounds__(SS_THREADS, ss_ctas(N, COMMIT)) verify_step_sm
     }
 }
 
-template <int N, typename TOut, bool COMMIT> cudaError_t launch_typed(const StepSmallParams &p, LaunchInFront commit, cudaStream_t stream)
+template <int N, typename TOut, bool COMMIT, int CTAS> cudaError_t launch_kernel(const StepSmallParams &p, LaunchInFront commit, cudaStream_t stream)
 {
     static PerContext seen;
     int sms = 0;
-    cudaError_t e = device_sms(seen, reinterpret_cast<const void *>(verify_step_small_kernel<N, TOut, COMMIT>), sizeof(StepSmallSmem<N>), &sms);
+    const auto kernel = verify_step_small_kernel<N, TOut, COMMIT, CTAS>;
+    cudaError_t e = device_sms(seen, reinterpret_cast<const void *>(kernel), sizeof(StepSmallSmem<N>), &sms);
     if (e == cudaSuccess && commit) e = commit();
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
@@ -428,7 +437,20 @@ template <int N, typename TOut, bool COMMIT> cudaError_t launch_typed(const Step
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, verify_step_small_kernel<N, TOut, COMMIT>, p);
+    return cudaLaunchKernelEx(&cfg, kernel, p);
+}
+
+template <typename TOut> cudaError_t launch_typed(const StepSmallParams &p, bool with_commit, LaunchInFront commit, cudaStream_t stream)
+{
+    if (p.max_tree_nodes > 16)
+        return with_commit ? launch_kernel<32, TOut, true, 2>(p, commit, stream) : launch_kernel<32, TOut, false, 2>(p, commit, stream);
+    if (!with_commit) return launch_kernel<16, TOut, false, 4>(p, commit, stream);
+    static PerContext seen;
+    int sms = 0;
+    const cudaError_t e = device_sms(seen, nullptr, 0, &sms);
+    if (e != cudaSuccess) return e;
+    return commit_at_four(p.max_tree_nodes, (long long)p.n_seq * p.c.h_v, sms) ? launch_kernel<16, TOut, true, 4>(p, commit, stream)
+                                                                               : launch_kernel<16, TOut, true, 3>(p, commit, stream);
 }
 
 }  // namespace
@@ -460,13 +482,7 @@ cudaError_t launch_step_small(const gdn_shape_t &s, const CommitParams &prev, bo
     p.beta = static_cast<const __nv_bfloat16 *>(beta);
     p.parent = parent; p.node_offsets = node_offsets; p.o = o;
     p.t_pad = node_offsets ? 0 : s.max_tree_nodes; p.n_trees = n_trees; p.n_nodes = n_nodes;
-    const bool bf = s.out_dtype == GDN_BF16;
-    if (s.max_tree_nodes <= 16) {
-        if (with_commit) return bf ? launch_typed<16, __nv_bfloat16, true>(p, commit, stream) : launch_typed<16, float, true>(p, commit, stream);
-        return bf ? launch_typed<16, __nv_bfloat16, false>(p, commit, stream) : launch_typed<16, float, false>(p, commit, stream);
-    }
-    if (with_commit) return bf ? launch_typed<32, __nv_bfloat16, true>(p, commit, stream) : launch_typed<32, float, true>(p, commit, stream);
-    return bf ? launch_typed<32, __nv_bfloat16, false>(p, commit, stream) : launch_typed<32, float, false>(p, commit, stream);
+    return s.out_dtype == GDN_BF16 ? launch_typed<__nv_bfloat16>(p, with_commit, commit, stream) : launch_typed<float>(p, with_commit, commit, stream);
 }
 
 }  // namespace gdn

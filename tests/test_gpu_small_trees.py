@@ -10,7 +10,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.fixture(scope="module")
-def tl():
+def tl(cuda_device):
     from tests import gdn_testlib
     return gdn_testlib
 
