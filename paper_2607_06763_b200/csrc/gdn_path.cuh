@@ -111,10 +111,17 @@ __device__ __forceinline__ int path_check_and_scalars(const CommitParams &p, int
 // Trees of at most SS_MAX_NODES nodes on the shapes of the tensor-core path (gdn_step_small.cu): the verification, behind the commit of
 // `prev` in the same pass over the state if with_commit, else on prev.S as it is (of prev only the sizes, raw_gates, S and
 // status_dev count then).  node_offsets == nullptr: padded layout.
+// plan: the padded layout with node counts and root paths out of a plan (no parent, n_nodes), verification alone.
 constexpr int SS_MAX_NODES = 32;
+struct SmallTreePlan {
+    const uint4 *unit_list = nullptr;
+    const int32_t *unit_count = nullptr;   // [0] records in the list, [1] what plan_magic says of the plan's shape
+    const uint8_t *anc8 = nullptr;
+    int capacity = 0, magic = 0;
+};
 bool step_small_supported(const gdn_shape_t &s);
 cudaError_t launch_step_small(const gdn_shape_t &s, const CommitParams &prev, bool with_commit, const void *q, const void *k, const void *v,
                               const void *g, const void *beta, const int32_t *parent, const int32_t *node_offsets, int n_trees,
-                              const int32_t *n_nodes, void *o, cudaStream_t stream, LaunchInFront commit = {});
+                              const int32_t *n_nodes, void *o, cudaStream_t stream, LaunchInFront commit = {}, const SmallTreePlan &plan = {});
 
 }  // namespace gdn

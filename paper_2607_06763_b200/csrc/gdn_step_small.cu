@@ -34,6 +34,8 @@ struct StepSmallParams {
     void *o;
     int t_pad, n_trees;   // padded layout (0: ragged packing): slot b keeps its rows at b * t_pad and carries tree b % n_trees
     const int32_t *n_nodes;
+    // PLANNED: padded layout, node counts and root paths out of a plan of the n_trees trees (unit list, its count and shape mark, paths)
+    SmallTreePlan plan;
 };
 
 // CTAs per SM: what the registers give without spilling more than a few words (N = 16 alone at three instead of four: 36.2 us for
@@ -128,8 +130,8 @@ __device__ __forceinline__ void state_passes(float *S, float (&x)[2][4][4], int 
         }
 }
 
-// CTAS: per SM.
-template <int N, typename TOut, bool COMMIT, int CTAS>
+// CTAS: per SM.  PLANNED: the trees come from a plan.
+template <int N, typename TOut, bool COMMIT, int CTAS, bool PLANNED>
 __global__ void __launch_bounds__(SS_THREADS, CTAS) verify_step_small_kernel(const StepSmallParams p)
 {
     extern __shared__ __align__(16) uint8_t ss_smem[];
@@ -146,7 +148,27 @@ __global__ void __launch_bounds__(SS_THREADS, CTAS) verify_step_small_kernel(con
     const int tree = p.t_pad ? b % p.n_trees : b;
     int base, T;
     bool off_ok;
-    if (p.t_pad) {
+    if (PLANNED) {
+        // a tree of at most 64 nodes has one record, anywhere in the list; a rejected or empty one has none
+        // (48 layers, commit and planned verification each, a tree of 8 / 16 / 32 nodes: 609 / 625 / 646 us with the kernel of grouped
+        // trees, 489 / 497 / 589 so)
+        base = b * p.t_pad;
+        T = 0;
+        const int n_rec = p.plan.unit_count[0];
+        if (p.plan.unit_count[1] != p.plan.magic || n_rec < 0 || n_rec > p.plan.capacity) {   // not a plan of this shape
+            if (tid == 0) report_status(c.status_dev, GDN_ERR_WORKSPACE);
+            return;
+        }
+        for (int r0 = 0; r0 < n_rec; r0 += 32) {
+            const uint4 rec = r0 + lane < n_rec ? p.plan.unit_list[r0 + lane] : make_uint4(0xFFFFFFFFu, 0u, 0u, 0u);
+            const uint32_t found = __ballot_sync(0xffffffffu, rec.x == (uint32_t)tree);
+            if (found) {
+                T = (int)((__shfl_sync(0xffffffffu, rec.z, __ffs(found) - 1) >> 16) & 0xFFu);
+                break;
+            }
+        }
+        off_ok = T <= p.t_pad;
+    } else if (p.t_pad) {
         base = b * p.t_pad;
         T = p.n_nodes[tree];
         off_ok = T >= 0 && T <= p.t_pad;
@@ -207,24 +229,37 @@ __global__ void __launch_bounds__(SS_THREADS, CTAS) verify_step_small_kernel(con
         // lane i: node i.  Ancestor masks by pointer doubling (five rounds cover 32 nodes).
         const bool mine = lane < T;
         const size_t n = (size_t)(base + lane) * c.h_v + h;
-        int up = mine ? p.parent[(p.t_pad ? tree * p.t_pad : base) + lane] : -1;
         const uint32_t g16 = mine ? reinterpret_cast<const unsigned short *>(p.g)[n] : 0u;
         const uint32_t b16 = mine ? reinterpret_cast<const unsigned short *>(p.beta)[n] : 0u;
-        int err = up < -1 || (mine && up >= lane) ? GDN_ERR_TREE : 0;
-        if (err) up = -1;
         uint32_t m = 1u << lane;
+        bool bad = false;
+        if constexpr (PLANNED) {
+            if (mine) {   // the root path as bytes, 0xFF behind its end
+                const uint4 path = *reinterpret_cast<const uint4 *>(p.plan.anc8 + ((size_t)tree * p.t_pad + lane) * 16);
+                const uint32_t w[4] = {path.x, path.y, path.z, path.w};
 #pragma unroll
-        for (int r = 1; r < N; r *= 2) {
-            const uint32_t above = __shfl_sync(0xffffffffu, m, max(up, 0));
-            const int next = __shfl_sync(0xffffffffu, up, max(up, 0));
-            if (up >= 0) {
-                m |= above;
-                up = next;
+                for (int e = 0; e < 16; ++e) {
+                    const uint32_t id = (w[e >> 2] >> (8 * (e & 3))) & 0xFFu;
+                    if (id != 0xFFu) m |= 1u << (id & 31u);
+                }
             }
+        } else {
+            int up = mine ? p.parent[(p.t_pad ? tree * p.t_pad : base) + lane] : -1;
+            int err = up < -1 || (mine && up >= lane) ? GDN_ERR_TREE : 0;
+            if (err) up = -1;
+#pragma unroll
+            for (int r = 1; r < N; r *= 2) {
+                const uint32_t above = __shfl_sync(0xffffffffu, m, max(up, 0));
+                const int next = __shfl_sync(0xffffffffu, up, max(up, 0));
+                if (up >= 0) {
+                    m |= above;
+                    up = next;
+                }
+            }
+            if (mine && !err && __popc(m) > c.max_depth) err = GDN_ERR_DEPTH;
+            if (err) report_status(c.status_dev, err);
+            bad = __any_sync(0xffffffffu, err != 0);
         }
-        if (mine && !err && __popc(m) > c.max_depth) err = GDN_ERR_DEPTH;
-        if (err) report_status(c.status_dev, err);
-        const bool bad = __any_sync(0xffffffffu, err != 0);
         if (lane < N) {
             sm.mask[lane] = mine ? m : 0u;
             sm.g[lane] = gate_log_decay(g16, c.raw_gates != 0);
@@ -419,11 +454,11 @@ __global__ void __launch_bounds__(SS_THREADS, CTAS) verify_step_small_kernel(con
     }
 }
 
-template <int N, typename TOut, bool COMMIT, int CTAS> cudaError_t launch_kernel(const StepSmallParams &p, LaunchInFront commit, cudaStream_t stream)
+template <int N, typename TOut, bool COMMIT, int CTAS, bool PLANNED = false> cudaError_t launch_kernel(const StepSmallParams &p, LaunchInFront commit, cudaStream_t stream)
 {
     static PerContext seen;
     int sms = 0;
-    const auto kernel = verify_step_small_kernel<N, TOut, COMMIT, CTAS>;
+    const auto kernel = verify_step_small_kernel<N, TOut, COMMIT, CTAS, PLANNED>;
     cudaError_t e = device_sms(seen, reinterpret_cast<const void *>(kernel), sizeof(StepSmallSmem<N>), &sms);
     if (e == cudaSuccess && commit) e = commit();
     if (e != cudaSuccess) return e;
@@ -442,6 +477,8 @@ template <int N, typename TOut, bool COMMIT, int CTAS> cudaError_t launch_kernel
 
 template <typename TOut> cudaError_t launch_typed(const StepSmallParams &p, bool with_commit, LaunchInFront commit, cudaStream_t stream)
 {
+    if (p.plan.unit_list)
+        return p.max_tree_nodes > 16 ? launch_kernel<32, TOut, false, 2, true>(p, commit, stream) : launch_kernel<16, TOut, false, 4, true>(p, commit, stream);
     if (p.max_tree_nodes > 16)
         return with_commit ? launch_kernel<32, TOut, true, 2>(p, commit, stream) : launch_kernel<32, TOut, false, 2>(p, commit, stream);
     if (!with_commit) return launch_kernel<16, TOut, false, 4>(p, commit, stream);
@@ -471,7 +508,7 @@ bool step_small_supported(const gdn_shape_t &s)
 
 cudaError_t launch_step_small(const gdn_shape_t &s, const CommitParams &prev, bool with_commit, const void *q, const void *k, const void *v,
                               const void *g, const void *beta, const int32_t *parent, const int32_t *node_offsets, int n_trees,
-                              const int32_t *n_nodes, void *o, cudaStream_t stream, LaunchInFront commit)
+                              const int32_t *n_nodes, void *o, cudaStream_t stream, LaunchInFront commit, const SmallTreePlan &plan)
 {
     if (s.n_seq == 0 || s.total_nodes == 0) return cudaSuccess;
     StepSmallParams p{};
@@ -482,6 +519,7 @@ cudaError_t launch_step_small(const gdn_shape_t &s, const CommitParams &prev, bo
     p.beta = static_cast<const __nv_bfloat16 *>(beta);
     p.parent = parent; p.node_offsets = node_offsets; p.o = o;
     p.t_pad = node_offsets ? 0 : s.max_tree_nodes; p.n_trees = n_trees; p.n_nodes = n_nodes;
+    p.plan = plan;
     return s.out_dtype == GDN_BF16 ? launch_typed<__nv_bfloat16>(p, with_commit, commit, stream) : launch_typed<float>(p, with_commit, commit, stream);
 }
 

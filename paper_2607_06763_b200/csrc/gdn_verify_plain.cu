@@ -982,13 +982,17 @@ cudaError_t launch_verify_sm100_planned(const gdn_shape_t &s, int n_trees, bool 
                                         const PlanPtrs &plan, void *o, int32_t *status_dev, cudaStream_t stream)
 {
     if (s.n_seq == 0 || s.total_nodes == 0) return cudaSuccess;
-    VerifyPlainParams p = make_params(s, S0, q, k, v, g, beta, nullptr, o, plan, status_dev);
-    p.t_pad = s.max_tree_nodes; p.n_trees = n_trees; p.raw_gates = raw_gates ? 1 : 0;
     gdn_shape_t ps = s;   // the shape the plan was built for: n_trees trees of t_pad rows
     ps.n_seq = n_trees;
     ps.total_nodes = n_trees * s.max_tree_nodes;
-    p.unit_capacity = (int)unit_list_capacity(ps);
-    p.plan_magic = plan_magic(n_trees, s.max_tree_nodes, s.max_depth);
+    const int capacity = (int)unit_list_capacity(ps), magic = plan_magic(n_trees, s.max_tree_nodes, s.max_depth);
+    if (step_small_supported(s))
+        return launch_step_small(s, state_only(s, S0, raw_gates, status_dev), false, q, k, v, g, beta, nullptr, nullptr, n_trees, nullptr, o,
+                                 stream, {}, {plan.unit_list, plan.unit_count, plan.anc8, capacity, magic});
+    VerifyPlainParams p = make_params(s, S0, q, k, v, g, beta, nullptr, o, plan, status_dev);
+    p.t_pad = s.max_tree_nodes; p.n_trees = n_trees; p.raw_gates = raw_gates ? 1 : 0;
+    p.unit_capacity = capacity;
+    p.plan_magic = magic;
     return launch_plain<true>(s, p, {}, stream);
 }
 

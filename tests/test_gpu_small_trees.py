@@ -70,3 +70,30 @@ def test_small_trees_are_as_exact_as_large_ones(tl, T):
     assert dc.verify() == 0 and dc.device_status() == 0
     ref = tl.oracle_verify(w)
     assert np.linalg.norm(dc.o_host() - ref) <= 2.0 ** -17 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("raw_gates", [False, True])
+@pytest.mark.parametrize("t_pad,sizes,n_layers,out_dtype", [(1, (1,), 2, synth.BF16), (16, (16, 9), 3, synth.F32), (16, tuple(range(1, 17)) * 3, 1, synth.BF16),
+                                                            (32, (32,), 3, synth.BF16), (31, (17, 31, 2), 2, synth.F32)])
+def test_planned_verification_of_small_trees(tl, t_pad, sizes, n_layers, out_dtype, raw_gates):
+    """Trees found in the plan's list (more than a warp of records among them); an empty tree has none, a plan of another
+    shape is refused on the device."""
+    import torch
+    import paper_2607_06763_b200 as gdn
+    from tests.test_gpu_padded import _plan
+    rng = np.random.default_rng(sum(sizes) + t_pad)
+    w = synth.padded_case(740 + t_pad + len(sizes), [synth.tree_geo(rng, n) for n in sizes], n_layers, t_pad, raw_gates, out_dtype=out_dtype)
+    d = PaddedDevice(w)
+    plan = _plan(d, w)
+    call = lambda plan: gdn.gdn_tree_verify_planned(d.shape, w.n_trees, raw_gates, d.S0, d.q, d.k, d.v, d.g_in, d.beta_in, plan, d.o, d.status)
+    assert call(plan) == 0 and d.status_value() == 0
+    _assert_outputs(tl, d, _oracle_verify(w), f"planned, {t_pad} rows")
+    d.n_nodes[0] = 0
+    plan = _plan(d, w)
+    d.o.fill_(7.0)
+    assert call(plan) == 0 and d.status_value() == 0
+    o = d.o_host()
+    assert np.all(o[:: w.n_trees] == 7.0) and (w.n_trees == 1 or np.any(o[1] != 7.0))
+    d.o.fill_(7.0)
+    assert call(torch.zeros_like(plan)) == 0 and d.status_value() == -10
+    assert np.all(d.o_host() == 7.0)
