@@ -567,6 +567,10 @@ def main():
             sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
             if fused and w.n_seq * w.h_v <= sms // 2:   # few units: commit and verify kernels side by side
                 kernel_name, launches_per_step = "commit_tile128_kernel + verify_plain_kernel", 2
+            largest = int(np.diff(w.node_offsets).max())
+            if largest <= 16 or (largest <= 32 and w.n_seq * w.h_v <= 2 * sms):   # small trees: one kernel of their own
+                kernel_name = "verify_step_small_kernel"
+                launches_per_step = 2 if args.mode == "separate" else 1
             dom_bytes = sbytes if fused else vbytes
             dom_ms = ms_per_step if args.mode != "separate" else split[0]
         else:   # larger trees: tree plan + the verify kernel in its grouped mode; the fused call builds the plan in

@@ -114,7 +114,8 @@ struct VerifyFastParams {
 // and its per-node tables, decay tables and accepted path are fetched in stages, each global load one phase before
 // its value is used.  The state tile is asked for at the top of the unit and is needed only after the Gram /
 // coefficient phases; the v rows land by TMA in an area that is free until the state operand is written.
-// SMALL (every tree of the call has at most 32 nodes, the largest more than 16: gdn_step_small.cu has the others): the R and output phases skip the 16-node pieces beyond the tree.
+// SMALL (every tree of the call has at most 32 nodes, the largest more than 16: gdn_step_small.cu has the others): the R and output
+// phases skip the 16-node pieces beyond the tree.
 template <typename TOut, bool SMALL, bool PADDED>
 __global__ void __launch_bounds__(FV_THREADS, 2) commit_verify_kernel(const __grid_constant__ VerifyFastParams p)
 {
