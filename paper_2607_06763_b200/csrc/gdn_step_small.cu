@@ -12,7 +12,7 @@
 //
 // Measured (us, 32 heads; the kernels of 64-node tiles / this one), trees of 16 nodes: 64 chains, accepted paths of 0 / 1 / 7 / 16
 // nodes 66.5 / 82.2 / 100.6 / 132.5 -> 44.4 / 75.7 / 80.7 / 91.2 (the state read and written once at the copy bandwidth: 41), verification
-// alone 44.6 -> 35.0; 48 geometric trees, paths of 0 / 1 / 7 47.8 / 60.2 / 67.6 -> 33.1 / 59.1 / 62.2; one layer, path of 7 11.4 -> 9.1.
+// alone 44.6 -> 35.0; 48 geometric trees, paths of 0 / 1 / 7 47.8 / 60.2 / 67.6 -> 33.1 / 59.1 / 62.2; one layer, path of 7 11.4 -> 8.2.
 // Error of fp32 outputs against 64 bits, in the norm, 40 trees of 16 nodes: verification 2.9e-6 -> 2.8e-6, step 4.3e-6 -> 2.6e-6 (its
 // state 5.9e-8 -> 5.1e-8).  Bound by HBM latency and the chain of a unit.
 #include "gdn_path.cuh"
@@ -50,24 +50,46 @@ inline bool commit_at_four(int max_tree_nodes, long long units, int sms)
     return units > 3LL * sms && (units <= 4LL * sms || max_tree_nodes <= 8);
 }
 
+// CTAs of a unit behind a commit (PARTS): one, or, while every one of them has an SM of its own, four or two that take 32 or 64 value
+// components each, every warp on the key positions of one or two chunks of its rows, which then stay in its registers.  With the whole
+// tile on one CTA the passes over it are 5300 of a unit's 11300 cycles (path of 1; 7500 behind one of 16), and its second half and both
+// halves once more are waited for; the coefficients, which every CTA makes for itself, are done in less time than the rows take to
+// come.  Calls back to back in a CUDA graph, us, commit and 64-node verification as two kernels / one CTA a unit / split, 32 heads,
+// paths of 1 / 8 / 9 / 16 nodes: one sequence of 16 nodes (four parts) 8.3 8.3 8.3 9.5 / 7.9 8.7 10.2 10.6 / 5.4 6.1 6.9 7.3, of 32 nodes
+// 8.5 8.5 8.5 9.6 / 9.4 9.8 10.8 11.2 / 7.6 7.9 8.7 9.1; two sequences (two parts) 8.6 9.3 9.9 11.9 / 8.0 8.8 10.3 10.8 / 6.3 6.9 7.6 8.1
+// and 9.0 9.4 10.0 11.9 / 9.7 10.1 11.0 11.4 / 9.2 9.5 10.3 10.7 (four parts, two CTAs on most SMs: 6.7 7.5 8.6 9.2 and 9.9 10.6 11.8 12.3).
+// Three sequences in two parts, two on some SMs: 16 nodes 7.9 8.9 9.8 10.4 instead of 8.0 8.8 10.4 10.8, 32 nodes 12.2 12.9 14.2 14.4 instead of
+// 9.7 10.1 11.1 11.5.
+inline int commit_parts(long long units, int sms) { return units <= sms / 4 ? 4 : units <= sms / 2 ? 2 : 1; }
+
 // N: nodes a tree may have here (16 or 32).
-template <int N> struct StepSmallSmem {
+template <int N, int PARTS> struct StepSmallSmem {
     static constexpr int W_ROW = 2 * N + 16;   // bytes from one row of w, z' to the next
     static constexpr int G_ROW = N + 4;        // floats from one row of the Gram block to the next
-    // k, q, v rows (zero beyond the tree); over k and q, once q' is there, the outputs on their way out
+    // k, q, v rows (zero beyond the tree); over k and q, once q' is there, the outputs on their way out (PARTS > 1: the warps' shares of them)
     alignas(16) uint8_t rows[3][N * SS_ROW];
     alignas(16) uint8_t qp[2][N * SS_ROW];     // q' as bf16 hi, lo; before that the Gram block [k;q].k^T
     alignas(16) uint8_t wz[4][N * W_ROW];      // -sa w hi, lo; z' hi, lo
     alignas(16) uint8_t pk[CF_MD * SS_ROW];
     alignas(16) uint16_t pv[CF_MD * SS_D];
     alignas(16) float couple[CF_MD * 16];
+    alignas(16) float products[PARTS == 1 ? 4 : 8 * 8 * 32];   // the warps' shares of the path's products with the old state
     float4 scal[CF_MD];
     uint32_t mask[N];                          // nodes on the root path
     float g[N], beta[N], sa[N];
     int len, bad;
     float decay;
     static_assert(2 * N * G_ROW * 4 <= 2 * N * SS_ROW, "the Gram block fits q'");
+    static_assert(8 * N / 2 * 32 * 4 <= 2 * N * SS_ROW, "so do the shares of the outputs k and q");
 };
+
+// The sum of what the PARTS warps on the same rows have of an entry (s: the first one's, stride: from one warp to the next).
+template <int PARTS> __device__ __forceinline__ float sum_shares(const float *s, int stride)
+{
+    constexpr int GROUPS = 8 / PARTS;
+    if constexpr (PARTS == 2) return s[0] + s[GROUPS * stride];
+    else return (s[0] + s[GROUPS * stride]) + (s[2 * GROUPS * stride] + s[3 * GROUPS * stride]);
+}
 
 // Acc[nodes] += S.q'^T of one chunk of 32 key positions: hi.hi, lo.hi, hi.lo (lo.lo is below 2^-18 of the result).
 template <int N>
@@ -131,18 +153,58 @@ __device__ __forceinline__ void state_passes(float *S, float (&x)[2][4][4], int 
         }
 }
 
+// The same of one of PARTS CTAs: PARTS warps share 16 rows, each with 4 / PARTS chunks of them (jj and on) that stay in its registers
+// (x).  Of the products with the old state and of those with q' a warp has a share; the first are summed here, by every warp for
+// itself, acc is left as it is.  share: this lane's place in products[], sum: its place in that of the first warp on the same rows.
+template <int N, int TILES, int PARTS>
+__device__ __forceinline__ void state_share(float *S, float (&x)[4 / PARTS][4][4], int jj, int len, uint32_t operand, const PathTile &path, int row,
+                                            int lane, float *share, const float *sum, float A_L, uint32_t q_hi, float (&acc)[N / 8][4], bool nodes)
+{
+    PathUpdate<TILES ? TILES : 1> up;
+    if constexpr (TILES != 0) {
+        PathProducts<TILES> a;
+#pragma unroll
+        for (int i = 0; i < TILES; ++i)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) a.z[i][e] = a.rest[i][e] = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4 / PARTS; ++j) path_products_chunk(x[j], jj + j, operand, a);
+#pragma unroll
+        for (int i = 0; i < TILES; ++i)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) share[(i * 4 + e) * 32] = a.z[i][e] + a.rest[i][e];
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < TILES; ++i)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                a.z[i][e] = sum_shares<PARTS>(sum + (i * 4 + e) * 32, 8 * 32);
+                a.rest[i][e] = 0.f;
+            }
+        path_solve(a, len, path, row, lane, up);
+    }
+#pragma unroll
+    for (int j = 0; j < 4 / PARTS; ++j) {
+        if constexpr (TILES != 0) {
+            path_update_chunk(x[j], jj + j, operand, A_L, up);
+            store_chunk(S, jj + j, x[j]);
+        }
+        if (nodes) output_chunk<N>(x[j], jj + j, q_hi, acc);
+    }
+}
+
 // CTAS: per SM.  PLANNED: the trees come from a plan.
-template <int N, typename TOut, bool COMMIT, int CTAS, bool PLANNED>
+template <int N, typename TOut, bool COMMIT, int CTAS, bool PLANNED, int PARTS>
 __global__ void __launch_bounds__(SS_THREADS, CTAS) verify_step_small_kernel(const StepSmallParams p)
 {
     extern __shared__ __align__(16) uint8_t ss_smem[];
-    using Smem = StepSmallSmem<N>;
+    using Smem = StepSmallSmem<N, PARTS>;
     Smem &sm = *reinterpret_cast<Smem *>(ss_smem);
     const CommitParams &c = p.c;
-    const int unit = blockIdx.x, b = unit / c.h_v, h = unit - b * c.h_v, hk = h / (c.h_v / c.h_qk);
+    const int unit = blockIdx.x / PARTS, part = blockIdx.x % PARTS, b = unit / c.h_v, h = unit - b * c.h_v, hk = h / (c.h_v / c.h_qk);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid < 4)   // L2 may be asked for the tile meanwhile (a prefetch consumes nothing)
-        prefetch_l2_bulk(c.S + (size_t)unit * SS_D * SS_D + (size_t)tid * 4096, 16384);
+    if (tid < 4 / PARTS)   // L2 may be asked for the tile meanwhile (a prefetch consumes nothing)
+        prefetch_l2_bulk(c.S + (size_t)unit * SS_D * SS_D + (size_t)(part * (4 / PARTS) + tid) * 4096, 16384);
     wait_for_previous_kernel();
 
     // the new tree; one with inconsistent node_offsets[] is reported and runs as a tree of no nodes
@@ -194,17 +256,21 @@ __global__ void __launch_bounds__(SS_THREADS, CTAS) verify_step_small_kernel(con
     if (len == 0 && T == 0) return;
 
     // the state first: its latency covers what is fetched and worked out below
-    const int row = warp * 16 + (lane >> 2);
+    // a warp's 16 rows and its chunks (PARTS == 1: all four, two at a time)
+    constexpr int GROUPS = 8 / PARTS, COMPS = SS_D / PARTS, CHUNKS = PARTS == 1 ? 2 : 4 / PARTS;
+    const int rg = PARTS == 1 ? warp : warp % GROUPS, jj = PARTS == 1 ? 0 : warp / GROUPS * CHUNKS;
+    const int comp0 = part * COMPS + rg * 16, row = comp0 + (lane >> 2);
     float *S = c.S + (size_t)unit * SS_D * SS_D + (size_t)row * SS_D + (lane & 3) * 8;
-    float x[2][4][4];
-    load_chunk(S, 0, x[0]);
-    load_chunk(S, 1, x[1]);
+    float x[CHUNKS][4][4];
+#pragma unroll
+    for (int j = 0; j < CHUNKS; ++j) load_chunk(S, jj + j, x[j]);
 
     const uint32_t rows = smem_u32(sm.rows[0]), pk = smem_u32(sm.pk);
     if (T > 0) {
 #pragma unroll
         for (int e = 0; e < 3 * N * 16 / SS_THREADS; ++e) {
             const int idx = tid + e * SS_THREADS, what = idx / (N * 16), i = (idx >> 4) % N, c16 = idx & 15;
+            if (PARTS > 1 && what == 2 && c16 / (16 / PARTS) != part) continue;   // (of v its own components only)
             const bool on = i < T;
             const size_t n = (size_t)(base + (on ? i : 0));
             const __nv_bfloat16 *src = what == 2 ? p.v + (n * c.h_v + h) * SS_D : (what ? p.q : p.k) + (n * c.h_qk + hk) * SS_D;
@@ -404,15 +470,23 @@ __global__ void __launch_bounds__(SS_THREADS, CTAS) verify_step_small_kernel(con
 #pragma unroll
         for (int e = 0; e < 4; ++e) acc[n][e] = 0.f;
     const PathTile path{sm.pv, sm.scal, sm.couple};
-    if (COMMIT && len > 8) state_passes<N, 2>(S, x, len, path_operand(pk, lane), path, row, lane, sm.decay, q_hi, acc, T > 0);
+    if constexpr (PARTS > 1) {
+        const uint32_t operand = path_operand(pk, lane);
+        float *const share = sm.products + warp * 256 + lane;
+        const float *const sum = sm.products + rg * 256 + lane;
+        if (len > 8) state_share<N, 2, PARTS>(S, x, jj, len, operand, path, row, lane, share, sum, sm.decay, q_hi, acc, T > 0);
+        else if (len > 0) state_share<N, 1, PARTS>(S, x, jj, len, operand, path, row, lane, share, sum, sm.decay, q_hi, acc, T > 0);
+        else state_share<N, 0, PARTS>(S, x, jj, 0, 0, path, row, lane, share, sum, 1.f, q_hi, acc, true);
+    } else if (COMMIT && len > 8) state_passes<N, 2>(S, x, len, path_operand(pk, lane), path, row, lane, sm.decay, q_hi, acc, T > 0);
     else if (COMMIT && len > 0) state_passes<N, 1>(S, x, len, path_operand(pk, lane), path, row, lane, sm.decay, q_hi, acc, T > 0);
     else state_passes<N, 0>(S, x, 0, 0, path, row, lane, 1.f, q_hi, acc, true);
     // (5) the v rows' part of the outputs, then a warp's sixteen components of every node through its own piece of shared memory, then 16-byte stores
     if (T > 0) {
-        const uint32_t v_at = rows + 2 * N * SS_ROW + ((lane & 7) + 8 * (lane >> 4)) * SS_ROW + warp * 32 + ((lane >> 3) & 1) * 16;
+        const uint32_t v_at = rows + 2 * N * SS_ROW + ((lane & 7) + 8 * (lane >> 4)) * SS_ROW + comp0 * 2 + ((lane >> 3) & 1) * 16;
         const uint32_t z_at = wz + 2 * N * Smem::W_ROW + ((lane & 7) + 8 * (lane >> 4)) * Smem::W_ROW + ((lane >> 3) & 1) * 16;
 #pragma unroll
         for (int ks = 0; ks < N / 16; ++ks) {
+            if (PARTS > 1 && warp / GROUPS != ks) continue;
             uint32_t a[4], zb[4];
             ldmatrix_x4_trans(v_at + ks * 16 * SS_ROW, a);
 #pragma unroll
@@ -424,49 +498,66 @@ __global__ void __launch_bounds__(SS_THREADS, CTAS) verify_step_small_kernel(con
                     mma_16816(acc[n + 1], a, zb[2], zb[3]);
                 }
         }
-        uint8_t *const stage = sm.rows[0] + warp * (N * 64);
-        constexpr int ROW_BYTES = 16 * (int)sizeof(TOut), PIECES = ROW_BYTES / 16;
-        if constexpr (sizeof(TOut) == 2) {
-            const uint32_t at = smem_u32(stage) + ((lane & 7) + 8 * (lane >> 4)) * ROW_BYTES + ((lane >> 3) & 1) * 16;
-#pragma unroll
-            for (int n = 0; n < N / 8; n += 2)
-                stmatrix_x4_trans(at + n * 8 * ROW_BYTES, pack_bf16(acc[n][0], acc[n][1]), pack_bf16(acc[n][2], acc[n][3]),
-                                  pack_bf16(acc[n + 1][0], acc[n + 1][1]), pack_bf16(acc[n + 1][2], acc[n + 1][3]));
-        } else {
-            float *const st = reinterpret_cast<float *>(stage);   // component c of node i at place c ^ 8 (i / 2 mod 2)
+        if constexpr (PARTS > 1) {   // the warps' shares, summed a component of a node per thread
+            float *const shares = reinterpret_cast<float *>(sm.rows[0]);
+            constexpr int SHARE = N / 2 * 32;   // of a warp
 #pragma unroll
             for (int n = 0; n < N / 8; ++n)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int i = n * 8 + 2 * l4 + (e & 1);
-                    st[i * 16 + ((g8 + 8 * (e >> 1)) ^ (8 * (l4 & 1)))] = acc[n][e];
-                }
-        }
-        __syncwarp();
-        uint8_t *const o = static_cast<uint8_t *>(p.o) + (((size_t)base * c.h_v + h) * SS_D + warp * 16) * sizeof(TOut);
+                for (int e = 0; e < 4; ++e) shares[warp * SHARE + (n * 4 + e) * 32 + lane] = acc[n][e];
+            __syncthreads();
+            TOut *const o = static_cast<TOut *>(p.o) + ((size_t)base * c.h_v + h) * SS_D + part * COMPS;
+            for (int idx = tid; idx < T * COMPS; idx += SS_THREADS) {
+                const int i = idx / COMPS, cc = idx % COMPS;   // held by lane 4 (cc mod 8) + (i mod 8) / 2 of the warps of row group cc / 16
+                const float *s = shares + cc / 16 * SHARE + (i / 8 * 4 + 2 * (cc / 8 % 2) + i % 2) * 32 + cc % 8 * 4 + i % 8 / 2;
+                store_from_float(o + (size_t)i * c.h_v * SS_D + cc, sum_shares<PARTS>(s, SHARE));
+            }
+        } else {
+            uint8_t *const stage = sm.rows[0] + warp * (N * 64);
+            constexpr int ROW_BYTES = 16 * (int)sizeof(TOut), PIECES = ROW_BYTES / 16;
+            if constexpr (sizeof(TOut) == 2) {
+                const uint32_t at = smem_u32(stage) + ((lane & 7) + 8 * (lane >> 4)) * ROW_BYTES + ((lane >> 3) & 1) * 16;
 #pragma unroll
-        for (int e = 0; e < N * PIECES / 32; ++e) {
-            const int i = (e * 32 + lane) / PIECES, piece = (e * 32 + lane) % PIECES;
-            const int at = sizeof(TOut) == 2 ? piece : piece ^ (2 * ((i >> 1) & 1));
-            if (i < T)
-                *reinterpret_cast<uint4 *>(o + (size_t)i * c.h_v * SS_D * sizeof(TOut) + piece * 16) =
-                    *reinterpret_cast<const uint4 *>(stage + i * ROW_BYTES + at * 16);
+                for (int n = 0; n < N / 8; n += 2)
+                    stmatrix_x4_trans(at + n * 8 * ROW_BYTES, pack_bf16(acc[n][0], acc[n][1]), pack_bf16(acc[n][2], acc[n][3]),
+                                      pack_bf16(acc[n + 1][0], acc[n + 1][1]), pack_bf16(acc[n + 1][2], acc[n + 1][3]));
+            } else {
+                float *const st = reinterpret_cast<float *>(stage);   // component c of node i at place c ^ 8 (i / 2 mod 2)
+#pragma unroll
+                for (int n = 0; n < N / 8; ++n)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int i = n * 8 + 2 * l4 + (e & 1);
+                        st[i * 16 + ((g8 + 8 * (e >> 1)) ^ (8 * (l4 & 1)))] = acc[n][e];
+                    }
+            }
+            __syncwarp();
+            uint8_t *const o = static_cast<uint8_t *>(p.o) + (((size_t)base * c.h_v + h) * SS_D + warp * 16) * sizeof(TOut);
+#pragma unroll
+            for (int e = 0; e < N * PIECES / 32; ++e) {
+                const int i = (e * 32 + lane) / PIECES, piece = (e * 32 + lane) % PIECES;
+                const int at = sizeof(TOut) == 2 ? piece : piece ^ (2 * ((i >> 1) & 1));
+                if (i < T)
+                    *reinterpret_cast<uint4 *>(o + (size_t)i * c.h_v * SS_D * sizeof(TOut) + piece * 16) =
+                        *reinterpret_cast<const uint4 *>(stage + i * ROW_BYTES + at * 16);
+            }
         }
     }
 }
 
-template <int N, typename TOut, bool COMMIT, int CTAS, bool PLANNED = false> cudaError_t launch_kernel(const StepSmallParams &p, LaunchInFront commit, cudaStream_t stream)
+template <int N, typename TOut, bool COMMIT, int CTAS, bool PLANNED = false, int PARTS = 1>
+cudaError_t launch_kernel(const StepSmallParams &p, LaunchInFront commit, cudaStream_t stream)
 {
     static PerContext seen;
     int sms = 0;
-    const auto kernel = verify_step_small_kernel<N, TOut, COMMIT, CTAS, PLANNED>;
-    cudaError_t e = device_sms(seen, reinterpret_cast<const void *>(kernel), sizeof(StepSmallSmem<N>), &sms);
+    const auto kernel = verify_step_small_kernel<N, TOut, COMMIT, CTAS, PLANNED, PARTS>;
+    cudaError_t e = device_sms(seen, reinterpret_cast<const void *>(kernel), sizeof(StepSmallSmem<N, PARTS>), &sms);
     if (e == cudaSuccess && commit) e = commit();
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(p.n_seq * p.c.h_v));
+    cfg.gridDim = dim3((unsigned)(p.n_seq * p.c.h_v * PARTS));
     cfg.blockDim = dim3(SS_THREADS);
-    cfg.dynamicSmemBytes = sizeof(StepSmallSmem<N>);
+    cfg.dynamicSmemBytes = sizeof(StepSmallSmem<N, PARTS>);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -480,15 +571,22 @@ template <typename TOut> cudaError_t launch_typed(const StepSmallParams &p, bool
 {
     if (p.plan.unit_list)
         return p.max_tree_nodes > 16 ? launch_kernel<32, TOut, false, 2, true>(p, commit, stream) : launch_kernel<16, TOut, false, 4, true>(p, commit, stream);
-    if (p.max_tree_nodes > 16)
-        return with_commit ? launch_kernel<32, TOut, true, 2>(p, commit, stream) : launch_kernel<32, TOut, false, 2>(p, commit, stream);
-    if (!with_commit) return launch_kernel<16, TOut, false, 4>(p, commit, stream);
+    if (!with_commit)
+        return p.max_tree_nodes > 16 ? launch_kernel<32, TOut, false, 2>(p, commit, stream) : launch_kernel<16, TOut, false, 4>(p, commit, stream);
     static PerContext seen;
     int sms = 0;
     const cudaError_t e = device_sms(seen, nullptr, 0, &sms);
     if (e != cudaSuccess) return e;
-    return commit_at_four(p.max_tree_nodes, (long long)p.n_seq * p.c.h_v, sms) ? launch_kernel<16, TOut, true, 4>(p, commit, stream)
-                                                                               : launch_kernel<16, TOut, true, 3>(p, commit, stream);
+    const long long units = (long long)p.n_seq * p.c.h_v;
+    const int parts = commit_parts(units, sms);
+    if (p.max_tree_nodes > 16)
+        return parts == 4   ? launch_kernel<32, TOut, true, 2, false, 4>(p, commit, stream)
+               : parts == 2 ? launch_kernel<32, TOut, true, 2, false, 2>(p, commit, stream)
+                            : launch_kernel<32, TOut, true, 2>(p, commit, stream);
+    if (parts == 4) return launch_kernel<16, TOut, true, 2, false, 4>(p, commit, stream);
+    if (parts == 2) return launch_kernel<16, TOut, true, 2, false, 2>(p, commit, stream);
+    return commit_at_four(p.max_tree_nodes, units, sms) ? launch_kernel<16, TOut, true, 4>(p, commit, stream)
+                                                        : launch_kernel<16, TOut, true, 3>(p, commit, stream);
 }
 
 }  // namespace

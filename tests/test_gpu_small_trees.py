@@ -97,3 +97,84 @@ def test_planned_verification_of_small_trees(tl, t_pad, sizes, n_layers, out_dty
     d.o.fill_(7.0)
     assert call(torch.zeros_like(plan)) == 0 and d.status_value() == -10
     assert np.all(d.o_host() == 7.0)
+
+
+def _units(limit):
+    """(units, nodes a tree may have) at both sides of the rules of the small-tree kernel, from the number of SMs."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    return {"four parts, 16": (sms // 4, 16), "four parts, 32": (sms // 4, 32), "two parts, first, 16": (sms // 4 + 1, 16),
+            "two parts, last, 16": (sms // 2, 16), "two parts, 32": (sms // 2, 32), "one part, 16": (sms // 2 + 1, 16),
+            "one part, 32": (sms // 2 + 1, 32), "last of 32": (2 * sms, 32), "first beyond 32": (2 * sms + 1, 32),
+            "last at three": (3 * sms, 16), "first at four": (3 * sms + 1, 16), "last at four": (4 * sms, 16),
+            "three again": (4 * sms + 1, 16), "four, 8 nodes": (4 * sms + 1, 8)}[limit]
+
+
+@pytest.mark.parametrize("out_dtype", [synth.BF16, synth.F32])
+@pytest.mark.parametrize("packing", ["ragged", "padded"])
+@pytest.mark.parametrize("limit", ["four parts, 16", "four parts, 32", "two parts, first, 16", "two parts, last, 16", "two parts, 32",
+                                   "one part, 16", "one part, 32", "last of 32", "first beyond 32", "last at three", "first at four",
+                                   "last at four", "three again", "four, 8 nodes"])
+def test_step_on_both_sides_of_every_rule(tl, limit, packing, out_dtype):
+    """One head a slot, so that the units can be counted out; paths of 0, 1, 7, 8, 9 and 16 nodes, trees of all sizes, one of them
+    empty, one with a parent[] that points forward, one path that is not a chain.  The state that the small-tree kernel commits is
+    held to fp32 rounding (see test_commit_is_as_exact_in_every_form)."""
+    import paper_2607_06763_b200 as gdn
+    from oracle import gdn_oracle as orc
+    slots, T = _units(limit)
+    rng = np.random.default_rng(slots + T)
+    lens = [(0, 1, 7, 8, 9, 16)[i % 6] for i in range(slots)]
+    sizes = [T] + [1 + (5 * i) % T for i in range(1, slots)]
+    trees = [synth.tree_geo(rng, n) if n > 1 else np.array([-1], np.int32) for n in sizes]
+    prev_trees = [synth.tree_chain(16)] * slots
+    paths = [np.arange(n, dtype=np.int32) for n in lens]
+    paths_ok = list(paths)
+    paths[5], paths_ok[5] = np.array([0, 2], np.int32), np.zeros(0, np.int32)
+    bad = next(i for i in range(8, slots) if sizes[i] > 2)
+    if packing == "ragged":
+        trees[4] = np.zeros(0, np.int32)
+        prev, prev_ok = (synth.random_case(750, prev_trees, 1, 1, 128, 128, synth.BF16, out_dtype, paths=p) for p in (paths, paths_ok))
+        new = synth.random_case(751, trees, 1, 1, 128, 128, synth.BF16, out_dtype)
+        dp, dn = tl.DeviceCase(prev), tl.DeviceCase(new)
+        dn.parent[int(new.node_offsets[bad]) + 1] = 2
+        S = dp.S0.clone()
+        rc = gdn.gdn_tree_commit_verify(dn.shape, S, dp.k, dp.v, dp.g, dp.beta, dp.parent, dp.node_offsets, dp.path, dp.path_offsets,
+                                        dn.q, dn.k, dn.v, dn.g, dn.beta, dn.parent, dn.node_offsets, dn.o, dn.ws, dn.ws_bytes, dn.status)
+        S_ref = tl.oracle_commit(prev_ok)
+        o_ref = orc.verify(S_ref, *(new.f64(n) for n in ("q", "k", "v", "g", "beta")), new.parent, new.node_offsets, new.scale)
+        rows = [slice(int(a), int(b)) for a, b in zip(new.node_offsets, new.node_offsets[1:])]
+        untouched, status = 0.0, dn.device_status
+    else:
+        prev, prev_ok = (synth.padded_case(752, prev_trees, 1, 16, True, h_qk=1, h_v=1, paths=p, out_dtype=out_dtype) for p in (paths, paths_ok))
+        new = synth.padded_case(753, trees, 1, T, True, h_qk=1, h_v=1, out_dtype=out_dtype)
+        dp, dn = PaddedDevice(prev), PaddedDevice(new)
+        dn.n_nodes[4] = 0
+        dn.parent[bad, 1] = 2
+        S = dp.S0.clone()
+        rc = gdn.gdn_tree_commit_verify_padded(dn.shape, new.n_trees, True, S, 16, dp.k, dp.v, dp.g_in, dp.beta_in, dp.parent, dp.n_nodes,
+                                               dp.path, dp.path_len, dn.q, dn.k, dn.v, dn.g_in, dn.beta_in, dn.parent, dn.n_nodes,
+                                               dn.o, dn.status)
+        S_ref = _oracle_commit(prev_ok, prev.S0.astype(np.float64))
+        o_ref = _oracle_verify(new, S_ref)
+        rows = [(i, slice(0, 0 if i == 4 else sizes[i])) for i in range(slots)]
+        untouched, status = 7.0, dn.status_value
+    assert rc == 0 and status() in (-7, -9)
+    o, S = dn.o_host(), S.cpu().numpy().astype(np.float64)
+    tl.assert_state_close(S, S_ref, what="state")
+    if limit != "first beyond 32":   # (the kernel of 64-node tiles takes the path step by step, scaled: a rounding of the state each)
+        assert np.linalg.norm(S - S_ref) <= 7.2e-8 * np.linalg.norm(S_ref)
+    assert np.array_equal(S[5], prev.S0[5]) and np.array_equal(S[0], prev.S0[0])
+    # value by value (seven rows at a time: too few for the norm-wise bound on bf16 rounding, a statistical one, which would be asked
+    # of 600 slots one by one), and that bound over all slots
+    err = ref = 0.0
+    for i, r in enumerate(rows):
+        if i == bad:
+            assert np.all(o[r] == untouched)
+        elif i != 4:
+            err, ref = err + ((o[r] - o_ref[r]) ** 2).sum(), ref + (o_ref[r] ** 2).sum()
+            for j in range(0, sizes[i], 7):
+                x, y = o[r][j:j + 7], o_ref[r][j:j + 7]
+                tl.assert_close_per_head(x, y, np.array([0, len(x)]), f"{limit}, {packing}, slot {i}", bf16_out=out_dtype == synth.BF16)
+    assert err <= (tl.TOL_BF16_NORMWISE if out_dtype == synth.BF16 else 2.0 ** -17) ** 2 * ref
+    if packing == "padded":
+        assert all(np.all(o[i, (0 if i in (4, bad) else sizes[i]):] == 7.0) for i in range(slots))

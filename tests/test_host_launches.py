@@ -80,6 +80,12 @@ FUSED = [
     (_fused, _shape(4, 256), A, ["commit_plan_kernel", "verify_plain_kernel"]),
     (_fused, _shape(4, 64, in_dtype=0), A, ["commit_generic_kernel", "verify_generic_small_kernel"]),
     (_fused, _shape(4, 100, d=64), A, ["plan_kernel", "commit_generic_kernel", "verify_generic_kernel"]),
+    # trees of at most 32 nodes: one pass, as long as units or nodes are few
+    (_fused, _shape(1, 16), A, ["verify_step_small_kernel"]),
+    (_fused_padded, _shape(2, 16), A, ["verify_step_small_kernel"]),
+    (_fused, _shape(48, 16), A, ["verify_step_small_kernel"]),
+    (_fused_padded, _shape(4, 32), A, ["verify_step_small_kernel"]),
+    (_fused, _shape(10, 32), A, ["commit_verify_kernel"]),
     # a state off a 32-byte boundary
     (_fused, _shape(1, 64), A + 16, ["commit_generic_kernel", "verify_generic_small_kernel"]),
     (_fused, _shape(48, 256), A + 16, ["plan_kernel", "commit_generic_kernel", "verify_generic_kernel"]),
@@ -102,6 +108,18 @@ def test_fused_call_commits_only_once_the_verification_is_prepared(fake_path, ca
             assert fresh.launches() in (kernels, ["commit_verify_kernel"])
         else:
             assert rc == -6 and not any("commit" in x for x in fresh.launches()), f"call {k} of {n} failed behind the commit"
+
+
+@pytest.mark.parametrize("units,T,form", [(1, 16, (16, 2, 4)), (37, 16, (16, 2, 4)), (38, 16, (16, 2, 2)), (74, 1, (16, 2, 2)), (75, 16, (16, 3, 1)),
+                                          (444, 16, (16, 3, 1)), (445, 16, (16, 4, 1)), (592, 16, (16, 4, 1)), (593, 16, (16, 3, 1)),
+                                          (593, 8, (16, 4, 1)), (37, 17, (32, 2, 4)), (74, 32, (32, 2, 2)), (75, 32, (32, 2, 1)), (296, 32, (32, 2, 1))])
+def test_forms_of_the_step_of_small_trees(fake_path, units, T, form):
+    """On 148 SMs: nodes of a tile, CTAs per SM and CTAs per unit of the kernel that a fused call takes."""
+    fake = Fake(fake_path)
+    s = gdn.GdnShape(units, 1, 1, 128, 128, 1, 1, 16, units * T, T, 0.0883883)
+    assert _fused(fake, s) == 0
+    n, ctas, parts = form
+    assert f"verify_step_small_kernelILi{n}E13__nv_bfloat16Lb1ELi{ctas}ELb0ELi{parts}EE" in fake.lib.fake_log().decode()
 
 
 @pytest.mark.parametrize("call,shape,S,kernels", FUSED, ids=range(len(FUSED)))
