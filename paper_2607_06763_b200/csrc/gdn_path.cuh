@@ -13,14 +13,14 @@ struct CommitParams {
     const void *k, *v, *g, *beta;
     const int32_t *parent, *node_offsets, *path, *path_offsets;
     int32_t *status_dev;
-    // padded layout (tile kernel only; t_pad = 0: ragged packing): slot b keeps its rows at b * t_pad and carries
+    // padded layout (d_k = d_v = 128, bf16 only; t_pad = 0: ragged packing): slot b keeps its rows at b * t_pad and carries
     // tree b % n_trees, whose parent[] row, node count and accepted path are shared by its slots
     int t_pad, n_trees, path_stride, raw_gates;
     const int32_t *n_nodes, *path_len;
 };
 
-// The commit kernels are launched with programmatic stream serialization: a grid may become resident under the tail of
-// the kernel in front of it and waits here before it reads or writes anything; the kernel behind it (a verification that
+// The commit kernels and that of small trees are launched with programmatic stream serialization: a grid may become resident under
+// the tail of the kernel in front of it and waits here before it reads or writes anything; the kernel behind it (a verification that
 // waits for this grid in turn) may be made resident as the last CTAs run.  48 layers of two calls each (121 nodes, 32
 // heads): 994 -> 850 us; verification and commit of 48 slots as two calls: 95.7 -> 92.3 us.
 __device__ __forceinline__ void wait_for_previous_kernel()
@@ -122,6 +122,6 @@ struct SmallTreePlan {
 bool step_small_supported(const gdn_shape_t &s);
 cudaError_t launch_step_small(const gdn_shape_t &s, const CommitParams &prev, bool with_commit, const void *q, const void *k, const void *v,
                               const void *g, const void *beta, const int32_t *parent, const int32_t *node_offsets, int n_trees,
-                              const int32_t *n_nodes, void *o, cudaStream_t stream, LaunchInFront commit = {}, const SmallTreePlan &plan = {});
+                              const int32_t *n_nodes, void *o, cudaStream_t stream, const SmallTreePlan &plan = {});
 
 }  // namespace gdn

@@ -546,13 +546,12 @@ __global__ void __launch_bounds__(SS_THREADS, CTAS) verify_step_small_kernel(con
 }
 
 template <int N, typename TOut, bool COMMIT, int CTAS, bool PLANNED = false, int PARTS = 1>
-cudaError_t launch_kernel(const StepSmallParams &p, LaunchInFront commit, cudaStream_t stream)
+cudaError_t launch_kernel(const StepSmallParams &p, cudaStream_t stream)
 {
     static PerContext seen;
     int sms = 0;
     const auto kernel = verify_step_small_kernel<N, TOut, COMMIT, CTAS, PLANNED, PARTS>;
     cudaError_t e = device_sms(seen, reinterpret_cast<const void *>(kernel), sizeof(StepSmallSmem<N, PARTS>), &sms);
-    if (e == cudaSuccess && commit) e = commit();
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(p.n_seq * p.c.h_v * PARTS));
@@ -567,12 +566,12 @@ cudaError_t launch_kernel(const StepSmallParams &p, LaunchInFront commit, cudaSt
     return cudaLaunchKernelEx(&cfg, kernel, p);
 }
 
-template <typename TOut> cudaError_t launch_typed(const StepSmallParams &p, bool with_commit, LaunchInFront commit, cudaStream_t stream)
+template <typename TOut> cudaError_t launch_typed(const StepSmallParams &p, bool with_commit, cudaStream_t stream)
 {
     if (p.plan.unit_list)
-        return p.max_tree_nodes > 16 ? launch_kernel<32, TOut, false, 2, true>(p, commit, stream) : launch_kernel<16, TOut, false, 4, true>(p, commit, stream);
+        return p.max_tree_nodes > 16 ? launch_kernel<32, TOut, false, 2, true>(p, stream) : launch_kernel<16, TOut, false, 4, true>(p, stream);
     if (!with_commit)
-        return p.max_tree_nodes > 16 ? launch_kernel<32, TOut, false, 2>(p, commit, stream) : launch_kernel<16, TOut, false, 4>(p, commit, stream);
+        return p.max_tree_nodes > 16 ? launch_kernel<32, TOut, false, 2>(p, stream) : launch_kernel<16, TOut, false, 4>(p, stream);
     static PerContext seen;
     int sms = 0;
     const cudaError_t e = device_sms(seen, nullptr, 0, &sms);
@@ -580,13 +579,13 @@ template <typename TOut> cudaError_t launch_typed(const StepSmallParams &p, bool
     const long long units = (long long)p.n_seq * p.c.h_v;
     const int parts = commit_parts(units, sms);
     if (p.max_tree_nodes > 16)
-        return parts == 4   ? launch_kernel<32, TOut, true, 2, false, 4>(p, commit, stream)
-               : parts == 2 ? launch_kernel<32, TOut, true, 2, false, 2>(p, commit, stream)
-                            : launch_kernel<32, TOut, true, 2>(p, commit, stream);
-    if (parts == 4) return launch_kernel<16, TOut, true, 2, false, 4>(p, commit, stream);
-    if (parts == 2) return launch_kernel<16, TOut, true, 2, false, 2>(p, commit, stream);
-    return commit_at_four(p.max_tree_nodes, units, sms) ? launch_kernel<16, TOut, true, 4>(p, commit, stream)
-                                                        : launch_kernel<16, TOut, true, 3>(p, commit, stream);
+        return parts == 4   ? launch_kernel<32, TOut, true, 2, false, 4>(p, stream)
+               : parts == 2 ? launch_kernel<32, TOut, true, 2, false, 2>(p, stream)
+                            : launch_kernel<32, TOut, true, 2>(p, stream);
+    if (parts == 4) return launch_kernel<16, TOut, true, 2, false, 4>(p, stream);
+    if (parts == 2) return launch_kernel<16, TOut, true, 2, false, 2>(p, stream);
+    return commit_at_four(p.max_tree_nodes, units, sms) ? launch_kernel<16, TOut, true, 4>(p, stream)
+                                                        : launch_kernel<16, TOut, true, 3>(p, stream);
 }
 
 }  // namespace
@@ -607,7 +606,7 @@ bool step_small_supported(const gdn_shape_t &s)
 
 cudaError_t launch_step_small(const gdn_shape_t &s, const CommitParams &prev, bool with_commit, const void *q, const void *k, const void *v,
                               const void *g, const void *beta, const int32_t *parent, const int32_t *node_offsets, int n_trees,
-                              const int32_t *n_nodes, void *o, cudaStream_t stream, LaunchInFront commit, const SmallTreePlan &plan)
+                              const int32_t *n_nodes, void *o, cudaStream_t stream, const SmallTreePlan &plan)
 {
     if (s.n_seq == 0 || s.total_nodes == 0) return cudaSuccess;
     StepSmallParams p{};
@@ -619,7 +618,7 @@ cudaError_t launch_step_small(const gdn_shape_t &s, const CommitParams &prev, bo
     p.parent = parent; p.node_offsets = node_offsets; p.o = o;
     p.t_pad = node_offsets ? 0 : s.max_tree_nodes; p.n_trees = n_trees; p.n_nodes = n_nodes;
     p.plan = plan;
-    return s.out_dtype == GDN_BF16 ? launch_typed<__nv_bfloat16>(p, with_commit, commit, stream) : launch_typed<float>(p, with_commit, commit, stream);
+    return s.out_dtype == GDN_BF16 ? launch_typed<__nv_bfloat16>(p, with_commit, stream) : launch_typed<float>(p, with_commit, stream);
 }
 
 }  // namespace gdn

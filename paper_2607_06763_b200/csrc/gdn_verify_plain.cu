@@ -968,9 +968,9 @@ cudaError_t launch_verify_sm100_padded(const gdn_shape_t &s, int n_trees, bool r
                                        cudaStream_t stream, LaunchInFront commit)
 {
     if (s.n_seq == 0 || s.total_nodes == 0) return cudaSuccess;
-    if (step_small_supported(s))
+    if (!commit && step_small_supported(s))
         return launch_step_small(s, state_only(s, S0, raw_gates, status_dev), false, q, k, v, g, beta, parent, nullptr, n_trees, n_nodes, o,
-                                 stream, commit);
+                                 stream);
     VerifyPlainParams p = make_params(s, S0, q, k, v, g, beta, nullptr, o, PlanPtrs{}, status_dev);
     p.parent = parent;
     p.t_pad = s.max_tree_nodes; p.n_trees = n_trees; p.n_nodes = n_nodes; p.raw_gates = raw_gates ? 1 : 0;
@@ -988,7 +988,7 @@ cudaError_t launch_verify_sm100_planned(const gdn_shape_t &s, int n_trees, bool 
     const int capacity = (int)unit_list_capacity(ps), magic = plan_magic(n_trees, s.max_tree_nodes, s.max_depth);
     if (step_small_supported(s))
         return launch_step_small(s, state_only(s, S0, raw_gates, status_dev), false, q, k, v, g, beta, nullptr, nullptr, n_trees, nullptr, o,
-                                 stream, {}, {plan.unit_list, plan.unit_count, plan.anc8, capacity, magic});
+                                 stream, {plan.unit_list, plan.unit_count, plan.anc8, capacity, magic});
     VerifyPlainParams p = make_params(s, S0, q, k, v, g, beta, nullptr, o, plan, status_dev);
     p.t_pad = s.max_tree_nodes; p.n_trees = n_trees; p.raw_gates = raw_gates ? 1 : 0;
     p.unit_capacity = capacity;
@@ -1010,9 +1010,9 @@ cudaError_t launch_verify_sm100(const gdn_shape_t &s, const float *S0, const voi
                                 int32_t *status_dev, cudaStream_t stream, LaunchInFront commit)
 {
     if (s.n_seq == 0 || s.total_nodes == 0) return cudaSuccess;
-    if (step_small_supported(s))
+    if (!commit && step_small_supported(s))
         return launch_step_small(s, state_only(s, S0, false, status_dev), false, q, k, v, g, beta, parent, node_offsets, 1, nullptr, o,
-                                 stream, commit);
+                                 stream);
     VerifyPlainParams p = make_params(s, S0, q, k, v, g, beta, node_offsets, o, plan, status_dev);
     p.parent = parent;
     if (!verify_sm100_single_group(s)) return launch_plain<true>(s, p, commit, stream);
