@@ -214,7 +214,9 @@ __global__ void __launch_bounds__(SS_THREADS, CTAS) verify_step_small_kernel(con
     if (PLANNED) {
         // a tree of at most 64 nodes has one record, anywhere in the list; a rejected or empty one has none
         // (48 layers, commit and planned verification each, a tree of 8 / 16 / 32 nodes: 609 / 625 / 646 us with the kernel of grouped
-        // trees, 489 / 497 / 589 so)
+        // trees, 489 / 497 / 589 so).  The trees' CTAs claimed their places about in their order, so that the search begins at the tree's own
+        // place and goes on to both sides of it, 32 records at a time (1024 trees of 16 nodes, one layer: 545 us from the head of the list on, 471 so;
+        // units in the order of the list, which need no search, find the tile that they had L2 fetch in another unit: 588)
         base = b * p.t_pad;
         T = 0;
         const int n_rec = p.plan.unit_count[0];
@@ -222,8 +224,11 @@ __global__ void __launch_bounds__(SS_THREADS, CTAS) verify_step_small_kernel(con
             if (tid == 0) report_status(c.status_dev, GDN_ERR_WORKSPACE);
             return;
         }
-        for (int r0 = 0; r0 < n_rec; r0 += 32) {
-            const uint4 rec = r0 + lane < n_rec ? p.plan.unit_list[r0 + lane] : make_uint4(0xFFFFFFFFu, 0u, 0u, 0u);
+        const int n_win = (n_rec + 31) >> 5, w0 = min(tree >> 5, n_win - 1);
+        for (int i = 0; i < 2 * n_win; ++i) {   // windows w0, w0 + 1, w0 - 1, w0 + 2, ...
+            const int w = w0 + (i & 1 ? (i + 1) >> 1 : -(i >> 1)), r = w * 32 + lane;
+            if (w < 0 || w >= n_win) continue;
+            const uint4 rec = r < n_rec ? p.plan.unit_list[r] : make_uint4(0xFFFFFFFFu, 0u, 0u, 0u);
             const uint32_t found = __ballot_sync(0xffffffffu, rec.x == (uint32_t)tree);
             if (found) {
                 T = (int)((__shfl_sync(0xffffffffu, rec.z, __ffs(found) - 1) >> 16) & 0xFFu);

@@ -178,3 +178,33 @@ def test_step_on_both_sides_of_every_rule(tl, limit, packing, out_dtype):
     assert err <= (tl.TOL_BF16_NORMWISE if out_dtype == synth.BF16 else 2.0 ** -17) ** 2 * ref
     if packing == "padded":
         assert all(np.all(o[i, (0 if i in (4, bad) else sizes[i]):] == 7.0) for i in range(slots))
+
+
+@pytest.mark.parametrize("t_pad", [5, 16])
+def test_planned_verification_of_many_small_trees(tl, t_pad):
+    """300 trees in each of two layers, some empty, some rejected when the plan is built: the records of the others stand in the list
+    in any order, and every slot finds its own tree."""
+    import paper_2607_06763_b200 as gdn
+    from tests.test_gpu_padded import _plan
+    rng = np.random.default_rng(t_pad)
+    sizes = rng.integers(1, t_pad + 1, size=300)
+    w = synth.padded_case(760 + t_pad, [synth.tree_geo(rng, int(n)) if n > 1 else np.array([-1], np.int32) for n in sizes], 2, t_pad, False, h_qk=1, h_v=2)
+    d = PaddedDevice(w)
+    empty, bad = {0, 31, 32, 150, 299}, {1, 33, 298} | {int(i) for i in range(0, 300, 37)}
+    bad = {i for i in bad - empty if sizes[i] > 2}
+    for i in empty:
+        d.n_nodes[i] = 0
+    for i in bad:
+        d.parent[i, 1] = 2
+    plan = _plan(d, w)
+    assert d.status_value() == -7
+    d.status.zero_()
+    assert gdn.gdn_tree_verify_planned(d.shape, w.n_trees, False, d.S0, d.q, d.k, d.v, d.g_in, d.beta_in, plan, d.o, d.status) == 0
+    assert d.status_value() == 0
+    o, ref = d.o_host(), _oracle_verify(w)
+    for s in range(w.n_slots):
+        t = s % 300
+        n = 0 if t in empty | bad else int(sizes[t])
+        assert np.all(o[s, n:] == 7.0)
+        for j in range(0, n, 7):   # (see above)
+            tl.assert_close_per_head(o[s, j:min(n, j + 7)], ref[s, j:min(n, j + 7)], np.array([0, min(n, j + 7) - j]), f"slot {s}", bf16_out=True)
