@@ -107,12 +107,25 @@ def test_commit_verify_padded(tl, raw_gates):
 
 @pytest.mark.parametrize("n_trees,rejected", [(1, None), (1, 0), (2, None), (2, 1)])
 def test_commit_verify_padded_shares_tables_between_units(tl, n_trees, rejected):
-    """640 units, several per CTA, whose trees repeat or alternate; a rejected tree is reported, nothing of its slots is
+    """640 units whose trees repeat or alternate; a rejected tree is reported, nothing of its slots is
     stored, and their accepted paths are committed all the same."""
+    _shared_tables(tl, n_trees, rejected, 16, (13, 16), synth.BF16)
+
+
+@pytest.mark.parametrize("out_dtype", [synth.BF16, synth.F32])
+@pytest.mark.parametrize("t_pad,sizes", [(64, (50, 64)), (32, (32, 19))])
+@pytest.mark.parametrize("n_trees,rejected", [(1, None), (1, 0), (2, None), (2, 1)])
+def test_commit_verify_padded_carries_tables_from_unit_to_unit(tl, n_trees, rejected, t_pad, sizes, out_dtype):
+    """The same on the kernel of 64-node tiles, whose CTAs take several units in a row and keep a tree's tables and verdict
+    where the next unit has the same tree (trees of up to 64 nodes, and its form for up to 32)."""
+    _shared_tables(tl, n_trees, rejected, t_pad, sizes, out_dtype)
+
+
+def _shared_tables(tl, n_trees, rejected, t_pad, sizes, out_dtype):
     import paper_2607_06763_b200 as gdn
     rng = np.random.default_rng(805)
     prev = synth.padded_case(830, _trees(rng, (16, 9)[:n_trees]), 20 // n_trees, 16, False, h_qk=16, h_v=32)
-    new = synth.padded_case(831, _trees(rng, (13, 16)[:n_trees]), 20 // n_trees, 16, False, h_qk=16, h_v=32)
+    new = synth.padded_case(831, _trees(rng, sizes[:n_trees]), 20 // n_trees, t_pad, False, h_qk=16, h_v=32, out_dtype=out_dtype)
     dp, dn = PaddedDevice(prev), PaddedDevice(new)
     if rejected is not None:
         dn.parent[rejected, 5] = 9
@@ -128,7 +141,7 @@ def test_commit_verify_padded_shares_tables_between_units(tl, n_trees, rejected)
         t = s % n_trees
         n = 0 if t == rejected else int(new.n_nodes[t])
         if n:
-            tl.assert_close_per_head(o[s, :n], ref[s, :n], np.array([0, n]), f"slot {s}", bf16_out=True)
+            tl.assert_close_per_head(o[s, :n], ref[s, :n], np.array([0, n]), f"slot {s}", bf16_out=out_dtype == synth.BF16)
         assert np.all(o[s, n:] == 7.0)
 
 

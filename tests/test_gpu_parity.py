@@ -545,6 +545,17 @@ def test_fused_commit_with_extreme_decay_takes_the_plain_replay(tl):
     _fused_case(tl, prev, new, "fused extreme decay")
 
 
+def test_fused_commit_with_extreme_decay_on_large_tiles(tl):
+    """The same on the kernel of 64-node tiles (new trees of more than 32 nodes, 120 units): the scaled replay would divide by
+    1e-47, so that the plain form has to take over."""
+    paths = [np.arange(12 if i % 2 else 5, dtype=np.int32) for i in range(30)]
+    prev = synth.random_case(43, [synth.tree_chain(12)] * 30, 2, 4, 128, 128, synth.BF16, synth.F32, paths=paths, name="prev")
+    prev.g = synth.store(np.full(prev.g.shape, -9.0, np.float32), synth.BF16)
+    rng = np.random.default_rng(44)
+    new = synth.random_case(45, [synth.tree_geo(rng, 33 + i) for i in range(30)], 2, 4, 128, 128, synth.BF16, synth.F32)
+    _fused_case(tl, prev, new, "fused extreme decay, large tiles")
+
+
 def test_rows_of_a_neighbouring_tree_never_leak(tl):
     """The tensor-core path stages 64-row boxes, so a short tree's tile also holds rows of the next tree.  Poison
     that neighbour with NaNs: the short tree's outputs and committed state must be unaffected."""
@@ -562,6 +573,35 @@ def test_rows_of_a_neighbouring_tree_never_leak(tl):
     tl.assert_close_per_head(o[:10], clean[:10], np.array([0, 10]), "short tree next to a poisoned one")
     assert dc.commit() == 0 and dc.device_status() == 0
     assert bool(torch_isfinite(dc.S0[0]))
+
+
+@pytest.mark.parametrize("kind,slots", [("verify", 2), ("verify", 30), ("fused", 2), ("fused", 30)])
+def test_rows_of_a_neighbouring_tree_never_leak_into_a_tile(tl, kind, slots):
+    """The same with trees of 33 to 62 nodes, which the kernels of 64-node tiles take: every other tree holds NaNs, in its rows and
+    (its accepted path) in those of the step before.  2 slots of 4 heads are a commit and a verification, 30 one kernel."""
+    import paper_2607_06763_b200 as gdn
+    rng = np.random.default_rng(62)
+    new = synth.random_case(63, [synth.tree_geo(rng, 33 + i) for i in range(slots)], 2, 4, 128, 128, synth.BF16, synth.F32)
+    prev = synth.random_case(64, [synth.tree_chain(10)] * slots, 2, 4, 128, 128, synth.BF16, synth.F32,
+                             paths=[np.arange(4 if i % 2 == 0 else 0, dtype=np.int32) for i in range(slots)])
+    S_ref = tl.oracle_commit(prev) if kind == "fused" else new.f64("S0")
+    clean = tl.oracle_verify(dataclass_replace_S0(new, S_ref))
+    for w in (prev, new):
+        for b in range(1, slots, 2):
+            for name in ("q", "k", "v", "g", "beta"):
+                getattr(w, name)[w.node_offsets[b]:w.node_offsets[b + 1]] = np.uint16(0x7FC0)
+    dp, dn = tl.DeviceCase(prev), tl.DeviceCase(new)
+    if kind == "verify":
+        assert dn.verify() == 0
+    else:
+        assert gdn.gdn_tree_commit_verify(dn.shape, dp.S0, dp.k, dp.v, dp.g, dp.beta, dp.parent, dp.node_offsets, dp.path, dp.path_offsets,
+                                          dn.q, dn.k, dn.v, dn.g, dn.beta, dn.parent, dn.node_offsets, dn.o, dn.ws, dn.ws_bytes, dn.status) == 0
+        tl.assert_state_close(dp.S0.cpu().numpy().astype(np.float64), S_ref, what="state")
+    assert dn.device_status() == 0
+    o = dn.o_host()
+    for b in range(0, slots, 2):
+        r = slice(int(new.node_offsets[b]), int(new.node_offsets[b + 1]))
+        tl.assert_close_per_head(o[r], clean[r], np.array([0, len(o[r])]), f"tree {b} next to a poisoned one")
 
 
 def torch_isfinite(t):
@@ -789,7 +829,8 @@ def test_commit_behind_a_strong_decay(tl, slots, g_strong, at):
 @pytest.mark.parametrize("at", [0, 2])
 @pytest.mark.parametrize("g_strong", [-3000.0, -30000.0, -np.inf])
 @pytest.mark.parametrize("kind,slots,T", [("verify", 2, 60), ("verify", 2, 200), ("fused", 2, 60), ("fused", 20, 60),
-                                          ("fused", 2, 200)])
+                                          ("fused", 2, 200), ("verify", 2, 16), ("verify", 2, 32), ("fused", 2, 16), ("fused", 20, 16),
+                                          ("fused", 2, 32), ("fused", 20, 32)])
 def test_verify_behind_a_strong_decay(tl, kind, slots, T, g_strong, at):
     """The same for the verification, alone and fused, of trees within one tile and of larger ones: node `at` of every tree
     has the strong decay, and the outputs of the nodes below it keep their precision."""
@@ -811,7 +852,8 @@ def test_verify_behind_a_strong_decay(tl, kind, slots, T, g_strong, at):
 
 
 @pytest.mark.parametrize("b", [2, 8, 128])
-@pytest.mark.parametrize("kind,slots,T", [("verify", 2, 60), ("verify", 2, 200), ("fused", 20, 60)])
+@pytest.mark.parametrize("kind,slots,T", [("verify", 2, 60), ("verify", 2, 200), ("fused", 20, 60), ("verify", 2, 16), ("verify", 2, 32),
+                                          ("fused", 2, 16), ("fused", 20, 16), ("fused", 2, 32), ("fused", 20, 32)])
 def test_verify_with_keys_of_any_length(tl, kind, slots, T, b):
     """Keys that are not normalised: beta |k|^2 = b at every node, nearly parallel, under decays of 1 / (b - 1), so that the state
     neither grows nor vanishes down a path.  The verification solves without the decays, where a weight grows up to (b - 1)^15
@@ -881,7 +923,8 @@ def test_fused_step_on_both_sides_of_the_two_kernel_rule(tl, side):
             tl.assert_close_per_head(o.cpu().numpy().astype(np.float64), o_ref, w.node_offsets, f"fused, {slots} slots, o")
 
 
-@pytest.mark.parametrize("in_dtype,sizes", [(synth.F32, (40, 9, 64)), (synth.BF16, (300, 20)), (synth.BF16, (40, 9, 64))])
+@pytest.mark.parametrize("in_dtype,sizes", [(synth.F32, (40, 9, 64)), (synth.BF16, (300, 20)), (synth.BF16, (40, 9, 64)),
+                                            (synth.BF16, (16, 5, 9)), (synth.BF16, (32, 7))])
 def test_verify_and_commit_in_turn_without_a_wait(tl, in_dtype, sizes):
     """Kernels of this library move in while the one in front still runs, here with the state, the trees and the workspace
     that the ones before have just read: every verification has to see what is written in between."""
@@ -912,7 +955,7 @@ def test_verify_and_commit_in_turn_without_a_wait(tl, in_dtype, sizes):
         tl.assert_state_close(S1.cpu().numpy().astype(np.float64), S, what=f"state behind pass {i}")
 
 
-@pytest.mark.parametrize("sizes", [(64, 1, 33), (20, 130), (64,) * 19, (300,)])
+@pytest.mark.parametrize("sizes", [(64, 1, 33), (20, 130), (64,) * 19, (300,), (16, 3), (32, 9)])
 def test_state_off_a_32_byte_boundary(tl, sizes):
     """A state at 16 mod 32 bytes, which the ragged entry points accept: verification, commit and fused call on the general
     kernels, against the oracle.  The words around the state stay as they are."""
