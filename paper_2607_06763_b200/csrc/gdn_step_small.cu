@@ -54,12 +54,20 @@ inline bool commit_at_four(int max_tree_nodes, long long units, int sms)
 // components each, every warp on the key positions of one or two chunks of its rows, which then stay in its registers.  With the whole
 // tile on one CTA the passes over it are 5300 of a unit's 11300 cycles (path of 1; 7500 behind one of 16), and its second half and both
 // halves once more are waited for; the coefficients, which every CTA makes for itself, are done in less time than the rows take to
-// come.  Calls back to back in a CUDA graph, us, commit and 64-node verification as two kernels / one CTA a unit / split, 32 heads,
-// paths of 1 / 8 / 9 / 16 nodes: one sequence of 16 nodes (four parts) 8.3 8.3 8.3 9.5 / 7.9 8.7 10.2 10.6 / 5.4 6.1 6.9 7.3, of 32 nodes
-// 8.5 8.5 8.5 9.6 / 9.4 9.8 10.8 11.2 / 7.6 7.9 8.7 9.1; two sequences (two parts) 8.6 9.3 9.9 11.9 / 8.0 8.8 10.3 10.8 / 6.3 6.9 7.6 8.1
-// and 9.0 9.4 10.0 11.9 / 9.7 10.1 11.0 11.4 / 9.2 9.5 10.3 10.7 (four parts, two CTAs on most SMs: 6.7 7.5 8.6 9.2 and 9.9 10.6 11.8 12.3).
-// Three sequences in two parts, two on some SMs: 16 nodes 7.9 8.9 9.8 10.4 instead of 8.0 8.8 10.4 10.8, 32 nodes 12.2 12.9 14.2 14.4 instead of
-// 9.7 10.1 11.1 11.5.
+// come.  Calls in a row, us, paths of 1 / 8 / 9 / 16 nodes, 32 heads ("two kernels": commit, then the verification of 64-node tiles):
+//                                                   two kernels             one CTA a unit         four or two parts
+//   in a graph, in L2:      1 sequence, 16 nodes     8.3  8.3  8.3  9.5      7.9  8.7 10.2 10.6     5.4  6.1  6.9  7.3
+//                           1 sequence, 32 nodes     8.5  8.5  8.5  9.6      9.4  9.8 10.8 11.2     7.6  7.9  8.7  9.1
+//                           2 sequences, 16 nodes    8.6  9.3  9.9 11.9      8.0  8.8 10.3 10.8     6.3  6.9  7.6  8.1   (four: 6.7  7.5  8.6  9.2)
+//                           2 sequences, 32 nodes    9.0  9.4 10.0 11.9      9.7 10.1 11.0 11.4     9.2  9.5 10.3 10.7   (four: 9.9 10.6 11.8 12.3)
+//   in a graph, not in L2:  1 sequence, 16 nodes     9.0  9.0  9.6 11.0      9.3 10.2 12.0 12.4     7.0  7.7  8.7  9.1
+//                           1 sequence, 32 nodes     9.3  9.3  9.7 11.1     10.9 11.3 12.6 13.0     9.1  9.5 10.5 10.9
+//                           2 sequences, 16 nodes    9.2 10.6 11.4 13.5      9.7 10.6 12.3 12.8     8.1  8.7  9.8 10.2
+//                           2 sequences, 32 nodes    9.5 10.6 11.5 13.5     11.4 11.8 13.0 13.4    10.9 11.2 12.2 12.7
+//   by the host, not in L2: 2 sequences, 32 nodes   11.5 11.6 12.3 14.4     11.8 12.2 13.4 13.9    11.4 11.7 12.7 13.3
+// (Two kernels stay faster for two sequences of 32 nodes and short paths in a graph; their commit goes step by step for so few tiles,
+// which leaves the state up to 1.6e-7 off in the norm with raw gates, this one below 7e-8.)  Three sequences in two parts, two on some
+// SMs: 16 nodes 7.9 8.9 9.8 10.4 instead of 8.0 8.8 10.4 10.8, 32 nodes 12.2 12.9 14.2 14.4 instead of 9.7 10.1 11.1 11.5.
 inline int commit_parts(long long units, int sms) { return units <= sms / 4 ? 4 : units <= sms / 2 ? 2 : 1; }
 
 // N: nodes a tree may have here (16 or 32).
@@ -596,7 +604,7 @@ template <typename TOut> cudaError_t launch_typed(const StepSmallParams &p, bool
 }  // namespace
 
 // Trees of at most 16 nodes, always; of up to 32 only while all units are resident at once.  Measured (us; the kernels of 64-node
-// tiles / this one), trees of 32 nodes, 32 heads, path of 7 and verification alone: 1 tree 11.1 / 10.4 and 8.4 / 7.9, 4 trees 13.7 / 10.8
+// tiles / this one), trees of 32 nodes, 32 heads, path of 7 and verification alone: 1 tree 11.1 / 8.5 and 8.4 / 7.9, 4 trees 13.7 / 10.8
 // and 8.4 / 7.8, 8 trees 18.8 / 14.9 and 10.6 / 9.8, 9 trees 19.6 / 15.5 and 11.0 / 10.0; beyond that the 64-node tiles share the
 // coefficients of a key head's value heads: 12 trees 32.2 / 26.3 and 15.5 / 15.7, 16 trees 32.3 / 31.4 and 16.3 / 18.8, 48 trees 74.7 / 78.3
 // and 35.6 / 47.5.
