@@ -29,6 +29,7 @@ constexpr int SS_ROW = GDN_PK_STRIDE;   // bytes from one row of an operand to t
 struct StepSmallParams {
     CommitParams c;   // the previous step (COMMIT); c.S: the state, of either form
     int n_seq, total_nodes, max_tree_nodes;
+    int rows_early;   // L2 is asked for the rows before the kernel in front has completed
     float scale;
     const __nv_bfloat16 *q, *k, *v, *g, *beta;
     const int32_t *parent, *node_offsets;
@@ -60,10 +61,10 @@ inline bool commit_at_four(int max_tree_nodes, long long units, int sms)
 //                           1 sequence, 32 nodes     8.5  8.5  8.5  9.6      9.4  9.8 10.8 11.2     7.6  7.9  8.7  9.1
 //                           2 sequences, 16 nodes    8.6  9.3  9.9 11.9      8.0  8.8 10.3 10.8     6.3  6.9  7.6  8.1   (four: 6.7  7.5  8.6  9.2)
 //                           2 sequences, 32 nodes    9.0  9.4 10.0 11.9      9.7 10.1 11.0 11.4     9.2  9.5 10.3 10.7   (four: 9.9 10.6 11.8 12.3)
-//   in a graph, not in L2:  1 sequence, 16 nodes     9.0  9.0  9.6 11.0      9.3 10.2 12.0 12.4     7.0  7.7  8.7  9.1
-//                           1 sequence, 32 nodes     9.3  9.3  9.7 11.1     10.9 11.3 12.6 13.0     9.1  9.5 10.5 10.9
-//                           2 sequences, 16 nodes    9.2 10.6 11.4 13.5      9.7 10.6 12.3 12.8     8.1  8.7  9.8 10.2
-//                           2 sequences, 32 nodes    9.5 10.6 11.5 13.5     11.4 11.8 13.0 13.4    10.9 11.2 12.2 12.7
+//   in a graph, not in L2:  1 sequence, 16 nodes     9.0  9.0  9.6 11.0      9.3 10.2 12.0 12.4     6.5  7.3  8.4  8.7
+//                           1 sequence, 32 nodes     9.3  9.3  9.7 11.1     10.9 11.3 12.6 13.0     8.5  8.9 10.0 10.4
+//                           2 sequences, 16 nodes    9.2 10.6 11.4 13.5      9.7 10.6 12.3 12.8     7.7  8.4  9.4  9.8
+//                           2 sequences, 32 nodes    9.5 10.6 11.5 13.5     11.4 11.8 13.0 13.4    10.4 10.7 11.7 12.2
 //   by the host, not in L2: 2 sequences, 32 nodes   11.5 11.6 12.3 14.4     11.8 12.2 13.4 13.9    11.4 11.7 12.7 13.3
 // (Two kernels stay faster for two sequences of 32 nodes and short paths in a graph; their commit goes step by step for so few tiles,
 // which leaves the state up to 1.6e-7 off in the norm with raw gates, this one below 7e-8.)  Three sequences in two parts, two on some
@@ -213,6 +214,21 @@ __global__ void __launch_bounds__(SS_THREADS, CTAS) verify_step_small_kernel(con
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid < 4 / PARTS)   // L2 may be asked for the tile meanwhile (a prefetch consumes nothing)
         prefetch_l2_bulk(c.S + (size_t)unit * SS_D * SS_D + (size_t)(part * (4 / PARTS) + tid) * 4096, 16384);
+    if ((!COMMIT || CTAS <= 2) && p.rows_early && tid >= SS_THREADS - N && tid - (SS_THREADS - N) < p.max_tree_nodes) {
+        // ... and for the rows; node_offsets[] only steers here: clamped to the tensors, and by way
+        // of L2, so that nothing stays in L1 for the read that counts.  Over buffers that L2 does not hold (us, in a graph, 64-node kernels
+        // / without / with): verification of 1 / 4 / 6 trees of 32 nodes 6.6 7.3 9.6 / 6.8 7.9 10.1 / 6.1 6.8 9.3, of 16 nodes 6.4 7.0 8.4 /
+        // 5.3 6.2 7.8 / 4.7 5.2 6.5; planned layer of one tree of 32 nodes, commit included, 12.8 / 13.5 / 13.2.  (A commit at three or four
+        // CTAs per SM: 12 trees of 16 nodes, path of 8, 18.1 without, 18.5 with.)
+        const int row = (p.t_pad ? b * p.t_pad : __ldcg(p.node_offsets + b)) + tid - (SS_THREADS - N);
+        if (row >= 0 && row < p.total_nodes) {
+            prefetch_l2_bulk(p.k + ((size_t)row * c.h_qk + hk) * SS_D, 256);
+            prefetch_l2_bulk(p.q + ((size_t)row * c.h_qk + hk) * SS_D, 256);
+            prefetch_l2_bulk(p.v + ((size_t)row * c.h_v + h) * SS_D, 256);
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(p.g + (size_t)row * c.h_v + h));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(p.beta + (size_t)row * c.h_v + h));
+        }
+    }
     wait_for_previous_kernel();
 
     // the new tree; one with inconsistent node_offsets[] is reported and runs as a tree of no nodes
@@ -559,7 +575,7 @@ __global__ void __launch_bounds__(SS_THREADS, CTAS) verify_step_small_kernel(con
 }
 
 template <int N, typename TOut, bool COMMIT, int CTAS, bool PLANNED = false, int PARTS = 1>
-cudaError_t launch_kernel(const StepSmallParams &p, cudaStream_t stream)
+cudaError_t launch_kernel(StepSmallParams p, cudaStream_t stream)
 {
     static PerContext seen;
     int sms = 0;
@@ -568,6 +584,8 @@ cudaError_t launch_kernel(const StepSmallParams &p, cudaStream_t stream)
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(p.n_seq * p.c.h_v * PARTS));
+    // (up to three quarters of what is resident at once: 9 trees of 32 nodes take 10.7 us without and 10.2 with, but 9.4 and 9.6 out of L2)
+    p.rows_early = cfg.gridDim.x <= (unsigned)(CTAS * sms * 3 / 4);
     cfg.blockDim = dim3(SS_THREADS);
     cfg.dynamicSmemBytes = sizeof(StepSmallSmem<N, PARTS>);
     cfg.stream = stream;
