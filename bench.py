@@ -37,7 +37,7 @@ UNIT = "nodes/s"
 CONFIG_WORKLOADS = {"stack48_T64": 5, "layer_T64": 1, "stack48_T256": 2, "ragged32": 3, "chains64x16": 4}
 SWEEP_T = (32, 64, 128, 256, 512)
 WORKLOADS = sorted(CONFIG_WORKLOADS) + [f"sweep_T{t}" for t in SWEEP_T] + ["stack48_T64_deep", "stack48_T64_bestfirst"]
-DTYPE = "bf16 inputs/outputs, fp32 state; contractions as bf16 hi+lo splits on tcgen05 with fp32 accumulation"
+DTYPE = "bf16 inputs/outputs, fp32 state; contractions as bf16 hi+lo splits on tcgen05 (trees of at most 16 nodes, 32 for few units: mma.sync) with fp32 accumulation"
 
 
 def make_workload(args) -> synth.Workload:
